@@ -38,9 +38,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 // Bounded wait.  `dead` points to the CTA's latch in shared memory (0 at kernel start).  Returns false when the wait
 // gave up: because this one ran out of time (the latch and the status word are then set), or because the latch was
-// already set by an earlier one.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status, volatile int* dead,
-                                          unsigned long long limit_ns = WAIT_LIMIT_NS) {
+// already set by an earlier one.  The polling loop is out of line: a barrier that is complete already -- most are, in a
+// pipeline that keeps up -- costs one try_wait (13 cycles on a B200); with the loop and the latch check inlined ahead of
+// it the same wait took 150 cycles, and 370 in the one-lane form of mbar_wait_warp.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int* status, volatile int* dead,
+                                            unsigned long long limit_ns) {
     if (*dead) return false;
     // a healthy wait ends within these polls; the timer is consulted only after them
 #pragma unroll 1
@@ -60,10 +62,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     if (status) atomicExch(status, STATUS_TIMEOUT);
     return false;
 }
-// The same for a whole (converged) warp: one lane polls, so that 31 lanes do not spend shared-memory cycles on it.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status, volatile int* dead,
+                                          unsigned long long limit_ns = WAIT_LIMIT_NS) {
+    return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, status, dead, limit_ns);
+}
+// The same for a whole (converged) warp: one answer for all lanes; past the first try one lane polls, so that 31 lanes do
+// not spend shared-memory cycles on it.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status, volatile int* dead) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
     int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, status, dead);
+    if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow(bar, parity, status, dead, WAIT_LIMIT_NS);
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 // Last wait of a CTA that is giving up: waits (bounded, whatever the latch says) for a copy or MMA group still in
