@@ -26,6 +26,30 @@ inline bool use_tc(int32_t dtype, int32_t dk, int32_t dv, uint32_t flags) {
     return !(flags & HARTS_FLAG_FMA_KERNELS) && harts::tc_supported(dtype, dk, dv);
 }
 
+// Chunk-parallel path over sequences [range[0], range[n]), range[r]..range[r+1] per round: the scan, then all chunks at once.
+harts::RoundOrder round_order(const int32_t* range, int32_t n) {
+    harts::RoundOrder ro;
+    ro.n = n > 1 ? n : 0;
+    for (int32_t r = 0; r <= n; r++) ro.ptr[r] = range[r];
+    return ro;
+}
+int32_t chunk_parallel_fwd(harts::FwdArgs a, const int32_t* range, int32_t n) {
+    a.seq_lo = range[0];
+    a.seq_hi = range[n];
+    int* flags = reinterpret_cast<int*>(static_cast<char*>(a.chunk_states) + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::scan_fwd(a, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::chunk_fwd(a);
+}
+int32_t chunk_parallel_bwd(harts::BwdArgs a, const int32_t* range, int32_t n) {
+    a.seq_lo = range[0];
+    a.seq_hi = range[n];
+    char* ws = const_cast<char*>(static_cast<const char*>(a.chunk_states));
+    void* ds = ws + harts::ds_tiles_offset(a.tb, a.H, a.dk, a.dv);
+    int* flags = reinterpret_cast<int*>(ws + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::scan_bwd(a, ds, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::chunk_bwd(a, ds);
+}
+
 }  // namespace
 
 extern "C" {
@@ -53,12 +77,15 @@ int32_t harts_la_plan_upload(const harts_la_plan_t* plan, void* dev_blob, void* 
 }
 
 int32_t harts_la_workspace_bytes(const harts_la_tables_t* tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype,
-                                 uint32_t /*flags*/, size_t* chunk_state_bytes, size_t* scratch_bytes) {
+                                 uint32_t flags, size_t* chunk_state_bytes, size_t* scratch_bytes) {
     if (!tb || H < 1 || dk < 1 || dv < 1) return HARTS_EINVAL;
     if (dtype != HARTS_FP32 && dtype != HARTS_BF16) return HARTS_EUNSUPPORTED;
     size_t elem = dtype == HARTS_FP32 ? 4 : 2;
-    if (chunk_state_bytes)      // the states, then the flags of the one-launch forms
+    (void)flags;
+    if (chunk_state_bytes) {    // the states, then the flags of the one-launch forms, then what the chunk-parallel path adds
         *chunk_state_bytes = harts::chunk_state_payload(*tb, H, dk, dv, elem) + harts::fused_flag_bytes(*tb, H);
+        if (harts::chunk_parallel(*tb, H, dk, dv, dtype, 0)) *chunk_state_bytes = harts::chunk_parallel_bytes(*tb, H, dk, dv);
+    }
     if (scratch_bytes) *scratch_bytes = harts::scratch_layout(*tb, H, dk, dv).total;
     return HARTS_OK;
 }
@@ -76,6 +103,10 @@ int32_t harts_la_fwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
                      static_cast<cudaStream_t>(stream)};
     if (flags & HARTS_FLAG_CHECK_TABLES)
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
+    if (chunk_states && harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) {
+        const int32_t range[2] = {seq_lo, seq_hi};
+        return chunk_parallel_fwd(a, range, 1);
+    }
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_fwd(a);
     return harts::fma_fwd(a);
 }
@@ -94,6 +125,10 @@ int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
                      flags, dev_status, static_cast<cudaStream_t>(stream)};
     if (flags & HARTS_FLAG_CHECK_TABLES)
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
+    if (harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) {
+        const int32_t range[2] = {seq_lo, seq_hi};
+        return chunk_parallel_bwd(a, range, 1);
+    }
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_bwd(a);
     return harts::fma_bwd(a);
 }
@@ -132,6 +167,8 @@ int32_t harts_la_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
             if (!dev_status) return HARTS_EINVAL;
             if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
         }
+        if (harts::chunk_parallel(tb, H, dk, dv, dtype, flags))
+            return chunk_parallel_fwd(a, p->round_seq_ptr.data(), p->n_rounds);
         int* fl = reinterpret_cast<int*>(static_cast<char*>(chunk_states) + harts::chunk_state_payload(tb, H, dk, dv, 2));
         rc = harts::tc_fwd_fused(a, fl, fl + harts::fused_flag_count(tb, H));
         if (rc != HARTS_EUNSUPPORTED) return rc;         // else: not all CTAs can be resident, launch round by round
@@ -168,6 +205,10 @@ int32_t harts_la_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
         if (flags & HARTS_FLAG_CHECK_TABLES) {
             if (!dev_status) return HARTS_EINVAL;
             if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
+        }
+        if (harts::chunk_parallel(tb, H, dk, dv, dtype, flags)) {
+            if ((rc = chunk_parallel_bwd(a, p->round_seq_ptr.data(), p->n_rounds)) != HARTS_OK) return rc;
+            return harts_la_bwd_finish(&tb, dk_, dv_, dg, scratch, H, dk, dv, dtype, stream);
         }
         // the flags sit behind the chunk states; the backward's come after the forward's (n_slots * H), the two
         // ticket counters after both

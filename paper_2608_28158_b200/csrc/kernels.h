@@ -135,6 +135,35 @@ struct RoundOrder {
     int n;
     int ptr[MAX_FUSED_ROUNDS + 1];
 };
+// Chunk-parallel path (bf16, d_k = d_v = 128): a scan leaves the state of every chunk boundary (backward: its gradient) in
+// memory, then every (chunk, head) is a work item of its own.
+int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      // la_scan.cu: states, exported slots
+int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
+int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
+int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles);     // la_chunk_bwd.cu
+// Taken up to 28,672 (chunk, head) items.  The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 400 KB:
+// with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.6 against 11.2 ms a step; 2,389 x 16: 3.0
+// against 3.1), with few the chain of its 3-6 us chunks is what takes the time (walk -> chunk-parallel: 304 chunks x 4 heads,
+// forward + backward, 0.74 -> 0.24 ms; 1,047 x 16, forward, 0.87 -> 0.52).  Many sequences of a chunk or two (fewer than
+// four chunks each, more than 128 (sequence, head) pairs) stay with the walk: the scan pays about 5 us for each of them.  The
+// line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
+constexpr int64_t CHUNK_PARALLEL_MAX = 28672;
+inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
+    return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 &&
+           (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
+           (tb.n_chunks >= 4 * (int64_t)tb.n_seq || (int64_t)tb.n_seq * H <= 128);
+}
+// the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then the scan's
+// ticket and counters
+inline size_t ds_tiles_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return align_up(chunk_state_payload(tb, H, dk, dv, 2) + fused_flag_bytes(tb, H), 1024);
+}
+inline size_t scan_flags_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return ds_tiles_offset(tb, H, dk, dv) + align_up(chunk_state_payload(tb, H, dk, dv, 2), 1024);
+}
+inline size_t chunk_parallel_bytes(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return scan_flags_offset(tb, H, dk, dv) + (4 + (size_t)(tb.n_seq > tb.n_slots ? tb.n_seq : tb.n_slots) * H * 4) * sizeof(int);
+}
 int32_t gk_mma_fwd_all(const FwdArgs& a, int* flags, int* ticket);     // all rounds in one launch (la_gk_mma.cu)
 int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrder& rounds);
 int32_t tc_bwd(const BwdArgs& a);

@@ -134,6 +134,34 @@ __device__ __forceinline__ bool flag_wait(const int* flag, int* status, volatile
     return false;
 }
 
+// Counting form for producers that finish warp by warp: a (converged) warp adds one once its lanes' data is written; the
+// consumer warp waits until `target` warps have.
+__device__ __forceinline__ void flag_add_warp(int* flag) {
+    __threadfence();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(flag) : "memory");
+}
+static __device__ __noinline__ bool flag_wait_warp(const int* flag, int target, int* status, volatile int* dead) {
+    int ok = 1;
+    if ((threadIdx.x & 31) == 0) {
+        const unsigned long long t0 = global_ns();
+        for (int round = 0;; round++) {
+            int v;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+            if (v >= target) break;
+            if ((round & 15) != 15) continue;
+            // another CTA of the launch has already given up: what this one waits for may never come
+            const bool gave_up = *dead || (status && *reinterpret_cast<volatile int*>(status) != 0);
+            if (!gave_up && round < (1 << 30) && global_ns() - t0 <= FLAG_WAIT_LIMIT_NS) continue;
+            if (!gave_up && status) atomicExch(status, STATUS_TIMEOUT);
+            *dead = 1;
+            ok = 0;
+            break;
+        }
+    }
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
 // ---- fences ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

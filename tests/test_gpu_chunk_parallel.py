@@ -1,0 +1,38 @@
+"""The chunk-parallel linear-attention path at its edges and at the line where the walk kernels take over."""
+import pytest
+import torch
+
+import paper_2608_28158_b200 as H
+from parity_util import compare, oracle_subset, run_gpu
+from test_gpu_parity import check
+from workloads import make_forest, make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lens", [(1,), (63,), (64,), (65, 1), (129, 64, 63), (64 * 40 + 1, 64, 1)])
+def test_chunk_parallel_edges(lens):
+    """One row, one row short of and past a chunk, single-chunk sequences, a boundary exported by the last chunk but one --
+    in every width of the scan's state slices (1, 50 and 100 heads: 32, 64 and 128 columns)."""
+    fo = make_forest([([-1] + [0] * (len(lens) - 1), [0] + [lens[0]] * (len(lens) - 2) + [max(1, lens[0] - 1)] * (len(lens) > 1), list(lens))])
+    for heads in (1, 50, 100):
+        inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 31)
+        plan, out = run_gpu(fo, inp)
+        pick = [0, heads - 1] if heads > 1 else [0]
+        tok, ref = oracle_subset(fo, inp, [0], pick)
+        check(compare(out, tok, pick, ref, rows=True), "bf16")
+
+
+@pytest.mark.parametrize("heads", [63, 64])
+def test_both_sides_of_the_chunk_parallel_line(heads):
+    """454 chunks x 63 heads take the chunk-parallel path, x 64 the walk kernels in their one-launch form: both against the
+    oracle, and bit-equal to one launch per round."""
+    fo = make_forest([([-1, 0, 0, 1], [0, 14000, 6001, 4000], [14000, 8000, 3000, 3901])])
+    inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 12, device="cuda")
+    plan, out = run_gpu(fo, inp)
+    assert (plan.n_chunks * heads <= 28672) == (heads == 63), plan.n_chunks
+    tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1])
+    check(compare(out, tok, [0, heads - 1], ref, rows=True), "bf16")
+    _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
+    for n in out:
+        assert torch.equal(out[n], rounds[n]), n
