@@ -160,8 +160,8 @@ int32_t harts_la_plan_tables(const harts_la_plan_t* plan, const void* dev_blob, 
  * chunk-boundary states, the backward recomputes everything inside a chunk from them).
  *   chunk_state_bytes: [n_chunks, H, dk, dv] start-of-chunk states in the run dtype, written by the
  *                      forward, read by the backward, followed by (n_slots + n_seq) * H int32 flags that the
- *                      one-launch forms of round 0 use (the library clears them itself) and, for small problems
- *                      in bf16 with dk = dv = 128, by the gradients of the boundary states.
+ *                      one-launch forms of round 0 use (the library clears them itself) and, in fp32 and
+ *                      for small problems in bf16 with dk = dv = 128, by the gradients of the boundary states.
  *   scratch_bytes:     backward scratch: per-sequence initial-state gradients [n_seq, H, dk, dv] fp32
  *                      and replay-row gradients [n_replay, H, dk + dv + 1] fp32.
  */

@@ -26,6 +26,9 @@ inline bool use_tc(int32_t dtype, int32_t dk, int32_t dv, uint32_t flags) {
     return !(flags & HARTS_FLAG_FMA_KERNELS) && harts::tc_supported(dtype, dk, dv);
 }
 
+float* f32_extra(const harts_la_tables_t& tb, const void* chunk_states, int32_t H, int32_t dk, int32_t dv) {
+    return reinterpret_cast<float*>(const_cast<char*>(static_cast<const char*>(chunk_states)) + harts::f32_extra_offset(tb, H, dk, dv));
+}
 // Chunk-parallel path over sequences [range[0], range[n]), range[r]..range[r+1] per round: the scan, then all chunks at once.
 harts::RoundOrder round_order(const int32_t* range, int32_t n) {
     harts::RoundOrder ro;
@@ -84,6 +87,7 @@ int32_t harts_la_workspace_bytes(const harts_la_tables_t* tb, int32_t H, int32_t
     (void)flags;
     if (chunk_state_bytes) {    // the states, then the flags of the one-launch forms, then what the chunk-parallel path adds
         *chunk_state_bytes = harts::chunk_state_payload(*tb, H, dk, dv, elem) + harts::fused_flag_bytes(*tb, H);
+        if (harts::f32_chunks(dk, dv, dtype)) *chunk_state_bytes += harts::f32_extra_bytes(*tb, H, dk, dv);
         if (harts::chunk_parallel(*tb, H, dk, dv, dtype, 0)) *chunk_state_bytes = harts::chunk_parallel_bytes(*tb, H, dk, dv);
     }
     if (scratch_bytes) *scratch_bytes = harts::scratch_layout(*tb, H, dk, dv).total;
@@ -103,10 +107,9 @@ int32_t harts_la_fwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
                      static_cast<cudaStream_t>(stream)};
     if (flags & HARTS_FLAG_CHECK_TABLES)
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
-    if (chunk_states && harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) {
-        const int32_t range[2] = {seq_lo, seq_hi};
-        return chunk_parallel_fwd(a, range, 1);
-    }
+    const int32_t range[2] = {seq_lo, seq_hi};
+    if (chunk_states && harts::f32_chunks(dk, dv, dtype)) return harts::f32_fwd(a, f32_extra(a.tb, chunk_states, H, dk, dv), range, 1);
+    if (chunk_states && harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) return chunk_parallel_fwd(a, range, 1);
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_fwd(a);
     return harts::fma_fwd(a);
 }
@@ -125,10 +128,9 @@ int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
                      flags, dev_status, static_cast<cudaStream_t>(stream)};
     if (flags & HARTS_FLAG_CHECK_TABLES)
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
-    if (harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) {
-        const int32_t range[2] = {seq_lo, seq_hi};
-        return chunk_parallel_bwd(a, range, 1);
-    }
+    const int32_t range[2] = {seq_lo, seq_hi};
+    if (harts::f32_chunks(dk, dv, dtype)) return harts::f32_bwd(a, f32_extra(a.tb, chunk_states, H, dk, dv), range, 1);
+    if (harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) return chunk_parallel_bwd(a, range, 1);
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_bwd(a);
     return harts::fma_bwd(a);
 }
@@ -152,7 +154,7 @@ int32_t harts_la_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
     int32_t r0 = round == 0 ? 1 : round, r1 = round == 0 ? p->n_rounds : round;
     if (round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && chunk_states &&
         !(flags & HARTS_FLAG_ROUND_LAUNCHES) &&
-        use_tc(dtype, dk, dv, flags)) {
+        (use_tc(dtype, dk, dv, flags) || harts::f32_chunks(dk, dv, dtype))) {
         // every round in one launch: a sequence waits for the flag of the state it starts from instead of for the
         // end of the previous round's kernel
         rc = check_common(&tb, 0, tb.n_seq, H, dk, dv, dtype);
@@ -167,6 +169,8 @@ int32_t harts_la_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
             if (!dev_status) return HARTS_EINVAL;
             if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
         }
+        if (harts::f32_chunks(dk, dv, dtype))
+            return harts::f32_fwd(a, f32_extra(tb, chunk_states, H, dk, dv), p->round_seq_ptr.data(), p->n_rounds);
         if (harts::chunk_parallel(tb, H, dk, dv, dtype, flags))
             return chunk_parallel_fwd(a, p->round_seq_ptr.data(), p->n_rounds);
         int* fl = reinterpret_cast<int*>(static_cast<char*>(chunk_states) + harts::chunk_state_payload(tb, H, dk, dv, 2));
@@ -193,7 +197,7 @@ int32_t harts_la_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
     int32_t r1 = round == 0 ? p->n_rounds : round, r0 = round == 0 ? 1 : round;
     bool done = false;
     if (round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && !(flags & HARTS_FLAG_ROUND_LAUNCHES) &&
-        use_tc(dtype, dk, dv, flags)) {
+        (use_tc(dtype, dk, dv, flags) || harts::f32_chunks(dk, dv, dtype))) {
         rc = check_common(&tb, 0, tb.n_seq, H, dk, dv, dtype);
         if (rc != HARTS_OK) return rc;
         if (!q || !k || !v || !g || !dO || !dq || !dk_ || !dv_ || !dg || !chunk_states || !scratch) return HARTS_EINVAL;
@@ -205,6 +209,11 @@ int32_t harts_la_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
         if (flags & HARTS_FLAG_CHECK_TABLES) {
             if (!dev_status) return HARTS_EINVAL;
             if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
+        }
+        if (harts::f32_chunks(dk, dv, dtype)) {
+            rc = harts::f32_bwd(a, f32_extra(tb, chunk_states, H, dk, dv), p->round_seq_ptr.data(), p->n_rounds);
+            if (rc != HARTS_OK) return rc;
+            return harts_la_bwd_finish(&tb, dk_, dv_, dg, scratch, H, dk, dv, dtype, stream);
         }
         if (harts::chunk_parallel(tb, H, dk, dv, dtype, flags)) {
             if ((rc = chunk_parallel_bwd(a, p->round_seq_ptr.data(), p->n_rounds)) != HARTS_OK) return rc;

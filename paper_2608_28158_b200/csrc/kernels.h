@@ -164,6 +164,17 @@ inline size_t scan_flags_offset(const harts_la_tables_t& tb, int32_t H, int32_t 
 inline size_t chunk_parallel_bytes(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
     return scan_flags_offset(tb, H, dk, dv) + (4 + (size_t)(tb.n_seq > tb.n_slots ? tb.n_seq : tb.n_slots) * H * 4) * sizeof(int);
 }
+// The same for fp32 inputs, d_k = d_v = 64 (la_f32.cu): every problem that brings a chunk-state workspace.  extra: e^{b_n}
+// [n_chunks, H] and the gradients of the boundary states [n_chunks, H, dk, dv], fp32, behind the flags.
+inline bool f32_chunks(int32_t dk, int32_t dv, int32_t dtype) { return dtype == HARTS_FP32 && dk == 64 && dv == 64; }
+inline size_t f32_extra_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return chunk_state_payload(tb, H, dk, dv, 4) + fused_flag_bytes(tb, H);
+}
+inline size_t f32_extra_bytes(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return align_up((size_t)tb.n_chunks * H, 64) * sizeof(float) + chunk_state_payload(tb, H, dk, dv, 4);
+}
+int32_t f32_fwd(const FwdArgs& a, float* extra, const int32_t* range, int32_t n);
+int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n);
 int32_t gk_mma_fwd_all(const FwdArgs& a, int* flags, int* ticket);     // all rounds in one launch (la_gk_mma.cu)
 int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrder& rounds);
 int32_t tc_bwd(const BwdArgs& a);

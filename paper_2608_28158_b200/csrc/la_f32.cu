@@ -1,0 +1,445 @@
+// Chunk-parallel path for fp32 inputs, d_k = d_v = 64, chunk 64, on the CUDA cores (no reduced-precision product anywhere).
+//
+//   outer_kernel   U_c = sum_j (w_j k_j)^T v_j of every chunk, w_j = e^{b_n-b_j} (backward: W_c = sum_t (e^{b_t} q_t)^T dO_t), e^{b_n}
+//   walk_kernel    S_{c+1} = e^{b_n} S_c + U_c along the chunks of a sequence, element by element, one launch per round; the
+//                  state at the start of a chunk replaces the chunk's sum in the workspace (backward: the gradient at its end)
+//   out_kernel     o_t = e^{b_t} q_t S_c + sum_{j<=t} A_tj v_j
+//   grad_kernel    dq, dk, dv, dg of a chunk from its rows, S_c and dS_{c+1} (formulas: la_fma.cu)
+// The kernels of la_fma.cu walk a sequence's chunks with everything in one CTA: 84 us per chunk, forward and backward, one
+// after the other.  Only the walk is serial here, and its step is one multiply-add per element with the operand prefetched;
+// the 64^3 products of different chunks run side by side.  What bounds it: launches and the latency of one product (256
+// threads x 4x4 outputs, 2,048 cycles at 128 multiply-adds a clock) on small forests, the CUDA cores on large ones.  718
+// tokens x 1 head (two rounds), forward + backward: 1.18 -> 0.080 ms (outer 7 + 7, walk 3 per round, out 13, grad 25 us).
+#include "chunk_item.cuh"
+
+namespace harts {
+namespace {
+
+using chunk::BT;
+using chunk::find_item;
+using chunk::Item;
+using chunk::RowData;
+using tc::ex2;
+
+constexpr int D = 64, NT = 256, LD = D + 4;      // rows of shared-memory tiles are padded: 16-byte aligned, conflict-free by column
+constexpr int TILE = BT * LD;                    // floats
+
+// Thread (ty, tx) = (tid / 16, tid % 16) owns outputs (4 ty + r, tx + 16 c), r, c = 0..3; a warp owns eight rows.
+using Acc = float[4][4];
+__device__ __forceinline__ void clear(Acc& a) {
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) a[r][c] = 0.f;
+}
+// a += X Y^T over column blocks 0..n_col-1 of 16
+template <int N_COL>
+__device__ __forceinline__ void mul_nt(Acc& a, const float* x, const float* y, int ty, int tx) {
+#pragma unroll 4
+    for (int i = 0; i < D; i += 4) {
+        float4 xv[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) xv[r] = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + i);
+#pragma unroll
+        for (int c = 0; c < N_COL; c++) {
+            const float4 yv = *reinterpret_cast<const float4*>(y + (tx + 16 * c) * LD + i);
+#pragma unroll
+            for (int r = 0; r < 4; r++) a[r][c] += xv[r].x * yv.x + xv[r].y * yv.y + xv[r].z * yv.z + xv[r].w * yv.w;
+        }
+    }
+}
+// the same where only columns <= the warp's last row are wanted (the rest of a stays as it is)
+__device__ __forceinline__ void mul_nt_causal(Acc& a, const float* x, const float* y, int ty, int tx) {
+    switch (ty >> 2) {                           // 16-row groups: two warps each
+        case 0: mul_nt<1>(a, x, y, ty, tx); break;
+        case 1: mul_nt<2>(a, x, y, ty, tx); break;
+        case 2: mul_nt<3>(a, x, y, ty, tx); break;
+        default: mul_nt<4>(a, x, y, ty, tx);
+    }
+}
+// a += X[:, k0..k1) Y[k0..k1, :)
+__device__ __forceinline__ void mul_nn(Acc& a, const float* x, const float* y, int k0, int k1, int ty, int tx) {
+#pragma unroll 2
+    for (int k = k0; k < k1; k += 4) {
+        float4 xv[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) xv[r] = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + k);
+#pragma unroll
+        for (int kk = 0; kk < 4; kk++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const float yv = y[(k + kk) * LD + tx + 16 * c];
+#pragma unroll
+                for (int r = 0; r < 4; r++) a[r][c] += (kk == 0 ? xv[r].x : kk == 1 ? xv[r].y : kk == 2 ? xv[r].z : xv[r].w) * yv;
+            }
+    }
+}
+// a += X[t0..64, :)^T Y[t0..64, :)
+__device__ __forceinline__ void mul_tn(Acc& a, const float* x, const float* y, int t0, int ty, int tx) {
+#pragma unroll 4
+    for (int t = t0; t < BT; t++) {
+        const float4 xv = *reinterpret_cast<const float4*>(x + t * LD + 4 * ty);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const float yv = y[t * LD + tx + 16 * c];
+            a[0][c] += xv.x * yv;
+            a[1][c] += xv.y * yv;
+            a[2][c] += xv.z * yv;
+            a[3][c] += xv.w * yv;
+        }
+    }
+}
+
+// Rows of a chunk into a tile; `own`: replayed rows (and rows past the end) are zero, else only rows past the end.
+__device__ __forceinline__ void load_tile(float* dst, const float* src, const RowData& rd, bool own, int h, int H) {
+    for (int e = threadIdx.x; e < BT * 16; e += NT) {
+        const int t = e >> 4, ch = e & 15, code = rd.code[t], r = code >= 0 ? code : -2 - code;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (own ? code >= 0 : code != -1) x = *reinterpret_cast<const float4*>(src + ((size_t)r * H + h) * D + ch * 4);
+        *reinterpret_cast<float4*>(dst + t * LD + ch * 4) = x;
+    }
+}
+__device__ __forceinline__ void load_state(float* dst, const float* src) {
+    for (int e = threadIdx.x; e < D * 16; e += NT)
+        *reinterpret_cast<float4*>(dst + (e >> 4) * LD + (e & 15) * 4) = *reinterpret_cast<const float4*>(src + e * 4);
+}
+// The CTA's item: warp 0 finds it and prepares its row data.
+__device__ __forceinline__ bool begin_item(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int H, const float* g, RowData& rd, Item& it) {
+    const int gc = tb.seq_chunk_ptr[seq_lo] + (int)blockIdx.x / H;
+    if (gc >= tb.seq_chunk_ptr[seq_hi]) return false;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const Item x = find_item(tb, seq_lo, seq_hi, gc, (int)blockIdx.x % H, lane);
+        int code[2];
+        float gv[2];
+        chunk::load_rows(tb, x, g, H, lane, code, gv);
+        chunk::store_rows(rd, code, gv, lane);
+        if (lane == 0) it = x;
+    }
+    __syncthreads();
+    return true;
+}
+
+struct __align__(16) OuterSmem {
+    float x[TILE], y[TILE];
+    RowData rd;
+    Item it;
+};
+template <bool BWD>
+__global__ void __launch_bounds__(NT) outer_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ a,
+                                                   const float* __restrict__ b, const float* __restrict__ g, float* __restrict__ sums,
+                                                   float* __restrict__ gammas, const int32_t* gate) {
+    if (gate_closed(gate)) return;
+    __shared__ OuterSmem s;
+    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    const Item& it = s.it;
+    if (BWD ? it.zero_state : it.last) return;   // this chunk's sum enters nothing
+    load_tile(s.x, a, s.rd, BWD, it.h, H);
+    for (int e = threadIdx.x; e < BT * 16; e += NT) {         // the weighted operand
+        const int t = e >> 4, ch = e & 15, code = s.rd.code[t], r = code >= 0 ? code : -2 - code;
+        const float w = BWD ? s.rd.eb[t] : s.rd.w[t];
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (BWD ? code >= 0 : code != -1) x = *reinterpret_cast<const float4*>(b + ((size_t)r * H + it.h) * D + ch * 4);
+        *reinterpret_cast<float4*>(s.y + t * LD + ch * 4) = make_float4(x.x * w, x.y * w, x.z * w, x.w * w);
+    }
+    __syncthreads();
+    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+    Acc acc;
+    clear(acc);
+    mul_tn(acc, s.x, s.y, 0, ty, tx);
+    float* dst = sums + ((size_t)it.gc * H + it.h) * (D * D);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) dst[(4 * ty + r) * D + tx + 16 * c] = acc[r][c];
+    if (threadIdx.x == 0) gammas[(size_t)it.gc * H + it.h] = s.rd.gamma;
+}
+
+// One thread walks four elements of the state along a sequence; four CTAs per (sequence, head).
+constexpr int AHEAD = 8;                         // sums in flight per thread
+template <bool BWD>
+__global__ void __launch_bounds__(NT) walk_kernel(const harts_la_tables_t tb, int seq_lo, int H, float* tiles, const float* gammas,
+                                                  float* slots, float* ds0, const int32_t* gate) {
+    if (gate_closed(gate)) return;
+    const int part = blockIdx.x & 3, item = blockIdx.x >> 2, h = item % H;
+    const int pos = seq_lo + item / H, seq = tb.seq_order ? tb.seq_order[pos] : pos;
+    const int chunk_base = tb.seq_chunk_ptr[seq], n_chunks = tb.seq_chunk_ptr[seq + 1] - chunk_base;
+    const int init_slot = tb.seq_init_slot[seq], req_lo = tb.seq_req_ptr[seq], req_hi = tb.seq_req_ptr[seq + 1];
+    const int n_steps = BWD && init_slot >= 0 ? n_chunks : n_chunks - 1;
+    const size_t stride = (size_t)H * (D * D), el = (size_t)h * (D * D) + part * 1024 + threadIdx.x * 4;
+    auto chunk_of = [&](int i) { return BWD ? n_chunks - 1 - i : i; };
+    auto load = [&](int i0, float4 (&u)[AHEAD], float (&gm)[AHEAD]) {
+#pragma unroll
+        for (int j = 0; j < AHEAD; j++)
+            if (i0 + j < n_steps) {
+                const size_t gc = chunk_base + chunk_of(i0 + j);
+                u[j] = *reinterpret_cast<const float4*>(tiles + gc * stride + el);
+                gm[j] = gammas[gc * H + h];
+            }
+    };
+    float4 u[AHEAD], un[AHEAD], x = make_float4(0.f, 0.f, 0.f, 0.f);
+    float gm[AHEAD], gn[AHEAD];
+    load(0, u, gm);
+    if (!BWD && init_slot >= 0) x = *reinterpret_cast<const float4*>(slots + (size_t)init_slot * stride + el);
+    int req = BWD ? req_hi - 1 : req_lo;
+    int boundary = (BWD ? req >= req_lo : req < req_hi) ? tb.slot_chunk[req] : -1;
+    for (int i0 = 0; i0 < n_chunks; i0 += AHEAD) {
+        load(i0 + AHEAD, un, gn);
+#pragma unroll
+        for (int j = 0; j < AHEAD; j++) {
+            const int i = i0 + j, c = chunk_of(i);
+            if (i >= n_chunks) break;
+            if (BWD && boundary == c + 1) {      // gradients of every sequence that started from this boundary, in table order
+                for (int q = tb.slot_cons_ptr[req]; q < tb.slot_cons_ptr[req + 1]; q++) {
+                    const float4 y = *reinterpret_cast<const float4*>(ds0 + (size_t)tb.slot_cons_seq[q] * stride + el);
+                    x.x += y.x, x.y += y.y, x.z += y.z, x.w += y.w;
+                }
+                req--;
+                boundary = req >= req_lo ? tb.slot_chunk[req] : -1;
+            }
+            // in place: this thread has read the chunk's sum already; backward: zero after the last chunk, not read
+            if (!BWD || i > 0) *reinterpret_cast<float4*>(tiles + (size_t)(chunk_base + c) * stride + el) = x;
+            if (!BWD && boundary == c) {
+                *reinterpret_cast<float4*>(slots + (size_t)req * stride + el) = x;
+                req++;
+                boundary = req < req_hi ? tb.slot_chunk[req] : -1;
+            }
+            if (i < n_steps) {
+                x.x = __fmaf_rn(gm[j], x.x, u[j].x), x.y = __fmaf_rn(gm[j], x.y, u[j].y);
+                x.z = __fmaf_rn(gm[j], x.z, u[j].z), x.w = __fmaf_rn(gm[j], x.w, u[j].w);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < AHEAD; j++) u[j] = un[j], gm[j] = gn[j];
+    }
+    if (BWD && init_slot >= 0) *reinterpret_cast<float4*>(ds0 + (size_t)seq * stride + el) = x;
+}
+
+struct __align__(16) OutSmem {
+    float q[TILE], k[TILE], v[TILE], s[TILE], p[TILE];
+    RowData rd;
+    Item it;
+};
+__global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
+                                                 const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
+                                                 const float* __restrict__ states, float* __restrict__ o, const int32_t* gate) {
+    if (gate_closed(gate)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OutSmem& s = *reinterpret_cast<OutSmem*>(smem_raw);
+    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    const Item& it = s.it;
+    load_tile(s.q, q, s.rd, true, it.h, H);
+    load_tile(s.k, k, s.rd, false, it.h, H);
+    load_tile(s.v, v, s.rd, false, it.h, H);
+    if (!it.zero_state) load_state(s.s, states + ((size_t)it.gc * H + it.h) * (D * D));
+    __syncthreads();
+    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16, warp = threadIdx.x / 32;
+    Acc acc;
+    clear(acc);
+    mul_nt_causal(acc, s.q, s.k, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int t = 4 * ty + r, j = tx + 16 * c;
+            s.p[t * LD + j] = j <= t ? acc[r][c] * ex2(s.rd.b2[t] - s.rd.b2[j]) : 0.f;
+        }
+    __syncwarp();                                // a warp reads the rows it wrote
+    clear(acc);
+    if (!it.zero_state) {
+        mul_nn(acc, s.q, s.s, 0, D, ty, tx);
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
+    }
+    mul_nn(acc, s.p, s.v, 0, 8 * warp + 8, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const int code = s.rd.code[4 * ty + r];
+        if (code >= 0)
+#pragma unroll
+            for (int c = 0; c < 4; c++) o[((size_t)code * H + it.h) * D + tx + 16 * c] = acc[r][c];
+    }
+}
+
+struct __align__(16) GradSmem {
+    float q[TILE], k[TILE], v[TILE], dO[TILE], s[TILE], ds[TILE], p[TILE], dp[TILE];
+    RowData rd;
+    Item it;
+    float z[BT], part[NT / 32];
+};
+__global__ void __launch_bounds__(NT) grad_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
+                                                  const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
+                                                  const float* __restrict__ dO, const float* __restrict__ states,
+                                                  const float* __restrict__ ds_tiles, float* __restrict__ dq, float* __restrict__ dk_,
+                                                  float* __restrict__ dv_, float* __restrict__ dg, float* __restrict__ rk,
+                                                  float* __restrict__ rv, float* __restrict__ rg, const int32_t* gate) {
+    if (gate_closed(gate)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
+    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    const Item& it = s.it;
+    const int h = it.h;
+    const bool has_s = !it.zero_state, has_ds = !it.last;
+    load_tile(s.q, q, s.rd, true, h, H);
+    load_tile(s.k, k, s.rd, false, h, H);
+    load_tile(s.v, v, s.rd, false, h, H);
+    load_tile(s.dO, dO, s.rd, true, h, H);
+    const size_t tile = ((size_t)it.gc * H + h) * (D * D);
+    if (has_s) load_state(s.s, states + tile);
+    if (has_ds) load_state(s.ds, ds_tiles + tile);
+    __syncthreads();
+    const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, warp = tid / 32, lane = tid & 31;
+    Acc acc, dacc;
+    clear(acc);
+    clear(dacc);
+    mul_nt_causal(acc, s.q, s.k, ty, tx);
+    mul_nt_causal(dacc, s.dO, s.v, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int t = 4 * ty + r, j = tx + 16 * c;
+            const float w = j <= t ? ex2(s.rd.b2[t] - s.rd.b2[j]) : 0.f;
+            s.p[t * LD + j] = j <= t ? acc[r][c] * w : 0.f;
+            s.dp[t * LD + j] = j <= t ? dacc[r][c] * w : 0.f;
+        }
+    __syncthreads();
+    const float gamma = s.rd.gamma;
+    float g_part = 0.f;                          // this thread's share of <S_{c+1}, dS_{c+1}>
+    float z[4] = {0.f, 0.f, 0.f, 0.f};           // its share of q.dq - k.dk, per row
+    // ---- dq = e^{b_t} dO S^T + dP K
+    clear(acc);
+    if (has_s) mul_nt<4>(acc, s.dO, s.s, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
+    mul_nn(acc, s.dp, s.k, 0, 8 * warp + 8, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const int t = 4 * ty + r, code = s.rd.code[t];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            z[r] += s.q[t * LD + tx + 16 * c] * acc[r][c];
+            if (code >= 0) dq[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
+        }
+    }
+    // ---- dk = w_j V dS^T + dP^T Q
+    clear(acc);
+    if (has_ds) mul_nt<4>(acc, s.v, s.ds, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int t = 4 * ty + r;
+            acc[r][c] *= s.rd.w[t];
+            g_part += s.k[t * LD + tx + 16 * c] * acc[r][c];
+        }
+    mul_tn(acc, s.dp, s.q, 8 * warp, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const int t = 4 * ty + r, code = s.rd.code[t];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            z[r] -= s.k[t * LD + tx + 16 * c] * acc[r][c];
+            if (code >= 0) dk_[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
+            else if (code < -1) rk[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = acc[r][c];
+        }
+    }
+    // ---- dv = w_j K dS + P^T dO
+    clear(acc);
+    if (has_ds) mul_nn(acc, s.k, s.ds, 0, D, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.w[4 * ty + r];
+    mul_tn(acc, s.p, s.dO, 8 * warp, ty, tx);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const int t = 4 * ty + r, code = s.rd.code[t];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            if (code >= 0) dv_[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
+            else if (code < -1) rv[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = acc[r][c];
+        }
+    }
+    // ---- dg_t = sum_{tau>=t} z_tau + e^{b_n} <S_c, dS> + sum_j k_j . (w_j dS v_j), every sum in a fixed order
+    if (has_s && has_ds) {
+        float dot = 0.f;
+        for (int e = tid; e < D * D; e += NT) dot += s.s[(e >> 6) * LD + (e & 63)] * s.ds[(e >> 6) * LD + (e & 63)];
+        g_part += gamma * dot;
+    }
+#pragma unroll
+    for (int o_ = 16; o_ > 0; o_ >>= 1) g_part += __shfl_xor_sync(~0u, g_part, o_);
+    if (lane == 0) s.part[warp] = g_part;
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+#pragma unroll
+        for (int o_ = 8; o_ > 0; o_ >>= 1) z[r] += __shfl_xor_sync(~0u, z[r], o_);
+        if (tx == 0) s.z[4 * ty + r] = z[r];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        float lo = s.z[lane], hi = s.z[lane + 32], G = 0.f;
+#pragma unroll
+        for (int o_ = 1; o_ < 32; o_ <<= 1) {
+            const float y0 = __shfl_down_sync(~0u, lo, o_), y1 = __shfl_down_sync(~0u, hi, o_);
+            if (lane + o_ < 32) {
+                lo += y0;
+                hi += y1;
+            }
+        }
+        const float half = __shfl_sync(~0u, hi, 0);
+#pragma unroll
+        for (int w = 0; w < NT / 32; w++) G += s.part[w];
+        const float out[2] = {lo + half + G, hi + G};
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            const int t = lane + 32 * r, code = s.rd.code[t];
+            if (code >= 0) dg[(size_t)code * H + h] = out[r];
+            else if (code < -1) rg[(size_t)(it.replay_base + t) * H + h] = out[r];
+        }
+    }
+}
+
+inline int32_t done() { return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA; }
+
+}  // namespace
+
+// Sequences [range[0], range[n]), range[r]..range[r+1] per round.  extra: f32_extra_bytes() behind the chunk states and flags.
+int32_t f32_fwd(const FwdArgs& a, float* extra, const int32_t* range, int32_t n) {
+    const int lo = range[0], hi = range[n], grid = a.tb.n_chunks * a.H;
+    if (lo == hi) return HARTS_OK;
+    const int32_t* gate = status_gate(a.flags, a.dev_status);
+    float *states = (float*)a.chunk_states, *gammas = extra;
+    outer_kernel<false><<<grid, NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.k, (const float*)a.v, a.g, states, gammas, gate);
+    for (int32_t r = 0; r < n; r++)
+        if (range[r] < range[r + 1])
+            walk_kernel<false><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, states, gammas, a.slots, nullptr, gate);
+    if (cudaFuncSetAttribute(out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(OutSmem)) != cudaSuccess) return HARTS_ECUDA;
+    out_kernel<<<grid, NT, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g,
+                                                        states, (float*)a.o, gate);
+    return done();
+}
+
+int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n) {
+    const int lo = range[0], hi = range[n], grid = a.tb.n_chunks * a.H;
+    if (lo == hi) return HARTS_OK;
+    const int32_t* gate = status_gate(a.flags, a.dev_status);
+    const ScratchLayout sl = scratch_layout(a.tb, a.H, a.dk, a.dv);
+    char* base = static_cast<char*>(a.scratch);
+    float *gammas = extra, *tiles = extra + align_up((size_t)a.tb.n_chunks * a.H, 64), *ds0 = (float*)(base + sl.ds0);
+    outer_kernel<true><<<grid, NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.dO, a.g, tiles, gammas, gate);
+    for (int32_t r = n - 1; r >= 0; r--)
+        if (range[r] < range[r + 1])
+            walk_kernel<true><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, tiles, gammas, nullptr, ds0, gate);
+    if (cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem)) != cudaSuccess) return HARTS_ECUDA;
+    grad_kernel<<<grid, NT, sizeof(GradSmem), a.stream>>>(
+        a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g, (const float*)a.dO, (const float*)a.chunk_states,
+        tiles, (float*)a.dq, (float*)a.dk_, (float*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv), (float*)(base + sl.rg), gate);
+    return done();
+}
+
+}  // namespace harts

@@ -569,7 +569,6 @@ int32_t handoff_reduce(const BwdArgs& a) {
 int32_t fma_bwd(const BwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     if (int32_t rc = handoff_reduce(a); rc != HARTS_OK) return rc;
-    if (a.dtype == HARTS_FP32 && a.dk == 64 && a.dv == 64) return launch_bwd<float, 64, 64>(a);
     if (a.dtype == HARTS_BF16 && a.dk == 64 && a.dv == 64) return launch_bwd<__nv_bfloat16, 64, 64>(a);
     if (a.dtype == HARTS_BF16 && a.dk == 128 && a.dv == 128) return launch_bwd<__nv_bfloat16, 128, 128>(a);
     return HARTS_EUNSUPPORTED;

@@ -23,6 +23,16 @@ def test_chunk_parallel_edges(lens):
         check(compare(out, tok, pick, ref, rows=True), "bf16")
 
 
+@pytest.mark.parametrize("lens", [(1,), (63,), (64,), (65, 1), (129, 64, 63), (64 * 20 + 1, 64, 1)])
+def test_fp32_edges(lens):
+    """The same edges through the fp32 kernels (d = 64); 20 chunks exceed the sums one walking thread keeps in flight."""
+    fo = make_forest([([-1] + [0] * (len(lens) - 1), [0] + [lens[0]] * (len(lens) - 2) + [max(1, lens[0] - 1)] * (len(lens) > 1), list(lens))])
+    inp = make_inputs(fo.n_tokens, 3, 64, 64, "fp32", 32)
+    plan, out = run_gpu(fo, inp)
+    tok, ref = oracle_subset(fo, inp, [0], [0, 1, 2])
+    check(compare(out, tok, [0, 1, 2], ref, rows=True), "fp32")
+
+
 @pytest.mark.parametrize("heads", [63, 64])
 def test_both_sides_of_the_chunk_parallel_line(heads):
     """454 chunks x 63 heads take the chunk-parallel path, x 64 the walk kernels in their one-launch form: both against the
