@@ -86,6 +86,22 @@ struct TileWalkT {      // enumerates the key tiles (W rows) of one item in orde
 };
 using TileWalk = TileWalkT<BK>;
 
+// dK / dV work of small problems, cut into units (attn_split.cu): a unit is a run of the query tiles of one key tile, in the
+// order of QWalk; slot: where its partial sums go, -1: the item is not cut.
+struct DkvUnit {
+    int piece, kt, n_tiles, slot, g, in_own, off, d;
+};
+struct SplitItem {
+    int n_tiles, n_units, first_unit, first_slot;
+};
+struct SplitTable {
+    int* n_units;
+    SplitItem* item;         // [n_kv_items]
+    DkvUnit* unit;
+    float* sums;             // [slot][Hkv][dV, dK][128][D]
+    int cap_slots;
+};
+
 // The query tiles (64 rows) that see the key tile `kt` (128 rows) of a piece: for every query head of the group,
 // the rest of the piece from the key tile's first row on (causal inside), then all rows of every descendant piece.
 // Key row i is seen by query column j iff jmin(i) <= j < n_valid, with jmin(i) = max(0, i - lead) for own tiles
@@ -96,6 +112,7 @@ struct QTile {
 struct QWalk {
     const Index& ix;
     int piece, k0, own_len, own_row0, G, head0, g, off, d, d_end, cur_len, cur_row0;
+    int left = 0x7fffffff;              // tiles still to deliver (a unit of a cut item)
     bool in_own;
     __device__ QWalk(const Index& ix_, int piece_, int kt, int hk, int G_) : ix(ix_), piece(piece_), G(G_) {
         k0 = kt * 128;
@@ -104,6 +121,17 @@ struct QWalk {
         head0 = hk * G;
         d_end = ix.desc_ptr[piece + 1];
         start_head(0);
+    }
+    __device__ void start_at(const DkvUnit& u) {
+        g = u.g;
+        in_own = u.in_own;
+        off = u.off;
+        d = u.d;
+        left = u.n_tiles;
+        if (!in_own && d < d_end) {
+            cur_len = ix.piece_len[ix.desc_piece[d]];
+            cur_row0 = ix.piece_row0[ix.desc_piece[d]];
+        }
     }
     __device__ void start_head(int g_) {
         g = g_;
@@ -117,6 +145,7 @@ struct QWalk {
         return n * G;
     }
     __device__ bool next(QTile& t) {
+        if (left-- <= 0) return false;
         while (true) {
             if (g >= G) return false;
             if (in_own) {

@@ -44,13 +44,15 @@ struct Misc {
     uint32_t tmem;
 };
 
+// SPLIT: the work is the unit list of attn_split.cu, and a unit of a cut item leaves fp32 sums.
+template <bool SPLIT>
 __global__ void __launch_bounds__(NT, 1)
 attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_constant__ CUtensorMap map_q,
                 const __grid_constant__ CUtensorMap map_do, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_dk,
                 const __grid_constant__ CUtensorMap map_dv, const float* __restrict__ lse,
                 const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk_, __nv_bfloat16* __restrict__ dv_,
-                int* status) {
+                int* status, SplitTable split) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     unsigned char* sK = smem + Smem::k;
@@ -80,20 +82,24 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
     const float scale_log2 = scale * LOG2E;
 
     uint32_t ph_kv = 0, ph_q[STAGES] = {}, ph_free[STAGES] = {}, ph_s[2] = {0, 0}, ph_p[2] = {0, 0}, ph_o = 0;
-    const int n_work = ix.n_kv_items * Hkv;
+    const int n_work = (SPLIT ? split.n_units[0] : ix.n_kv_items) * Hkv;
     // work items come most work first; dealt in a snake pattern (tier by tier, every second tier in reverse), so that no
     // CTA gets the largest item of every tier
     for (int tier = 0; tier * (int)gridDim.x < n_work; tier++) {
         const int w = tier * (int)gridDim.x + ((tier & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
         if (w >= n_work) continue;
         const int item = w / Hkv, hk = w % Hkv;
-        const int piece = ix.kv_item[2 * item], kt = ix.kv_item[2 * item + 1];
+        DkvUnit unit{};
+        if (SPLIT) unit = split.unit[item];
+        const int piece = SPLIT ? unit.piece : ix.kv_item[2 * item], kt = SPLIT ? unit.kt : ix.kv_item[2 * item + 1];
+        const bool partial = SPLIT && unit.slot >= 0;
         const int kv_row0 = ix.piece_row0[piece] + kt * BKV;
         const int kv_valid = min(BKV, ix.piece_len[piece] - kt * BKV);
 
         if (is_producer) {
             // ---- TMA producer: the K and V tiles, then the query / dO tiles STAGES deep -----------------------------
             QWalk lw(ix, piece, kt, hk, G);
+            if (SPLIT) lw.start_at(unit);
             QTile lt;
             mbar_expect_tx(&m.bar_kv, 2 * KV_TILE);
             for (int p = 0; p < 2; p++)
@@ -119,7 +125,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         }
         if (is_issuer) {
             // ---- MMA issue: this thread does nothing else, a tcgen05.mma holds it until the pipe has room ---------
-            const int n_tiles = QWalk(ix, piece, kt, hk, G).count();
+            const int n_tiles = SPLIT ? unit.n_tiles : QWalk(ix, piece, kt, hk, G).count();
             auto issue_s = [&](int n) {      // S^T(n), dP^T(n) into buffer n & 1
                 const int stage = n % STAGES, b = n & 1;
                 mbar_wait(&m.bar_q[stage], ph_q[stage], status, &m.dead);
@@ -159,6 +165,10 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         }
         if (is_softmax) {
             QWalk walk(ix, piece, kt, hk, G), ahead(ix, piece, kt, hk, G);
+            if (SPLIT) {
+                walk.start_at(unit);
+                ahead.start_at(unit);
+            }
             QTile t, ta;
             const int i = tid & 127, c = tid >> 7;             // key row inside the tile, and which 32 of the 64 query columns
             const bool row_ok = i < kv_valid;
@@ -232,6 +242,14 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
                     uint32_t x[32];
                     tmem_ld32(tm_lane + (which ? COL_DK : COL_DV) + c4 * 32, x);
                     tmem_ld_wait();
+                    if (partial) {                                       // fp32 sums of this unit
+                        float4* to = reinterpret_cast<float4*>(split.sums + (((size_t)unit.slot * Hkv + hk) * 2 + which) * (BKV * D) + i * D + c4 * 32);
+#pragma unroll
+                        for (int v = 0; v < 8; v++)
+                            to[v] = make_float4(__uint_as_float(x[4 * v]), __uint_as_float(x[4 * v + 1]), __uint_as_float(x[4 * v + 2]),
+                                                __uint_as_float(x[4 * v + 3]));
+                        continue;
+                    }
 #pragma unroll
                     for (int v4 = 0; v4 < 4; v4++) {
                         uint4 pk;
@@ -253,7 +271,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         tc_fence_before();
         if (__syncthreads_or(m.dead)) break;
         tc_fence_after();
-        if (is_issuer && kv_valid == BKV) {
+        if (is_issuer && kv_valid == BKV && !partial) {
             for (int p = 0; p < 2; p++)
                 for (int r = 0; r < 2; r++) {
                     tma_store_3d(&map_dv, sV + p * (KV_TILE / 2) + r * (KV_TILE / 4), p * 64, hk, kv_row0 + r * 64);
@@ -281,7 +299,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
 
 int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* k, const void* v, const float* lse,
                         const void* dO, const float* delta, void* dk_, void* dv_, int Hq, int Hkv, float scale,
-                        int32_t* status, cudaStream_t st) {
+                        int32_t* status, const SplitTable* split, cudaStream_t st) {
     CUtensorMap mq, mdo, mk, mv, mdk, mdv;
     int32_t rc;
     if ((rc = make_row_map(&mq, q, n_rows, Hq)) != HARTS_OK) return rc;
@@ -290,13 +308,13 @@ int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* 
     if ((rc = make_row_map(&mv, v, n_rows, Hkv)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mdk, dk_, n_rows, Hkv)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mdv, dv_, n_rows, Hkv)) != HARTS_OK) return rc;
-    if (cudaFuncSetAttribute(attn_dkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::bytes + 1024) !=
-        cudaSuccess)
-        return HARTS_ECUDA;
+    const auto kernel = split ? attn_dkv_kernel<true> : attn_dkv_kernel<false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::bytes + 1024) != cudaSuccess) return HARTS_ECUDA;
     const long long n_work = (long long)ix.n_kv_items * Hkv;
-    const int grid = (int)(n_work < sm_count() ? n_work : sm_count());
-    attn_dkv_kernel<<<grid, NT, Smem::bytes + 1024, st>>>(ix, Hq, Hkv, Hq / Hkv, scale, mq, mdo, mk, mv, mdk, mdv, lse,
-                                                          delta, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_, status);
+    const int grid = split || n_work > sm_count() ? sm_count() : (int)n_work;
+    kernel<<<grid, NT, Smem::bytes + 1024, st>>>(ix, Hq, Hkv, Hq / Hkv, scale, mq, mdo, mk, mv, mdk, mdv, lse,
+                                                          delta, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_, status,
+                                                 split ? *split : SplitTable{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

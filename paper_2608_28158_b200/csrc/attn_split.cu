@@ -1,0 +1,181 @@
+// Split of the dK / dV work of small problems.  A key tile near the root is seen by every query below it -- for every query
+// head of its group -- so on one tree with grouped queries a few work items are most of the work, and the CTA that draws the
+// largest one is what the launch takes (9,001 tokens, 16 query heads on 4 key heads: 1.02 ms, 0.33 ms with this split).  Here
+// one CTA cuts every item into units of about a quarter of an SM's share of the whole, attn_dkv_kernel leaves the sums of
+// a cut item in fp32, unit by unit, and reduce_kernel adds them in unit order (no atomics: same bits every run).
+// The table and the partial sums live in the dq tensor, which is written only afterwards (the dQ kernel runs last then).
+#include "kernels.h"
+
+#include "../../include/harts_attn.h"
+#include "attn_common.cuh"
+
+namespace harts {
+
+int sm_count();
+
+namespace {
+
+using namespace attn;
+
+__device__ __forceinline__ int warp_sum(int x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(~0u, x, o);
+    return x;
+}
+__device__ __forceinline__ int tiles_of(int rows) { return (rows + 63) / 64; }
+
+// One CTA of 1024 threads, a warp per item.
+__global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, int sms, SplitTable t) {
+    __shared__ int total, slots, len;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    for (int i = warp; i < ix.n_kv_items; i += 32) {          // tiles of every item
+        const int piece = ix.kv_item[2 * i], kt = ix.kv_item[2 * i + 1];
+        int n = 0;
+        for (int d = ix.desc_ptr[piece] + lane; d < ix.desc_ptr[piece + 1]; d += 32) n += tiles_of(ix.piece_len[ix.desc_piece[d]]);
+        n = (warp_sum(n) + tiles_of(ix.piece_len[piece] - kt * 128)) * G;
+        if (lane == 0) {
+            t.item[i].n_tiles = n;
+            atomicAdd(&total, n);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) len = max(16, (int)(((long long)total * Hkv + 4 * sms - 1) / (4 * sms)));
+    for (int tries = 0; tries < 20; tries++) {                // the longest unit such that the partial sums fit
+        if (threadIdx.x == 0) slots = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < ix.n_kv_items; i += 1024) {
+            const int n = t.item[i].n_tiles;
+            if (n > len) atomicAdd(&slots, (n + len - 1) / len);
+        }
+        __syncthreads();
+        const bool fits = slots <= t.cap_slots;
+        __syncthreads();
+        if (fits) break;
+        if (threadIdx.x == 0) len *= 2;
+    }
+    __syncthreads();
+    const int L = slots <= t.cap_slots ? len : 0x3fffffff;
+    if (warp == 0) {                                          // units and slots before every item
+        int units = 0, used = 0;
+        for (int i0 = 0; i0 < ix.n_kv_items; i0 += 32) {
+            const int i = i0 + lane, n = i < ix.n_kv_items ? t.item[i].n_tiles : 0;
+            const int k = i < ix.n_kv_items ? (n + L - 1) / L : 0, s = k > 1 ? k : 0;
+            int ku = k, su = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(~0u, ku, o), z = __shfl_up_sync(~0u, su, o);
+                if (lane >= o) {
+                    ku += y;
+                    su += z;
+                }
+            }
+            if (i < ix.n_kv_items) {
+                t.item[i].n_units = k;
+                t.item[i].first_unit = units + ku - k;
+                t.item[i].first_slot = used + su - s;
+            }
+            units += __shfl_sync(~0u, ku, 31);
+            used += __shfl_sync(~0u, su, 31);
+        }
+        if (lane == 0) t.n_units[0] = units;
+    }
+    __syncthreads();
+    for (int i = warp; i < ix.n_kv_items; i += 32) {          // where every unit begins
+        const SplitItem it = t.item[i];
+        const int piece = ix.kv_item[2 * i], kt = ix.kv_item[2 * i + 1], own = tiles_of(ix.piece_len[piece] - kt * 128);
+        const int per_head = it.n_tiles / G, step = (it.n_tiles + it.n_units - 1) / it.n_units;
+        for (int u = 0; u < it.n_units; u++) {
+            DkvUnit x;
+            x.piece = piece;
+            x.kt = kt;
+            x.n_tiles = max(0, min(step, it.n_tiles - u * step));
+            x.slot = it.n_units > 1 ? it.first_slot + u : -1;
+            const int at = min(u * step, it.n_tiles - 1);
+            x.g = at / per_head;
+            int r = at % per_head;
+            x.in_own = r < own;
+            x.off = kt * 128 + r * 64;
+            x.d = ix.desc_ptr[piece];
+            if (!x.in_own) {
+                r -= own;
+                for (int d0 = x.d; d0 < ix.desc_ptr[piece + 1]; d0 += 32) {
+                    const int d = d0 + lane, n = d < ix.desc_ptr[piece + 1] ? tiles_of(ix.piece_len[ix.desc_piece[d]]) : 0;
+                    int sum = n;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(~0u, sum, o);
+                        if (lane >= o) sum += y;
+                    }
+                    const unsigned here = __ballot_sync(~0u, r < sum);
+                    if (here) {
+                        const int l = __ffs(here) - 1;
+                        x.d = d0 + l;
+                        x.off = (r - (__shfl_sync(~0u, sum, l) - __shfl_sync(~0u, n, l))) * 64;
+                        break;
+                    }
+                    r -= __shfl_sync(~0u, sum, 31);
+                }
+            }
+            if (lane == 0) t.unit[it.first_unit + u] = x;
+        }
+    }
+}
+
+// dV and dK of the items that were cut: their units' sums in unit order, eight CTAs per (item, key head).
+__global__ void __launch_bounds__(256) reduce_kernel(Index ix, int Hkv, SplitTable t, __nv_bfloat16* __restrict__ dk_,
+                                                     __nv_bfloat16* __restrict__ dv_) {
+    const int part = blockIdx.x & 7, i = (blockIdx.x >> 3) / Hkv, hk = (blockIdx.x >> 3) % Hkv;
+    const SplitItem it = t.item[i];
+    if (it.n_units < 2) return;
+    const int piece = ix.kv_item[2 * i], kt = ix.kv_item[2 * i + 1];
+    const int row0 = ix.piece_row0[piece] + kt * 128, valid = min(128, ix.piece_len[piece] - kt * 128);
+#pragma unroll
+    for (int which = 0; which < 2; which++) {
+        const int r = part * 16 + threadIdx.x / 16, ch = threadIdx.x % 16;
+        if (r >= valid) return;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+#pragma unroll 4
+        for (int u = 0; u < it.n_units; u++) {
+            const float4* src = reinterpret_cast<const float4*>(t.sums + (((size_t)(it.first_slot + u) * Hkv + hk) * 2 + which) * (128 * D) +
+                                                                r * D + ch * 8);
+            const float4 x = src[0], y = src[1];
+            a.x += x.x, a.y += x.y, a.z += x.z, a.w += x.w;
+            b.x += y.x, b.y += y.y, b.z += y.z, b.w += y.w;
+        }
+        __nv_bfloat162 o[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w), __floats2bfloat162_rn(b.x, b.y),
+                               __floats2bfloat162_rn(b.z, b.w)};
+        *reinterpret_cast<uint4*>((which ? dk_ : dv_) + ((size_t)(row0 + r) * Hkv + hk) * D + ch * 8) = *reinterpret_cast<uint4*>(o);
+    }
+}
+
+}  // namespace
+
+// The table and the partial sums in `buf`; false: too small a buffer, or so much work that it balances by itself (16 items
+// and more per SM: the largest item of 16k-token trees is then 1 in 25 of an SM's share).
+bool attn_split_table(const Index& ix, int Hkv, void* buf, size_t bytes, SplitTable* t) {
+    if ((long long)ix.n_kv_items * Hkv >= 16LL * sm_count()) return false;
+    const size_t max_units = (size_t)ix.n_kv_items + 5 * sm_count() + 64;       // units of a quarter share, plus one per item
+    char* p = static_cast<char*>(buf);
+    size_t off = 256;
+    t->n_units = reinterpret_cast<int*>(p);
+    t->item = reinterpret_cast<SplitItem*>(p + off);
+    off = align_up(off + (size_t)ix.n_kv_items * sizeof(SplitItem), 256);
+    t->unit = reinterpret_cast<DkvUnit*>(p + off);
+    off = align_up(off + max_units * sizeof(DkvUnit), 256);
+    t->sums = reinterpret_cast<float*>(p + off);
+    if (bytes <= off) return false;
+    t->cap_slots = (int)((bytes - off) / ((size_t)Hkv * 2 * 128 * D * sizeof(float)));
+    return t->cap_slots > 1;
+}
+int32_t attn_split_launch(const Index& ix, int G, int Hkv, const SplitTable& t, cudaStream_t st) {
+    split_kernel<<<1, 1024, 0, st>>>(ix, G, Hkv, sm_count(), t);
+    return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
+}
+int32_t attn_split_reduce(const Index& ix, int Hkv, const SplitTable& t, void* dk_, void* dv_, cudaStream_t st) {
+    reduce_kernel<<<ix.n_kv_items * Hkv * 8, 256, 0, st>>>(ix, Hkv, t, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_);
+    return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
+}
+
+}  // namespace harts
