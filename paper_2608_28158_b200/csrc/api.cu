@@ -53,6 +53,23 @@ int32_t chunk_parallel_bwd(harts::BwdArgs a, const int32_t* range, int32_t n) {
     return rc != HARTS_OK ? rc : harts::chunk_bwd(a, ds);
 }
 
+int32_t gk_chunk_parallel_fwd(harts::FwdArgs a, const int32_t* range, int32_t n) {
+    a.seq_lo = range[0];
+    a.seq_hi = range[n];
+    int* flags = reinterpret_cast<int*>(static_cast<char*>(a.chunk_states) + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::gk_scan_fwd(a, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::gk_chunk_fwd(a);
+}
+int32_t gk_chunk_parallel_bwd(harts::BwdArgs a, const int32_t* range, int32_t n) {
+    a.seq_lo = range[0];
+    a.seq_hi = range[n];
+    char* ws = const_cast<char*>(static_cast<const char*>(a.chunk_states));
+    void* ds = ws + harts::ds_tiles_offset(a.tb, a.H, a.dk, a.dv);
+    int* flags = reinterpret_cast<int*>(ws + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::gk_scan_bwd(a, ds, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::gk_chunk_bwd(a, ds);
+}
+
 }  // namespace
 
 extern "C" {
@@ -280,6 +297,8 @@ int32_t harts_la_gk_workspace_bytes(const harts_la_tables_t* tb, int32_t H, int3
     const size_t elem = dtype == HARTS_FP32 ? 4 : 2;
     if (chunk_state_bytes)      // the states, then the flags of the one-launch forms
         *chunk_state_bytes = harts::chunk_state_payload(*tb, H, dk, dv, elem) + harts::fused_flag_bytes(*tb, H);
+    if (chunk_state_bytes && harts::gk_chunk_parallel(*tb, H, dk, dv, dtype, 0))
+        *chunk_state_bytes = harts::chunk_parallel_bytes(*tb, H, dk, dv);
     if (scratch_bytes) *scratch_bytes = harts::gk_scratch_layout(*tb, H, dk, dv).total;
     return HARTS_OK;
 }
@@ -299,7 +318,15 @@ int32_t harts_la_gk_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32
         return HARTS_EINVAL;
     if ((flags & HARTS_FLAG_CHECK_TABLES) && !dev_status) return HARTS_EINVAL;
     const int32_t r0 = round == 0 ? 1 : round, r1 = round == 0 ? p->n_rounds : round;
-    const bool one_launch = round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && chunk_states &&
+    const bool chunks = chunk_states && harts::gk_chunk_parallel(tb, H, dk, dv, dtype, flags);
+    if (chunks && round == 0 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && !(flags & HARTS_FLAG_ROUND_LAUNCHES)) {
+        harts::FwdArgs a{tb, 0, tb.n_seq, q, k, v, gk, o, slots, chunk_states, H, dk, dv, dtype, flags, dev_status,
+                         static_cast<cudaStream_t>(stream)};
+        if (flags & HARTS_FLAG_CHECK_TABLES)
+            if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
+        return gk_chunk_parallel_fwd(a, p->round_seq_ptr.data(), p->n_rounds);
+    }
+    const bool one_launch = !chunks && round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && chunk_states &&
                             !(flags & (HARTS_FLAG_ROUND_LAUNCHES | HARTS_FLAG_FMA_KERNELS)) &&
                             harts::gk_mma_supported(dtype, dk, dv);
     if (one_launch) {           // flags and tickets sit behind the chunk states, as for the scalar-gate calls
@@ -316,7 +343,7 @@ int32_t harts_la_gk_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32
                          dtype, flags, dev_status, static_cast<cudaStream_t>(stream)};
         if (flags & HARTS_FLAG_CHECK_TABLES)
             if ((rc = harts::check_tables(tb, a.seq_lo, a.seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
-        if ((rc = harts::gk_fwd(a)) != HARTS_OK) return rc;
+        if ((rc = chunks ? gk_chunk_parallel_fwd(a, &p->round_seq_ptr[r - 1], 1) : harts::gk_fwd(a)) != HARTS_OK) return rc;
     }
     return HARTS_OK;
 }
@@ -338,7 +365,16 @@ int32_t harts_la_gk_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32
     if ((flags & HARTS_FLAG_CHECK_TABLES) && !dev_status) return HARTS_EINVAL;
     const int32_t r1 = round == 0 ? p->n_rounds : round, r0 = round == 0 ? 1 : round;
     bool done = false;
-    if (round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS &&
+    const bool chunks = harts::gk_chunk_parallel(tb, H, dk, dv, dtype, flags);
+    if (chunks && round == 0 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && !(flags & HARTS_FLAG_ROUND_LAUNCHES)) {
+        harts::BwdArgs a{tb, 0, tb.n_seq, q, k, v, gk, dO, dq, dk_, dv_, dgk, chunk_states, scratch, H, dk, dv, dtype, flags,
+                         dev_status, static_cast<cudaStream_t>(stream)};
+        if (flags & HARTS_FLAG_CHECK_TABLES)
+            if ((rc = harts::check_tables(tb, 0, tb.n_seq, dev_status, a.stream)) != HARTS_OK) return rc;
+        if ((rc = gk_chunk_parallel_bwd(a, p->round_seq_ptr.data(), p->n_rounds)) != HARTS_OK) return rc;
+        done = true;
+    }
+    if (!chunks && round == 0 && p->n_rounds > 1 && p->n_rounds <= harts::MAX_FUSED_ROUNDS &&
         !(flags & (HARTS_FLAG_ROUND_LAUNCHES | HARTS_FLAG_FMA_KERNELS)) && harts::gk_mma_supported(dtype, dk, dv)) {
         harts::BwdArgs a{tb, 0, tb.n_seq, q, k, v, gk, dO, dq, dk_, dv_, dgk, chunk_states, scratch, H, dk, dv, dtype, flags,
                          dev_status, static_cast<cudaStream_t>(stream)};
@@ -358,7 +394,7 @@ int32_t harts_la_gk_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32
                          chunk_states, scratch, H, dk, dv, dtype, flags, dev_status, static_cast<cudaStream_t>(stream)};
         if (flags & HARTS_FLAG_CHECK_TABLES)
             if ((rc = harts::check_tables(tb, a.seq_lo, a.seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
-        if ((rc = harts::gk_bwd(a)) != HARTS_OK) return rc;
+        if ((rc = chunks ? gk_chunk_parallel_bwd(a, &p->round_seq_ptr[r - 1], 1) : harts::gk_bwd(a)) != HARTS_OK) return rc;
     }
     if (r0 == 1)
         return harts::gk_replay_reduce(tb, dk_, dv_, dgk, scratch, H, dk, dv, dtype, static_cast<cudaStream_t>(stream));

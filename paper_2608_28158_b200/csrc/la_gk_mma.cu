@@ -378,13 +378,14 @@ __device__ __forceinline__ void scores_diagonal(const unsigned char* sQ, const u
 }
 
 // q <- q .* e^{b_t} and k <- k .* e^{b_n - b_t} written to (possibly other) swizzled tiles
+template <bool Q = true, bool K = true>
 __device__ __forceinline__ void scale_qk(const unsigned char* sQ, const unsigned char* sK, const float* sB,
                                          unsigned char* dQ, unsigned char* dK) {
 #pragma unroll
     for (int u = 0; u < BT * 16 / NT; u++) {
         const int p = threadIdx.x + u * NT, t = p >> 4, c16 = p & 15;
         const uint32_t off = sw256(t, c16);
-        uint4 qv = *reinterpret_cast<const uint4*>(sQ + off), kv = *reinterpret_cast<const uint4*>(sK + off);
+        uint4 qv = *reinterpret_cast<const uint4*>((Q ? sQ : sK) + off), kv = *reinterpret_cast<const uint4*>((K ? sK : sQ) + off);
         uint32_t* qw = reinterpret_cast<uint32_t*>(&qv);
         uint32_t* kw = reinterpret_cast<uint32_t*>(&kv);
 #pragma unroll
@@ -394,11 +395,11 @@ __device__ __forceinline__ void scale_qk(const unsigned char* sQ, const unsigned
             const float2 bn = *reinterpret_cast<const float2*>(sB + (BT - 1) * D + i);
             const float2 qf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qw[e]));
             const float2 kf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kw[e]));
-            qw[e] = pack2(qf.x * ex2(bt.x), qf.y * ex2(bt.y));
-            kw[e] = pack2(kf.x * ex2(bn.x - bt.x), kf.y * ex2(bn.y - bt.y));
+            if (Q) qw[e] = pack2(qf.x * ex2(bt.x), qf.y * ex2(bt.y));
+            if (K) kw[e] = pack2(kf.x * ex2(bn.x - bt.x), kf.y * ex2(bn.y - bt.y));
         }
-        *reinterpret_cast<uint4*>(dQ + off) = qv;
-        *reinterpret_cast<uint4*>(dK + off) = kv;
+        if (Q) *reinterpret_cast<uint4*>(dQ + off) = qv;
+        if (K) *reinterpret_cast<uint4*>(dK + off) = kv;
     }
 }
 
@@ -478,17 +479,46 @@ __device__ __forceinline__ void tile_to_global(const unsigned char* tile, __nv_b
         reinterpret_cast<uint4*>(dst)[p] = *reinterpret_cast<const uint4*>(tile + sw256(p >> 4, p & 15));
 }
 
+// plain row-major [128][128] bf16 in global memory -> swizzled tile
+__device__ __forceinline__ void global_to_tile128(const __nv_bfloat16* src, unsigned char* tile) {
+    uint4 buf[D * 16 / NT];
+#pragma unroll
+    for (int u = 0; u < D * 16 / NT; u++) buf[u] = reinterpret_cast<const uint4*>(src)[threadIdx.x + u * NT];
+#pragma unroll
+    for (int u = 0; u < D * 16 / NT; u++) {
+        const int p = threadIdx.x + u * NT;
+        *reinterpret_cast<uint4*>(tile + sw256(p >> 4, p & 15)) = buf[u];
+    }
+}
+
+// the sequence of [seq_lo, seq_hi) that owns chunk gc (every warp searches, 32 ways at a time)
+__device__ __forceinline__ int owner_of(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int gc) {
+    const int lane = threadIdx.x & 31;
+    int lo = seq_lo, hi = seq_hi;
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32, i = lo + lane * step;
+        const unsigned m = __ballot_sync(~0u, i < hi && tb.seq_chunk_ptr[i] <= gc);
+        lo += (__popc(m) - 1) * step;
+        hi = min(hi, lo + step);
+    }
+    return lo;
+}
+
+// How a kernel is driven.
+// ROUND: one launch per round, item = (sequence, head) = block index, no flags.
+// CHUNKS: the boundary states (backward: their gradients too) are in memory (la_scan.cu), item = (chunk, head).
 // ONE_LAUNCH: the grid covers the sequences of ALL rounds (numbered round by round).  Every CTA draws its work item
 // from `ticket`, so an item is only ever held by a running CTA; a sequence that starts from an exported state waits for
 // the flag its producer (an earlier round, a smaller ticket, hence running or done) sets after writing the slot.
-// Otherwise: one launch per round, item = block index, no flags.
-template <bool ONE_LAUNCH>
+enum Mode { ROUND, ONE_LAUNCH_MODE, CHUNKS_MODE };
+template <int MODE>
 __global__ void __launch_bounds__(NT, 1)
-gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* __restrict__ q,
+gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                   __nv_bfloat16* __restrict__ o, float* __restrict__ slots, __nv_bfloat16* __restrict__ chunk_states,
                   const int32_t* gate, int* status, int* slot_flags, int* ticket) {
     if (gate_closed(gate)) return;
+    constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE, CHUNKS = MODE == CHUNKS_MODE;
     __shared__ int s_item, s_dead;
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sQ = sm + Shared::q, *sK = sm + Shared::k, *sV = sm + Shared::v, *sP = sm + Shared::p,
@@ -511,14 +541,18 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         __syncthreads();
         item = s_item;
     }
-    const int seq_pos = seq_lo + item / H, h = item % H;
-    const int seq = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
     const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
-    const SeqInfo s = seq_info(tb, seq);
     const size_t state_elems = (size_t)D * D;
+    const int chunk_lo = CHUNKS ? tb.seq_chunk_ptr[seq_lo] : 0, n_items = CHUNKS ? (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H : 0;
+    do {
+    if (CHUNKS && item >= n_items) break;
+    const int seq_pos = seq_lo + item / H, h = item % H, gc = chunk_lo + item / H;
+    const int seq = CHUNKS ? owner_of(tb, seq_lo, seq_hi, gc) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+    const SeqInfo s = seq_info(tb, seq);
 
     float st[8][4];
-    if (s.init_slot < 0) {
+    if (CHUNKS) {
+    } else if (s.init_slot < 0) {
 #pragma unroll
         for (int n = 0; n < 8; n++) st[n][0] = st[n][1] = st[n][2] = st[n][3] = 0.f;
     } else {
@@ -530,7 +564,9 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
     }
 
     int next_req = s.req_lo;
-    for (int c = 0; c < s.n_chunks; c++) {
+    const int c_lo = CHUNKS ? gc - s.chunk_base : 0, c_hi = CHUNKS ? c_lo + 1 : s.n_chunks;
+    for (int c = c_lo; c < c_hi; c++) {
+        const bool has_s = !CHUNKS || c > 0 || s.init_slot >= 0;      // the state of a sequence that starts from zero is not read
         __syncthreads();                                   // the previous chunk's readers of every tile are through
         load_codes(tb, s, c, srow);
         __syncthreads();
@@ -538,15 +574,16 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         load_tile_bf16(q, H, h, srow, true, sQ);
         load_tile_bf16(v, H, h, srow, false, sV);
         load_g(gk, H, h, srow, sB);
-        if (c + 1 < s.n_chunks) {
+        if (!CHUNKS && c + 1 < s.n_chunks) {
             prefetch_rows(k, H, h, s, c + 1);
             prefetch_rows(q, H, h, s, c + 1);
             prefetch_rows(v, H, h, s, c + 1);
             prefetch_rows(gk, H, h, s, c + 1);
         }
         // start-of-chunk state: operand copy, kept for the backward, exported when the plan requests this boundary
-        state_to_operand(st, sSb, warp, lane);
-        const bool exported = next_req < s.req_hi && tb.slot_chunk[next_req] == c;
+        if (!CHUNKS) state_to_operand(st, sSb, warp, lane);
+        else if (has_s) global_to_tile128(chunk_states + ((size_t)gc * H + h) * state_elems, sSb);
+        const bool exported = !CHUNKS && next_req < s.req_hi && tb.slot_chunk[next_req] == c;
         if (exported) {
             state_to_global(st, slots + ((size_t)next_req * H + h) * state_elems, warp, lane);
             if (ONE_LAUNCH) __threadfence();               // this thread's part of the slot, before the flag below
@@ -554,7 +591,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         }
         __syncthreads();
         if (ONE_LAUNCH && exported && tid == 0) tc::flag_set(slot_flags + (size_t)(next_req - 1) * H + h);
-        if (chunk_states) tile_to_global<D>(sSb, chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems);
+        if (!CHUNKS && chunk_states) tile_to_global<D>(sSb, chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems);
         cumsum_rows(sB, sTmp);
         const bool mild = chunk_is_mild(sB);
         unsigned char* sKd = reinterpret_cast<unsigned char*>(sR);        // the two are never needed in the same chunk
@@ -565,7 +602,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         if (!mild) scores_diagonal(sQ, sK, sR, sP, warp, lane);
         scores_off_diagonal(s_u32(sQa), s_u32(sKa), sP, warp, lane, mild, s_u32(sKd));
         __syncthreads();
-        scale_qk(sQ, sK, sB, sQ, sK);
+        scale_qk<true, !CHUNKS>(sQ, sK, sB, sQ, sK);
         __syncthreads();
         // ---- o = P V + q~ S_c : warp -> rows 16 * mb, columns 32 * nq ----------------------------------------------
         {
@@ -584,6 +621,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
+            if (has_s)
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4];
@@ -596,17 +634,19 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
-            const int c_lo = srow[m0 + g], c_hi = srow[m0 + g + 8];
+            const int row_lo = srow[m0 + g], row_hi = srow[m0 + g + 8];
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = n_base + n * 8 + tq * 2;
-                if (c_lo >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)c_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
-                if (c_hi >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)c_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
+                if (row_lo >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
+                if (row_hi >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
             }
         }
         // ---- S <- Diag(e^{b_n}) S + k~^T V ---------------------------------------------------------------------------
-        state_update(st, sB, aK, aV, warp, lane);
+        if (!CHUNKS) state_update(st, sB, aK, aV, warp, lane);
     }
+    item += gridDim.x;
+    } while (CHUNKS);
 }
 
 // ---- backward ---------------------------------------------------------------------------------------------------------
@@ -637,18 +677,6 @@ struct SharedB {
 };
 static_assert(SharedB::bytes <= 232448, "backward tiles do not fit in shared memory");
 
-// plain row-major [128][128] bf16 in global memory -> swizzled tile
-__device__ __forceinline__ void global_to_tile128(const __nv_bfloat16* src, unsigned char* tile) {
-    uint4 buf[D * 16 / NT];
-#pragma unroll
-    for (int u = 0; u < D * 16 / NT; u++) buf[u] = reinterpret_cast<const uint4*>(src)[threadIdx.x + u * NT];
-#pragma unroll
-    for (int u = 0; u < D * 16 / NT; u++) {
-        const int p = threadIdx.x + u * NT;
-        *reinterpret_cast<uint4*>(tile + sw256(p >> 4, p & 15)) = buf[u];
-    }
-}
-
 __device__ __forceinline__ float2 ld_bf2(const unsigned char* tile, int r, int col) {      // [r][col], [r][col+1]; col even
     return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + sw256(r, col >> 3) + (col & 7) * 2));
 }
@@ -658,15 +686,17 @@ __device__ __forceinline__ float2 ld_bf2(const unsigned char* tile, int r, int c
 // inside a round the plan's order).  A sequence publishes a flag once its initial-state gradient is in the scratch area;
 // a sequence that exported a boundary waits for the flags of all sequences that started there (later rounds, smaller
 // tickets, hence running or done) and sums their gradients itself in the order handoff_reduce uses.
-template <bool ONE_LAUNCH>
+template <int MODE>
 __global__ void __launch_bounds__(NT, 1)
-gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* __restrict__ q,
+gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                   const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk_,
                   __nv_bfloat16* __restrict__ dv_, float* __restrict__ dgk, const __nv_bfloat16* __restrict__ chunk_states,
+                  const __nv_bfloat16* __restrict__ ds_tiles,
                   float* __restrict__ ds0, float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg,
                   const int32_t* gate, int* status, int* ds0_flags, int* ticket, const RoundOrder rounds) {
     if (gate_closed(gate)) return;
+    constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE, CHUNKS = MODE == CHUNKS_MODE;
     __shared__ int s_item, s_dead;
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sQ = sm + SharedB::q, *sK = sm + SharedB::k, *sV = sm + SharedB::v, *sDO = sm + SharedB::dO,
@@ -687,7 +717,12 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
     // blocks are handed to the SMs in index order: with the plan's order (longest sequence of the round first) the long
     // walks start first and the short ones fill the tail
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
-    int seq_pos = seq_lo + blockIdx.x / H, h = blockIdx.x % H;
+    const int chunk_lo = CHUNKS ? tb.seq_chunk_ptr[seq_lo] : 0, n_items = CHUNKS ? (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H : 0;
+    int item = blockIdx.x;
+    do {
+    if (CHUNKS && item >= n_items) break;
+    int seq_pos = seq_lo + item / H, h = item % H;
+    const int gc = chunk_lo + item / H;
     if constexpr (ONE_LAUNCH) {
         if (tid == 0) {
             s_item = atomicAdd(ticket, 1);
@@ -703,7 +738,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
             else j -= cnt;
         }
     }
-    const int seq = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+    const int seq = CHUNKS ? owner_of(tb, seq_lo, seq_hi, gc) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
     const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
     const SeqInfo s = seq_info(tb, seq);
     const size_t state_elems = (size_t)D * D;
@@ -713,11 +748,14 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
     for (int n = 0; n < 8; n++) ds[n][0] = ds[n][1] = ds[n][2] = ds[n][3] = 0.f;
 
     int next_req = s.req_hi - 1;                      // slots of this sequence are ordered by chunk index
-    for (int c = s.n_chunks - 1; c >= 0; c--) {
+    const int c_hi = CHUNKS ? gc - s.chunk_base : s.n_chunks - 1, c_lo = CHUNKS ? c_hi : 0;
+    for (int c = c_hi; c >= c_lo; c--) {
+        // zero, and neither read nor multiplied: the state of a sequence that starts from zero, the gradient after a last chunk
+        const bool has_s = !CHUNKS || c > 0 || s.init_slot >= 0, has_ds = !CHUNKS || c + 1 < s.n_chunks;
         __syncthreads();                              // the previous chunk's readers of every tile are through
         // gradient arriving at boundary c+1 from the sequences that started there: one launch per round -- summed into
         // the first consumer's buffer by handoff_reduce; all rounds in one launch -- awaited and summed here, same order
-        if (next_req >= s.req_lo && tb.slot_chunk[next_req] == c + 1) {
+        if (!CHUNKS && next_req >= s.req_lo && tb.slot_chunk[next_req] == c + 1) {
             const int cons_lo = tb.slot_cons_ptr[next_req], cons_hi = tb.slot_cons_ptr[next_req + 1];
             if constexpr (ONE_LAUNCH) {
                 for (int u = cons_lo + tid; u < cons_hi; u += NT)
@@ -747,8 +785,8 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         load_tile_bf16(v, H, h, srow, false, sV);
         load_tile_bf16(dO, H, h, srow, true, sDO);
         load_g(gk, H, h, srow, sB);
-        global_to_tile128(chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems, sSc);
-        if (c >= 1) {      // the next chunk of the walk (chunk 0 of a sequence with replayed rows is not consecutive)
+        if (has_s) global_to_tile128(chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems, sSc);
+        if (!CHUNKS && c >= 1) {      // the next chunk of the walk (chunk 0 of a sequence with replayed rows is not consecutive)
             if (c - 1 >= 1 || s.n_replay == 0) {
                 prefetch_rows(k, H, h, s, c - 1);
                 prefetch_rows(q, H, h, s, c - 1);
@@ -759,7 +797,8 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
             const char* st = reinterpret_cast<const char*>(chunk_states + ((size_t)(s.chunk_base + c - 1) * H + h) * state_elems);
             for (int p = tid; p < D * D * 2 / 128; p += NT) asm volatile("prefetch.global.L2 [%0];" ::"l"(st + p * 128));
         }
-        state_to_operand(ds, sdSb, warp, lane);
+        if (!CHUNKS) state_to_operand(ds, sdSb, warp, lane);
+        else if (has_ds) global_to_tile128(ds_tiles + ((size_t)gc * H + h) * state_elems, sdSb);
         __syncthreads();
         cumsum_rows(sB, sTmp);
         const bool mild = chunk_is_mild(sB);          // diagonal blocks as dense products too (see chunk_is_mild)
@@ -782,12 +821,14 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                 frag_b_nk<256>(b, aV, ks * 16, 16 * nq, lane);          // dA: columns (keys) 16 * nq ..
                 mma16816(da[0], a, b[0], b[1]);
                 mma16816(da[1], a, b[2], b[3]);
+                if (has_s)
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
                     frag_b_nk<256>(b, aSc, ks * 16, 32 * nq + 16 * n2, lane);
                     mma16816(iq[2 * n2], a, b[0], b[1]);
                     mma16816(iq[2 * n2 + 1], a, b[2], b[3]);
                 }
+                if (!has_ds) continue;
                 frag_a<256>(a, aV, 16 * mb, ks * 16, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
@@ -816,11 +857,18 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         {   // <S_c[i,:], dS[i,:]> over this warp's 64 columns of its 16 state rows i (the two column halves meet later)
             const int i0 = (warp & 7) * 16 + g, c0 = (warp >> 3) * 64 + tq * 2;
             float d_lo = 0.f, d_hi = 0.f;
+            if (has_s && has_ds)
 #pragma unroll
             for (int n = 0; n < 8; n++) {
                 const float2 s_lo = ld_bf2(sSc, i0, c0 + n * 8), s_hi = ld_bf2(sSc, i0 + 8, c0 + n * 8);
-                d_lo += s_lo.x * ds[n][0] + s_lo.y * ds[n][1];
-                d_hi += s_hi.x * ds[n][2] + s_hi.y * ds[n][3];
+                if constexpr (CHUNKS) {
+                    const float2 x_lo = ld_bf2(sdSb, i0, c0 + n * 8), x_hi = ld_bf2(sdSb, i0 + 8, c0 + n * 8);
+                    d_lo += s_lo.x * x_lo.x + s_lo.y * x_lo.y;
+                    d_hi += s_hi.x * x_hi.x + s_hi.y * x_hi.y;
+                } else {
+                    d_lo += s_lo.x * ds[n][0] + s_lo.y * ds[n][1];
+                    d_hi += s_hi.x * ds[n][2] + s_hi.y * ds[n][3];
+                }
             }
             d_lo += __shfl_xor_sync(0xffffffffu, d_lo, 1); d_lo += __shfl_xor_sync(0xffffffffu, d_lo, 2);
             d_hi += __shfl_xor_sync(0xffffffffu, d_hi, 1); d_hi += __shfl_xor_sync(0xffffffffu, d_hi, 2);
@@ -1002,7 +1050,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                 *reinterpret_cast<float4*>(dst + 4) = k1;
             }
         }
-        scale_qk(sQ, sK, sB, sQ, sK);                 // q~, k~ over the raw tiles, which nobody reads any more
+        scale_qk<!CHUNKS, true>(sQ, sK, sB, sQ, sK);  // q~, k~ over the raw tiles, which nobody reads any more
         __syncthreads();
         // ---- dv_j = sum_{t>=j} A_tj dO_t + k~_j dS : warp -> rows 16 * mb, columns 32 * nq -------------------------------
         {
@@ -1019,6 +1067,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
+            if (has_ds)
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4], b[4];
@@ -1030,20 +1079,20 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
-            const int c_lo = srow[r_lo], c_hi = srow[r_hi];
+            const int row_lo = srow[r_lo], row_hi = srow[r_hi];
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = 32 * nq + 8 * n + 2 * tq;
-                if (c_lo >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)c_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
-                else if (c_lo < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_lo) * H + h) * D + col) = make_float2(acc[n][0], acc[n][1]);
-                if (c_hi >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)c_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
-                else if (c_hi < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_hi) * H + h) * D + col) = make_float2(acc[n][2], acc[n][3]);
+                if (row_lo >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)row_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
+                else if (row_lo < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_lo) * H + h) * D + col) = make_float2(acc[n][0], acc[n][1]);
+                if (row_hi >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)row_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
+                else if (row_hi < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_hi) * H + h) * D + col) = make_float2(acc[n][2], acc[n][3]);
             }
         }
         // ---- dS <- Diag(e^{b_n}) dS + q~^T dO ---------------------------------------------------------------------------
-        state_update(ds, sB, aQ, aDO, warp, lane);
+        if (!CHUNKS) state_update(ds, sB, aQ, aDO, warp, lane);
     }
-    if (s.init_slot >= 0) {
+    if (!CHUNKS && s.init_slot >= 0) {
         state_to_global(ds, ds0 + ((size_t)seq * H + h) * state_elems, warp, lane);
         if constexpr (ONE_LAUNCH) {
             __threadfence();                           // this thread's part, before the flag that follows the barrier
@@ -1051,6 +1100,8 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
             if (tid == 0) tc::flag_set(ds0_flags + (size_t)seq * H + h);
         }
     }
+    item += gridDim.x;
+    } while (CHUNKS);
 }
 
 }  // namespace
@@ -1059,12 +1110,12 @@ int32_t gk_mma_supported(int32_t dtype, int32_t dk, int32_t dv) { return dtype =
 
 int32_t gk_mma_fwd(const FwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) !=
+    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<ROUND>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) !=
         cudaSuccess)
         return HARTS_ECUDA;
     const int n = (a.seq_hi - a.seq_lo) * a.H;
-    gk_mma_fwd_kernel<false><<<n, NT, Shared::fwd_bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+    gk_mma_fwd_kernel<ROUND><<<n, NT, Shared::fwd_bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
         nullptr, nullptr);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -1072,16 +1123,16 @@ int32_t gk_mma_fwd(const FwdArgs& a) {
 
 int32_t gk_mma_bwd(const BwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    if (cudaFuncSetAttribute(gk_mma_bwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) !=
+    if (cudaFuncSetAttribute(gk_mma_bwd_kernel<ROUND>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) !=
         cudaSuccess)
         return HARTS_ECUDA;
     const int n = (a.seq_hi - a.seq_lo) * a.H;
     const GkScratchLayout sl = gk_scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
-    gk_mma_bwd_kernel<false><<<n, NT, SharedB::bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+    gk_mma_bwd_kernel<ROUND><<<n, NT, SharedB::bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
@@ -1093,15 +1144,15 @@ int32_t gk_mma_fwd_all(const FwdArgs& a, int* flags, int* ticket) {
     const int64_t n = (int64_t)(a.seq_hi - a.seq_lo) * a.H;
     if (n == 0) return HARTS_OK;
     if (n > (int64_t)ONE_LAUNCH_ITEMS_PER_CTA * sm_count()) return HARTS_EUNSUPPORTED;
-    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) !=
+    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<ONE_LAUNCH_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) !=
         cudaSuccess)
         return HARTS_ECUDA;
     if (a.tb.n_slots > 0 &&
         cudaMemsetAsync(flags, 0, (size_t)a.tb.n_slots * a.H * sizeof(int), a.stream) != cudaSuccess)
         return HARTS_ECUDA;
     if (cudaMemsetAsync(ticket, 0, sizeof(int), a.stream) != cudaSuccess) return HARTS_ECUDA;
-    gk_mma_fwd_kernel<true><<<(int)n, NT, Shared::fwd_bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+    gk_mma_fwd_kernel<ONE_LAUNCH_MODE><<<(int)n, NT, Shared::fwd_bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
         flags, ticket);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -1112,18 +1163,45 @@ int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrd
     if (n == 0) return HARTS_OK;
     if (rounds.n < 1 || rounds.ptr[0] != a.seq_lo || rounds.ptr[rounds.n] != a.seq_hi) return HARTS_EINVAL;
     if (n > (int64_t)ONE_LAUNCH_ITEMS_PER_CTA * sm_count()) return HARTS_EUNSUPPORTED;
-    if (cudaFuncSetAttribute(gk_mma_bwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) !=
+    if (cudaFuncSetAttribute(gk_mma_bwd_kernel<ONE_LAUNCH_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) !=
         cudaSuccess)
         return HARTS_ECUDA;
     if (cudaMemsetAsync(flags, 0, (size_t)a.tb.n_seq * a.H * sizeof(int), a.stream) != cudaSuccess) return HARTS_ECUDA;
     if (cudaMemsetAsync(ticket, 0, sizeof(int), a.stream) != cudaSuccess) return HARTS_ECUDA;
     const GkScratchLayout sl = gk_scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
-    gk_mma_bwd_kernel<true><<<(int)n, NT, SharedB::bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+    gk_mma_bwd_kernel<ONE_LAUNCH_MODE><<<(int)n, NT, SharedB::bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, flags, ticket, rounds);
+    return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
+}
+
+// Every (chunk, head) of sequences [seq_lo, seq_hi) on its own; the scan has left the states (and their gradients).
+int32_t gk_chunk_fwd(const FwdArgs& a) {
+    if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<CHUNKS_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) != cudaSuccess)
+        return HARTS_ECUDA;
+    const int64_t n = (int64_t)a.tb.n_chunks * a.H;
+    gk_mma_fwd_kernel<CHUNKS_MODE><<<(int)(n < sm_count() ? n : sm_count()), NT, Shared::fwd_bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+        (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
+        nullptr, nullptr);
+    return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
+}
+int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
+    if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    if (cudaFuncSetAttribute(gk_mma_bwd_kernel<CHUNKS_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) != cudaSuccess)
+        return HARTS_ECUDA;
+    const int64_t n = (int64_t)a.tb.n_chunks * a.H;
+    const GkScratchLayout sl = gk_scratch_layout(a.tb, a.H, a.dk, a.dv);
+    char* base = static_cast<char*>(a.scratch);
+    gk_mma_bwd_kernel<CHUNKS_MODE><<<(int)(n < sm_count() ? n : sm_count()), NT, SharedB::bytes, a.stream>>>(
+        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+        (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
+        (const __nv_bfloat16*)a.chunk_states, (const __nv_bfloat16*)ds_tiles, (float*)(base + sl.ds0), (float*)(base + sl.rk),
+        (float*)(base + sl.rv), (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

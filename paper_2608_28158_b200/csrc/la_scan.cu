@@ -24,6 +24,7 @@ namespace harts {
 int32_t make_row_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
 int32_t make_state_map(CUtensorMap* map, const void* base, int64_t n);
 int32_t make_state_slice_map(CUtensorMap* map, const void* base, int64_t n);
+int32_t make_gate_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
 int sm_count();
 
 namespace {
@@ -31,19 +32,21 @@ namespace {
 using namespace tc;
 
 constexpr int BT = 64, D = 128;
-constexpr int GATES = 4, RAW = 8, OUTS = 3, ITEMS = 4;      // rings: weights, raw log-decays, tiles on their way out, items
+constexpr int GATES = 4, RAW = 8, ITEMS = 4;      // rings: weights, raw log-decays, items
 constexpr int PANEL = BT * 128, S_PANEL = D * 128;
 constexpr float LOG2E = 1.4426950408889634f;
 
-template <int NV>
+template <int NV, bool GK>
 struct Shape {
     static constexpr int NS = NV == 32 ? 128 : 256, NWT = NS, NT = NS + NWT + 128;   // state threads, weighting threads, four warps
     static constexpr int CW = NV * 128 / NS;               // state columns per state thread
-    static constexpr int STAGES = NV == 64 ? 5 : 3;        // chunks of rows in shared memory
+    static constexpr int STAGES = GK ? 2 : NV == 64 ? 5 : 3;        // chunks of rows in shared memory
+    static constexpr int OUTS = GK ? 2 : 3;                // state tiles on their way out
     // a 32-column slice loads the 64-column panel it lies in
-    static constexpr int A = 2 * PANEL, B = (NV + 63) / 64 * PANEL, O = D * NV * 2;
-    static constexpr int a = 0, b = STAGES * A, out = b + STAGES * B, misc = out + OUTS * O,
-                         bytes = misc + 4096 + 1024;      // 1024: alignment of the dynamic area
+    static constexpr int A = 2 * PANEL, B = (NV + 63) / 64 * PANEL, G = GK ? BT * D * 4 : 0,
+                         O = D * NV * 2;
+    static constexpr int a = 0, b = STAGES * A, g = b + STAGES * B, out = g + STAGES * G, misc = out + OUTS * O,
+                         bytes = misc + 12288 + 1024;      // 1024: alignment of the dynamic area
 };
 struct Item {                // one (sequence, head, slice); seq < 0: no more
     int seq, h, slice, own_begin, n_replay, n_virtual, n_chunks, chunk_base, replay_base, init_slot, req_lo, req_hi;
@@ -53,28 +56,32 @@ struct Misc {
     float w[GATES][BT];
     float gamma[GATES];
     float raw[RAW][BT];
-    uint64_t full[5], weighted[5], stage_empty[5], u_full[2], u_empty[2], gates_full[GATES], gates_empty[GATES], out_full[OUTS],
-        out_empty[OUTS], item_full[ITEMS], item_empty[ITEMS];
+    float gammas[GATES][D];      // per-channel decay: e^{b_n} of every state row
+    float part[2][4][D];         // and the sums of four groups of 16 rows, of every second step
+    uint64_t full[5], weighted[5], stage_empty[5], u_full[2], u_empty[2], gates_full[GATES], gates_empty[GATES], out_full[3],
+        out_empty[3], item_full[ITEMS], item_empty[ITEMS], part_full[2];
     Item items[ITEMS];
     uint32_t tmem;
     int dead;
 };
-static_assert(sizeof(Misc) <= 4096, "misc area");
+static_assert(sizeof(Misc) <= 12288, "misc area");
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
 // a: the operand that spans the state's rows (k forward, q backward), b: the one that spans its columns (v / dO).
-template <bool BWD, int NV>
-__global__ void __launch_bounds__(Shape<NV>::NT, NV == 32 ? 2 : 1)
+// GK: a log-decay per row and state row (g [rows, H, 128]): its tile travels with the rows, and the weights go onto a.
+template <bool BWD, int NV, bool GK>
+__global__ void __launch_bounds__(Shape<NV, GK>::NT, NV == 32 ? 2 : 1)
 scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __grid_constant__ CUtensorMap map_a,
-            const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_tiles,
+            const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_g,
+            const __grid_constant__ CUtensorMap map_tiles,
             const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ b, const float* __restrict__ g,
             float* slots, float* ds0, int* status, const int32_t* gate, int* flags, int* ticket, const RoundOrder order) {
     if (gate_closed(gate)) return;
-    using S = Shape<NV>;
-    constexpr int SLICES = D / NV, NS = S::NS, NWT = S::NWT, CW = S::CW, STAGES = S::STAGES;
+    using S = Shape<NV, GK>;
+    constexpr int SLICES = D / NV, NS = S::NS, NWT = S::NWT, CW = S::CW, STAGES = S::STAGES, OUTS = S::OUTS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     Misc& m = *reinterpret_cast<Misc*>(smem + S::misc);
@@ -86,11 +93,12 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             mbar_init(&m.stage_empty[i], 1);
         }
         for (int i = 0; i < GATES; i++) {
-            mbar_init(&m.gates_full[i], 1);
-            mbar_init(&m.gates_empty[i], (NS + NWT) / 32);
+            mbar_init(&m.gates_full[i], GK ? NWT / 32 : 1);
+            mbar_init(&m.gates_empty[i], GK ? NS / 32 : (NS + NWT) / 32);
         }
         for (int i = 0; i < 2; i++) {
             mbar_init(&m.u_full[i], 1);
+            mbar_init(&m.part_full[i], NWT / 32);
             mbar_init(&m.u_empty[i], NS / 32);
         }
         for (int i = 0; i < OUTS; i++) {
@@ -99,7 +107,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
         }
         for (int i = 0; i < ITEMS; i++) {
             mbar_init(&m.item_full[i], 1);
-            mbar_init(&m.item_empty[i], (NS + NWT) / 32 + 3);
+            mbar_init(&m.item_empty[i], (NS + NWT) / 32 + (GK ? 2 : 3));
         }
         m.dead = 0;
         fence_barrier_init();
@@ -182,7 +190,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 }
                 if (i >= it.n_steps) break;
                 if (!wait_warp(&m.gates_full[gs % GATES], gs / GATES) || !wait_warp(&m.u_full[gs & 1], gs >> 1)) alive = false;
-                const float gamma = m.gamma[gs % GATES];
+                const float gamma = GK ? m.gammas[gs % GATES][L] : m.gamma[gs % GATES];
                 tc_fence_after();
 #pragma unroll
                 for (int blk = 0; blk < CW / 16; blk++) {
@@ -214,12 +222,53 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
         int gs = 0;
         bool alive = true;
         for (int k = 0; alive && wait_warp(&m.item_full[k % ITEMS], k / ITEMS); k++) {
-            const int seq = m.items[k % ITEMS].seq, n_steps = m.items[k % ITEMS].n_steps, slice = m.items[k % ITEMS].slice;
+            const Item it = m.items[k % ITEMS];
+            const int slice = it.slice;
             __syncwarp();
             if (lane == 0) mbar_arrive(&m.item_empty[k % ITEMS]);
-            if (seq < 0) break;
-            for (int i = 0; i < n_steps; i++, gs++) {
+            if (it.seq < 0) break;
+            for (int i = 0; i < it.n_steps; i++, gs++) {
                 const int st = gs % STAGES;
+                if constexpr (GK) {
+                    // thread = two channels x 16 rows: running sums of its rows, joined over the four row groups
+                    const int i0 = 2 * (wt & 63), grp = wt >> 6, n_rows = min(BT, it.n_virtual - chunk_of(it, i) * BT);
+                    const int first = BWD && chunk_of(it, i) == 0 ? it.n_replay : 0;      // rows before it carry no weight
+                    alive = (gs < GATES || wait_warp(&m.gates_empty[gs % GATES], gs / GATES - 1)) && wait_warp(&m.full[st], gs / STAGES);
+                    if (!alive) break;
+                    const float* sg = reinterpret_cast<const float*>(smem + S::g + st * S::G) + i0;
+                    float2 run[16];
+                    float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int u = 0; u < 16; u++) {
+                        const int t = 16 * grp + u;
+                        const float2 x = *reinterpret_cast<const float2*>(sg + t * D);
+                        sum.x += t < n_rows ? x.x * LOG2E : 0.f;
+                        sum.y += t < n_rows ? x.y * LOG2E : 0.f;
+                        run[u] = sum;
+                    }
+                    *reinterpret_cast<float2*>(&m.part[gs & 1][grp][i0]) = sum;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&m.part_full[gs & 1]);
+                    if (!(alive = wait_warp(&m.part_full[gs & 1], gs >> 1))) break;
+                    float2 before = make_float2(0.f, 0.f), bn = before;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const float2 x = *reinterpret_cast<const float2*>(&m.part[gs & 1][q][i0]);
+                        if (q < grp) before.x += x.x, before.y += x.y;
+                        bn.x += x.x, bn.y += x.y;
+                    }
+                    if (grp == 0) *reinterpret_cast<float2*>(&m.gammas[gs % GATES][i0]) = make_float2(ex2(bn.x), ex2(bn.y));
+                    unsigned char* sa = smem + S::a + st * S::A + (i0 >> 6) * PANEL + (i0 & 7) * 2;
+#pragma unroll
+                    for (int u = 0; u < 16; u++) {
+                        const int t = 16 * grp + u;
+                        uint32_t* at = reinterpret_cast<uint32_t*>(sa + sw128_chunk(t, (i0 & 63) >> 3));
+                        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(at));
+                        const float b0 = before.x + run[u].x, b1 = before.y + run[u].y;
+                        const uint32_t y = pack_bf16(f.x * ex2(BWD ? b0 : bn.x - b0), f.y * ex2(BWD ? b1 : bn.y - b1));
+                        *at = BWD && (t < first || t >= n_rows) ? 0u : y;
+                    }
+                } else {
                 alive = wait_warp(&m.gates_full[gs % GATES], gs / GATES) && wait_warp(&m.full[st], gs / STAGES);
                 if (!alive) break;
                 unsigned char* sb = smem + S::b + st * S::B;
@@ -239,11 +288,12 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     }
                     *at = BWD && wv == 0.f ? make_uint4(0, 0, 0, 0) : y;
                 }
+                }
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(&m.weighted[st]);
-                    mbar_arrive(&m.gates_empty[gs % GATES]);
+                    mbar_arrive(GK ? &m.gates_full[gs % GATES] : &m.gates_empty[gs % GATES]);
                 }
             }
         }
@@ -299,28 +349,36 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 unsigned char *sa = smem + S::a + st * S::A, *sb = smem + S::b + st * S::B;
                 const int b0 = it.slice * NV / 64 * 64;
                 if (gs >= STAGES && !(alive = wait_warp(&m.stage_empty[st], gs / STAGES - 1))) break;
-                if (!BWD && i == 0 && it.n_replay > 0) {      // chunk 0 begins with rows from anywhere: row by row
+                // chunk 0 begins with rows from anywhere: row by row (backward: only the gates of replayed rows count)
+                if ((GK || !BWD) && chunk_of(it, i) == 0 && it.n_replay > 0) {
                     int row[2];
 #pragma unroll
                     for (int u = 0; u < 2; u++) {
                         const int t = lane + 32 * u;
-                        row[u] = t < it.n_replay ? tb.replay_row[it.replay_base + t] : it.own_begin + t - it.n_replay;
+                        row[u] = t < it.n_replay ? tb.replay_row[it.replay_base + t] : min(it.own_begin + t - it.n_replay, tb.n_rows - 1);
                     }
 #pragma unroll 4
                     for (int t = 0; t < BT; t++) {
                         const size_t r = ((size_t)__shfl_sync(~0u, t < 32 ? row[0] : row[1], t & 31) * H + it.h) * D;
                         const int ch = lane & 15;
-                        if (lane < 16)
-                            cp_async16(smem_u32(sa + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), a + r + ch * 8);
-                        else if (ch < S::B / PANEL * 8)
-                            cp_async16(smem_u32(sb + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), b + r + b0 + ch * 8);
+                        if (!BWD || t >= it.n_replay) {
+                            if (lane < 16)
+                                cp_async16(smem_u32(sa + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), a + r + ch * 8);
+                            else if (ch < S::B / PANEL * 8)
+                                cp_async16(smem_u32(sb + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), b + r + b0 + ch * 8);
+                        } else {
+                            *reinterpret_cast<uint4*>((lane < 16 ? sa : sb) + (lane < 16 || S::B > PANEL ? (ch >> 3) * PANEL : 0) + sw128_chunk(t, ch & 7)) =
+                                make_uint4(0, 0, 0, 0);
+                        }
+                        if (GK) cp_async16(smem_u32(smem + S::g + st * S::G + t * (D * 4) + lane * 16), g + r + lane * 4);
                     }
                     asm volatile("cp.async.wait_all;" ::: "memory");
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&m.full[st]);
                 } else if (lane == 0) {
-                    mbar_expect_tx(&m.full[st], S::A + S::B);
+                    mbar_expect_tx(&m.full[st], S::A + S::B + S::G);
+                    if (GK) tma_load_3d(smem + S::g + st * S::G, &map_g, 0, it.h, row0, &m.full[st]);
                     for (int p = 0; p < 2; p++) tma_load_3d(sa + p * PANEL, &map_a, p * 64, it.h, row0, &m.full[st]);
                     for (int p = 0; p < S::B / PANEL; p++) tma_load_3d(sb + p * PANEL, &map_b, b0 + p * 64, it.h, row0, &m.full[st]);
                 }
@@ -351,6 +409,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 }
             }
     } else if (warp == (NS + NWT) / 32 + 2) {
+        if constexpr (!GK) {
         // ---- gates: log-decays (four bytes each, rows are H apart) five steps ahead, running sums -> weights --------------------
         int gs = 0;
         bool alive = true;
@@ -399,6 +458,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             __syncwarp();
         }
+        }
     } else {
         // ---- tile stores ---------------------------------------------------------------------------------------------------------
         int gt = 0;
@@ -442,23 +502,26 @@ struct Launch {
     cudaStream_t stream;
 };
 
-template <bool BWD, int NV>
+template <bool BWD, int NV, bool GK>
 int32_t launch(const Launch& x) {
-    CUtensorMap ma, mb, mt;
+    using S = Shape<NV, GK>;
+    CUtensorMap ma, mb, mg, mt;
     int32_t rc;
     const int64_t n_tiles = (int64_t)x.tb.n_chunks * x.H;
     if ((rc = make_row_map(&ma, x.a, x.tb.n_rows, x.H)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mb, x.b, x.tb.n_rows, x.H)) != HARTS_OK) return rc;
+    mg = ma;
+    if (GK && (rc = make_gate_map(&mg, x.g, x.tb.n_rows, x.H)) != HARTS_OK) return rc;
     if ((rc = NV == 32 ? make_state_slice_map(&mt, x.tiles, n_tiles) : make_state_map(&mt, x.tiles, n_tiles)) != HARTS_OK) return rc;
-    if (cudaFuncSetAttribute(scan_kernel<BWD, NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<NV>::bytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(scan_kernel<BWD, NV, GK>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int n = (x.seq_hi - x.seq_lo) * x.H * (D / NV), resident = (NV == 32 ? 2 : 1) * sm_count();
     if (x.order.n) {
         const size_t n_flags = (size_t)(BWD ? x.tb.n_seq : x.tb.n_slots) * x.H * (D / NV);
         if (cudaMemsetAsync(x.flags, 0, (4 + n_flags) * sizeof(int), x.stream) != cudaSuccess) return HARTS_ECUDA;
     }
-    scan_kernel<BWD, NV><<<n < resident ? n : resident, Shape<NV>::NT, Shape<NV>::bytes, x.stream>>>(
-        x.tb, x.seq_lo, n, x.H, ma, mb, mt, (const __nv_bfloat16*)x.a, (const __nv_bfloat16*)x.b, x.g, x.slots, x.ds0, x.status, x.gate,
+    scan_kernel<BWD, NV, GK><<<n < resident ? n : resident, S::NT, S::bytes, x.stream>>>(
+        x.tb, x.seq_lo, n, x.H, ma, mb, mg, mt, (const __nv_bfloat16*)x.a, (const __nv_bfloat16*)x.b, x.g, x.slots, x.ds0, x.status, x.gate,
         x.flags + 4, x.flags, x.order);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
@@ -468,7 +531,7 @@ int32_t launch(const Launch& x) {
 template <bool BWD>
 int32_t launch_sliced(const Launch& x) {
     const int chains = (x.order.n ? x.order.ptr[1] - x.order.ptr[0] : x.seq_hi - x.seq_lo) * x.H;
-    return 4 * chains <= sm_count() ? launch<BWD, 32>(x) : 2 * chains <= sm_count() ? launch<BWD, 64>(x) : launch<BWD, 128>(x);
+    return 4 * chains <= sm_count() ? launch<BWD, 32, false>(x) : 2 * chains <= sm_count() ? launch<BWD, 64, false>(x) : launch<BWD, 128, false>(x);
 }
 
 }  // namespace
@@ -489,6 +552,25 @@ int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder&
     float* ds0 = (float*)((char*)a.scratch + scratch_layout(a.tb, a.H, a.dk, a.dv).ds0);
     return launch_sliced<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, nullptr, ds0, a.dev_status,
                                 status_gate(a.flags, a.dev_status), flags, order, a.stream});
+}
+
+// The same with a log-decay per key channel (FwdArgs::g / BwdArgs::g point to [rows, H, 128]): two slices of 64 columns while
+// that leaves every SM at most one CTA, else one of 128 (the gate tile is as large as k and v together, so slices cost more).
+template <bool BWD>
+static int32_t launch_gk(const Launch& x) {
+    const int chains = (x.order.n ? x.order.ptr[1] - x.order.ptr[0] : x.seq_hi - x.seq_lo) * x.H;
+    return 2 * chains <= sm_count() ? launch<BWD, 64, true>(x) : launch<BWD, 128, true>(x);
+}
+int32_t gk_scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order) {
+    if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    return launch_gk<false>({a.tb, a.seq_lo, a.seq_hi, a.H, a.k, a.v, a.g, a.chunk_states, a.slots, nullptr, a.dev_status,
+                             status_gate(a.flags, a.dev_status), flags, order, a.stream});
+}
+int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order) {
+    if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    float* ds0 = (float*)((char*)a.scratch + gk_scratch_layout(a.tb, a.H, a.dk, a.dv).ds0);
+    return launch_gk<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, nullptr, ds0, a.dev_status,
+                            status_gate(a.flags, a.dev_status), flags, order, a.stream});
 }
 
 }  // namespace harts

@@ -528,6 +528,18 @@ int32_t make_state_slice_map(CUtensorMap* map, const void* base, int64_t n) {
     return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
 }
 
+// [rows][H][128] fp32 tensor, box = 64 rows x 1 head x 128 columns, plain rows
+int32_t make_gate_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return HARTS_ECUDA;
+    cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)rows}, strides[2] = {512, (cuuint64_t)H * 512};
+    cuuint32_t box[3] = {128, 1, 64}, es[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+}
+
 // [rows][H][128] bf16 output tensor, box = 64 rows x 1 head x 128 columns, plain (unswizzled) rows
 int32_t make_out_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H) {
     EncodeTiledFn fn = encode_fn();
