@@ -171,6 +171,21 @@ __device__ __forceinline__ void prefetch_rows(const T* base, int H, int h, const
     }
 }
 
+// The same for the CTA's next (chunk, head) item of the chunk-parallel kernels, where that is a chunk of the same sequence.
+struct NextItem {
+    int c, h, gc;            // c < 0: none
+};
+__device__ __forceinline__ NextItem next_item(const SeqInfo& s, int c, int gc, int item, int H, int n_items) {
+    const int nx = item + gridDim.x, d = nx / H - item / H;
+    NextItem n{c + d, nx % H, gc + d};
+    if (nx >= n_items || n.c >= s.n_chunks) n.c = -1;
+    return n;
+}
+__device__ __forceinline__ void prefetch_state(const __nv_bfloat16* tiles, int gc, int h, int H) {
+    const char* st = reinterpret_cast<const char*>(tiles + ((size_t)gc * H + h) * (D * D));
+    for (int p = threadIdx.x; p < D * D * 2 / 128; p += NT) asm volatile("prefetch.global.L2 [%0];" ::"l"(st + p * 128));
+}
+
 // running sum over the rows, per channel: four threads per channel (16 rows each, scanned in registers), joined through
 // sTmp[4][128]
 __device__ __forceinline__ void cumsum_rows(float* sB, float* sTmp) {
@@ -574,7 +589,16 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         load_tile_bf16(q, H, h, srow, true, sQ);
         load_tile_bf16(v, H, h, srow, false, sV);
         load_g(gk, H, h, srow, sB);
-        if (!CHUNKS && c + 1 < s.n_chunks) {
+        if (CHUNKS) {
+            const NextItem nx = next_item(s, c, gc, item, H, n_items);
+            if (nx.c >= 0) {
+                prefetch_rows(k, H, nx.h, s, nx.c);
+                prefetch_rows(q, H, nx.h, s, nx.c);
+                prefetch_rows(v, H, nx.h, s, nx.c);
+                prefetch_rows(gk, H, nx.h, s, nx.c);
+                prefetch_state(chunk_states, nx.gc, nx.h, H);
+            }
+        } else if (c + 1 < s.n_chunks) {
             prefetch_rows(k, H, h, s, c + 1);
             prefetch_rows(q, H, h, s, c + 1);
             prefetch_rows(v, H, h, s, c + 1);
@@ -786,7 +810,18 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         load_tile_bf16(dO, H, h, srow, true, sDO);
         load_g(gk, H, h, srow, sB);
         if (has_s) global_to_tile128(chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems, sSc);
-        if (!CHUNKS && c >= 1) {      // the next chunk of the walk (chunk 0 of a sequence with replayed rows is not consecutive)
+        if (CHUNKS) {
+            const NextItem nx = next_item(s, c, gc, item, H, n_items);
+            if (nx.c >= 0) {
+                prefetch_rows(k, H, nx.h, s, nx.c);
+                prefetch_rows(q, H, nx.h, s, nx.c);
+                prefetch_rows(v, H, nx.h, s, nx.c);
+                prefetch_rows(dO, H, nx.h, s, nx.c);
+                prefetch_rows(gk, H, nx.h, s, nx.c);
+                prefetch_state(chunk_states, nx.gc, nx.h, H);
+                prefetch_state(ds_tiles, nx.gc, nx.h, H);
+            }
+        } else if (c >= 1) {      // the next chunk of the walk (chunk 0 of a sequence with replayed rows is not consecutive)
             if (c - 1 >= 1 || s.n_replay == 0) {
                 prefetch_rows(k, H, h, s, c - 1);
                 prefetch_rows(q, H, h, s, c - 1);
