@@ -51,8 +51,7 @@ struct Costs {
     }
     i64 W(int a, int b) const { return plen[b + 1] - plen[a] - (pL[b + 1] - pL[a + 1]); }      // interval a..b
     int lcp(int a, int b) const {                 // a < b: minimum of L[a+1..b]
-        int lo = a + 1, n = b - a, k = 0;
-        while ((2 << k) <= n) ++k;
+        const int lo = a + 1, k = 31 - __builtin_clz(static_cast<unsigned>(b - a));
         return std::min(sparse[k][lo], sparse[k][b + 1 - (1 << k)]);
     }
 };
@@ -164,82 +163,121 @@ struct ExactDP {
 };
 
 // ---- merge / split evolution of the natural partition towards a target K (contiguous throughout) --------------------
-bool evolve(const Costs& c, i64 T, std::vector<int> starts, int target, Grouping* out) {
-    const int N = c.N;
+// Merges and splits are chosen without regard to the target, so the way to a far target passes through every nearer
+// one: each direction is walked once, and `out` gets the targets in the order of `pick` (ascending; targets that the
+// walk cannot reach are left out).
+void evolve(const Costs& c, i64 T, const std::vector<int>& natural, const std::vector<int>& pick, std::vector<Grouping>& out) {
+    const int N = c.N, K0 = static_cast<int>(natural.size());
+    std::vector<int> starts = natural;
     auto end_of = [&](size_t k) { return (k + 1 < starts.size() ? starts[k + 1] : N) - 1; };
-    while (static_cast<int>(starts.size()) > target) {           // merge the feasible neighbours that save most
-        int best = -1;
-        i64 best_save = -1;
-        for (size_t k = 0; k + 1 < starts.size(); ++k) {
-            if (c.W(starts[k], end_of(k + 1)) > T) continue;
-            const i64 save = c.L[starts[k + 1]];                 // Eq. 6
-            if (save > best_save) {
+    std::vector<Grouping> down;
+    for (size_t j = pick.size(); j-- > 0;) {                     // targets below K0, nearest first
+        if (pick[j] >= K0) continue;
+        bool reached = true;
+        while (static_cast<int>(starts.size()) > pick[j]) {      // merge the feasible neighbours that save most
+            int best = -1;
+            i64 best_save = -1;
+            for (size_t k = 0; k + 1 < starts.size(); ++k) {
+                const i64 save = c.L[starts[k + 1]];             // Eq. 6
+                if (save <= best_save || c.W(starts[k], end_of(k + 1)) > T) continue;
                 best_save = save;
                 best = static_cast<int>(k);
             }
+            if (best < 0) {
+                reached = false;
+                break;
+            }
+            starts.erase(starts.begin() + best + 1);
         }
-        if (best < 0) return false;
-        starts.erase(starts.begin() + best + 1);
+        if (!reached) break;                                     // nor can any lower target be
+        down.push_back(from_cuts(starts, N, HARTS_MB_EVOLVED));
     }
-    while (static_cast<int>(starts.size()) < target) {           // split where it costs least
-        int best_t = -1, best_l = std::numeric_limits<int>::max();
-        for (size_t k = 0; k < starts.size(); ++k)
-            for (int t = starts[k] + 1; t <= end_of(k); ++t)
-                if (c.L[t] < best_l) {
-                    best_l = c.L[t];
-                    best_t = t;
-                }
-        if (best_t < 0) return false;
-        starts.insert(std::upper_bound(starts.begin(), starts.end(), best_t), best_t);
+    for (size_t j = down.size(); j-- > 0;) out.push_back(std::move(down[j]));
+    // The splits taken are the positions of least adjacent LCP (the lower index on ties) that are not cuts yet.
+    starts = natural;
+    std::vector<int> cut(N, 0), order;
+    for (int t : starts) cut[t] = 1;
+    for (int t = 1; t < N; ++t)
+        if (!cut[t]) order.push_back(t);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c.L[a] < c.L[b]; });
+    size_t used = 0;
+    for (int target : pick) {
+        if (target < K0) continue;
+        const size_t want = target - K0;
+        if (target > N || want > order.size()) break;
+        starts.insert(starts.end(), order.begin() + used, order.begin() + want);
+        used = want;
+        std::sort(starts.begin(), starts.end());
+        out.push_back(from_cuts(starts, N, HARTS_MB_EVOLVED));
     }
-    *out = from_cuts(starts, N, HARTS_MB_EVOLVED);
-    return true;
 }
 
 // ---- trie-aware greedy placement (Eq. 10) ------------------------------------------------------------------------------
 struct Bin {
-    std::set<int> members;
+    std::vector<int> members;                     // ascending
     i64 work = 0;
 };
-// exact work increase of inserting x (Eq. 10) and the amount it shares
-i64 insert_delta(const Costs& c, const Bin& b, int x) {
-    auto it = b.members.lower_bound(x);
-    const bool has_q = it != b.members.end(), has_p = it != b.members.begin();
-    const int q = has_q ? *it : -1, p = has_p ? *std::prev(it) : -1;
-    i64 d = c.len[x];
-    if (has_p) d -= c.lcp(p, x);
-    if (has_q) d -= c.lcp(x, q);
-    if (has_p && has_q) d += c.lcp(p, q);
-    return d;
-}
-// the same with one member left out of the microbatch (skip < 0: nobody); x itself is never counted as a neighbour
-i64 insert_delta_without(const Costs& c, const Bin& b, int x, int skip) {
-    auto hi = b.members.upper_bound(x);
-    while (hi != b.members.end() && *hi == skip) ++hi;
-    auto lo = b.members.lower_bound(x);
-    int p = -1;
-    while (lo != b.members.begin()) {
-        --lo;
-        if (*lo != skip) {
-            p = *lo;
-            break;
-        }
-    }
-    const int q = hi != b.members.end() ? *hi : -1;
-    i64 d = c.len[x];
-    if (p >= 0) d -= c.lcp(p, x);
-    if (q >= 0) d -= c.lcp(x, q);
-    if (p >= 0 && q >= 0) d += c.lcp(p, q);
-    return d;
+// What trajectory x shares with the members of a microbatch (x itself and `skip` are not counted).  Its exact work
+// increase (Eq. 10) is len(x) - LCP(p, x) - LCP(x, q) + LCP(p, q) with its neighbours p, q among the members; LCP(p, q)
+// is the smaller of the other two, so the increase is len(x) - max(LCP(p, x), LCP(x, q)).
+int shared_with(const Costs& c, const Bin& b, int x, int skip = -1) {
+    const int *first = b.members.data(), *last = first + b.members.size();
+    const int* it = std::lower_bound(first, last, x);
+    const int *lo = it, *hi = it;
+    int s = 0;
+    if (lo != first && lo[-1] == skip) --lo;
+    if (lo != first) s = c.lcp(lo[-1], x);
+    while (hi != last && (*hi == x || *hi == skip)) ++hi;
+    return hi != last ? std::max(s, c.lcp(x, *hi)) : s;
 }
 void bin_insert(const Costs& c, Bin& b, int x) {
-    b.work += insert_delta(c, b, x);
-    b.members.insert(x);
+    b.work += c.len[x] - shared_with(c, b, x);
+    b.members.insert(std::lower_bound(b.members.begin(), b.members.end(), x), x);
 }
 void bin_erase(const Costs& c, Bin& b, int x) {
-    b.members.erase(x);
-    b.work -= insert_delta(c, b, x);
+    b.members.erase(std::lower_bound(b.members.begin(), b.members.end(), x));
+    b.work -= c.len[x] - shared_with(c, b, x);
 }
+
+// What x shares with every microbatch at once.  The LCP falls with the distance and is zero outside x's own tree, so a
+// walk to both sides meets the nearest member of every microbatch that shares anything; a walk that is still inside
+// the tree after WALK trajectories gives up, and the microbatches are asked one by one.  `of` is the microbatch of
+// each trajectory (-1: none); `touched` lists the entries of `shared` that are not zero.
+struct SharedWithAll {
+    static constexpr int WALK = 256;
+    std::vector<int> shared, touched;
+    void find(const Costs& c, const std::vector<Bin>& bins, const std::vector<int>& of, int x) {
+        for (int k : touched) shared[k] = 0;
+        touched.clear();
+        if (shared.size() < bins.size()) shared.resize(bins.size(), 0);
+        auto note = [&](int y, int v) {
+            const int k = of[y];
+            if (k < 0 || shared[k] >= v) return;
+            if (shared[k] == 0) touched.push_back(k);
+            shared[k] = v;
+        };
+        int y = x, v = std::numeric_limits<int>::max();
+        const int lo = std::max(0, x - WALK), hi = std::min(c.N - 1, x + WALK);
+        for (; y > lo; --y) {
+            v = std::min(v, c.L[y]);
+            if (v == 0) break;
+            note(y - 1, v);
+        }
+        const bool left_open = y == lo && lo > 0 && v > 0;
+        v = std::numeric_limits<int>::max();
+        for (y = x; y < hi; ++y) {
+            v = std::min(v, c.L[y + 1]);
+            if (v == 0) break;
+            note(y + 1, v);
+        }
+        if (!left_open && !(y == hi && hi < c.N - 1 && v > 0)) return;
+        for (size_t k = 0; k < bins.size(); ++k) {
+            const int s = shared_with(c, bins[k], x);
+            if (s > 0 && shared[k] == 0) touched.push_back(static_cast<int>(k));
+            shared[k] = s;
+        }
+    }
+};
 
 // One placement step as the greedy saw it: trajectory x went to microbatch dest (a new one when created == 1) with
 // work increase delta (Eq. 10).
@@ -250,28 +288,60 @@ struct GreedyStep {
 // The placement pass of the greedy: every trajectory, in the given order, goes to the capacity-feasible microbatch
 // with the largest work after insertion (best-fit) or the largest shared amount |x| - delta (max-shared); ties go to
 // the earliest microbatch; a new microbatch is opened when none fits.
+// A microbatch that shares nothing with x costs len(x) wherever it stands, so only those that share something are looked
+// at one by one.  Of the others max-shared wants the earliest that fits; best-fit wants the heaviest that fits, which
+// `heavy` (heaviest first, the earlier one first on ties) finds by bisection.
 void greedy_place(const Costs& c, i64 T, const std::vector<int>& order, bool best_fit, std::vector<Bin>& bins,
-                  std::vector<GreedyStep>* trace) {
+                  std::vector<int>& of, SharedWithAll& all, std::vector<GreedyStep>* trace) {
+    of.assign(c.N, -1);
+    std::vector<i64> work;
+    std::vector<std::pair<i64, int>> heavy;                      // (-work, microbatch), ascending
     for (int x : order) {
+        all.find(c, bins, of, x);
         int best = -1;
         i64 best_key = -1, best_delta = 0;
-        for (size_t k = 0; k < bins.size(); ++k) {
-            const i64 d = insert_delta(c, bins[k], x);
-            if (bins[k].work + d > T) continue;
-            const i64 key = best_fit ? bins[k].work + d : c.len[x] - d;     // work after insertion | shared amount
-            if (key > best_key) {
+        auto offer = [&](int k, i64 d) {
+            if (work[k] + d > T) return;
+            const i64 key = best_fit ? work[k] + d : c.len[x] - d;     // work after insertion | shared amount
+            if (key > best_key || (key == best_key && k < best)) {
                 best_key = key;
                 best_delta = d;
-                best = static_cast<int>(k);
+                best = k;
             }
+        };
+        for (int k : all.touched)
+            if (all.shared[k] > 0) offer(k, c.len[x] - all.shared[k]);
+        if (best_fit) {
+            auto it = std::lower_bound(heavy.begin(), heavy.end(), std::make_pair(c.len[x] - T, 0));
+            while (it != heavy.end() && all.shared[it->second] > 0) ++it;
+            if (it != heavy.end()) offer(it->second, c.len[x]);
+        } else if (best < 0) {
+            for (size_t k = 0; k < work.size() && best < 0; ++k)
+                if (all.shared[k] == 0) offer(static_cast<int>(k), c.len[x]);
         }
         const bool created = best < 0;
         if (created) {
-            bins.emplace_back();
-            best = static_cast<int>(bins.size()) - 1;
+            best = static_cast<int>(bins.size());
             best_delta = c.len[x];
+            bins.emplace_back();
+            work.push_back(0);
         }
-        bin_insert(c, bins[best], x);
+        Bin& b = bins[best];
+        if (best_fit) {
+            const std::pair<i64, int> now(-(work[best] + best_delta), best);
+            auto to = std::lower_bound(heavy.begin(), heavy.end(), now);
+            if (created) {
+                heavy.insert(to, now);
+            } else {
+                auto was = std::lower_bound(to, heavy.end(), std::make_pair(-work[best], best));
+                std::move_backward(to, was, was + 1);            // a microbatch only gets heavier
+                *to = now;
+            }
+        }
+        work[best] += best_delta;
+        b.work = work[best];
+        b.members.insert(std::lower_bound(b.members.begin(), b.members.end(), x), x);
+        of[x] = best;
         if (trace) trace->push_back({x, best, created ? 1 : 0, best_delta});
     }
 }
@@ -280,45 +350,57 @@ void greedy_place(const Costs& c, i64 T, const std::vector<int>& order, bool bes
 std::vector<std::vector<int>> greedy_orders(const Costs& c) {
     const int N = static_cast<int>(c.len.size());
     std::vector<std::vector<int>> orders(4, std::vector<int>(N));
-    for (int i = 0; i < N; ++i) orders[0][i] = i, orders[1][i] = N - 1 - i, orders[2][i] = i, orders[3][i] = i;
-    std::stable_sort(orders[2].begin(), orders[2].end(), [&](int a, int b) { return c.len[a] > c.len[b]; });
-    std::vector<int> uniq(N);
-    for (int i = 0; i < N; ++i) uniq[i] = c.len[i] - std::max(c.L[i], i + 1 < N ? c.L[i + 1] : 0);
-    std::stable_sort(orders[3].begin(), orders[3].end(), [&](int a, int b) { return uniq[a] > uniq[b]; });
+    for (int i = 0; i < N; ++i) orders[0][i] = i, orders[1][i] = N - 1 - i;
+    std::vector<std::pair<int, int>> by(N);       // (-key, index): ascending order is descending key, stable
+    auto sorted = [&](std::vector<int>& out) {
+        std::sort(by.begin(), by.end());
+        for (int i = 0; i < N; ++i) out[i] = by[i].second;
+    };
+    for (int i = 0; i < N; ++i) by[i] = {-c.len[i], i};
+    sorted(orders[2]);
+    for (int i = 0; i < N; ++i) by[i] = {std::max(c.L[i], i + 1 < N ? c.L[i + 1] : 0) - c.len[i], i};
+    sorted(orders[3]);
     return orders;
 }
 
 bool greedy_plan(const Costs& c, i64 T, int D, const std::vector<int>& order, bool best_fit, Grouping* out) {
     std::vector<Bin> bins;
-    greedy_place(c, T, order, best_fit, bins, nullptr);
-    // eliminate small microbatches: re-place all members of the lightest one (max-shared destination), all or nothing
-    while (bins.size() > 1) {
-        size_t lightest = 0;
-        for (size_t k = 1; k < bins.size(); ++k)
-            if (bins[k].work < bins[lightest].work) lightest = k;
-        std::vector<Bin> trial = bins;
-        trial.erase(trial.begin() + lightest);
-        bool ok = true;
-        for (int x : bins[lightest].members) {
+    std::vector<int> of;
+    SharedWithAll all;
+    greedy_place(c, T, order, best_fit, bins, of, all, nullptr);
+    // eliminate small microbatches: re-place all members of the lightest one (max-shared destination), all or nothing.
+    // Numbers stay as they are while microbatches go (an emptied one is skipped), which keeps their order for ties.
+    size_t alive = bins.size();
+    while (alive > 1) {
+        int lightest = -1;
+        for (size_t k = 0; k < bins.size(); ++k)
+            if (!bins[k].members.empty() && (lightest < 0 || bins[k].work < bins[lightest].work)) lightest = static_cast<int>(k);
+        Bin moved = std::move(bins[lightest]);
+        bins[lightest] = Bin();
+        for (int x : moved.members) of[x] = -1;
+        std::vector<GreedyStep> done;
+        for (int x : moved.members) {
+            all.find(c, bins, of, x);
             int best = -1;
             i64 best_shared = -1;
-            for (size_t k = 0; k < trial.size(); ++k) {
-                const i64 d = insert_delta(c, trial[k], x);
-                if (trial[k].work + d > T) continue;
-                if (c.len[x] - d > best_shared) {
-                    best_shared = c.len[x] - d;
-                    best = static_cast<int>(k);
-                }
+            for (size_t k = 0; k < bins.size(); ++k) {
+                if (all.shared[k] <= best_shared || bins[k].members.empty() || bins[k].work + c.len[x] - all.shared[k] > T) continue;
+                best_shared = all.shared[k];
+                best = static_cast<int>(k);
             }
-            if (best < 0) {
-                ok = false;
-                break;
-            }
-            bin_insert(c, trial[best], x);
+            if (best < 0) break;
+            bin_insert(c, bins[best], x);
+            of[x] = best;
+            done.push_back({x, best, 0, 0});
         }
-        if (!ok) break;
-        bins.swap(trial);
+        if (done.size() < moved.members.size()) {                // put everything back
+            for (size_t i = done.size(); i-- > 0;) bin_erase(c, bins[done[i].dest], done[i].x);
+            bins[lightest] = std::move(moved);
+            break;
+        }
+        --alive;
     }
+    bins.erase(std::remove_if(bins.begin(), bins.end(), [](const Bin& b) { return b.members.empty(); }), bins.end());
     // align K to D: split off the single trajectory whose own microbatch costs least extra
     while (bins.size() % D != 0) {
         int best_bin = -1, best_x = -1;
@@ -326,7 +408,7 @@ bool greedy_plan(const Costs& c, i64 T, int D, const std::vector<int>& order, bo
         for (size_t k = 0; k < bins.size(); ++k) {
             if (bins[k].members.size() < 2) continue;
             for (int x : bins[k].members) {
-                const i64 inc = c.len[x] - insert_delta_without(c, bins[k], x, -1);      // own microbatch minus what it frees
+                const i64 inc = shared_with(c, bins[k], x);      // its own microbatch minus what it frees here
                 if (inc < best_inc) {
                     best_inc = inc;
                     best_bin = static_cast<int>(k);
@@ -341,7 +423,7 @@ bool greedy_plan(const Costs& c, i64 T, int D, const std::vector<int>& order, bo
     }
     out->mb.clear();
     out->source = HARTS_MB_GREEDY;
-    for (auto& b : bins) out->mb.emplace_back(b.members.begin(), b.members.end());
+    for (auto& b : bins) out->mb.push_back(std::move(b.members));
     return true;
 }
 
@@ -375,29 +457,37 @@ bool refine_boundaries(const Costs& c, i64 T, std::vector<int>& starts) {
     return any;
 }
 
-// Sparse repair: at most four single moves or swaps between microbatches that are close in lexicographic order.
+// Sparse repair: at most four single moves or swaps between microbatches that are close in lexicographic order.  A move
+// gains (shared with B) - (shared with A), and nothing shares more with x than a lexicographic neighbour does: `slack`,
+// what the best neighbour shares minus what x shares where it is, bounds the gain of moving x, and the sum of two
+// slacks the gain of a swap.  Most trajectories sit beside their best neighbour (slack 0) and are passed over.
 bool sparse_repair(const Costs& c, i64 T, Grouping& g) {
     const int N = c.N;
     std::vector<Bin> bins(g.mb.size());
     std::vector<int> of(N);
     for (size_t k = 0; k < g.mb.size(); ++k)
         for (int x : g.mb[k]) {
-            bin_insert(c, bins[k], x);
+            bins[k].members.push_back(x);
             of[x] = static_cast<int>(k);
         }
+    for (Bin& b : bins) b.work = work_of(c, b.members);
+    std::vector<int> here(N), slack(N);
     bool any = false;
     for (int iter = 0; iter < 4; ++iter) {
         i64 best_gain = 0;
         int mv_x = -1, mv_to = -1, sw_x = -1, sw_y = -1;
+        for (int x = 0; x < N; ++x) {
+            here[x] = shared_with(c, bins[of[x]], x);
+            slack[x] = std::max(c.L[x], x + 1 < N ? c.L[x + 1] : 0) - here[x];
+        }
         for (int x = 0; x < N; ++x) {                       // moves out of non-singleton microbatches
             const int A = of[x];
-            if (bins[A].members.size() < 2) continue;
+            if (slack[x] <= best_gain || bins[A].members.size() < 2) continue;
             for (int y = std::max(0, x - H_WIN); y <= std::min(N - 1, x + H_WIN); ++y) {
                 const int B = of[y];
                 if (B == A) continue;
-                const i64 d = insert_delta(c, bins[B], x);
-                if (bins[B].work + d > T) continue;
-                const i64 gain = insert_delta_without(c, bins[A], x, -1) - d;      // freed in A minus added in B
+                const i64 s = shared_with(c, bins[B], x), gain = s - here[x];      // freed in A minus added in B
+                if (bins[B].work + c.len[x] - s > T) continue;
                 if (gain > best_gain) {
                     best_gain = gain;
                     mv_x = x;
@@ -409,11 +499,10 @@ bool sparse_repair(const Costs& c, i64 T, Grouping& g) {
             for (int x = 0; x < N; ++x)
                 for (int y = x + 1; y <= std::min(N - 1, x + H_WIN); ++y) {
                     const int A = of[x], B = of[y];
-                    if (A == B) continue;
-                    const i64 a_new = bins[A].work - insert_delta_without(c, bins[A], x, -1) +
-                                      insert_delta_without(c, bins[A], y, x);
-                    const i64 b_new = bins[B].work - insert_delta_without(c, bins[B], y, -1) +
-                                      insert_delta_without(c, bins[B], x, y);
+                    if (A == B || i64(slack[x]) + slack[y] <= best_gain) continue;
+                    const i64 x_len = c.len[x], y_len = c.len[y];
+                    const i64 a_new = bins[A].work - (x_len - here[x]) + (y_len - shared_with(c, bins[A], y, x));
+                    const i64 b_new = bins[B].work - (y_len - here[y]) + (x_len - shared_with(c, bins[B], x, y));
                     if (a_new > T || b_new > T) continue;
                     const i64 gain = (bins[A].work + bins[B].work) - (a_new + b_new);
                     if (gain > best_gain) {
@@ -441,7 +530,7 @@ bool sparse_repair(const Costs& c, i64 T, Grouping& g) {
         any = true;
     }
     if (any)
-        for (size_t k = 0; k < g.mb.size(); ++k) g.mb[k].assign(bins[k].members.begin(), bins[k].members.end());
+        for (size_t k = 0; k < g.mb.size(); ++k) g.mb[k] = std::move(bins[k].members);
     return any;
 }
 
@@ -513,52 +602,57 @@ bool forest_ok(int32_t n_trees, const int32_t* ptr, const int32_t* par, const in
     return true;
 }
 
-// Trajectories in depth-first order (explicit stack: trees may be deep chains).
+// Trajectories in depth-first order (no recursion: trees may be deep chains).
 void enumerate(const harts_mb_plan_t& p, int32_t n_trees, std::vector<Traj>& out) {
     const auto& ptr = p.tree_node_ptr;
     const auto& par = p.node_parent;
     const auto& off = p.node_fork_off;
     const auto& len = p.node_len;
     const int n_nodes = ptr[n_trees];
-    std::vector<std::vector<int>> kids(n_nodes);
+    // children of every node by fork offset (the earlier child first on ties), as one array
+    std::vector<int> kid_ptr(n_nodes + 1, 0), kids(std::max(n_nodes - n_trees, 1)), next(n_nodes), depth(n_nodes, 0);
     std::vector<char> continued(n_nodes, 0);
     for (int t = 0; t < n_trees; ++t)
         for (int i = ptr[t] + 1; i < ptr[t + 1]; ++i) {
             const int q = ptr[t] + par[i];
-            kids[q].push_back(i);
+            ++kid_ptr[q + 1];
+            depth[i] = depth[q] + 1;
             if (off[i] == len[q]) continued[q] = 1;
         }
-    for (auto& k : kids) std::stable_sort(k.begin(), k.end(), [&](int a, int b) { return off[a] < off[b]; });
-    std::vector<int> root_of(n_nodes);
+    for (int i = 0; i < n_nodes; ++i) {
+        kid_ptr[i + 1] += kid_ptr[i];
+        next[i] = kid_ptr[i];
+    }
     for (int t = 0; t < n_trees; ++t)
-        for (int i = ptr[t]; i < ptr[t + 1]; ++i) root_of[i] = ptr[t];
+        for (int i = ptr[t] + 1; i < ptr[t + 1]; ++i) kids[next[ptr[t] + par[i]]++] = i;
+    auto by_offset = [&](int a, int b) { return off[a] < off[b] || (off[a] == off[b] && a < b); };
+    for (int i = 0; i < n_nodes; ++i) {
+        next[i] = kid_ptr[i];
+        if (!std::is_sorted(kids.begin() + kid_ptr[i], kids.begin() + kid_ptr[i + 1], by_offset))
+            std::sort(kids.begin() + kid_ptr[i], kids.begin() + kid_ptr[i + 1], by_offset);
+    }
+    out.reserve(n_nodes - std::count(continued.begin(), continued.end(), 1));
     for (int t = 0; t < n_trees; ++t) {
-        std::vector<std::pair<int, size_t>> stack;
-        stack.push_back({ptr[t], size_t(0)});
-        while (!stack.empty()) {
-            auto& top = stack.back();
-            const int v = top.first;
-            if (top.second < kids[v].size()) {
-                const int child = kids[v][top.second++];
-                stack.push_back({child, size_t(0)});
+        const int root = ptr[t];
+        for (int v = root; v >= 0;) {
+            if (next[v] < kid_ptr[v + 1]) {
+                v = kids[next[v]++];
                 continue;
             }
             if (!continued[v]) {
-                Traj tr;
+                out.emplace_back();
+                Traj& tr = out.back();
                 tr.leaf = v;
-                int node = v, upto = len[v];
-                while (true) {
-                    tr.path.push_back({node, upto});
-                    if (node == root_of[node]) break;
-                    upto = off[node];
-                    node = root_of[node] + par[node];
-                }
-                std::reverse(tr.path.begin(), tr.path.end());
                 tr.len = 0;
-                for (auto& e : tr.path) tr.len += e.second;
-                out.push_back(std::move(tr));
+                tr.path.resize(depth[v] + 1);
+                for (int node = v, upto = len[v], j = depth[v]; j >= 0; --j) {
+                    tr.path[j] = {node, upto};
+                    tr.len += upto;
+                    upto = off[node];
+                    node = root + par[node];
+                }
             }
-            stack.pop_back();
+            v = v == root ? -1 : root + par[v];
         }
     }
 }
@@ -612,10 +706,7 @@ int32_t build(harts_mb_plan_t& p, int32_t n_trees, int32_t D, i64 T) {
             for (int i = 0; i < 14; ++i) chosen.insert(ks[16 + (ks.size() - 17) * (i + 1) / 15]);
             pick.assign(chosen.begin(), chosen.end());
         }
-        for (int K : pick) {
-            Grouping g;
-            if (K <= N && evolve(c, T, nat, K, &g)) cands.push_back(std::move(g));
-        }
+        evolve(c, T, nat, pick, cands);
     }
     const size_t n_base_end = cands.size();
 
@@ -764,8 +855,10 @@ extern "C" int32_t harts_mb_greedy_trace(const harts_mb_plan_t* plan, int32_t or
         c.L.assign(plan->traj_lcp.begin(), plan->traj_lcp.end());
         c.build();
         std::vector<Bin> bins;
+        std::vector<int> of;
+        SharedWithAll all;
         std::vector<GreedyStep> trace;
-        greedy_place(c, plan->view.T, greedy_orders(c)[order], policy == 0, bins, &trace);
+        greedy_place(c, plan->view.T, greedy_orders(c)[order], policy == 0, bins, of, all, &trace);
         *n_steps = N;
         if (!step_traj && !step_mb && !step_created && !step_delta) return HARTS_OK;
         if (cap < N || !step_traj || !step_mb || !step_created || !step_delta) return HARTS_EINVAL;
