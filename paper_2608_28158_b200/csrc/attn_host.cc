@@ -33,42 +33,35 @@ extern "C" int32_t harts_attn_index(int32_t n_trees, const int32_t* tree_node_pt
     const int64_t C = base[n_nodes];
     if (C >= INT32_MAX) return HARTS_EINVAL;
     auto row = [&](int64_t canon) { return row_of_token ? row_of_token[canon] : static_cast<int32_t>(canon); };
-    if (row_of_token) {
-        std::vector<char> seen(C, 0);
-        for (int64_t c = 0; c < C; ++c) {
-            const int32_t r = row_of_token[c];
-            if (r < 0 || r >= C || seen[r]) return HARTS_EINVAL;
-            seen[r] = 1;
-        }
-    }
-    // predecessor and number of successors of every physical row
-    std::vector<int32_t> prev(C), n_child(C, 0);
+    // predecessor of every physical row and whether it has several successors, in one walk in canonical order
+    // (row_of_token must be a permutation of 0..C-1)
+    constexpr int32_t UNSEEN = -2;
+    std::vector<int32_t> prev(C, UNSEEN);
+    std::vector<unsigned char> n_child(C, 0);         // 0, 1 or 2 for "several"
     for (int32_t t = 0; t < n_trees; ++t) {
         const int32_t lo = tree_node_ptr[t], hi = tree_node_ptr[t + 1];
         for (int32_t i = lo; i < hi; ++i) {
-            const int64_t p0 = i == lo ? -1 : base[lo + node_parent[i]] + node_fork_off[i] - 1;
-            prev[row(base[i])] = p0 < 0 ? -1 : row(p0);
-            for (int64_t c = base[i] + 1; c < base[i + 1]; ++c) prev[row(c)] = row(c - 1);
+            int32_t p = i == lo ? -1 : row(base[lo + node_parent[i]] + node_fork_off[i] - 1);
+            for (int64_t c = base[i]; c < base[i + 1]; ++c) {
+                const int32_t r = row(c);
+                if (r < 0 || r >= C || prev[r] != UNSEEN) return HARTS_EINVAL;
+                prev[r] = p;
+                if (p >= 0) n_child[p] = n_child[p] == 0 ? 1 : 2;
+                p = r;
+            }
         }
     }
-    for (int64_t r = 0; r < C; ++r)
-        if (prev[r] >= 0) ++n_child[prev[r]];
     // pieces: row r continues the piece of row r-1 iff r-1 is its predecessor and r is r-1's only successor
-    std::vector<int32_t> piece_of(C), p_row0, p_len, p_parent;
-    for (int64_t r = 0; r < C; ++r) {
-        const bool cont = r > 0 && prev[r] == r - 1 && n_child[r - 1] == 1;
-        if (!cont) {
-            p_row0.push_back(static_cast<int32_t>(r));
-            p_len.push_back(0);
-        }
-        piece_of[r] = static_cast<int32_t>(p_row0.size()) - 1;
-        ++p_len.back();
-    }
+    std::vector<int32_t> p_row0, p_len, p_parent;
+    for (int64_t r = 0; r < C; ++r)
+        if (r == 0 || prev[r] != r - 1 || n_child[r - 1] != 1) p_row0.push_back(static_cast<int32_t>(r));
     const int32_t P = static_cast<int32_t>(p_row0.size());
+    p_len.resize(P);
     p_parent.resize(P);
+    for (int32_t p = 0; p < P; ++p) p_len[p] = (p + 1 < P ? p_row0[p + 1] : static_cast<int32_t>(C)) - p_row0[p];
     for (int32_t p = 0; p < P; ++p) {
         const int32_t a = prev[p_row0[p]];
-        p_parent[p] = a < 0 ? -1 : piece_of[a];
+        p_parent[p] = a < 0 ? -1 : static_cast<int32_t>(std::upper_bound(p_row0.begin(), p_row0.end(), a) - p_row0.begin()) - 1;
         // the predecessor must close its piece, so that ancestors are whole pieces
         if (a >= 0 && a != p_row0[p_parent[p]] + p_len[p_parent[p]] - 1) return HARTS_EINTERNAL;
     }

@@ -29,32 +29,29 @@ extern "C" int32_t harts_conv_index(int32_t n_trees, const int32_t* tree_node_pt
     if (C >= INT32_MAX) return HARTS_EINVAL;
     if (C - n_trees > 0 && !child_row) return HARTS_EINVAL;
     auto row = [&](int64_t canon) { return row_of_token ? row_of_token[canon] : static_cast<int32_t>(canon); };
-    if (row_of_token) {                               // must be a permutation of 0..C-1
-        std::vector<char> seen(C, 0);
-        for (int64_t c = 0; c < C; ++c) {
-            const int32_t r = row_of_token[c];
-            if (r < 0 || r >= C || seen[r]) return HARTS_EINVAL;
-            seen[r] = 1;
-        }
-    }
-    // canonical predecessor of every token, then the same in physical rows
-    std::vector<int64_t> pred(C);
+    constexpr int32_t UNSEEN = -2;
+    for (int64_t r = 0; r < C; ++r) prev_row[r] = UNSEEN;
+    for (int64_t r = 0; r < C; ++r) next_row[r] = 0;  // the number of children, while the tables are built
+    // one walk in canonical order; row_of_token must be a permutation of 0..C-1
     for (int32_t t = 0; t < n_trees; ++t) {
         const int32_t lo = tree_node_ptr[t], hi = tree_node_ptr[t + 1];
         for (int32_t i = lo; i < hi; ++i) {
-            pred[base[i]] = i == lo ? -1 : base[lo + node_parent[i]] + node_fork_off[i] - 1;
-            for (int64_t c = base[i] + 1; c < base[i + 1]; ++c) pred[c] = c - 1;
+            int32_t p = i == lo ? -1 : row(base[lo + node_parent[i]] + node_fork_off[i] - 1);
+            for (int64_t c = base[i]; c < base[i + 1]; ++c) {
+                const int32_t r = row(c);
+                if (r < 0 || r >= C || prev_row[r] != UNSEEN) return HARTS_EINVAL;
+                prev_row[r] = p;
+                if (p >= 0) ++next_row[p];
+                p = r;
+            }
         }
     }
-    for (int64_t r = 0; r <= C; ++r) child_ptr[r] = 0;
-    for (int64_t c = 0; c < C; ++c) {
-        prev_row[row(c)] = pred[c] < 0 ? -1 : row(pred[c]);
-        if (pred[c] >= 0) ++child_ptr[row(pred[c]) + 1];
+    child_ptr[0] = 0;
+    for (int64_t r = 0; r < C; ++r) child_ptr[r + 1] = child_ptr[r] + next_row[r];
+    for (int64_t c = C; c-- > 0;) {                   // canonical order of the children of one row, the last one first
+        const int32_t r = row(c), p = prev_row[r];
+        if (p >= 0) child_row[child_ptr[p] + --next_row[p]] = r;
     }
-    for (int64_t r = 0; r < C; ++r) child_ptr[r + 1] += child_ptr[r];
-    std::vector<int32_t> fill(child_ptr, child_ptr + C);
-    for (int64_t c = 0; c < C; ++c)                   // canonical order of the children of one row
-        if (pred[c] >= 0) child_row[fill[row(pred[c])]++] = row(c);
     for (int64_t r = 0; r < C; ++r) {
         const int32_t n = child_ptr[r + 1] - child_ptr[r];
         next_row[r] = n == 0 ? -1 : (n == 1 ? child_row[child_ptr[r]] : -2);

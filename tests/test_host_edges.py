@@ -1,0 +1,43 @@
+"""Edges of the host side's tables: runs of positions in the row grouping, and a tree that is wider than the planner's
+walk over neighbours."""
+import random
+
+import numpy as np
+import pytest
+
+import paper_2608_28158_b200 as H
+from oracle import mb_oracle as mo
+from test_mb_plan import _lex_trajs, _plan
+from test_plan_oracle import random_tree
+from workloads import make_forest
+
+
+def _runs(seed):
+    rng = np.random.default_rng(seed)
+    return np.concatenate([np.arange(a, a + n) for a, n in zip(rng.integers(0, 150, 60), rng.integers(1, 50, 60))])
+
+
+@pytest.mark.parametrize("m", [
+    [], [0], [199], list(range(200)), [7] * 40, list(range(199, -1, -1)), [3, 4, 5, 4, 5, 6, 5, 3], _runs(1), _runs(2),
+    np.random.default_rng(3).integers(0, 200, 700)], ids=range(10))
+def test_rows_are_grouped_in_position_order(m):
+    m = np.asarray(m, np.int32)
+    ptr, pos = H.harts_logp_csr(200, m)
+    assert np.array_equal(ptr, np.concatenate([[0], np.cumsum(np.bincount(m, minlength=200))]))
+    assert np.array_equal(pos, np.argsort(m, kind="stable"))
+    for bad in (-1, 200, 2147483647):
+        with pytest.raises(H.HartsError):
+            H.harts_logp_csr(200, np.append(m, bad))
+
+
+@pytest.mark.parametrize("leaves", [255, 258, 300])
+def test_greedy_in_a_tree_wider_than_the_walk(leaves):
+    rnd = random.Random(leaves)
+    wide = ([-1] + [0] * leaves, [0] + [rnd.randint(1, 3) for _ in range(leaves)], [3] + [rnd.randint(1, 2) for _ in range(leaves)])
+    fo = make_forest([wide, random_tree(rnd, 9, 12)])
+    plan = _plan(fo, 1, 80)
+    trajs = _lex_trajs(fo, plan)
+    orders = mo.greedy_orders(trajs)
+    for order, policy in ((1, 0), (3, 1)):
+        got = list(zip(*(a.tolist() for a in plan.greedy_trace(order, policy))))
+        assert got == mo.greedy_place(trajs, orders[order], 80, best_fit=policy == 0)
