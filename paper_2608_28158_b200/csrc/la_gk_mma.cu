@@ -188,11 +188,12 @@ __device__ __forceinline__ void prefetch_state(const __nv_bfloat16* tiles, int g
 
 // running sum over the rows, per channel: four threads per channel (16 rows each, scanned in registers), joined through
 // sTmp[4][128]
+template <bool RAW = false>      // RAW: sB still holds the log-decays themselves, not yet in log2 units
 __device__ __forceinline__ void cumsum_rows(float* sB, float* sTmp) {
     const int tid = threadIdx.x, i = tid & (D - 1), part = tid >> 7;
     float x[16];
 #pragma unroll
-    for (int u = 0; u < 16; u++) x[u] = sB[(part * 16 + u) * D + i];
+    for (int u = 0; u < 16; u++) x[u] = sB[(part * 16 + u) * D + i] * (RAW ? LOG2E : 1.f);
 #pragma unroll
     for (int u = 1; u < 16; u++) x[u] += x[u - 1];
     sTmp[part * D + i] = x[15];
@@ -521,19 +522,19 @@ __device__ __forceinline__ int owner_of(const harts_la_tables_t& tb, int seq_lo,
 
 // How a kernel is driven.
 // ROUND: one launch per round, item = (sequence, head) = block index, no flags.
-// CHUNKS: the boundary states (backward: their gradients too) are in memory (la_scan.cu), item = (chunk, head).
+// CHUNKS (backward only): the boundary states and their gradients are in memory (la_scan.cu), item = (chunk, head).
 // ONE_LAUNCH: the grid covers the sequences of ALL rounds (numbered round by round).  Every CTA draws its work item
 // from `ticket`, so an item is only ever held by a running CTA; a sequence that starts from an exported state waits for
 // the flag its producer (an earlier round, a smaller ticket, hence running or done) sets after writing the slot.
 enum Mode { ROUND, ONE_LAUNCH_MODE, CHUNKS_MODE };
 template <int MODE>
 __global__ void __launch_bounds__(NT, 1)
-gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
+gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                   __nv_bfloat16* __restrict__ o, float* __restrict__ slots, __nv_bfloat16* __restrict__ chunk_states,
                   const int32_t* gate, int* status, int* slot_flags, int* ticket) {
     if (gate_closed(gate)) return;
-    constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE, CHUNKS = MODE == CHUNKS_MODE;
+    constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE;
     __shared__ int s_item, s_dead;
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sQ = sm + Shared::q, *sK = sm + Shared::k, *sV = sm + Shared::v, *sP = sm + Shared::p,
@@ -558,16 +559,12 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
     }
     const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
     const size_t state_elems = (size_t)D * D;
-    const int chunk_lo = CHUNKS ? tb.seq_chunk_ptr[seq_lo] : 0, n_items = CHUNKS ? (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H : 0;
-    do {
-    if (CHUNKS && item >= n_items) break;
-    const int seq_pos = seq_lo + item / H, h = item % H, gc = chunk_lo + item / H;
-    const int seq = CHUNKS ? owner_of(tb, seq_lo, seq_hi, gc) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+    const int seq_pos = seq_lo + item / H, h = item % H;
+    const int seq = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
     const SeqInfo s = seq_info(tb, seq);
 
     float st[8][4];
-    if (CHUNKS) {
-    } else if (s.init_slot < 0) {
+    if (s.init_slot < 0) {
 #pragma unroll
         for (int n = 0; n < 8; n++) st[n][0] = st[n][1] = st[n][2] = st[n][3] = 0.f;
     } else {
@@ -579,9 +576,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
     }
 
     int next_req = s.req_lo;
-    const int c_lo = CHUNKS ? gc - s.chunk_base : 0, c_hi = CHUNKS ? c_lo + 1 : s.n_chunks;
-    for (int c = c_lo; c < c_hi; c++) {
-        const bool has_s = !CHUNKS || c > 0 || s.init_slot >= 0;      // the state of a sequence that starts from zero is not read
+    for (int c = 0; c < s.n_chunks; c++) {
         __syncthreads();                                   // the previous chunk's readers of every tile are through
         load_codes(tb, s, c, srow);
         __syncthreads();
@@ -589,25 +584,15 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         load_tile_bf16(q, H, h, srow, true, sQ);
         load_tile_bf16(v, H, h, srow, false, sV);
         load_g(gk, H, h, srow, sB);
-        if (CHUNKS) {
-            const NextItem nx = next_item(s, c, gc, item, H, n_items);
-            if (nx.c >= 0) {
-                prefetch_rows(k, H, nx.h, s, nx.c);
-                prefetch_rows(q, H, nx.h, s, nx.c);
-                prefetch_rows(v, H, nx.h, s, nx.c);
-                prefetch_rows(gk, H, nx.h, s, nx.c);
-                prefetch_state(chunk_states, nx.gc, nx.h, H);
-            }
-        } else if (c + 1 < s.n_chunks) {
+        if (c + 1 < s.n_chunks) {
             prefetch_rows(k, H, h, s, c + 1);
             prefetch_rows(q, H, h, s, c + 1);
             prefetch_rows(v, H, h, s, c + 1);
             prefetch_rows(gk, H, h, s, c + 1);
         }
         // start-of-chunk state: operand copy, kept for the backward, exported when the plan requests this boundary
-        if (!CHUNKS) state_to_operand(st, sSb, warp, lane);
-        else if (has_s) global_to_tile128(chunk_states + ((size_t)gc * H + h) * state_elems, sSb);
-        const bool exported = !CHUNKS && next_req < s.req_hi && tb.slot_chunk[next_req] == c;
+        state_to_operand(st, sSb, warp, lane);
+        const bool exported = next_req < s.req_hi && tb.slot_chunk[next_req] == c;
         if (exported) {
             state_to_global(st, slots + ((size_t)next_req * H + h) * state_elems, warp, lane);
             if (ONE_LAUNCH) __threadfence();               // this thread's part of the slot, before the flag below
@@ -615,7 +600,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         }
         __syncthreads();
         if (ONE_LAUNCH && exported && tid == 0) tc::flag_set(slot_flags + (size_t)(next_req - 1) * H + h);
-        if (!CHUNKS && chunk_states) tile_to_global<D>(sSb, chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems);
+        if (chunk_states) tile_to_global<D>(sSb, chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems);
         cumsum_rows(sB, sTmp);
         const bool mild = chunk_is_mild(sB);
         unsigned char* sKd = reinterpret_cast<unsigned char*>(sR);        // the two are never needed in the same chunk
@@ -626,7 +611,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         if (!mild) scores_diagonal(sQ, sK, sR, sP, warp, lane);
         scores_off_diagonal(s_u32(sQa), s_u32(sKa), sP, warp, lane, mild, s_u32(sKd));
         __syncthreads();
-        scale_qk<true, !CHUNKS>(sQ, sK, sB, sQ, sK);
+        scale_qk(sQ, sK, sB, sQ, sK);
         __syncthreads();
         // ---- o = P V + q~ S_c : warp -> rows 16 * mb, columns 32 * nq ----------------------------------------------
         {
@@ -645,7 +630,6 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
-            if (has_s)
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4];
@@ -667,10 +651,184 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             }
         }
         // ---- S <- Diag(e^{b_n}) S + k~^T V ---------------------------------------------------------------------------
-        if (!CHUNKS) state_update(st, sB, aK, aV, warp, lane);
+        state_update(st, sB, aK, aV, warp, lane);
     }
-    item += gridDim.x;
-    } while (CHUNKS);
+}
+
+
+// ---- forward, every (chunk, head) on its own -----------------------------------------------------------------------------
+// The boundary states are in memory (la_scan.cu).  What bounds an item is its chain of phases (load, running sums, operands,
+// scores, outputs), each far below the machine's rates, so two CTAs share an SM: 115 KB of shared memory and 64 registers a
+// thread.  To fit, everything is worked on in place or over something dead: the running sums' scratch lies under the
+// scores, k becomes the keys anchored at their own block, q becomes q~, V comes in over the anchored queries once the
+// scores are done, the state over the running sums.  One pass over q and k makes all four operands of a mild chunk.
+// Measured, 1,047 chunks x 16 heads: 0.78 ms (one CTA per SM with every tile in a place of its own: 1.08).
+struct SharedC {
+    static constexpr int q = 0, k = 16384;                              // bf16 [64][128]; then q~, keys anchored at their block
+    static constexpr int b = 32768;                                     // fp32 [64][128] running log-decay; then the state
+    static constexpr int qa = 65536, ka = qa + 16384;                   // anchored operands; then V; step factors (not mild)
+    static constexpr int p = ka + 96 * 256, row = p + 8192, bytes = row + 256;
+};
+static_assert(2 * (SharedC::bytes + 1024 + 64) <= 228 * 1024, "two CTAs per SM");
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool take) {      // zeros where nothing is taken
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(take ? 16 : 0) : "memory");
+}
+
+// all operands of a mild chunk: a thread's 16-byte piece of q and of k, in place and into the anchored tiles
+__device__ __forceinline__ void mild_operands(unsigned char* sQ, unsigned char* sK, const float* sB, unsigned char* sQa,
+                                              unsigned char* sKa) {
+#pragma unroll
+    for (int u = 0; u < BT * 16 / NT; u++) {
+        const int p = threadIdx.x + u * NT, t = p >> 4, c16 = p & 15, blk = t >> 4;
+        const uint32_t off = sw256(t, c16);
+        float bs[8], ba[8];
+        auto row8 = [&](float (&x)[8], int r) {
+            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(sB + r * D + c16 * 8);
+            *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(sB + r * D + c16 * 8 + 4);
+        };
+        auto scaled = [&](const uint4& x, auto exponent) {
+            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+            uint32_t y[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
+                y[e] = pack2(f.x * ex2(exponent(2 * e)), f.y * ex2(exponent(2 * e + 1)));
+            }
+            return make_uint4(y[0], y[1], y[2], y[3]);
+        };
+        row8(bs, t);
+        row8(ba, 16 * blk);
+        const uint4 qv = *reinterpret_cast<const uint4*>(sQ + off), kv = *reinterpret_cast<const uint4*>(sK + off);
+        *reinterpret_cast<uint4*>(sQa + off) = scaled(qv, [&](int e) { return bs[e] - ba[e]; });
+        *reinterpret_cast<uint4*>(sQ + off) = scaled(qv, [&](int e) { return bs[e]; });
+        *reinterpret_cast<uint4*>(sK + off) = scaled(kv, [&](int e) { return ba[e] - bs[e]; });
+        for (int I = blk + 1; I < 4; I++) {
+            row8(ba, 16 * I);
+            *reinterpret_cast<uint4*>(sKa + sw256(ka_row0(I) + t, c16)) = scaled(kv, [&](int e) { return ba[e] - bs[e]; });
+        }
+    }
+}
+
+__global__ void __launch_bounds__(NT, 2)
+gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
+                    const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
+                    __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ chunk_states, const int32_t* gate) {
+    if (gate_closed(gate)) return;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *sQ = sm + SharedC::q, *sK = sm + SharedC::k, *sQa = sm + SharedC::qa, *sKa = sm + SharedC::ka,
+                  *sP = sm + SharedC::p, *sV = sQa;
+    float *sB = reinterpret_cast<float*>(sm + SharedC::b), *sTmp = reinterpret_cast<float*>(sP), *sR = reinterpret_cast<float*>(sQa);
+    int* srow = reinterpret_cast<int*>(sm + SharedC::row);
+    const uint32_t aQ = s_u32(sQ), aK = s_u32(sK), aB = s_u32(sB), aP = s_u32(sP), aV = s_u32(sV), aS = aB;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
+    const int chunk_lo = tb.seq_chunk_ptr[seq_lo], n_items = (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H;
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const int h = item % H, gc = chunk_lo + item / H;
+        const SeqInfo s = seq_info(tb, owner_of(tb, seq_lo, seq_hi, gc));
+        const int c = gc - s.chunk_base;
+        const bool has_s = c > 0 || s.init_slot >= 0;     // the state of a sequence that starts from zero is not read
+        __syncthreads();                                   // the previous item's readers of every tile are through
+        load_codes(tb, s, c, srow);
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < BT * 16 / NT; u++) {
+            const int p = tid + u * NT, t = p >> 4, c16 = p & 15, code = srow[t];
+            const size_t off = ((size_t)(code >= 0 ? code : code == -1 ? 0 : -2 - code) * H + h) * D + c16 * 8;
+            cp_async16(aQ + sw256(t, c16), q + off, code >= 0);
+            cp_async16(aK + sw256(t, c16), k + off, code != -1);
+        }
+#pragma unroll
+        for (int u = 0; u < BT * 32 / NT; u++) {
+            const int p = tid + u * NT, t = p >> 5, code = srow[t];
+            cp_async16(aB + p * 16, gk + ((size_t)(code >= 0 ? code : code == -1 ? 0 : -2 - code) * H + h) * D + (p & 31) * 4, code != -1);
+        }
+        const NextItem nx = next_item(s, c, gc, item, H, n_items);
+        if (nx.c >= 0) {
+            prefetch_rows(k, H, nx.h, s, nx.c);
+            prefetch_rows(q, H, nx.h, s, nx.c);
+            prefetch_rows(v, H, nx.h, s, nx.c);
+            prefetch_rows(gk, H, nx.h, s, nx.c);
+            prefetch_state(chunk_states, nx.gc, nx.h, H);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        cumsum_rows<true>(sB, sTmp);
+        const bool mild = chunk_is_mild(sB);
+        if (mild) mild_operands(sQ, sK, sB, sQa, sKa);
+        else anchored_operands(sQ, sK, sB, sQa, sKa);
+        __syncthreads();
+        auto load_state = [&] {                            // over the running sums
+            const __nv_bfloat16* src = chunk_states + ((size_t)gc * H + h) * (D * D);
+#pragma unroll
+            for (int u = 0; u < D * 16 / NT; u++) {
+                const int p = tid + u * NT;
+                cp_async16(aS + sw256(p >> 4, p & 15), src + p * 8, true);
+            }
+        };
+        if (mild && has_s) load_state();
+        uint4 vv[BT * 16 / NT];                            // V, on its way while the scores are computed
+#pragma unroll
+        for (int u = 0; u < BT * 16 / NT; u++) {
+            const int p = tid + u * NT, code = srow[p >> 4], r = code >= 0 ? code : -2 - code;
+            vv[u] = code != -1 ? *reinterpret_cast<const uint4*>(v + ((size_t)r * H + h) * D + (p & 15) * 8) : make_uint4(0, 0, 0, 0);
+        }
+        scores_off_diagonal(s_u32(sQa), s_u32(sKa), sP, warp, lane, mild, aK);
+        __syncthreads();                                   // the anchored operands are dead
+        if (!mild) {
+            step_factors(sB, sR);
+            __syncthreads();
+            scores_diagonal(sQ, sK, sR, sP, warp, lane);
+            __syncthreads();
+            scale_qk<true, false>(sQ, sK, sB, sQ, sK);
+            __syncthreads();
+            if (has_s) load_state();
+        }
+#pragma unroll
+        for (int u = 0; u < BT * 16 / NT; u++) {
+            const int p = tid + u * NT;
+            *reinterpret_cast<uint4*>(sV + sw256(p >> 4, p & 15)) = vv[u];
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        // ---- o = P V + q~ S_c : warp -> rows 16 * mb, columns 32 * nq ----------------------------------------------
+        const int m0 = mb * 16, n_base = nq * 32;
+        float acc[4][4];
+#pragma unroll
+        for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+        for (int ks = 0; ks <= mb; ks++) {              // P is zero right of the diagonal block
+            uint32_t a[4];
+            frag_a<128>(a, aP, m0, ks * 16, lane);
+#pragma unroll
+            for (int n2 = 0; n2 < 2; n2++) {
+                uint32_t b[4];
+                frag_b_kn<256>(b, aV, ks * 16, n_base + n2 * 16, lane);
+                mma16816(acc[2 * n2], a, b[0], b[1]);
+                mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
+            }
+        }
+        if (has_s)
+#pragma unroll
+            for (int ks = 0; ks < 8; ks++) {
+                uint32_t a[4];
+                frag_a<256>(a, aQ, m0, ks * 16, lane);
+#pragma unroll
+                for (int n2 = 0; n2 < 2; n2++) {
+                    uint32_t b[4];
+                    frag_b_kn<256>(b, aS, ks * 16, n_base + n2 * 16, lane);
+                    mma16816(acc[2 * n2], a, b[0], b[1]);
+                    mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
+                }
+            }
+        const int row_lo = srow[m0 + g], row_hi = srow[m0 + g + 8];
+#pragma unroll
+        for (int n = 0; n < 4; n++) {
+            const int col = n_base + n * 8 + tq * 2;
+            if (row_lo >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
+            if (row_hi >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
+        }
+    }
 }
 
 // ---- backward ---------------------------------------------------------------------------------------------------------
@@ -1150,7 +1308,7 @@ int32_t gk_mma_fwd(const FwdArgs& a) {
         return HARTS_ECUDA;
     const int n = (a.seq_hi - a.seq_lo) * a.H;
     gk_mma_fwd_kernel<ROUND><<<n, NT, Shared::fwd_bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
         nullptr, nullptr);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -1187,7 +1345,7 @@ int32_t gk_mma_fwd_all(const FwdArgs& a, int* flags, int* ticket) {
         return HARTS_ECUDA;
     if (cudaMemsetAsync(ticket, 0, sizeof(int), a.stream) != cudaSuccess) return HARTS_ECUDA;
     gk_mma_fwd_kernel<ONE_LAUNCH_MODE><<<(int)n, NT, Shared::fwd_bytes, a.stream>>>(
-        a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
+        a.tb, a.seq_lo, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
         flags, ticket);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -1216,13 +1374,12 @@ int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrd
 // Every (chunk, head) of sequences [seq_lo, seq_hi) on its own; the scan has left the states (and their gradients).
 int32_t gk_chunk_fwd(const FwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    if (cudaFuncSetAttribute(gk_mma_fwd_kernel<CHUNKS_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shared::fwd_bytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(gk_chunk_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedC::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
-    gk_mma_fwd_kernel<CHUNKS_MODE><<<(int)(n < sm_count() ? n : sm_count()), NT, Shared::fwd_bytes, a.stream>>>(
+    gk_chunk_fwd_kernel<<<(int)(n < 2 * sm_count() ? n : 2 * sm_count()), NT, SharedC::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
-        (__nv_bfloat16*)a.o, a.slots, (__nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status), a.dev_status,
-        nullptr, nullptr);
+        (__nv_bfloat16*)a.o, (const __nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
