@@ -141,14 +141,13 @@ int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      //
 int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
 int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles);     // la_chunk_bwd.cu
-// Taken up to 38,912 (chunk, head) items.  The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 400 KB:
-// with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.1 against 11.1 ms a step; 46 k items of agentic
-// trees 3.45 / 3.48, 41 k of branchy ones 3.51 / 3.61), with few the chain of its 3-6 us chunks is what takes the time (walk ->
-// chunk-parallel: 304 chunks x 4 heads 0.74 -> 0.24 ms; 2,389 x 16 3.04 -> 2.84; 1,047 x 16, forward, 0.87 -> 0.52).  Many
-// sequences of a chunk or two (fewer than four chunks each, more than 128 (sequence, head) pairs) stay with the walk: the scan
-// pays about 5 us for each of them.  The line depends on the tables' totals only, so that a round issued alone takes the path
-// of the whole.
-constexpr int64_t CHUNK_PARALLEL_MAX = 38912;
+// Taken up to 28,672 (chunk, head) items.  The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 400 KB:
+// with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.6 against 11.2 ms a step; 2,389 x 16: 3.0
+// against 3.1), with few the chain of its 3-6 us chunks is what takes the time (walk -> chunk-parallel: 304 chunks x 4 heads,
+// forward + backward, 0.74 -> 0.24 ms; 1,047 x 16, forward, 0.87 -> 0.52).  Many sequences of a chunk or two (fewer than
+// four chunks each, more than 128 (sequence, head) pairs) stay with the walk: the scan pays about 5 us for each of them.  The
+// line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
+constexpr int64_t CHUNK_PARALLEL_MAX = 28672;
 inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
     return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 &&
            (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
