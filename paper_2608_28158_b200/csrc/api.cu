@@ -297,7 +297,7 @@ int32_t harts_la_gk_workspace_bytes(const harts_la_tables_t* tb, int32_t H, int3
     const size_t elem = dtype == HARTS_FP32 ? 4 : 2;
     if (chunk_state_bytes)      // the states, then the flags of the one-launch forms
         *chunk_state_bytes = harts::chunk_state_payload(*tb, H, dk, dv, elem) + harts::fused_flag_bytes(*tb, H);
-    if (chunk_state_bytes && harts::gk_chunk_parallel(*tb, H, dk, dv, dtype, 0))
+    if (chunk_state_bytes && harts::chunk_parallel(*tb, H, dk, dv, dtype, 0))
         *chunk_state_bytes = harts::chunk_parallel_bytes(*tb, H, dk, dv);
     if (scratch_bytes) *scratch_bytes = harts::gk_scratch_layout(*tb, H, dk, dv).total;
     return HARTS_OK;
@@ -318,7 +318,7 @@ int32_t harts_la_gk_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32
         return HARTS_EINVAL;
     if ((flags & HARTS_FLAG_CHECK_TABLES) && !dev_status) return HARTS_EINVAL;
     const int32_t r0 = round == 0 ? 1 : round, r1 = round == 0 ? p->n_rounds : round;
-    const bool chunks = chunk_states && harts::gk_chunk_parallel(tb, H, dk, dv, dtype, flags);
+    const bool chunks = chunk_states && harts::chunk_parallel(tb, H, dk, dv, dtype, flags);
     if (chunks && round == 0 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && !(flags & HARTS_FLAG_ROUND_LAUNCHES)) {
         harts::FwdArgs a{tb, 0, tb.n_seq, q, k, v, gk, o, slots, chunk_states, H, dk, dv, dtype, flags, dev_status,
                          static_cast<cudaStream_t>(stream)};
@@ -365,7 +365,7 @@ int32_t harts_la_gk_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32
     if ((flags & HARTS_FLAG_CHECK_TABLES) && !dev_status) return HARTS_EINVAL;
     const int32_t r1 = round == 0 ? p->n_rounds : round, r0 = round == 0 ? 1 : round;
     bool done = false;
-    const bool chunks = harts::gk_chunk_parallel(tb, H, dk, dv, dtype, flags);
+    const bool chunks = harts::chunk_parallel(tb, H, dk, dv, dtype, flags);
     if (chunks && round == 0 && p->n_rounds <= harts::MAX_FUSED_ROUNDS && !(flags & HARTS_FLAG_ROUND_LAUNCHES)) {
         harts::BwdArgs a{tb, 0, tb.n_seq, q, k, v, gk, dO, dq, dk_, dv_, dgk, chunk_states, scratch, H, dk, dv, dtype, flags,
                          dev_status, static_cast<cudaStream_t>(stream)};
