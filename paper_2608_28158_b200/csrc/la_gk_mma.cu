@@ -118,11 +118,8 @@ __device__ __forceinline__ void load_codes(const harts_la_tables_t& tb, const Se
 }
 
 // The loads of a chunk go to shared memory by cp.async, all of them in flight at once (through registers they were a round
-// trip each: backward, 1,047 chunks x 16 heads, 2.59 -> 2.20 ms); loads_done() before the barrier that publishes them.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool take) {      // zeros where nothing is taken
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(take ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void loads_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// trip each: backward, 1,047 chunks x 16 heads, 2.59 -> 2.20 ms); cp_async_wait_all() before the barrier that publishes them.
+using tc::cp_async16;
 
 // One [BT][128] bf16 tile of a [rows, H, 128] tensor into a swizzled tile, 16 bytes at a time.  need_own: only rows
 // with an output are taken (q, dO); otherwise every valid row (k, v).  Rows that are not taken become zero.
@@ -132,7 +129,7 @@ __device__ __forceinline__ void load_tile_bf16(const __nv_bfloat16* src, int H, 
     for (int u = 0; u < BT * 16 / NT; u++) {
         const int p = threadIdx.x + u * NT, t = p >> 4, c16 = p & 15, code = srow[t];
         const int r = code >= 0 ? code : code == -1 ? 0 : -2 - code;
-        cp_async16(s_u32(dst) + sw256(t, c16), src + ((size_t)r * H + h) * D + c16 * 8, need_own ? code >= 0 : code != -1);
+        cp_async16(dst + sw256(t, c16), src + ((size_t)r * H + h) * D + c16 * 8, need_own ? code >= 0 : code != -1);
     }
 }
 
@@ -142,7 +139,7 @@ __device__ __forceinline__ void load_g(const float* gk, int H, int h, const int*
     for (int u = 0; u < BT * 32 / NT; u++) {
         const int p = threadIdx.x + u * NT, t = p >> 5, c4 = p & 31, code = srow[t];
         const int r = code >= 0 ? code : code == -1 ? 0 : -2 - code;
-        cp_async16(s_u32(sB) + p * 16, gk + ((size_t)r * H + h) * D + c4 * 4, code != -1);
+        cp_async16(reinterpret_cast<unsigned char*>(sB) + p * 16, gk + ((size_t)r * H + h) * D + c4 * 4, code != -1);
     }
 }
 
@@ -514,7 +511,7 @@ __device__ __forceinline__ void global_to_tile128(const __nv_bfloat16* src, unsi
 #pragma unroll
     for (int u = 0; u < D * 16 / NT; u++) {
         const int p = threadIdx.x + u * NT;
-        cp_async16(s_u32(tile) + sw256(p >> 4, p & 15), src + p * 8, true);
+        cp_async16(tile + sw256(p >> 4, p & 15), src + p * 8, true);
     }
 }
 
@@ -609,7 +606,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
             if (ONE_LAUNCH) __threadfence();               // this thread's part of the slot, before the flag below
             next_req++;
         }
-        loads_done();
+        tc::cp_async_wait_all();
         __syncthreads();
         if (ONE_LAUNCH && exported && tid == 0) tc::flag_set(slot_flags + (size_t)(next_req - 1) * H + h);
         if (chunk_states) tile_to_global<D>(sSb, chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems);
@@ -722,7 +719,7 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
             prefetch_rows(gk, H, nx.h, s, nx.c);
             prefetch_state(chunk_states, nx.gc, nx.h, H);
         }
-        loads_done();
+        tc::cp_async_wait_all();
         __syncthreads();
         cumsum_rows(sB, sTmp);
         const bool mild = chunk_is_mild(sB);
@@ -753,7 +750,7 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
             const int p = tid + u * NT;
             *reinterpret_cast<uint4*>(sV + sw256(p >> 4, p & 15)) = vv[u];
         }
-        loads_done();
+        tc::cp_async_wait_all();
         __syncthreads();
         // ---- o = P V + q~ S_c : warp -> rows 16 * mb, columns 32 * nq ----------------------------------------------
         const int m0 = mb * 16, n_base = nq * 32;
@@ -955,7 +952,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
         }
         if (!CHUNKS) state_to_operand(ds, sdSb, warp, lane);
         else if (has_ds) global_to_tile128(ds_tiles + ((size_t)gc * H + h) * state_elems, sdSb);
-        loads_done();
+        tc::cp_async_wait_all();
         __syncthreads();
         cumsum_rows(sB, sTmp);
         const bool mild = chunk_is_mild(sB);          // diagonal blocks as dense products too (see chunk_is_mild)

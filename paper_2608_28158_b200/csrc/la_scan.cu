@@ -66,10 +66,6 @@ struct Misc {
 };
 static_assert(sizeof(Misc) <= 12288, "misc area");
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-
 // a: the operand that spans the state's rows (k forward, q backward), b: the one that spans its columns (v / dO).
 // GK: a log-decay per row and state row (g [rows, H, 128]): its tile travels with the rows, and the weights go onto a.
 template <bool BWD, int NV, bool GK>
@@ -363,16 +359,16 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                         const int ch = lane & 15;
                         if (!BWD || t >= it.n_replay) {
                             if (lane < 16)
-                                cp_async16(smem_u32(sa + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), a + r + ch * 8);
+                                cp_async16(sa + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7), a + r + ch * 8, true);
                             else if (ch < S::B / PANEL * 8)
-                                cp_async16(smem_u32(sb + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7)), b + r + b0 + ch * 8);
+                                cp_async16(sb + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7), b + r + b0 + ch * 8, true);
                         } else {
                             *reinterpret_cast<uint4*>((lane < 16 ? sa : sb) + (lane < 16 || S::B > PANEL ? (ch >> 3) * PANEL : 0) + sw128_chunk(t, ch & 7)) =
                                 make_uint4(0, 0, 0, 0);
                         }
-                        if (GK) cp_async16(smem_u32(smem + S::g + st * S::G + t * (D * 4) + lane * 16), g + r + lane * 4);
+                        if (GK) cp_async16(smem + S::g + st * S::G + t * (D * 4) + lane * 16, g + r + lane * 4, true);
                     }
-                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    cp_async_wait_all();
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&m.full[st]);

@@ -26,6 +26,7 @@ namespace harts {
 
 int32_t make_row_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
 int32_t make_state_map(CUtensorMap* map, const void* base, int64_t n);
+int32_t make_state32_map(CUtensorMap* map, const void* base, int64_t n);
 int32_t make_out_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
 int sm_count();
 
@@ -213,7 +214,8 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
               const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
               const __grid_constant__ CUtensorMap map_do, const __grid_constant__ CUtensorMap map_cs,
               const __grid_constant__ CUtensorMap map_dq, const __grid_constant__ CUtensorMap map_dk,
-              const __grid_constant__ CUtensorMap map_dv, const __nv_bfloat16* __restrict__ q,
+              const __grid_constant__ CUtensorMap map_dv, const __grid_constant__ CUtensorMap map_ds0,
+              const __nv_bfloat16* __restrict__ q,
               const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ g,
               const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk_,
               __nv_bfloat16* __restrict__ dv_, float* __restrict__ dg, float* __restrict__ ds0, float* __restrict__ rk,
@@ -291,6 +293,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     const int seq = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
     // the item's record lives in shared memory and is read where it is needed: held in registers over the whole walk it
     // would push the kernel over its register budget
+    if (is_issuer) tma_store_wait_read();          // the previous item's dS0 has left the state tiles
     __syncthreads();                               // the previous item's last readers of the record are through
     if (tid == 0) {
         m.seq = seq_info(tb, seq);
@@ -411,23 +414,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         if (gathered) {
             for (int e = tid; e < BT * 16; e += NT) {
                 int row = e >> 4, ch = e & 15, code = rd.code[row];
-                uint4 zero = make_uint4(0, 0, 0, 0), kq = zero, vq = zero, qq = zero, dq4 = zero;
-                if (code != -1) {
-                    int r = code >= 0 ? code : -2 - code;
-                    size_t off = ((size_t)r * H + h) * D + ch * 8;
-                    kq = *reinterpret_cast<const uint4*>(k + off);
-                    vq = *reinterpret_cast<const uint4*>(v + off);
-                    if (code >= 0) {
-                        qq = *reinterpret_cast<const uint4*>(q + off);
-                        dq4 = *reinterpret_cast<const uint4*>(dO + off);
-                    }
-                }
-                uint32_t dst = (ch >> 3) * PANEL + sw128_chunk(row, ch & 7);
-                *reinterpret_cast<uint4*>(sQ + dst) = qq;
-                *reinterpret_cast<uint4*>(sK + dst) = kq;
-                *reinterpret_cast<uint4*>(sV + dst) = vq;
-                *reinterpret_cast<uint4*>(sDO + dst) = dq4;
+                const size_t off = ((size_t)(code >= 0 ? code : code == -1 ? 0 : -2 - code) * H + h) * D + ch * 8;
+                const uint32_t dst = (ch >> 3) * PANEL + sw128_chunk(row, ch & 7);
+                cp_async16(sQ + dst, q + off, code >= 0);
+                cp_async16(sK + dst, k + off, code != -1);
+                cp_async16(sV + dst, v + off, code != -1);
+                cp_async16(sDO + dst, dO + off, code >= 0);
             }
+            cp_async_wait_all();
             fence_async_smem();
             __syncthreads();
         }
@@ -818,7 +812,27 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (is_compute && s.init_slot >= 0) {
+    // One launch per round: staged over the state tiles (128-byte-swizzled panels of 32 columns) and stored by TMA, since a
+    // row per thread takes 32 lines per store instruction (6,949 one- and two-chunk sequence chunks x 16 heads: 8.68 -> 7.71
+    // ms).  All rounds in one launch: stored by the threads, so that each can
+    // fence its part before the flag.
+    if (!ONE_LAUNCH && s.init_slot >= 0) {
+        if (is_compute) {
+            uint32_t x[32];
+            tmem_ld32(tm_lane + COL_DS + grp * 32, x);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i4 = 0; i4 < 8; i4++)
+                *reinterpret_cast<uint4*>(sS + grp * S_PANEL + sw128_chunk(L, i4)) = make_uint4(x[i4 * 4], x[i4 * 4 + 1], x[i4 * 4 + 2], x[i4 * 4 + 3]);
+            fence_async_smem();
+        }
+        __syncthreads();
+        if (is_issuer) {
+            for (int p = 0; p < 4; p++) tma_store_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, seq * H + h);
+            tma_store_commit();
+        }
+    }
+    if (ONE_LAUNCH && is_compute && s.init_slot >= 0) {
         float* dst = ds0 + ((size_t)seq * H + h) * state_elems + (size_t)L * D;
         uint32_t x[32];
         tmem_ld32(tm_lane + COL_DS + grp * 32, x);
@@ -828,7 +842,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             reinterpret_cast<float4*>(dst + grp * 32)[i4] =
                 make_float4(__uint_as_float(x[i4 * 4]), __uint_as_float(x[i4 * 4 + 1]), __uint_as_float(x[i4 * 4 + 2]),
                             __uint_as_float(x[i4 * 4 + 3]));
-        if (ONE_LAUNCH) __threadfence();           // this thread's part, before the flag that follows the barrier below
+        __threadfence();                           // this thread's part, before the flag that follows the barrier below
     }
     if (ONE_LAUNCH && s.init_slot >= 0) {           // publish: the gradient of this sequence's initial state is in place
         if (!__syncthreads_or(m.dead) && tid == 0) flag_set(ds0_flags + (size_t)seq * H + h);
@@ -854,7 +868,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
 int32_t tc_bwd(const BwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     if (int32_t rc0 = handoff_reduce(a); rc0 != HARTS_OK) return rc0;
-    CUtensorMap mq, mk, mv, mdo, mcs, mdq, mdk, mdv;
+    CUtensorMap mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mds0;
     int32_t rc;
     if ((rc = make_row_map(&mq, a.q, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mk, a.k, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
@@ -869,10 +883,11 @@ int32_t tc_bwd(const BwdArgs& a) {
         return HARTS_ECUDA;
     ScratchLayout sl = scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
+    if ((rc = make_state32_map(&mds0, base + sl.ds0, (int64_t)a.tb.n_seq * a.H)) != HARTS_OK) return rc;
     int n = (a.seq_hi - a.seq_lo) * a.H;
     int grid = n < sm_count() ? n : sm_count();
     tc_bwd_kernel<false><<<grid, NT, Smem::bytes + 1024, a.stream>>>(
-        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
+        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mds0, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_,
         (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), a.dev_status, status_gate(a.flags, a.dev_status), nullptr, nullptr, RoundOrder{});
@@ -914,8 +929,9 @@ int32_t tc_bwd_fused(const BwdArgs& a, int* flags, int* ticket, const RoundOrder
     ScratchLayout sl = scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
     const int grid = n < sm_count() ? n : sm_count();
+    // (its hand-off gradients do not leave by TMA: any map in their place)
     tc_bwd_kernel<true><<<grid, NT, Smem::bytes + 1024, a.stream>>>(
-        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
+        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mdv, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_,
         (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), a.dev_status, status_gate(a.flags, a.dev_status), flags, ticket, rounds);

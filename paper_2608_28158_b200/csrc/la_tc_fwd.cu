@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(NT, 2)
 tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __grid_constant__ CUtensorMap map_q,
               const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
               const __grid_constant__ CUtensorMap map_cs, const __grid_constant__ CUtensorMap map_o,
-              const __nv_bfloat16* __restrict__ q,
+              const __grid_constant__ CUtensorMap map_slots, const __nv_bfloat16* __restrict__ q,
               const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ g,
               __nv_bfloat16* __restrict__ o, float* __restrict__ slots, int store_states, int* status,
               const int32_t* gate, int* slot_flags, int* ticket) {
@@ -180,18 +180,39 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         if (tid == 0) wait_for_slot(slot_flags + (size_t)s.init_slot * H + h, status, &m.dead);
         __syncthreads();
     }
-    // initial state into tensor memory: lane i = L holds S[i][:]
-    {
+    // initial state into tensor memory: lane i = L holds S[i][:].  One launch per round: 64 KB by TMA into 128-byte-swizzled
+    // panels of 32 columns over the (free) tiles, since a row per thread takes 32 lines per load instruction (a problem of
+    // one- and two-chunk sequences, 6,949 chunks x 16 heads: forward 3.60 -> 3.16 ms).
+    if (!ONE_LAUNCH && s.init_slot >= 0) {
+        if (tid == 0) {
+            tma_store_wait_read();                // the state store of the previous item has left sS
+            tma_pending = true;
+            mbar_expect_tx(&m.bar_tma, 4 * S_PANEL);
+            for (int p = 0; p < 4; p++)
+                tma_load_3d(smem + p * S_PANEL, &map_slots, p * 32, 0, s.init_slot * H + h, &m.bar_tma);
+        }
+        if (mbar_wait(&m.bar_tma, ph_tma, status, &m.dead)) {
+            ph_tma ^= 1;
+            tma_pending = false;
+        }
+        for (int blk = 2 * grp; blk < 2 * grp + 2; blk++) {
+            uint32_t x[32];
+#pragma unroll
+            for (int i4 = 0; i4 < 8; i4++)
+                *reinterpret_cast<uint4*>(x + 4 * i4) = *reinterpret_cast<const uint4*>(smem + blk * S_PANEL + sw128_chunk(L, i4));
+            tmem_st32(tm_lane + COL_S + blk * 32, x);
+        }
+        tmem_st_wait();
+        fence_async_smem();
+        __syncthreads();                          // the tiles are free again
+    } else {
         const float* src = s.init_slot < 0 ? nullptr : slots + ((size_t)s.init_slot * H + h) * state_elems + (size_t)L * D;
         for (int blk = 2 * grp; blk < 2 * grp + 2; blk++) {
             uint32_t x[32];
 #pragma unroll
             for (int i4 = 0; i4 < 8; i4++) {
-                // one launch: the slot was written during this launch by another CTA (read past L1); one launch per
-                // round: siblings that start from the same slot on this SM find it in L1
-                float4 a = !src ? make_float4(0.f, 0.f, 0.f, 0.f)
-                           : ONE_LAUNCH ? __ldcg(reinterpret_cast<const float4*>(src + blk * 32) + i4)
-                                        : reinterpret_cast<const float4*>(src + blk * 32)[i4];
+                // written during this launch by another CTA: read past L1
+                float4 a = !src ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcg(reinterpret_cast<const float4*>(src + blk * 32) + i4);
                 x[i4 * 4 + 0] = __float_as_uint(a.x);
                 x[i4 * 4 + 1] = __float_as_uint(a.y);
                 x[i4 * 4 + 2] = __float_as_uint(a.z);
@@ -260,19 +281,13 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             __syncthreads();
             for (int e = tid; e < BT * 16; e += NT) {
                 int row = e >> 4, ch = e & 15, code = m.code[row];
-                uint4 zero = make_uint4(0, 0, 0, 0), kq = zero, vq = zero, qq = zero;
-                if (code != -1) {
-                    int r = code >= 0 ? code : -2 - code;
-                    size_t off = ((size_t)r * H + h) * D + ch * 8;
-                    kq = *reinterpret_cast<const uint4*>(k + off);
-                    vq = *reinterpret_cast<const uint4*>(v + off);
-                    if (code >= 0) qq = *reinterpret_cast<const uint4*>(q + off);
-                }
-                uint32_t dst = (ch >> 3) * PANEL + sw128_chunk(row, ch & 7);
-                *reinterpret_cast<uint4*>(sQ + dst) = qq;
-                *reinterpret_cast<uint4*>(sK + dst) = kq;
-                *reinterpret_cast<uint4*>(sV + dst) = vq;
+                const size_t off = ((size_t)(code >= 0 ? code : code == -1 ? 0 : -2 - code) * H + h) * D + ch * 8;
+                const uint32_t dst = (ch >> 3) * PANEL + sw128_chunk(row, ch & 7);
+                cp_async16(sQ + dst, q + off, code >= 0);
+                cp_async16(sK + dst, k + off, code != -1);
+                cp_async16(sV + dst, v + off, code != -1);
             }
+            cp_async_wait_all();                  // all rows in flight at once; by registers it was four round trips
             fence_async_smem();
         }
         __syncthreads();                          // (2) codes, gathered tiles, partial sums visible
@@ -516,6 +531,18 @@ int32_t make_state_map(CUtensorMap* map, const void* base, int64_t n) {
     return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
 }
 
+// [n][128][128] fp32 states (exported slots, hand-off gradients), box = 1 state x 128 rows x 32 columns
+int32_t make_state32_map(CUtensorMap* map, const void* base, int64_t n) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return HARTS_ECUDA;
+    cuuint64_t dims[3] = {128, 128, (cuuint64_t)(n < 1 ? 1 : n)}, strides[2] = {512, 65536};
+    cuuint32_t box[3] = {32, 128, 1}, es[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+}
+
 // 32-column slices of [n][128][128] bf16 states, box = 1 state x 128 rows, 64-byte swizzle
 int32_t make_state_slice_map(CUtensorMap* map, const void* base, int64_t n) {
     EncodeTiledFn fn = encode_fn();
@@ -567,7 +594,7 @@ int32_t tc_supported(int32_t dtype, int32_t dk, int32_t dv) { return dtype == HA
 
 int32_t tc_fwd(const FwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    CUtensorMap mq, mk, mv, mcs, mo;
+    CUtensorMap mq, mk, mv, mcs, mo, ms;
     int32_t rc;
     if ((rc = make_row_map(&mq, a.q, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mk, a.k, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
@@ -575,13 +602,14 @@ int32_t tc_fwd(const FwdArgs& a) {
     const void* cs = a.chunk_states ? a.chunk_states : a.q;   // a valid address for the (unused) map
     if ((rc = make_state_map(&mcs, cs, a.chunk_states ? (int64_t)a.tb.n_chunks * a.H : 1)) != HARTS_OK) return rc;
     if ((rc = make_out_map(&mo, a.o, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
+    if ((rc = make_state32_map(&ms, a.slots ? (const void*)a.slots : a.q, (int64_t)a.tb.n_slots * a.H)) != HARTS_OK) return rc;
     if (cudaFuncSetAttribute(tc_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::bytes + 1024) !=
         cudaSuccess)
         return HARTS_ECUDA;
     int n = (a.seq_hi - a.seq_lo) * a.H;
     int grid = n < 2 * sm_count() ? n : 2 * sm_count();
     tc_fwd_kernel<false><<<grid, NT, Smem::bytes + 1024, a.stream>>>(
-        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mcs, mo, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
+        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mcs, mo, ms, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (__nv_bfloat16*)a.o, a.slots, a.chunk_states != nullptr, a.dev_status,
         status_gate(a.flags, a.dev_status), nullptr, nullptr);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -621,8 +649,9 @@ int32_t tc_fwd_fused(const FwdArgs& a, int* flags, int* ticket) {
     if (cudaMemsetAsync(ticket, 0, sizeof(int), a.stream) != cudaSuccess) return HARTS_ECUDA;
     int n = (a.seq_hi - a.seq_lo) * a.H;
     int grid = n < 2 * sm_count() ? n : 2 * sm_count();
+    // (its initial states do not come by TMA: any map in place of the slots')
     tc_fwd_kernel<true><<<grid, NT, Smem::bytes + 1024, a.stream>>>(
-        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mcs, mo, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
+        a.tb, a.seq_lo, n, a.H, mq, mk, mv, mcs, mo, mcs, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (__nv_bfloat16*)a.o, a.slots, a.chunk_states != nullptr, a.dev_status,
         status_gate(a.flags, a.dev_status), flags, ticket);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
