@@ -52,7 +52,7 @@ struct Smem {
     static constexpr int q = 0, k = TILE, v = 2 * TILE, dO = 3 * TILE, dOs = 4 * TILE, p = 5 * TILE,
                          dp = 5 * TILE + PANEL, s = 5 * TILE + 2 * PANEL, ds = s + 2 * S_PANEL,
                          stage_dq = ds + 2 * S_PANEL, stage_dk = stage_dq + TILE, stage_dv = stage_dk + TILE,
-                         misc = stage_dv + TILE;       // stage_*: outputs of a full chunk, [row][feature], for TMA stores
+                         misc = stage_dv + TILE;       // stage_*: outputs, swizzled [row][64 features] panels
     static constexpr int bytes = misc + 4096;
 };
 struct RowData {             // per-chunk row quantities, double-buffered (the next chunk's are prepared in the tail)
@@ -93,94 +93,14 @@ __device__ __forceinline__ SeqInfo seq_info(const harts_la_tables_t& tb, int seq
     return s;
 }
 
-// Sum over the 32 lanes of a warp for each of 16 per-lane values; lane l returns the total of z[l & 15].
-__device__ __forceinline__ float warp_transpose_reduce16(float (&z)[16], int lane) {
-#pragma unroll
-    for (int s = 8; s >= 1; s >>= 1) {
-        const bool upper = (lane & s) != 0;
-#pragma unroll
-        for (int i = 0; i < s; i++) {
-            float send = upper ? z[i] : z[i + s];
-            float keep = upper ? z[i + s] : z[i];
-            z[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-    return z[0] + __shfl_xor_sync(0xffffffffu, z[0], 16);
-}
-
-// ---- partial chunks (a ragged tail, or chunk 0 of a sequence that replays ancestor rows) ------------------------------
-// Epilogue for this thread's feature index L and its 16 rows, in three parts that follow the three commits of the MMA
-// batch (dk, dv, dq: the longest part first, so that little is left after the last MMA).  qk[e] holds q[t][L] (low
-// half) and k[t][L] (high half) as bf16 bits, read from the tiles before the batch so that the tiles can be reloaded
-// while the epilogue runs.  The outputs are staged in shared memory ([row][feature], plain layout); the compute warps
-// copy the valid rows out after the epilogue (own rows to the outputs, replayed rows, staged in fp32, to the scratch).
-__device__ __forceinline__ void epilogue_dq(const RowData& m, unsigned char* smem, uint32_t tm_lane, int grp, int L, int H,
-                                            int h, const uint32_t (&qk)[16], __nv_bfloat16* dq, float (&z)[16]) {
-    const int t0 = grp * 16;
-    uint32_t xq[16];
-    tmem_ld16(tm_lane + COL_DQ + t0, xq);
-    tmem_ld_wait();
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int t = t0 + e;
-        const float dqv = __uint_as_float(xq[e]);
-        const float qv = __uint_as_float(qk[e] << 16);
-        z[e] += (m.code[t] != -1) ? qv * dqv : 0.f;
-        // replayed rows have no dq; their row of this staging tile holds one half of their fp32 dk (epilogue_dk)
-        if (m.code[t] >= -1)
-            *reinterpret_cast<__nv_bfloat16*>(smem + Smem::stage_dq + t * 256 + L * 2) = __float2bfloat16_rn(dqv);
-    }
-}
-
-__device__ __forceinline__ void epilogue_dk(const RowData& m, unsigned char* smem, uint32_t tm_lane, int grp, int L, int H,
-                                            int h, int replay_base, const uint32_t (&qk)[16], __nv_bfloat16* dk_,
-                                            float* rk, float (&z)[16], float& g_part) {
-    const int t0 = grp * 16;
-    uint32_t xi[16], xe[16];
-    tmem_ld16(tm_lane + COL_DK + t0, xi);
-    tmem_ld16(tm_lane + COL_A + t0, xe);
-    tmem_ld_wait();
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int t = t0 + e;
-        const float kv = __uint_as_float(qk[e] & 0xffff0000u);
-        const float inter = m.w[t] * __uint_as_float(xe[e]);
-        const float dkv = __uint_as_float(xi[e]) + inter;
-        const bool row_ok = m.code[t] != -1;
-        z[e] = row_ok ? -kv * dkv : 0.f;
-        g_part += row_ok ? kv * inter : 0.f;
-        // replayed rows (chunk 0 only) keep fp32: features 0..63 in the row's 256 bytes of the dk staging tile,
-        // 64..127 in its row of the dq staging tile (replayed rows have no dq); every operand tile is still being read
-        if (m.code[t] < -1)
-            *reinterpret_cast<float*>(smem + (L < 64 ? Smem::stage_dk : Smem::stage_dq) + t * 256 + (L & 63) * 4) = dkv;
-        else
-            *reinterpret_cast<__nv_bfloat16*>(smem + Smem::stage_dk + t * 256 + L * 2) = __float2bfloat16_rn(dkv);
-    }
-}
-
-__device__ __forceinline__ void epilogue_dv(const RowData& m, unsigned char* smem, uint32_t tm_lane, int grp, int L, int H,
-                                            int h, int replay_base, __nv_bfloat16* dv_, float* rv) {
-    const int t0 = grp * 16;
-    uint32_t xi[16], xe[16];
-    tmem_ld16(tm_lane + COL_DV + t0, xi);
-    tmem_ld16(tm_lane + COL_DA + t0, xe);
-    tmem_ld_wait();
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int t = t0 + e;
-        const float dvv = __uint_as_float(xi[e]) + m.w[t] * __uint_as_float(xe[e]);
-        *reinterpret_cast<__nv_bfloat16*>(smem + Smem::stage_dv + t * 256 + L * 2) = __float2bfloat16_rn(dvv);
-        // replayed rows: fp32 over the bf16 copy of dS, which no MMA reads once the dk and dv groups are done
-        if (m.code[t] < -1) *reinterpret_cast<float*>(smem + Smem::ds + t * 512 + L * 4) = dvv;
-    }
-}
-
-// ---- full chunks: the epilogue in matrix-fragment layout -------------------------------------------------------------
-// All 64 rows of the chunk are own rows.  A warp covers 32 features (its tensor-memory lane quarter) x 16 rows t (its
+// ---- the epilogue in matrix-fragment layout ---------------------------------------------------------------------------
+// A warp covers 32 features (its tensor-memory lane quarter) x 16 rows t (its
 // column group); tcgen05.ld hands every thread 16 values as fragments of 8x8 matrices: features f = m + 8 fa
 // (m = lane >> 2, fa = 0..3), rows t = t0 + 8 ta + 2 c + {0, 1} (c = lane & 3, ta = 0, 1).  q and k arrive in the same
 // layout by ldmatrix (transposing), the outputs leave by stmatrix (transposing) into 128-byte-swizzled [row][64
-// features] panels that TMA stores pick up: no 2-byte shared-memory accesses and no transposed reads.
+// features] panels that TMA stores (a full chunk) or 16-byte copies (a ragged tail, a chunk with replayed rows) pick up:
+// no 2-byte shared-memory accesses and no transposed reads.  Replayed rows' fp32 gradients leave straight from the
+// fragments (6,949 one- and two-chunk sequence chunks x 16 heads: 6.76 against 7.71 ms with staged 2-byte stores).
 struct Frag {
     uint32_t q[2][4], k[2][4];      // [ta][fa], two bf16 per register: rows t, t + 1
 };
@@ -456,7 +376,6 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             }
         }
         float g_part = 0.f;                       // this thread's share of <S_{c+1}, dS_{c+1}>
-        uint32_t qk[16];                          // q[t][L] | k[t][L] << 16 of this thread's 16 rows (bf16 bits)
         if (is_compute) {
             // ---- dS pass: add hand-off gradients, bf16 operand copy, <S_c, dS>, pre-scale by gamma -----------------
             {
@@ -623,123 +542,106 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
         if (is_aux && c > 0) store_rows(m.rows[cur ^ 1], nx_code, nx_g);   // visible to the others at barrier (B)
         if (is_compute) {
-            if (full) {
-                const int c4 = lane & 3, Lq = (warp & 3) * 32, t0 = grp * 16;
-                Frag fr;
+            const int c4 = lane & 3, Lq = (warp & 3) * 32, t0 = grp * 16;
+            Frag fr;
 #pragma unroll
-                for (int ta = 0; ta < 2; ta++) {
-                    ldmatrix_x4_trans(frag_addr(aQ, lane, Lq, t0, ta), fr.q[ta]);
-                    ldmatrix_x4_trans(frag_addr(aK, lane, Lq, t0, ta), fr.k[ta]);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&m.bar_qk_read);
-                // e^{b_n - b_t} of this thread's four rows: t0 + 2c, +1, t0 + 8 + 2c, +1
-                const float2 wlo = *reinterpret_cast<const float2*>(rd.w + t0 + 2 * c4);
-                const float2 whi = *reinterpret_cast<const float2*>(rd.w + t0 + 8 + 2 * c4);
-                const float wv[4] = {wlo.x, wlo.y, whi.x, whi.y};
-                float zf[4] = {0.f, 0.f, 0.f, 0.f};              // q.dq - k.dk over this thread's features, per row
-                float val[2][8];
-                uint32_t xi[2][8], xe[2][8];
-                // ---- dk -----------------------------------------------------------------------------------------------
-                mbar_wait(&m.bar_o, ph_o, status, &m.dead);
-                tc_fence_after();
-#pragma unroll
-                for (int l = 0; l < 2; l++) {
-                    tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DK + t0, xi[l]);
-                    tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_A + t0, xe[l]);
-                }
-                tmem_ld_wait();
-#pragma unroll
-                for (int l = 0; l < 2; l++)
-#pragma unroll
-                    for (int r = 0; r < 8; r++) {
-                        const int ti = 2 * (r >> 2) + (r & 1);
-                        const float kv = frag_elem(fr.k, l, r);
-                        const float inter = wv[ti] * __uint_as_float(xe[l][r]);
-                        const float dkv = __uint_as_float(xi[l][r]) + inter;
-                        zf[ti] -= kv * dkv;
-                        g_part += kv * inter;
-                        val[l][r] = dkv;
-                    }
-                frag_store(smem_u32(smem + Smem::stage_dk), lane, Lq, t0, val);
-#pragma unroll
-                for (int o_ = 16; o_ > 0; o_ >>= 1) g_part += __shfl_xor_sync(0xffffffffu, g_part, o_);
-                if (lane == 0) m.gred[warp] = g_part;
-                // ---- dv -----------------------------------------------------------------------------------------------
-                mbar_wait(&m.bar_o2, ph_o, status, &m.dead);
-                tc_fence_after();
-#pragma unroll
-                for (int l = 0; l < 2; l++) {
-                    tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DV + t0, xi[l]);
-                    tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DA + t0, xe[l]);
-                }
-                tmem_ld_wait();
-#pragma unroll
-                for (int l = 0; l < 2; l++)
-#pragma unroll
-                    for (int r = 0; r < 8; r++)
-                        val[l][r] = __uint_as_float(xi[l][r]) + wv[2 * (r >> 2) + (r & 1)] * __uint_as_float(xe[l][r]);
-                frag_store(smem_u32(smem + Smem::stage_dv), lane, Lq, t0, val);
-                // ---- dq -----------------------------------------------------------------------------------------------
-                mbar_wait(&m.bar_o3, ph_o, status, &m.dead);
-                tc_fence_after();
-#pragma unroll
-                for (int l = 0; l < 2; l++) tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DQ + t0, xi[l]);
-                tmem_ld_wait();
-#pragma unroll
-                for (int l = 0; l < 2; l++)
-#pragma unroll
-                    for (int r = 0; r < 8; r++) {
-                        const float dqv = __uint_as_float(xi[l][r]);
-                        zf[2 * (r >> 2) + (r & 1)] += frag_elem(fr.q, l, r) * dqv;
-                        val[l][r] = dqv;
-                    }
-                frag_store(smem_u32(smem + Smem::stage_dq), lane, Lq, t0, val);
-                // rows are shared by the eight threads with the same c: sum over them, then one writer per row
-#pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 4);
-                    zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 8);
-                    zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 16);
-                }
-                if (lane < 4) {
-                    m.red[warp][2 * c4] = zf[0];
-                    m.red[warp][2 * c4 + 1] = zf[1];
-                    m.red[warp][8 + 2 * c4] = zf[2];
-                    m.red[warp][8 + 2 * c4 + 1] = zf[3];
-                }
-            } else {
-            // q[t][L], k[t][L] of this thread's 16 rows, for the dg terms (read while the first MMAs run; after this
-            // the epilogue does not touch the tiles, which are reloaded as soon as the MMAs are done)
-            {
-                const uint32_t qk_base = (L >> 6) * PANEL + (L & 7) * 2;
-                const uint32_t cL = (L & 63) >> 3;
-#pragma unroll
-                for (int e = 0; e < 16; e++) {
-                    const int t = grp * 16 + e;
-                    const uint32_t off = qk_base + t * 128 + ((cL ^ (uint32_t)(t & 7)) << 4);
-                    qk[e] = (uint32_t)*reinterpret_cast<const unsigned short*>(sQ + off) |
-                            ((uint32_t)*reinterpret_cast<const unsigned short*>(sK + off) << 16);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&m.bar_qk_read);
+            for (int ta = 0; ta < 2; ta++) {
+                ldmatrix_x4_trans(frag_addr(aQ, lane, Lq, t0, ta), fr.q[ta]);
+                ldmatrix_x4_trans(frag_addr(aK, lane, Lq, t0, ta), fr.k[ta]);
             }
-            // ---- epilogue in three parts, each as soon as its accumulators are complete -------------------------------
-            float z[16];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&m.bar_qk_read);
+            // e^{b_n - b_t} of this thread's four rows: t0 + 2c, +1, t0 + 8 + 2c, +1
+            const float2 wlo = *reinterpret_cast<const float2*>(rd.w + t0 + 2 * c4);
+            const float2 whi = *reinterpret_cast<const float2*>(rd.w + t0 + 8 + 2 * c4);
+            const float wv[4] = {wlo.x, wlo.y, whi.x, whi.y};
+            int code[4];
+            *reinterpret_cast<int2*>(code) = *reinterpret_cast<const int2*>(rd.code + t0 + 2 * c4);
+            *reinterpret_cast<int2*>(code + 2) = *reinterpret_cast<const int2*>(rd.code + t0 + 8 + 2 * c4);
+            auto replay_store = [&](float* dst, const float (&val)[2][8]) {      // eight lanes = one 32-byte piece
+                const int mrow = lane >> 2;
+#pragma unroll
+                for (int l = 0; l < 2; l++)
+#pragma unroll
+                    for (int r = 0; r < 8; r++) {
+                        const int t = t0 + 8 * (r >> 2) + 2 * c4 + (r & 1);
+                        if (code[2 * (r >> 2) + (r & 1)] < -1)
+                            dst[((size_t)(s.replay_base + t) * H + h) * D + Lq + 16 * l + 8 * ((r >> 1) & 1) + mrow] = val[l][r];
+                    }
+            };
+            float zf[4] = {0.f, 0.f, 0.f, 0.f};              // q.dq - k.dk over this thread's features, per row
+            float val[2][8];
+            uint32_t xi[2][8], xe[2][8];
+            // ---- dk -----------------------------------------------------------------------------------------------
             mbar_wait(&m.bar_o, ph_o, status, &m.dead);
             tc_fence_after();
-            epilogue_dk(rd, smem, tm_lane, grp, L, H, h, s.replay_base, qk, dk_, rk, z, g_part);
+#pragma unroll
+            for (int l = 0; l < 2; l++) {
+                tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DK + t0, xi[l]);
+                tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_A + t0, xe[l]);
+            }
+            tmem_ld_wait();
+#pragma unroll
+            for (int l = 0; l < 2; l++)
+#pragma unroll
+                for (int r = 0; r < 8; r++) {
+                    const int ti = 2 * (r >> 2) + (r & 1);
+                    const float kv = frag_elem(fr.k, l, r);
+                    const float inter = wv[ti] * __uint_as_float(xe[l][r]);
+                    const float dkv = __uint_as_float(xi[l][r]) + inter;
+                    const bool ok = code[ti] != -1;
+                    zf[ti] -= ok ? kv * dkv : 0.f;
+                    g_part += ok ? kv * inter : 0.f;
+                    val[l][r] = dkv;
+                }
+            frag_store(smem_u32(smem + Smem::stage_dk), lane, Lq, t0, val);
+            if (gathered) replay_store(rk, val);
 #pragma unroll
             for (int o_ = 16; o_ > 0; o_ >>= 1) g_part += __shfl_xor_sync(0xffffffffu, g_part, o_);
             if (lane == 0) m.gred[warp] = g_part;
+            // ---- dv -----------------------------------------------------------------------------------------------
             mbar_wait(&m.bar_o2, ph_o, status, &m.dead);
             tc_fence_after();
-            epilogue_dv(rd, smem, tm_lane, grp, L, H, h, s.replay_base, dv_, rv);
+#pragma unroll
+            for (int l = 0; l < 2; l++) {
+                tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DV + t0, xi[l]);
+                tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DA + t0, xe[l]);
+            }
+            tmem_ld_wait();
+#pragma unroll
+            for (int l = 0; l < 2; l++)
+#pragma unroll
+                for (int r = 0; r < 8; r++)
+                    val[l][r] = __uint_as_float(xi[l][r]) + wv[2 * (r >> 2) + (r & 1)] * __uint_as_float(xe[l][r]);
+            frag_store(smem_u32(smem + Smem::stage_dv), lane, Lq, t0, val);
+            if (gathered) replay_store(rv, val);
+            // ---- dq -----------------------------------------------------------------------------------------------
             mbar_wait(&m.bar_o3, ph_o, status, &m.dead);
             tc_fence_after();
-            epilogue_dq(rd, smem, tm_lane, grp, L, H, h, qk, dq, z);
-            const float row_total = warp_transpose_reduce16(z, lane);
-            if (lane < 16) m.red[warp][lane] = row_total;
+#pragma unroll
+            for (int l = 0; l < 2; l++) tmem_ld_frag16(tm_lane + ((uint32_t)(16 * l) << 16) + COL_DQ + t0, xi[l]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int l = 0; l < 2; l++)
+#pragma unroll
+                for (int r = 0; r < 8; r++) {
+                    const float dqv = __uint_as_float(xi[l][r]);
+                    zf[2 * (r >> 2) + (r & 1)] += code[2 * (r >> 2) + (r & 1)] >= 0 ? frag_elem(fr.q, l, r) * dqv : 0.f;
+                    val[l][r] = dqv;
+                }
+            frag_store(smem_u32(smem + Smem::stage_dq), lane, Lq, t0, val);
+            // rows are shared by the eight threads with the same c: sum over them, then one writer per row
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 4);
+                zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 8);
+                zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 16);
+            }
+            if (lane < 4) {
+                m.red[warp][2 * c4] = zf[0];
+                m.red[warp][2 * c4 + 1] = zf[1];
+                m.red[warp][8 + 2 * c4] = zf[2];
+                m.red[warp][8 + 2 * c4 + 1] = zf[3];
             }
             if (full) fence_async_smem();
         }
@@ -749,26 +651,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         tc_fence_after();
         if (gave_up) break;
         if (is_compute && !full) {
-            // partial chunk: the staged rows leave with 16-byte stores, own rows to the outputs (bf16), replayed rows
-            // to the scratch (fp32); rows past the end go nowhere
+            // partial chunk: the staged own rows leave with 16-byte stores
             for (int e = tid; e < BT * 16 * 3; e += NC) {
-                const int which = e / (BT * 16), t = (e / 16) % BT, j = e % 16, code = rd.code[t];
+                const int which = e / (BT * 16), t = (e / 16) % BT, ch = e % 16, code = rd.code[t];
                 if (code < 0) continue;
                 __nv_bfloat16* out = which == 0 ? dq : (which == 1 ? dk_ : dv_);
-                const int stage = which == 0 ? Smem::stage_dq : (which == 1 ? Smem::stage_dk : Smem::stage_dv);
-                *reinterpret_cast<uint4*>(out + ((size_t)code * H + h) * D + j * 8) =
-                    *reinterpret_cast<const uint4*>(smem + stage + t * 256 + j * 16);
+                *reinterpret_cast<uint4*>(out + ((size_t)code * H + h) * D + ch * 8) = *reinterpret_cast<const uint4*>(
+                    smem + Smem::stage_dq + which * TILE + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7));
             }
-            if (gathered)
-                for (int e = tid; e < BT * 32 * 2; e += NC) {
-                    const int which = e / (BT * 32), t = (e / 32) % BT, j = e % 32;
-                    if (rd.code[t] >= -1) continue;
-                    float* out = which == 0 ? rk : rv;
-                    const int src = which == 1 ? Smem::ds + t * 512 + j * 16
-                                               : (j < 16 ? Smem::stage_dk : Smem::stage_dq) + t * 256 + (j & 15) * 16;
-                    *reinterpret_cast<float4*>(out + ((size_t)(s.replay_base + t) * H + h) * D + j * 4) =
-                        *reinterpret_cast<const float4*>(smem + src);
-                }
         }
         if (is_issuer && full) {
             int row0 = s.own_begin - s.n_replay + c * BT;
