@@ -141,17 +141,20 @@ int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      //
 int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
 int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles);     // la_chunk_bwd.cu
-// Taken up to 28,672 (chunk, head) items.  The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 400 KB:
-// with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.6 against 11.2 ms a step; 2,389 x 16: 3.0
-// against 3.1), with few the chain of its 3-6 us chunks is what takes the time (walk -> chunk-parallel: 304 chunks x 4 heads,
-// forward + backward, 0.74 -> 0.24 ms; 1,047 x 16, forward, 0.87 -> 0.52).  Many sequences of a chunk or two (fewer than
-// four chunks each, more than 128 (sequence, head) pairs) stay with the walk: the scan pays about 5 us for each of them.  The
-// line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
-constexpr int64_t CHUNK_PARALLEL_MAX = 28672;
+// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs.  The walk kernels (la_tc_*.cu) move 240 KB per item in
+// a whole step, this path 400 KB: with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.7 against 11.2
+// ms a step; 2,389 x 16: 3.0 against 3.1; 685 chunks in 21 sequences x 32 heads: 1.70 against 1.85), with few the chain of its
+// 3-6 us chunks is what takes the time (walk -> chunk-parallel: 304 chunks x 4 heads, forward + backward, 0.74 -> 0.24 ms;
+// 1,047 chunks in 28 sequences x 16, forward, 0.87 -> 0.52).  With r = longest path of chunks over the average sequence (5 to
+// 10), the walk's chain is longer than this path's time while n_seq * H < about 100 r.  Many sequences of a chunk or two (fewer
+// than four chunks each, more than 128 pairs) stay with the walk: the scan pays about 5 us for each of them.  The line
+// depends on the tables' totals only, so that a round issued alone takes the path of the whole.
+constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640;
 inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
+    const int64_t chains = (int64_t)tb.n_seq * H;
     return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 &&
-           (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
-           (tb.n_chunks >= 4 * (int64_t)tb.n_seq || (int64_t)tb.n_seq * H <= 128);
+           (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX && chains <= CHUNK_PARALLEL_CHAINS &&
+           (tb.n_chunks >= 4 * (int64_t)tb.n_seq || chains <= 128);
 }
 // the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then the scan's
 // ticket and counters

@@ -46,3 +46,17 @@ def test_both_sides_of_the_chunk_parallel_line(heads):
     _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
     for n in out:
         assert torch.equal(out[n], rounds[n]), n
+
+
+@pytest.mark.parametrize("heads", [64, 65])
+def test_both_sides_of_the_chain_line(heads):
+    """Ten sequences of four or more chunks: 640 (sequence, head) pairs take the chunk-parallel path, 650 the walk."""
+    fo = make_forest([([-1] + [0] * 9, [0] + [256] * 9, [512] + [270] * 9)])
+    inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 13, device="cuda")
+    plan, out = run_gpu(fo, inp)
+    assert plan.n_seq == 10 and plan.n_chunks >= 40
+    tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1])
+    check(compare(out, tok, [0, heads - 1], ref, rows=True), "bf16")
+    _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
+    for n in out:
+        assert torch.equal(out[n], rounds[n]), n
