@@ -100,7 +100,7 @@ __device__ __forceinline__ SeqInfo seq_info(const harts_la_tables_t& tb, int seq
 // layout by ldmatrix (transposing), the outputs leave by stmatrix (transposing) into 128-byte-swizzled [row][64
 // features] panels that TMA stores (a full chunk) or 16-byte copies (a ragged tail, a chunk with replayed rows) pick up:
 // no 2-byte shared-memory accesses and no transposed reads.  Replayed rows' fp32 gradients leave straight from the
-// fragments (6,949 one- and two-chunk sequence chunks x 16 heads: 6.76 against 7.71 ms with staged 2-byte stores).
+// fragments (6,949 one- and two-chunk sequence chunks x 16 heads: 6.69 against 7.71 ms with staged 2-byte stores).
 struct Frag {
     uint32_t q[2][4], k[2][4];      // [ta][fa], two bf16 per register: rows t, t + 1
 };
@@ -569,7 +569,8 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                             dst[((size_t)(s.replay_base + t) * H + h) * D + Lq + 16 * l + 8 * ((r >> 1) & 1) + mrow] = val[l][r];
                     }
             };
-            float zf[4] = {0.f, 0.f, 0.f, 0.f};              // q.dq - k.dk over this thread's features, per row
+            // q.dq - k.dk and k.(inter-chunk dk) over this thread's features, per row; rows past the end are dropped from the sums
+            float zf[4] = {0.f, 0.f, 0.f, 0.f}, gs[4] = {0.f, 0.f, 0.f, 0.f};
             float val[2][8];
             uint32_t xi[2][8], xe[2][8];
             // ---- dk -----------------------------------------------------------------------------------------------
@@ -589,13 +590,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                     const float kv = frag_elem(fr.k, l, r);
                     const float inter = wv[ti] * __uint_as_float(xe[l][r]);
                     const float dkv = __uint_as_float(xi[l][r]) + inter;
-                    const bool ok = code[ti] != -1;
-                    zf[ti] -= ok ? kv * dkv : 0.f;
-                    g_part += ok ? kv * inter : 0.f;
+                    zf[ti] -= kv * dkv;
+                    gs[ti] += kv * inter;
                     val[l][r] = dkv;
                 }
             frag_store(smem_u32(smem + Smem::stage_dk), lane, Lq, t0, val);
             if (gathered) replay_store(rk, val);
+#pragma unroll
+            for (int u = 0; u < 4; u++) g_part += code[u] != -1 ? gs[u] : 0.f;
 #pragma unroll
             for (int o_ = 16; o_ > 0; o_ >>= 1) g_part += __shfl_xor_sync(0xffffffffu, g_part, o_);
             if (lane == 0) m.gred[warp] = g_part;
@@ -626,13 +628,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
 #pragma unroll
                 for (int r = 0; r < 8; r++) {
                     const float dqv = __uint_as_float(xi[l][r]);
-                    zf[2 * (r >> 2) + (r & 1)] += code[2 * (r >> 2) + (r & 1)] >= 0 ? frag_elem(fr.q, l, r) * dqv : 0.f;
+                    zf[2 * (r >> 2) + (r & 1)] += frag_elem(fr.q, l, r) * dqv;      // replayed rows: q is zero
                     val[l][r] = dqv;
                 }
             frag_store(smem_u32(smem + Smem::stage_dq), lane, Lq, t0, val);
             // rows are shared by the eight threads with the same c: sum over them, then one writer per row
 #pragma unroll
             for (int i = 0; i < 4; i++) {
+                zf[i] = code[i] != -1 ? zf[i] : 0.f;
                 zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 4);
                 zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 8);
                 zf[i] += __shfl_xor_sync(0xffffffffu, zf[i], 16);
