@@ -43,8 +43,9 @@ def harts_attn_index(tree_node_ptr, node_parent, node_fork_off, node_len, row_of
     rot = None if row_of_token is None else np.ascontiguousarray(np.asarray(row_of_token), dtype=np.int32)
     ip = lambda a: None if a is None else a.ctypes.data_as(_I32P)  # noqa: E731
     n = _i64(0)
-    # room for what forests usually need, so that the tables are built once; the call says how much it wants otherwise
-    blob = np.zeros(4096 + 64 * len(arrs[1]) + int(arrs[3].sum(dtype=np.int64)) // 16, np.int32)
+    # room for what forests usually need, so that the tables are built once; the call says how much it wants otherwise.
+    # The lengths are not checked yet, so they ask for 4 MB at most.
+    blob = np.zeros(4096 + 64 * len(arrs[1]) + min(max(int(arrs[3].sum(dtype=np.int64)), 0), 1 << 24) // 16, np.int32)
     build = lambda: lib.harts_attn_index(len(arrs[0]) - 1, *map(ip, arrs), ip(rot), len(blob), ip(blob), C.byref(n))  # noqa: E731
     code = build()
     if n.value > len(blob):

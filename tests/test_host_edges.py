@@ -1,12 +1,14 @@
 """Edges of the host side's tables: runs of positions in the row grouping, and a tree that is wider than the planner's
 walk over neighbours."""
 import random
+import tracemalloc
 
 import numpy as np
 import pytest
 
 import paper_2608_28158_b200 as H
 from oracle import mb_oracle as mo
+from test_attn_host import _check as _check_index
 from test_mb_plan import _lex_trajs, _plan
 from test_plan_oracle import random_tree
 from workloads import make_forest
@@ -41,3 +43,27 @@ def test_greedy_in_a_tree_wider_than_the_walk(leaves):
     for order, policy in ((1, 0), (3, 1)):
         got = list(zip(*(a.tolist() for a in plan.greedy_trace(order, policy))))
         assert got == mo.greedy_place(trajs, orders[order], 80, best_fit=policy == 0)
+
+
+@pytest.mark.parametrize("lens", [[-100000000], [-1, 5], [0], [2147483647] * 40], ids=["negative", "one_negative", "empty", "huge"])
+def test_attention_index_refuses_malformed_lengths(lens):
+    """A node length that no forest can have is refused as such, whatever it says about the size of the tables: the buffer
+    that is made before the lengths are checked stays small (40 nodes of 2^31 - 1 tokens would ask for 20 GB)."""
+    n = len(lens)
+    tracemalloc.start()
+    with pytest.raises(H.HartsError):
+        H.harts_attn_index([0, n], [-1] + [0] * (n - 1), [0] + [1] * (n - 1), lens)
+    peak = tracemalloc.get_traced_memory()[1]
+    tracemalloc.stop()
+    assert peak < 16 << 20
+
+
+def test_attention_index_beyond_the_first_guess():
+    """A comb of 300 nodes in a row, a leaf off each: the ancestor and descendant lists need more words than the first buffer
+    has, and the call is repeated with the size it asks for."""
+    n = 300
+    par = [-1] + [x for i in range(n - 1) for x in (2 * i, 2 * i)] + [2 * n - 2]
+    fo = make_forest([(par, [0] + [1] * (2 * n - 1), [1] * (2 * n))])
+    _check_index(fo, None)
+    ix = H.harts_attn_index(fo.tree_node_ptr, fo.node_parent, fo.node_fork_off, fo.node_len)
+    assert len(ix.host) > 4096 + 64 * 2 * n + 2 * n // 16
