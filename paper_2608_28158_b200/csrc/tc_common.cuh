@@ -67,12 +67,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, status, dead, limit_ns);
 }
 // The same for a whole (converged) warp: one answer for all lanes; past the first try one lane polls, so that 31 lanes do
-// not spend shared-memory cycles on it.
+// not spend shared-memory cycles on it.  Only that lane has acquired then, and a shuffle orders no memory: the warp barrier
+// behind it is what lets the other lanes read the data.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status, volatile int* dead) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow(bar, parity, status, dead, WAIT_LIMIT_NS);
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    return ok != 0;
 }
 // Last wait of a CTA that is giving up: waits (bounded, whatever the latch says) for a copy or MMA group still in
 // flight, so that nothing lands in shared or tensor memory after the CTA has gone.
@@ -111,16 +114,18 @@ constexpr unsigned long long FLAG_WAIT_LIMIT_NS = 4000ull * 1000 * 1000;
 __device__ __forceinline__ void flag_set(int* flag) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(flag), "r"(1) : "memory");
 }
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ bool flag_wait(const int* flag, int* status, volatile int* dead,
                                           unsigned long long limit_ns = FLAG_WAIT_LIMIT_NS) {
     const unsigned long long t0 = global_ns();
     for (int round = 0; round < (1 << 26); round++) {
-        int v;
 #pragma unroll 1
-        for (int i = 0; i < 16; i++) {
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-            if (v != 0) return true;
-        }
+        for (int i = 0; i < 16; i++)
+            if (ld_acquire(flag) != 0) return true;
         if (*dead) return false;
         // another CTA of the launch has already given up (its wait ran out): what this one waits for may never come
         if (status && *reinterpret_cast<volatile int*>(status) != 0) {
@@ -135,7 +140,7 @@ __device__ __forceinline__ bool flag_wait(const int* flag, int* status, volatile
 }
 
 // Counting form for producers that finish warp by warp: a (converged) warp adds one once its lanes' data is written; the
-// consumer warp waits until `target` warps have.
+// consumer warp waits until `target` warps have (its first lane acquires, the warp barrier hands that on to the others).
 __device__ __forceinline__ void flag_add_warp(int* flag) {
     __threadfence();
     __syncwarp();
@@ -146,9 +151,7 @@ static __device__ __noinline__ bool flag_wait_warp(const int* flag, int target, 
     if ((threadIdx.x & 31) == 0) {
         const unsigned long long t0 = global_ns();
         for (int round = 0;; round++) {
-            int v;
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-            if (v >= target) break;
+            if (ld_acquire(flag) >= target) break;
             if ((round & 15) != 15) continue;
             // another CTA of the launch has already given up: what this one waits for may never come
             const bool gave_up = *dead || (status && *reinterpret_cast<volatile int*>(status) != 0);
@@ -159,7 +162,9 @@ static __device__ __noinline__ bool flag_wait_warp(const int* flag, int target, 
             break;
         }
     }
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    return ok != 0;
 }
 
 // ---- fences ---------------------------------------------------------------------------------------
