@@ -13,6 +13,9 @@
 #include "chunk_item.cuh"
 
 namespace harts {
+
+int sm_count();
+
 namespace {
 
 using chunk::BT;
@@ -103,13 +106,15 @@ __device__ __forceinline__ void load_state(float* dst, const float* src) {
     for (int e = threadIdx.x; e < D * 16; e += NT)
         *reinterpret_cast<float4*>(dst + (e >> 4) * LD + (e & 15) * 4) = *reinterpret_cast<const float4*>(src + e * 4);
 }
-// The CTA's item: warp 0 finds it and prepares its row data.
-__device__ __forceinline__ bool begin_item(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int H, const float* g, RowData& rd, Item& it) {
-    const int gc = tb.seq_chunk_ptr[seq_lo] + (int)blockIdx.x / H;
+// The CTA's item `idx` of the range: warp 0 finds it and prepares its row data.  False: the range has no such item.
+__device__ __forceinline__ bool begin_item(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int H, const float* g, int idx, RowData& rd,
+                                           Item& it) {
+    const int gc = tb.seq_chunk_ptr[seq_lo] + idx / H;
     if (gc >= tb.seq_chunk_ptr[seq_hi]) return false;
+    __syncthreads();                             // the last readers of the item before are through
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        const Item x = find_item(tb, seq_lo, seq_hi, gc, (int)blockIdx.x % H, lane);
+        const Item x = find_item(tb, seq_lo, seq_hi, gc, idx % H, lane);
         int code[2];
         float gv[2];
         chunk::load_rows(tb, x, g, H, lane, code, gv);
@@ -131,9 +136,9 @@ __global__ void __launch_bounds__(NT) outer_kernel(const harts_la_tables_t tb, i
                                                    float* __restrict__ gammas, const int32_t* gate) {
     if (gate_closed(gate)) return;
     __shared__ OuterSmem s;
-    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
     const Item& it = s.it;
-    if (BWD ? it.zero_state : it.last) return;   // this chunk's sum enters nothing
+    if (BWD ? it.zero_state : it.last) continue; // this chunk's sum enters nothing
     load_tile(s.x, a, s.rd, BWD, it.h, H);
     for (int e = threadIdx.x; e < BT * 16; e += NT) {         // the weighted operand
         const int t = e >> 4, ch = e & 15, code = s.rd.code[t], r = code >= 0 ? code : -2 - code;
@@ -153,6 +158,7 @@ __global__ void __launch_bounds__(NT) outer_kernel(const harts_la_tables_t tb, i
 #pragma unroll
         for (int c = 0; c < 4; c++) dst[(4 * ty + r) * D + tx + 16 * c] = acc[r][c];
     if (threadIdx.x == 0) gammas[(size_t)it.gc * H + it.h] = s.rd.gamma;
+    }
 }
 
 // One thread walks four elements of the state along a sequence; four CTAs per (sequence, head).
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int
     if (gate_closed(gate)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OutSmem& s = *reinterpret_cast<OutSmem*>(smem_raw);
-    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
     const Item& it = s.it;
     load_tile(s.q, q, s.rd, true, it.h, H);
     load_tile(s.k, k, s.rd, false, it.h, H);
@@ -261,6 +267,7 @@ __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int
 #pragma unroll
             for (int c = 0; c < 4; c++) o[((size_t)code * H + it.h) * D + tx + 16 * c] = acc[r][c];
     }
+    }
 }
 
 struct __align__(16) GradSmem {
@@ -269,7 +276,7 @@ struct __align__(16) GradSmem {
     Item it;
     float z[BT], part[NT / 32];
 };
-__global__ void __launch_bounds__(NT) grad_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
+__global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
                                                   const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
                                                   const float* __restrict__ dO, const float* __restrict__ states,
                                                   const float* __restrict__ ds_tiles, float* __restrict__ dq, float* __restrict__ dk_,
@@ -278,7 +285,7 @@ __global__ void __launch_bounds__(NT) grad_kernel(const harts_la_tables_t tb, in
     if (gate_closed(gate)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
-    if (!begin_item(tb, seq_lo, seq_hi, H, g, s.rd, s.it)) return;
+    for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
     const Item& it = s.it;
     const int h = it.h;
     const bool has_s = !it.zero_state, has_ds = !it.last;
@@ -402,7 +409,16 @@ __global__ void __launch_bounds__(NT) grad_kernel(const harts_la_tables_t tb, in
             else if (code < -1) rg[(size_t)(it.replay_base + t) * H + h] = out[r];
         }
     }
+    }
 }
+
+// A grid no larger than what is resident at once: the number of items of a range is in the tables on the device, and one launch
+// per round would otherwise bring the whole forest's CTAs each time.
+inline int grid_of(const harts_la_tables_t& tb, int32_t H, int per_sm) {
+    const int64_t items = (int64_t)tb.n_chunks * H, most = (int64_t)per_sm * sm_count();
+    return (int)(items < most ? items : most);
+}
+constexpr int OUTER_PER_SM = 6, OUT_PER_SM = 2, GRAD_PER_SM = 1;       // 36, 88 and 140 KB of shared memory each
 
 inline int32_t done() { return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA; }
 
@@ -410,33 +426,33 @@ inline int32_t done() { return cudaGetLastError() == cudaSuccess ? HARTS_OK : HA
 
 // Sequences [range[0], range[n]), range[r]..range[r+1] per round.  extra: f32_extra_bytes() behind the chunk states and flags.
 int32_t f32_fwd(const FwdArgs& a, float* extra, const int32_t* range, int32_t n) {
-    const int lo = range[0], hi = range[n], grid = a.tb.n_chunks * a.H;
+    const int lo = range[0], hi = range[n];
     if (lo == hi) return HARTS_OK;
     const int32_t* gate = status_gate(a.flags, a.dev_status);
     float *states = (float*)a.chunk_states, *gammas = extra;
-    outer_kernel<false><<<grid, NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.k, (const float*)a.v, a.g, states, gammas, gate);
+    outer_kernel<false><<<grid_of(a.tb, a.H, OUTER_PER_SM), NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.k, (const float*)a.v, a.g, states, gammas, gate);
     for (int32_t r = 0; r < n; r++)
         if (range[r] < range[r + 1])
             walk_kernel<false><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, states, gammas, a.slots, nullptr, gate);
     if (cudaFuncSetAttribute(out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(OutSmem)) != cudaSuccess) return HARTS_ECUDA;
-    out_kernel<<<grid, NT, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g,
+    out_kernel<<<grid_of(a.tb, a.H, OUT_PER_SM), NT, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g,
                                                         states, (float*)a.o, gate);
     return done();
 }
 
 int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n) {
-    const int lo = range[0], hi = range[n], grid = a.tb.n_chunks * a.H;
+    const int lo = range[0], hi = range[n];
     if (lo == hi) return HARTS_OK;
     const int32_t* gate = status_gate(a.flags, a.dev_status);
     const ScratchLayout sl = scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
     float *gammas = extra, *tiles = extra + align_up((size_t)a.tb.n_chunks * a.H, 64), *ds0 = (float*)(base + sl.ds0);
-    outer_kernel<true><<<grid, NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.dO, a.g, tiles, gammas, gate);
+    outer_kernel<true><<<grid_of(a.tb, a.H, OUTER_PER_SM), NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.dO, a.g, tiles, gammas, gate);
     for (int32_t r = n - 1; r >= 0; r--)
         if (range[r] < range[r + 1])
             walk_kernel<true><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, tiles, gammas, nullptr, ds0, gate);
     if (cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem)) != cudaSuccess) return HARTS_ECUDA;
-    grad_kernel<<<grid, NT, sizeof(GradSmem), a.stream>>>(
+    grad_kernel<<<grid_of(a.tb, a.H, GRAD_PER_SM), NT, sizeof(GradSmem), a.stream>>>(
         a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g, (const float*)a.dO, (const float*)a.chunk_states,
         tiles, (float*)a.dq, (float*)a.dk_, (float*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv), (float*)(base + sl.rg), gate);
     return done();

@@ -3,7 +3,7 @@ import pytest
 import torch
 
 import paper_2608_28158_b200 as H
-from parity_util import compare, oracle_subset, run_gpu
+from parity_util import compare, oracle_subset, plan_of, run_gpu
 from test_gpu_parity import check
 from workloads import make_forest, make_inputs
 
@@ -60,3 +60,37 @@ def test_both_sides_of_the_chain_line(heads):
     _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
     for n in out:
         assert torch.equal(out[n], rounds[n]), n
+
+
+def test_fp32_more_items_than_resident_blocks():
+    """460 chunks x 2 heads: every kernel's CTAs take several items in turn, in one call and round by round."""
+    fo = make_forest([([-1, 0, 0, 1], [0, 14000, 6001, 4000], [14000, 8000, 3000, 4333])])
+    inp = make_inputs(fo.n_tokens, 2, 64, 64, "fp32", 14)
+    plan, out = run_gpu(fo, inp)
+    assert plan.n_chunks * 2 > 6 * torch.cuda.get_device_properties(0).multi_processor_count
+    tok, ref = oracle_subset(fo, inp, [0], [0, 1])
+    check(compare(out, tok, [0, 1], ref, rows=True), "fp32")
+    _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
+    for n in out:
+        assert torch.equal(out[n], rounds[n]), n
+
+
+def test_fp32_call_for_one_sequence_does_not_pay_for_the_forest():
+    """A packed call names a range of sequences: one sequence of one chunk takes about as long beside 6,000 chunks x 8 heads as
+    beside two (a grid of the whole forest's items made it 3 times as long)."""
+    def median_us(root):
+        fo = make_forest([([-1, 0], [0, root], [root + 64, 64])])
+        plan = plan_of(fo).upload()
+        x, g = torch.zeros(fo.n_tokens, 8, 64, device="cuda"), torch.zeros(fo.n_tokens, 8, device="cuda")
+        o, ws, n = torch.empty_like(x), H.Workspace(plan, 8, 64, 64, torch.float32), plan.n_seq
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(52)]
+        for e in ev:
+            H.harts_la_fwd_seqs(plan.tables, n - 1, n, x, x, x, g, o, ws.slots, ws.chunk_states, 0, ws.dev_status)
+            e.record()
+        torch.cuda.synchronize()
+        H.harts_la_check(ws.dev_status)
+        return sorted(a.elapsed_time(b) * 1e3 for a, b in zip(ev[1:-1], ev[2:]))[25]
+
+    few, many = median_us(128), median_us(64 * 6000)
+    print(f"one sequence: {few:.1f} us beside 2 chunks, {many:.1f} us beside 6,000")
+    assert many < 1.75 * few
