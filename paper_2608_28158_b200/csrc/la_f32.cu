@@ -93,6 +93,40 @@ __device__ __forceinline__ void mul_tn(Acc& a, const float* x, const float* y, i
     }
 }
 
+// The eight columns (rows) at the diagonal of a warp's rows: what lies past the diagonal is left out, not multiplied by zero, so
+// that an infinity or a NaN in a later row stays out of the rows before it.
+// a += P[:, k0..k0+8) Y[k0..k0+8, :), columns up to the row
+__device__ __forceinline__ void mul_nn_diagonal(Acc& a, const float* x, const float* y, int k0, int ty, int tx) {
+#pragma unroll
+    for (int k = k0; k < k0 + 8; k += 4) {
+        float xv[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) *reinterpret_cast<float4*>(xv[r]) = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + k);
+#pragma unroll
+        for (int kk = 0; kk < 4; kk++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const float yv = y[(k + kk) * LD + tx + 16 * c];
+#pragma unroll
+                for (int r = 0; r < 4; r++) a[r][c] = k + kk <= 4 * ty + r ? a[r][c] + xv[r][kk] * yv : a[r][c];
+            }
+    }
+}
+// a += P[t0..t0+8, :)^T Y[t0..t0+8, :), rows from the column on
+__device__ __forceinline__ void mul_tn_diagonal(Acc& a, const float* x, const float* y, int t0, int ty, int tx) {
+#pragma unroll
+    for (int t = t0; t < t0 + 8; t++) {
+        float xv[4];
+        *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(x + t * LD + 4 * ty);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const float yv = y[t * LD + tx + 16 * c];
+#pragma unroll
+            for (int r = 0; r < 4; r++) a[r][c] = t >= 4 * ty + r ? a[r][c] + xv[r] * yv : a[r][c];
+        }
+    }
+}
+
 // Rows of a chunk into a tile; `own`: replayed rows (and rows past the end) are zero, else only rows past the end.
 __device__ __forceinline__ void load_tile(float* dst, const float* src, const RowData& rd, bool own, int h, int H) {
     for (int e = threadIdx.x; e < BT * 16; e += NT) {
@@ -259,7 +293,8 @@ __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int
 #pragma unroll
             for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
     }
-    mul_nn(acc, s.p, s.v, 0, 8 * warp + 8, ty, tx);
+    mul_nn(acc, s.p, s.v, 0, 8 * warp, ty, tx);
+    mul_nn_diagonal(acc, s.p, s.v, 8 * warp, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int code = s.rd.code[4 * ty + r];
@@ -323,7 +358,8 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     for (int r = 0; r < 4; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
-    mul_nn(acc, s.dp, s.k, 0, 8 * warp + 8, ty, tx);
+    mul_nn(acc, s.dp, s.k, 0, 8 * warp, ty, tx);
+    mul_nn_diagonal(acc, s.dp, s.k, 8 * warp, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];
@@ -344,7 +380,8 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
             acc[r][c] *= s.rd.w[t];
             g_part += s.k[t * LD + tx + 16 * c] * acc[r][c];
         }
-    mul_tn(acc, s.dp, s.q, 8 * warp, ty, tx);
+    mul_tn_diagonal(acc, s.dp, s.q, 8 * warp, ty, tx);
+    mul_tn(acc, s.dp, s.q, 8 * warp + 8, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];
@@ -362,7 +399,8 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     for (int r = 0; r < 4; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.w[4 * ty + r];
-    mul_tn(acc, s.p, s.dO, 8 * warp, ty, tx);
+    mul_tn_diagonal(acc, s.p, s.dO, 8 * warp, ty, tx);
+    mul_tn(acc, s.p, s.dO, 8 * warp + 8, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];

@@ -94,3 +94,21 @@ def test_fp32_call_for_one_sequence_does_not_pay_for_the_forest():
     few, many = median_us(128), median_us(64 * 6000)
     print(f"one sequence: {few:.1f} us beside 2 chunks, {many:.1f} us beside 6,000")
     assert many < 1.75 * few
+
+
+@pytest.mark.parametrize("name", ["q", "k", "v", "dO"])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_fp32_non_finite_rows_keep_to_the_causal_side(name, bad):
+    """An infinity or NaN in one row must not reach what does not depend on it: outputs and dq of the rows before it (k, v), dk and
+    dv of the rows after it (q, dO), bit for bit -- wherever the row stands in its chunk."""
+    fo = make_forest([([-1], [0], [200])])
+    inp = make_inputs(fo.n_tokens, 2, 64, 64, "fp32", 16)
+    _, clean = run_gpu(fo, inp)
+    for t in (1, 6, 37, 63, 64, 127, 130, 198):
+        x = {n: y.clone() for n, y in inp.items()}
+        x[name][t, 0] = bad
+        _, out = run_gpu(fo, x)
+        for n in ("o", "dq") if name in "kv" else ("dk", "dv"):
+            rows = slice(0, t) if name in "kv" else slice(t + 1, None)
+            assert torch.equal(out[n][rows], clean[n][rows]), (n, t)
+            assert torch.equal(out[n][:, 1], clean[n][:, 1]), (n, t)
