@@ -127,8 +127,38 @@ __device__ __forceinline__ void mul_tn_diagonal(Acc& a, const float* x, const fl
     }
 }
 
+// Row data with the running log-decay to twice 32 bits (b2 + b2_lo): the decay between two rows is the exponential of a
+// difference of two running sums, and after a steep gate both are large.  Summed in 64 bits by the same warp scan.
+struct Rows : RowData {
+    float b2_lo[BT];
+    __device__ float decay(int t, int j) const { return ex2((b2[t] - b2[j]) + (b2_lo[t] - b2_lo[j])); }
+};
+__device__ __forceinline__ void store_gates(Rows& rd, const float (&gv)[2], int lane) {
+    double x0 = gv[0] * 1.4426950408889634074, x1 = gv[1] * 1.4426950408889634074;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double y0 = __shfl_up_sync(~0u, x0, o), y1 = __shfl_up_sync(~0u, x1, o);
+        if (lane >= o) {
+            x0 += y0;
+            x1 += y1;
+        }
+    }
+    x1 += __shfl_sync(~0u, x0, 31);
+    const double bn = __shfl_sync(~0u, x1, 31), x[2] = {x0, x1};
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+        const int t = lane + 32 * r;
+        const float hi = (float)x[r];
+        rd.b2[t] = hi;
+        rd.b2_lo[t] = isinf(hi) ? 0.f : (float)(x[r] - hi);
+        rd.eb[t] = ex2(hi);
+        rd.w[t] = ex2((float)(bn - x[r]));
+    }
+    if (lane == 0) rd.gamma = ex2((float)bn);
+}
+
 // Rows of a chunk into a tile; `own`: replayed rows (and rows past the end) are zero, else only rows past the end.
-__device__ __forceinline__ void load_tile(float* dst, const float* src, const RowData& rd, bool own, int h, int H) {
+__device__ __forceinline__ void load_tile(float* dst, const float* src, const Rows& rd, bool own, int h, int H) {
     for (int e = threadIdx.x; e < BT * 16; e += NT) {
         const int t = e >> 4, ch = e & 15, code = rd.code[t], r = code >= 0 ? code : -2 - code;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -140,32 +170,35 @@ __device__ __forceinline__ void load_state(float* dst, const float* src) {
     for (int e = threadIdx.x; e < D * 16; e += NT)
         *reinterpret_cast<float4*>(dst + (e >> 4) * LD + (e & 15) * 4) = *reinterpret_cast<const float4*>(src + e * 4);
 }
-// The CTA's item `idx` of the range: warp 0 finds it and prepares its row data.  False: the range has no such item.
-__device__ __forceinline__ bool begin_item(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int H, const float* g, int idx, RowData& rd,
+// The CTA's item `idx` of the range: warp 0 finds it and prepares its row data.  False: the range has no such item.  On return
+// the record and the row codes are there for all; the gates' sums and weights are after the CTA's next barrier, so that warp 0
+// works them out while the others load the tiles.
+__device__ __forceinline__ bool begin_item(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int H, const float* g, int idx, Rows& rd,
                                            Item& it) {
-    const int gc = tb.seq_chunk_ptr[seq_lo] + idx / H;
+    const int gc = tb.seq_chunk_ptr[seq_lo] + idx / H, lane = threadIdx.x;
     if (gc >= tb.seq_chunk_ptr[seq_hi]) return false;
     __syncthreads();                             // the last readers of the item before are through
+    float gv[2];
     if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
         const Item x = find_item(tb, seq_lo, seq_hi, gc, idx % H, lane);
         int code[2];
-        float gv[2];
         chunk::load_rows(tb, x, g, H, lane, code, gv);
-        chunk::store_rows(rd, code, gv, lane);
+        rd.code[lane] = code[0];
+        rd.code[lane + 32] = code[1];
         if (lane == 0) it = x;
     }
     __syncthreads();
+    if (threadIdx.x < 32) store_gates(rd, gv, lane);
     return true;
 }
 
 struct __align__(16) OuterSmem {
     float x[TILE], y[TILE];
-    RowData rd;
+    Rows rd;
     Item it;
 };
 template <bool BWD>
-__global__ void __launch_bounds__(NT) outer_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ a,
+__global__ void __launch_bounds__(NT, 5) outer_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ a,
                                                    const float* __restrict__ b, const float* __restrict__ g, float* __restrict__ sums,
                                                    float* __restrict__ gammas, const int32_t* gate) {
     if (gate_closed(gate)) return;
@@ -174,12 +207,19 @@ __global__ void __launch_bounds__(NT) outer_kernel(const harts_la_tables_t tb, i
     const Item& it = s.it;
     if (BWD ? it.zero_state : it.last) continue; // this chunk's sum enters nothing
     load_tile(s.x, a, s.rd, BWD, it.h, H);
-    for (int e = threadIdx.x; e < BT * 16; e += NT) {         // the weighted operand
-        const int t = e >> 4, ch = e & 15, code = s.rd.code[t], r = code >= 0 ? code : -2 - code;
+    float4 y[BT * 16 / NT];                      // the operand that is weighted
+#pragma unroll
+    for (int u = 0; u < BT * 16 / NT; u++) {
+        const int e = threadIdx.x + u * NT, code = s.rd.code[e >> 4], r = code >= 0 ? code : -2 - code;
+        y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (BWD ? code >= 0 : code != -1) y[u] = *reinterpret_cast<const float4*>(b + ((size_t)r * H + it.h) * D + (e & 15) * 4);
+    }
+    __syncthreads();                             // the weights
+#pragma unroll
+    for (int u = 0; u < BT * 16 / NT; u++) {
+        const int e = threadIdx.x + u * NT, t = e >> 4;
         const float w = BWD ? s.rd.eb[t] : s.rd.w[t];
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (BWD ? code >= 0 : code != -1) x = *reinterpret_cast<const float4*>(b + ((size_t)r * H + it.h) * D + ch * 4);
-        *reinterpret_cast<float4*>(s.y + t * LD + ch * 4) = make_float4(x.x * w, x.y * w, x.z * w, x.w * w);
+        *reinterpret_cast<float4*>(s.y + t * LD + (e & 15) * 4) = make_float4(y[u].x * w, y[u].y * w, y[u].z * w, y[u].w * w);
     }
     __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
@@ -257,7 +297,7 @@ __global__ void __launch_bounds__(NT) walk_kernel(const harts_la_tables_t tb, in
 
 struct __align__(16) OutSmem {
     float q[TILE], k[TILE], v[TILE], s[TILE], p[TILE];
-    RowData rd;
+    Rows rd;
     Item it;
 };
 __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
@@ -282,32 +322,29 @@ __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const int t = 4 * ty + r, j = tx + 16 * c;
-            s.p[t * LD + j] = j <= t ? acc[r][c] * ex2(s.rd.b2[t] - s.rd.b2[j]) : 0.f;
+            s.p[t * LD + j] = j <= t ? acc[r][c] * s.rd.decay(t, j) : 0.f;
         }
     __syncwarp();                                // a warp reads the rows it wrote
     clear(acc);
-    if (!it.zero_state) {
-        mul_nn(acc, s.q, s.s, 0, D, ty, tx);
-#pragma unroll
-        for (int r = 0; r < 4; r++)
-#pragma unroll
-            for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
-    }
-    mul_nn(acc, s.p, s.v, 0, 8 * warp, ty, tx);
-    mul_nn_diagonal(acc, s.p, s.v, 8 * warp, ty, tx);
+    if (!it.zero_state) mul_nn(acc, s.q, s.s, 0, D, ty, tx);
+    Acc in;                                      // the chunk's own share, summed by itself: it is small beside the state's
+    clear(in);
+    mul_nn(in, s.p, s.v, 0, 8 * warp, ty, tx);
+    mul_nn_diagonal(in, s.p, s.v, 8 * warp, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int code = s.rd.code[4 * ty + r];
         if (code >= 0)
 #pragma unroll
-            for (int c = 0; c < 4; c++) o[((size_t)code * H + it.h) * D + tx + 16 * c] = acc[r][c];
+            for (int c = 0; c < 4; c++)
+                o[((size_t)code * H + it.h) * D + tx + 16 * c] = it.zero_state ? in[r][c] : __fmaf_rn(s.rd.eb[4 * ty + r], acc[r][c], in[r][c]);
     }
     }
 }
 
 struct __align__(16) GradSmem {
     float q[TILE], k[TILE], v[TILE], dO[TILE], s[TILE], ds[TILE], p[TILE], dp[TILE];
-    RowData rd;
+    Rows rd;
     Item it;
     float z[BT], part[NT / 32];
 };
@@ -343,7 +380,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const int t = 4 * ty + r, j = tx + 16 * c;
-            const float w = j <= t ? ex2(s.rd.b2[t] - s.rd.b2[j]) : 0.f;
+            const float w = j <= t ? s.rd.decay(t, j) : 0.f;
             s.p[t * LD + j] = j <= t ? acc[r][c] * w : 0.f;
             s.dp[t * LD + j] = j <= t ? dacc[r][c] * w : 0.f;
         }
@@ -353,61 +390,52 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     float z[4] = {0.f, 0.f, 0.f, 0.f};           // its share of q.dq - k.dk, per row
     // ---- dq = e^{b_t} dO S^T + dP K
     clear(acc);
+    clear(dacc);
     if (has_s) mul_nt<4>(acc, s.dO, s.s, ty, tx);
-#pragma unroll
-    for (int r = 0; r < 4; r++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.eb[4 * ty + r];
-    mul_nn(acc, s.dp, s.k, 0, 8 * warp, ty, tx);
-    mul_nn_diagonal(acc, s.dp, s.k, 8 * warp, ty, tx);
+    mul_nn(dacc, s.dp, s.k, 0, 8 * warp, ty, tx);         // the chunk's own share by itself, as in out_kernel
+    mul_nn_diagonal(dacc, s.dp, s.k, 8 * warp, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            z[r] += s.q[t * LD + tx + 16 * c] * acc[r][c];
-            if (code >= 0) dq[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
+            const float x = has_s ? __fmaf_rn(s.rd.eb[t], acc[r][c], dacc[r][c]) : dacc[r][c];
+            z[r] += s.q[t * LD + tx + 16 * c] * x;
+            if (code >= 0) dq[((size_t)code * H + h) * D + tx + 16 * c] = x;
         }
     }
     // ---- dk = w_j V dS^T + dP^T Q
     clear(acc);
+    clear(dacc);
     if (has_ds) mul_nt<4>(acc, s.v, s.ds, ty, tx);
-#pragma unroll
-    for (int r = 0; r < 4; r++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const int t = 4 * ty + r;
-            acc[r][c] *= s.rd.w[t];
-            g_part += s.k[t * LD + tx + 16 * c] * acc[r][c];
-        }
-    mul_tn_diagonal(acc, s.dp, s.q, 8 * warp, ty, tx);
-    mul_tn(acc, s.dp, s.q, 8 * warp + 8, ty, tx);
+    mul_tn_diagonal(dacc, s.dp, s.q, 8 * warp, ty, tx);
+    mul_tn(dacc, s.dp, s.q, 8 * warp + 8, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            z[r] -= s.k[t * LD + tx + 16 * c] * acc[r][c];
-            if (code >= 0) dk_[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
-            else if (code < -1) rk[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = acc[r][c];
+            const float kv = s.k[t * LD + tx + 16 * c], inter = has_ds ? acc[r][c] * s.rd.w[t] : 0.f, x = dacc[r][c] + inter;
+            g_part += kv * inter;
+            z[r] -= kv * x;
+            if (code >= 0) dk_[((size_t)code * H + h) * D + tx + 16 * c] = x;
+            else if (code < -1) rk[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = x;
         }
     }
     // ---- dv = w_j K dS + P^T dO
     clear(acc);
+    clear(dacc);
     if (has_ds) mul_nn(acc, s.k, s.ds, 0, D, ty, tx);
-#pragma unroll
-    for (int r = 0; r < 4; r++)
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[r][c] *= s.rd.w[4 * ty + r];
-    mul_tn_diagonal(acc, s.p, s.dO, 8 * warp, ty, tx);
-    mul_tn(acc, s.p, s.dO, 8 * warp + 8, ty, tx);
+    mul_tn_diagonal(dacc, s.p, s.dO, 8 * warp, ty, tx);
+    mul_tn(dacc, s.p, s.dO, 8 * warp + 8, ty, tx);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t = 4 * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            if (code >= 0) dv_[((size_t)code * H + h) * D + tx + 16 * c] = acc[r][c];
-            else if (code < -1) rv[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = acc[r][c];
+            const float x = has_ds ? __fmaf_rn(s.rd.w[t], acc[r][c], dacc[r][c]) : dacc[r][c];
+            if (code >= 0) dv_[((size_t)code * H + h) * D + tx + 16 * c] = x;
+            else if (code < -1) rv[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = x;
         }
     }
     // ---- dg_t = sum_{tau>=t} z_tau + e^{b_n} <S_c, dS> + sum_j k_j . (w_j dS v_j), every sum in a fixed order
@@ -456,7 +484,7 @@ inline int grid_of(const harts_la_tables_t& tb, int32_t H, int per_sm) {
     const int64_t items = (int64_t)tb.n_chunks * H, most = (int64_t)per_sm * sm_count();
     return (int)(items < most ? items : most);
 }
-constexpr int OUTER_PER_SM = 6, OUT_PER_SM = 2, GRAD_PER_SM = 1;       // 36, 88 and 140 KB of shared memory each
+constexpr int OUTER_PER_SM = 5, OUT_PER_SM = 2, GRAD_PER_SM = 1;       // 47 registers a thread; 88 and 140 KB of shared memory
 
 inline int32_t done() { return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA; }
 

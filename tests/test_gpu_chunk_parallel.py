@@ -112,3 +112,18 @@ def test_fp32_non_finite_rows_keep_to_the_causal_side(name, bad):
             rows = slice(0, t) if name in "kv" else slice(t + 1, None)
             assert torch.equal(out[n][rows], clean[n][rows]), (n, t)
             assert torch.equal(out[n][:, 1], clean[n][:, 1]), (n, t)
+
+
+@pytest.mark.parametrize("reset", [-100.0, -3000.0])
+def test_fp32_keeps_its_precision_behind_steep_gates(reset):
+    """One token in a hundred forgets everything before it.  The running log-decay of a chunk is large from there on, and the
+    decay between two later rows is the exponential of a difference of two such sums: in 32 bits it was off by 2^-24 of the
+    sums (8e-5 at -3000).  64-term fp32 sums are off by at most 64 * 2^-24."""
+    fo = make_forest([([-1, 0, 0], [0, 700, 333], [700, 300, 250])])
+    inp = make_inputs(fo.n_tokens, 2, 64, 64, "fp32", 17)
+    gen = torch.Generator().manual_seed(17)
+    inp["g"] = torch.where(torch.rand(inp["g"].shape, generator=gen) < 0.01, torch.tensor(reset), inp["g"])
+    _, out = run_gpu(fo, inp)
+    tok, ref = oracle_subset(fo, inp, [0], [0, 1])
+    errs = compare(out, tok, [0, 1], ref)
+    assert all(e <= 64 * 2.0 ** -24 for e in errs.values()), errs
