@@ -161,7 +161,9 @@ int32_t harts_la_plan_tables(const harts_la_plan_t* plan, const void* dev_blob, 
  *   chunk_state_bytes: [n_chunks, H, dk, dv] start-of-chunk states in the run dtype, written by the
  *                      forward, read by the backward, followed by (n_slots + n_seq) * H int32 flags that the
  *                      one-launch forms of round 0 use (the library clears them itself) and, in fp32 and
- *                      for small problems in bf16 with dk = dv = 128, by the gradients of the boundary states.
+ *                      for small problems in bf16 with dk = dv = 128, by what the backward keeps there: the
+ *                      gradients of the boundary states and parts of their products with the states.  Calls that
+ *                      share this buffer must not run at the same time.
  *   scratch_bytes:     backward scratch: per-sequence initial-state gradients [n_seq, H, dk, dv] fp32
  *                      and replay-row gradients [n_replay, H, dk + dv + 1] fp32.
  */

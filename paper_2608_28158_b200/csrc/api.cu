@@ -49,8 +49,9 @@ int32_t chunk_parallel_bwd(harts::BwdArgs a, const int32_t* range, int32_t n) {
     char* ws = const_cast<char*>(static_cast<const char*>(a.chunk_states));
     void* ds = ws + harts::ds_tiles_offset(a.tb, a.H, a.dk, a.dv);
     int* flags = reinterpret_cast<int*>(ws + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
-    const int32_t rc = harts::scan_bwd(a, ds, flags, round_order(range, n));
-    return rc != HARTS_OK ? rc : harts::chunk_bwd(a, ds);
+    float* dots = reinterpret_cast<float*>(ws + harts::dots_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::scan_bwd(a, ds, dots, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::chunk_bwd(a, ds, dots);
 }
 
 int32_t gk_chunk_parallel_fwd(harts::FwdArgs a, const int32_t* range, int32_t n) {
@@ -66,8 +67,9 @@ int32_t gk_chunk_parallel_bwd(harts::BwdArgs a, const int32_t* range, int32_t n)
     char* ws = const_cast<char*>(static_cast<const char*>(a.chunk_states));
     void* ds = ws + harts::ds_tiles_offset(a.tb, a.H, a.dk, a.dv);
     int* flags = reinterpret_cast<int*>(ws + harts::scan_flags_offset(a.tb, a.H, a.dk, a.dv));
-    const int32_t rc = harts::gk_scan_bwd(a, ds, flags, round_order(range, n));
-    return rc != HARTS_OK ? rc : harts::gk_chunk_bwd(a, ds);
+    float* dots = reinterpret_cast<float*>(ws + harts::dots_offset(a.tb, a.H, a.dk, a.dv));
+    const int32_t rc = harts::gk_scan_bwd(a, ds, dots, flags, round_order(range, n));
+    return rc != HARTS_OK ? rc : harts::gk_chunk_bwd(a, ds, dots);
 }
 
 }  // namespace

@@ -138,9 +138,9 @@ struct RoundOrder {
 // Chunk-parallel path (bf16, d_k = d_v = 128): a scan leaves the state of every chunk boundary (backward: its gradient) in
 // memory, then every (chunk, head) is a work item of its own.
 int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      // la_scan.cu: states, exported slots
-int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
+int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
-int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles);     // la_chunk_bwd.cu
+int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);     // la_chunk_bwd.cu
 // Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs.  The walk kernels (la_tc_*.cu) move 240 KB per item in
 // a whole step, this path 400 KB: with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.7 against 11.2
 // ms a step; 2,389 x 16: 3.0 against 3.1; 685 chunks in 21 sequences x 32 heads: 1.70 against 1.85), with few the chain of its
@@ -156,13 +156,16 @@ inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, i
            (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX && chains <= CHUNK_PARALLEL_CHAINS &&
            (tb.n_chunks >= 4 * (int64_t)tb.n_seq || chains <= 128);
 }
-// the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then the scan's
-// ticket and counters
+// the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then
+// <S_c, dS_c> in parts, fp32 [n_chunks, H, 4 blocks of 32 columns, dk], then the scan's ticket and counters
 inline size_t ds_tiles_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
     return align_up(chunk_state_payload(tb, H, dk, dv, 2) + fused_flag_bytes(tb, H), 1024);
 }
-inline size_t scan_flags_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+inline size_t dots_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
     return ds_tiles_offset(tb, H, dk, dv) + align_up(chunk_state_payload(tb, H, dk, dv, 2), 1024);
+}
+inline size_t scan_flags_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
+    return dots_offset(tb, H, dk, dv) + (size_t)tb.n_chunks * H * (dv / 32) * dk * sizeof(float);
 }
 inline size_t chunk_parallel_bytes(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
     return scan_flags_offset(tb, H, dk, dv) + (4 + (size_t)(tb.n_seq > tb.n_slots ? tb.n_seq : tb.n_slots) * H * 4) * sizeof(int);
@@ -170,9 +173,9 @@ inline size_t chunk_parallel_bytes(const harts_la_tables_t& tb, int32_t H, int32
 // The same for the per-channel decay, under the same rule (walk -> chunk-parallel, forward + backward: 1,047 chunks x 16 heads
 // 7.7 -> 3.8 ms; 33 k items of agentic trees 7.4 -> 6.8, of branchy ones 7.0 -> 7.2; 64 k items 12.3 -> 12.9).
 int32_t gk_scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);
-int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order);
+int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);
 int32_t gk_chunk_fwd(const FwdArgs& a);
-int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles);
+int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);
 // The same for fp32 inputs, d_k = d_v = 64 (la_f32.cu): every problem that brings a chunk-state workspace.  extra: e^{b_n}
 // [n_chunks, H] and the gradients of the boundary states [n_chunks, H, dk, dv], fp32, behind the flags.
 inline bool f32_chunks(int32_t dk, int32_t dv, int32_t dtype) { return dtype == HARTS_FP32 && dk == 64 && dv == 64; }

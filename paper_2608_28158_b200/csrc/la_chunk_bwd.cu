@@ -4,7 +4,7 @@
 //     dq = dP K   + e^{b_t} (dO S^T)
 //     dk = dP^T Q + w_j (V dS^T)                      w_j = e^{b_n-b_j}
 //     dv = P^T dO + w_j (K dS)
-//     dg_t = sum_{tau>=t} (q.dq - k.dk) + e^{b_n} <S, dS> + sum_j k_j . (w_j dS v_j)
+//     dg_t = sum_{tau>=t} (q.dq - k.dk) + e^{b_n} <S, dS> + sum_j k_j . (w_j dS v_j)        <S, dS>: from the scan, where dS is fp32
 // tcgen05 MMAs, every product transposed (tensor-memory lane = feature, column = row of the chunk); the 24 MMAs of the
 // three state products do not need P or dP and run under the decay masking, so twelve are left after it.  One CTA per SM:
 // eight 64-column accumulators take all 512 tensor-memory columns, tiles and staging 198 KB of shared memory.  Sixteen
@@ -65,7 +65,8 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                  const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                  const float* __restrict__ g, const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq,
                  __nv_bfloat16* __restrict__ dk_, __nv_bfloat16* __restrict__ dv_, float* __restrict__ dg,
-                 float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg, int* status, const int32_t* gate) {
+                 float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg, const float* __restrict__ dots,
+                 int* status, const int32_t* gate) {
     if (gate_closed(gate)) return;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -203,6 +204,7 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
         if (is_aux && i + 1 < n_mine) store_rows(m.rows[(i + 1) % 3], nx_code, nx_g, lane);
         float g_part = 0.f;                // this thread's share of <S_{c+1}, dS_{c+1}>
         if (is_compute) {
+            if (has_s && has_ds) g_part = dots[((size_t)it.gc * H + h) * NC + tid];      // <S, dS>, one of its 512 parts per thread
             // ---- P (lanes 0..63), dP (lanes 64..127): 16 columns of one of them per thread --------------------------------
             mbar_wait(&m.bar_a, ph, status, &m.dead);
             tc_fence_after();
@@ -250,7 +252,7 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DQ, dKm + kstep_mnmajor(ks), dDPk + kstep_kmajor<BT>(ks), I_MK64, ks > 0);
             mma_commit(&m.bar_o3);
             mbar_wait(&m.bar_o3, ph, status, &m.dead);
-            mbar_wait(&m.bar_qk_read, ph, status, &m.dead);      // the compute warps have taken their q, k and state values
+            mbar_wait(&m.bar_qk_read, ph, status, &m.dead);      // the compute warps have taken their q and k values
             if (i + 1 < n_mine) {
                 issue_tiles(m.items[(i + 1) % 3]);
                 tiles_pending = true;
@@ -263,7 +265,6 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
         }
         if (is_compute) {
             mbar_wait(&m.bar_tiles, ph, status, &m.dead);        // long complete: orders this thread's reads of the tiles
-            mbar_wait(&m.bar_states, ph, status, &m.dead);
             const int c4 = lane & 3, mrow = lane >> 2, Lq = (warp & 3) * 32, t0 = grp * 16;
             uint32_t fq[2][4], fk[2][4];
 #pragma unroll
@@ -271,22 +272,7 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                 ldmatrix_x4_trans(frag_addr(aQ, lane, Lq, t0, ta), fq[ta]);
                 ldmatrix_x4_trans(frag_addr(aK, lane, Lq, t0, ta), fk[ta]);
             }
-            if (has_s && has_ds) {         // <S, dS>: row L, 32 columns
-                float dot = 0.f;
-#pragma unroll
-                for (int v4 = 0; v4 < 4; v4++) {
-                    const int ch = grp * 4 + v4;
-                    const uint32_t off = (ch >> 3) * S_PANEL + sw128_chunk(L, ch & 7);
-                    const uint4 x = *reinterpret_cast<const uint4*>(sS + off), y = *reinterpret_cast<const uint4*>(sDS + off);
-                    const __nv_bfloat162 *hx = reinterpret_cast<const __nv_bfloat162*>(&x), *hy = reinterpret_cast<const __nv_bfloat162*>(&y);
-#pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        const float2 fx = __bfloat1622float2(hx[e]), fy = __bfloat1622float2(hy[e]);
-                        dot += fx.x * fy.x + fx.y * fy.y;
-                    }
-                }
-                g_part = rd.gamma * dot;
-            }
+            g_part *= rd.gamma;
             __syncwarp();
             if (lane == 0) mbar_arrive(&m.bar_qk_read);
             // this thread's four rows: t0 + 2c, +1, t0 + 8 + 2c, +1
@@ -443,8 +429,8 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
 
 }  // namespace
 
-// Gradients of the chunks of sequences [seq_lo, seq_hi); states in a.chunk_states, their gradients in ds_tiles.
-int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
+// Gradients of the chunks of sequences [seq_lo, seq_hi); states in a.chunk_states, their gradients in ds_tiles, <S, dS> in dots.
+int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     CUtensorMap mq, mk, mv, mdo, ms, mds, mdq, mdk, mdv;
     int32_t rc;
@@ -467,7 +453,7 @@ int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
         a.tb, a.seq_lo, a.seq_hi, a.H, mq, mk, mv, mdo, ms, mds, mdq, mdk, mdv, (const __nv_bfloat16*)a.q,
         (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq,
         (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv),
-        (float*)(base + sl.rg), a.dev_status, status_gate(a.flags, a.dev_status));
+        (float*)(base + sl.rg), dots, a.dev_status, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

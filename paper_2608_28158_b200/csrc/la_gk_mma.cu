@@ -834,7 +834,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                   const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk_,
                   __nv_bfloat16* __restrict__ dv_, float* __restrict__ dgk, const __nv_bfloat16* __restrict__ chunk_states,
-                  const __nv_bfloat16* __restrict__ ds_tiles,
+                  const __nv_bfloat16* __restrict__ ds_tiles, const float* __restrict__ dots,
                   float* __restrict__ ds0, float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg,
                   const int32_t* gate, int* status, int* ds0_flags, int* ticket, const RoundOrder rounds) {
     if (gate_closed(gate)) return;
@@ -1008,21 +1008,19 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                 }
             }
         }
-        {   // <S_c[i,:], dS[i,:]> over this warp's 64 columns of its 16 state rows i (the two column halves meet later)
+        if constexpr (CHUNKS) {      // <S_c[i,:], dS[i,:]> in four parts of 32 columns, from the scan (dS is fp32 there)
+            if (tid < 2 * D) {
+                const float* part = dots + ((size_t)gc * H + h) * (4 * D) + (tid >> 7) * (2 * D) + (tid & (D - 1));
+                sRowdot[tid] = has_s && has_ds ? part[0] + part[D] : 0.f;
+            }
+        } else {   // <S_c[i,:], dS[i,:]> over this warp's 64 columns of its 16 state rows i (the two column halves meet later)
             const int i0 = (warp & 7) * 16 + g, c0 = (warp >> 3) * 64 + tq * 2;
             float d_lo = 0.f, d_hi = 0.f;
-            if (has_s && has_ds)
 #pragma unroll
             for (int n = 0; n < 8; n++) {
                 const float2 s_lo = ld_bf2(sSc, i0, c0 + n * 8), s_hi = ld_bf2(sSc, i0 + 8, c0 + n * 8);
-                if constexpr (CHUNKS) {
-                    const float2 x_lo = ld_bf2(sdSb, i0, c0 + n * 8), x_hi = ld_bf2(sdSb, i0 + 8, c0 + n * 8);
-                    d_lo += s_lo.x * x_lo.x + s_lo.y * x_lo.y;
-                    d_hi += s_hi.x * x_hi.x + s_hi.y * x_hi.y;
-                } else {
-                    d_lo += s_lo.x * ds[n][0] + s_lo.y * ds[n][1];
-                    d_hi += s_hi.x * ds[n][2] + s_hi.y * ds[n][3];
-                }
+                d_lo += s_lo.x * ds[n][0] + s_lo.y * ds[n][1];
+                d_hi += s_hi.x * ds[n][2] + s_hi.y * ds[n][3];
             }
             d_lo += __shfl_xor_sync(0xffffffffu, d_lo, 1); d_lo += __shfl_xor_sync(0xffffffffu, d_lo, 2);
             d_hi += __shfl_xor_sync(0xffffffffu, d_hi, 1); d_hi += __shfl_xor_sync(0xffffffffu, d_hi, 2);
@@ -1344,7 +1342,7 @@ int32_t gk_mma_bwd(const BwdArgs& a) {
     gk_mma_bwd_kernel<ROUND><<<n, NT, SharedB::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (const __nv_bfloat16*)a.chunk_states, nullptr, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
@@ -1385,7 +1383,7 @@ int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrd
     gk_mma_bwd_kernel<ONE_LAUNCH_MODE><<<(int)n, NT, SharedB::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (const __nv_bfloat16*)a.chunk_states, nullptr, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
         (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, flags, ticket, rounds);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
@@ -1401,7 +1399,7 @@ int32_t gk_chunk_fwd(const FwdArgs& a) {
         (__nv_bfloat16*)a.o, (const __nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
-int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
+int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     if (cudaFuncSetAttribute(gk_mma_bwd_kernel<CHUNKS_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) != cudaSuccess)
         return HARTS_ECUDA;
@@ -1411,7 +1409,7 @@ int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles) {
     gk_mma_bwd_kernel<CHUNKS_MODE><<<(int)(n < sm_count() ? n : sm_count()), NT, SharedB::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, (const __nv_bfloat16*)ds_tiles, (float*)(base + sl.ds0), (float*)(base + sl.rk),
+        (const __nv_bfloat16*)a.chunk_states, (const __nv_bfloat16*)ds_tiles, dots, (float*)(base + sl.ds0), (float*)(base + sl.rk),
         (float*)(base + sl.rv), (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }

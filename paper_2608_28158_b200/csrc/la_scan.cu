@@ -4,6 +4,8 @@
 // Backward: dS_{c-1} = e^{b_n} dS_c + sum_t q_t^T (e^{b_t} dO_t)   dS_c (gradient at the END of chunk c) -> workspace tile
 // With the tiles in memory every chunk is independent of every other (la_chunk_fwd.cu, la_chunk_bwd.cu), so a problem
 // whose (sequence, head) chains are fewer than the SMs still fills the GPU.
+// The backward also leaves <S_c[i,:], dS_c[i,:]> of every chunk, row and 32 columns, which dg needs: the gradient is fp32 only
+// here.  S_c arrives in the buffer that the gradient's tile leaves from, one to two tiles ahead, so it takes no room.
 //
 // What bounds it: the chain of chunks of one sequence while there are few of them, then 64 KB of traffic per (chunk, head).
 // So the products, which do not depend on the chain, are taken out of it: the sum of a chunk is a tcgen05 product of its
@@ -61,6 +63,7 @@ struct Misc {
     uint64_t full[5], weighted[5], stage_empty[5], u_full[2], u_empty[2], gates_full[GATES], gates_empty[GATES], out_full[3],
         out_empty[3], item_full[ITEMS], item_empty[ITEMS], part_full[2];
     Item items[ITEMS];
+    int2 tile[3];            // backward: the tile (index, slice) a buffer is for
     uint32_t tmem;
     int dead;
 };
@@ -72,9 +75,9 @@ template <bool BWD, int NV, bool GK>
 __global__ void __launch_bounds__(Shape<NV, GK>::NT, NV == 32 ? 2 : 1)
 scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __grid_constant__ CUtensorMap map_a,
             const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_g,
-            const __grid_constant__ CUtensorMap map_tiles,
+            const __grid_constant__ CUtensorMap map_tiles, const __grid_constant__ CUtensorMap map_s,
             const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ b, const float* __restrict__ g,
-            float* slots, float* ds0, int* status, const int32_t* gate, int* flags, int* ticket, const RoundOrder order) {
+            float* slots, float* ds0, float* __restrict__ dots, int* status, const int32_t* gate, int* flags, int* ticket, const RoundOrder order) {
     if (gate_closed(gate)) return;
     using S = Shape<NV, GK>;
     constexpr int SLICES = D / NV, NS = S::NS, NWT = S::NWT, CW = S::CW, STAGES = S::STAGES, OUTS = S::OUTS;
@@ -163,13 +166,31 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     boundary = req >= it.req_lo ? tb.slot_chunk[req] : -1;
                 }
                 if (!BWD || i > 0) {              // the state before this step as a bf16 tile (backward: zero after the last chunk)
-                    if (gt >= OUTS && !wait_warp(&m.out_empty[gt % OUTS], gt / OUTS - 1)) alive = false;
+                    // backward: the buffer holds S_c, which is multiplied with the gradient before that is rounded over it
+                    if ((BWD || gt >= OUTS) && !wait_warp(&m.out_empty[gt % OUTS], BWD ? gt / OUTS : gt / OUTS - 1)) alive = false;
                     unsigned char* dst = smem + S::out + (gt % OUTS) * S::O + (col0 >> 6) * S_PANEL;
+                    float* dot = BWD ? dots + ((size_t)(it.chunk_base + c) * H + it.h) * (4 * D) + (it.slice * NV + col0) / 32 * D + L : nullptr;
+                    float d0 = 0.f, d1 = 0.f;
 #pragma unroll
-                    for (int v = 0; v < CW / 8; v++)
-                        *reinterpret_cast<uint4*>(dst + (NV == 32 ? L * 64 + ((v ^ ((L >> 1) & 3)) << 4) : sw128_chunk(L, (col0 & 63) / 8 + v))) =
-                            make_uint4(pack_bf16(x[8 * v], x[8 * v + 1]), pack_bf16(x[8 * v + 2], x[8 * v + 3]),
-                                       pack_bf16(x[8 * v + 4], x[8 * v + 5]), pack_bf16(x[8 * v + 6], x[8 * v + 7]));
+                    for (int v = 0; v < CW / 8; v++) {
+                        uint4* at = reinterpret_cast<uint4*>(dst + (NV == 32 ? L * 64 + ((v ^ ((L >> 1) & 3)) << 4) : sw128_chunk(L, (col0 & 63) / 8 + v)));
+                        if constexpr (BWD) {
+                            const uint4 y = *at;
+                            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&y);
+#pragma unroll
+                            for (int e = 0; e < 4; e++) {
+                                const float2 f = __bfloat1622float2(h2[e]);
+                                d0 += f.x * x[8 * v + 2 * e];
+                                d1 += f.y * x[8 * v + 2 * e + 1];
+                            }
+                            if ((v & 3) == 3) {   // 32 columns: the same sums whatever the width of the slices
+                                dot[v / 4 * D] = d0 + d1;
+                                d0 = d1 = 0.f;
+                            }
+                        }
+                        *at = make_uint4(pack_bf16(x[8 * v], x[8 * v + 1]), pack_bf16(x[8 * v + 2], x[8 * v + 3]),
+                                         pack_bf16(x[8 * v + 4], x[8 * v + 5]), pack_bf16(x[8 * v + 6], x[8 * v + 7]));
+                    }
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&m.out_full[gt % OUTS]);
@@ -456,15 +477,51 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
         }
         }
     } else {
-        // ---- tile stores ---------------------------------------------------------------------------------------------------------
+        // ---- tile stores (backward: and the loads of S_c into their buffers) -----------------------------------------------------
         int gt = 0;
         bool alive = true;
-        if (lane == 0) {
+        if (BWD && lane == 0) {
+            int loaded = 0, k = 0, i = 0, n = 0, chunk_base = 0, h = 0, slice = 0;
+            // requests S_c for the next tile, in this item or the next that has one; false: there is none
+            auto request = [&] {
+                while (i >= n) {
+                    if (!wait(&m.item_full[k % ITEMS], k / ITEMS)) return false;
+                    const Item& it = m.items[k % ITEMS];
+                    const int seq = it.seq;
+                    n = it.n_chunks;
+                    chunk_base = it.chunk_base;
+                    h = it.h;
+                    slice = it.slice;
+                    mbar_arrive(&m.item_empty[k++ % ITEMS]);
+                    if (seq < 0) return false;
+                    i = 1;
+                }
+                const int buf = loaded++ % OUTS, idx = (chunk_base + n - 1 - i++) * H + h;
+                m.tile[buf] = make_int2(idx, slice);
+                mbar_expect_tx(&m.out_empty[buf], S::O);
+                for (int p = 0; p < (NV + 63) / 64; p++)
+                    tma_load_3d(smem + S::out + buf * S::O + p * S_PANEL, &map_s, slice * NV + p * 64, 0, idx, &m.out_empty[buf]);
+                return true;
+            };
+            bool more = true;
+            while (more && loaded < OUTS) more = request();
+            for (; gt < loaded; gt++) {
+                if (!wait(&m.out_full[gt % OUTS], gt / OUTS)) break;
+                const int2 tile = m.tile[gt % OUTS];
+                for (int p = 0; p < (NV + 63) / 64; p++)
+                    tma_store_3d(&map_tiles, smem + S::out + (gt % OUTS) * S::O + p * S_PANEL, tile.y * NV + p * 64, 0, tile.x);
+                tma_store_commit();
+                if (!more) continue;
+                tma_store_wait_read();
+                more = request();
+            }
+            tma_store_wait_all();
+        } else if (lane == 0) {
             for (int k = 0; alive && wait(&m.item_full[k % ITEMS], k / ITEMS); k++) {
                 const Item it = m.items[k % ITEMS];
                 mbar_arrive(&m.item_empty[k % ITEMS]);
                 if (it.seq < 0) break;
-                for (int i = BWD ? 1 : 0; i < it.n_chunks; i++, gt++) {
+                for (int i = 0; i < it.n_chunks; i++, gt++) {
                     if (!(alive = wait(&m.out_full[gt % OUTS], gt / OUTS))) break;
                     const int idx = (it.chunk_base + chunk_of(it, i)) * H + it.h;
                     for (int p = 0; p < (NV + 63) / 64; p++)
@@ -490,7 +547,8 @@ struct Launch {
     const void *a, *b;
     const float* g;
     void* tiles;
-    float *slots, *ds0;
+    const void* states;      // backward: the forward's tiles
+    float *slots, *ds0, *dots;
     int* status;
     const int32_t* gate;
     int* flags;              // all rounds in one launch (order.n > 0): the ticket, then counters per (slot | sequence, head, slice)
@@ -501,7 +559,7 @@ struct Launch {
 template <bool BWD, int NV, bool GK>
 int32_t launch(const Launch& x) {
     using S = Shape<NV, GK>;
-    CUtensorMap ma, mb, mg, mt;
+    CUtensorMap ma, mb, mg, mt, ms;
     int32_t rc;
     const int64_t n_tiles = (int64_t)x.tb.n_chunks * x.H;
     if ((rc = make_row_map(&ma, x.a, x.tb.n_rows, x.H)) != HARTS_OK) return rc;
@@ -509,6 +567,8 @@ int32_t launch(const Launch& x) {
     mg = ma;
     if (GK && (rc = make_gate_map(&mg, x.g, x.tb.n_rows, x.H)) != HARTS_OK) return rc;
     if ((rc = NV == 32 ? make_state_slice_map(&mt, x.tiles, n_tiles) : make_state_map(&mt, x.tiles, n_tiles)) != HARTS_OK) return rc;
+    ms = mt;
+    if (BWD && (rc = NV == 32 ? make_state_slice_map(&ms, x.states, n_tiles) : make_state_map(&ms, x.states, n_tiles)) != HARTS_OK) return rc;
     if (cudaFuncSetAttribute(scan_kernel<BWD, NV, GK>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int n = (x.seq_hi - x.seq_lo) * x.H * (D / NV), resident = (NV == 32 ? 2 : 1) * sm_count();
@@ -517,7 +577,7 @@ int32_t launch(const Launch& x) {
         if (cudaMemsetAsync(x.flags, 0, (4 + n_flags) * sizeof(int), x.stream) != cudaSuccess) return HARTS_ECUDA;
     }
     scan_kernel<BWD, NV, GK><<<n < resident ? n : resident, S::NT, S::bytes, x.stream>>>(
-        x.tb, x.seq_lo, n, x.H, ma, mb, mg, mt, (const __nv_bfloat16*)x.a, (const __nv_bfloat16*)x.b, x.g, x.slots, x.ds0, x.status, x.gate,
+        x.tb, x.seq_lo, n, x.H, ma, mb, mg, mt, ms, (const __nv_bfloat16*)x.a, (const __nv_bfloat16*)x.b, x.g, x.slots, x.ds0, x.dots, x.status, x.gate,
         x.flags + 4, x.flags, x.order);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
@@ -539,14 +599,14 @@ int32_t launch_sliced(const Launch& x) {
 // launch cannot deadlock.
 int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    return launch_sliced<false>({a.tb, a.seq_lo, a.seq_hi, a.H, a.k, a.v, a.g, a.chunk_states, a.slots, nullptr, a.dev_status,
+    return launch_sliced<false>({a.tb, a.seq_lo, a.seq_hi, a.H, a.k, a.v, a.g, a.chunk_states, nullptr, a.slots, nullptr, nullptr, a.dev_status,
                                  status_gate(a.flags, a.dev_status), flags, order, a.stream});
 }
 
-int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order) {
+int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     float* ds0 = (float*)((char*)a.scratch + scratch_layout(a.tb, a.H, a.dk, a.dv).ds0);
-    return launch_sliced<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, nullptr, ds0, a.dev_status,
+    return launch_sliced<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, a.chunk_states, nullptr, ds0, dots, a.dev_status,
                                 status_gate(a.flags, a.dev_status), flags, order, a.stream});
 }
 
@@ -559,13 +619,13 @@ static int32_t launch_gk(const Launch& x) {
 }
 int32_t gk_scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    return launch_gk<false>({a.tb, a.seq_lo, a.seq_hi, a.H, a.k, a.v, a.g, a.chunk_states, a.slots, nullptr, a.dev_status,
+    return launch_gk<false>({a.tb, a.seq_lo, a.seq_hi, a.H, a.k, a.v, a.g, a.chunk_states, nullptr, a.slots, nullptr, nullptr, a.dev_status,
                              status_gate(a.flags, a.dev_status), flags, order, a.stream});
 }
-int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, int* flags, const RoundOrder& order) {
+int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
     float* ds0 = (float*)((char*)a.scratch + gk_scratch_layout(a.tb, a.H, a.dk, a.dv).ds0);
-    return launch_gk<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, nullptr, ds0, a.dev_status,
+    return launch_gk<true>({a.tb, a.seq_lo, a.seq_hi, a.H, a.q, a.dO, a.g, ds_tiles, a.chunk_states, nullptr, ds0, dots, a.dev_status,
                             status_gate(a.flags, a.dev_status), flags, order, a.stream});
 }
 

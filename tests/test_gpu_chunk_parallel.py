@@ -1,11 +1,14 @@
 """The chunk-parallel linear-attention path at its edges and at the line where the walk kernels take over."""
+import numpy as np
 import pytest
 import torch
 
 import paper_2608_28158_b200 as H
-from parity_util import compare, oracle_subset, plan_of, run_gpu
+from oracle import gk_oracle as go
+from oracle import la_oracle as lo
+from parity_util import compare, oracle_subset, plan_of, rel_err, run_gpu, to_physical
 from test_gpu_parity import check
-from workloads import make_forest, make_inputs
+from workloads import make_forest, make_gk, make_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -127,3 +130,35 @@ def test_fp32_keeps_its_precision_behind_steep_gates(reset):
     tok, ref = oracle_subset(fo, inp, [0], [0, 1])
     errs = compare(out, tok, [0, 1], ref)
     assert all(e <= 64 * 2.0 ** -24 for e in errs.values()), errs
+
+
+def _gk_dg(fo, inp):
+    plan = plan_of(fo).upload()
+    x = to_physical(plan, inp)
+    n, heads, d = x["q"].shape
+    states, scratch = (torch.empty(b, dtype=torch.uint8, device="cuda") for b in H.harts_la_gk_workspace_bytes(plan.tables, heads, d, d, 1))
+    slots, status = torch.empty(max(plan.n_slots, 1) * heads * d * d, device="cuda"), torch.zeros(4, dtype=torch.int32, device="cuda")
+    o, dq, dk, dv, dg = (torch.empty_like(x[m]) for m in ("v", "q", "k", "v", "g"))
+    H.harts_la_gk_fwd(plan, 0, x["q"], x["k"], x["v"], x["g"], o, slots, states, 0, status)
+    H.harts_la_gk_bwd(plan, 0, x["q"], x["k"], x["v"], x["g"], x["dO"], dq, dk, dv, dg, states, scratch, 0, status)
+    H.harts_la_check(status)
+    return dg[torch.as_tensor(plan.row_of_token.astype(np.int64), device="cuda")]
+
+
+@pytest.mark.parametrize("gates", [1.0, 0.0])
+@pytest.mark.parametrize("form", ["scalar", "per_channel"])
+def test_dg_is_as_exact_as_in_the_walk(form, gates):
+    """Seven sequences x 4 heads take the chunk-parallel path, the same four heads 24 times over the walk kernels.  Both hold the
+    boundary gradient in 32 bits where dg needs it: against the oracle the one is not further off than the other (without decay
+    a bf16 gradient made it 1.4 times as far)."""
+    fo = make_forest([([-1] + [0] * 6, [0] + [700] * 6, [900] + [330] * 6)])
+    inp = make_inputs(fo.n_tokens, 4, 128, 128, "bf16", 18)
+    if form == "per_channel":
+        inp["g"] = make_gk(fo.n_tokens, 4, 128, 18)
+    inp["g"] = inp["g"] * gates
+    many = {n: x.repeat(1, 24, *[1] * (x.dim() - 2)) for n, x in inp.items()}
+    oracle, run = (go, _gk_dg) if form == "per_channel" else (lo, lambda fo, x: run_gpu(fo, x)[1]["dg"])
+    ref = oracle.forest_eval(fo, *(inp[n] for n in ("q", "k", "v", "g", "dO")))["dg"]
+    chunk, walk = (rel_err(run(fo, x)[:, :4].cpu().numpy(), ref) for x in (inp, many))
+    print(f"{form} x{gates}: dg error {chunk:.2e} chunk-parallel, {walk:.2e} walk")
+    assert chunk <= 1.1 * walk
