@@ -320,7 +320,7 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
 int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* k, const void* v, const float* lse,
                         const void* dO, const float* delta, void* dk_, void* dv_, int Hq, int Hkv, float scale,
                         int32_t* status, const SplitTable* split, cudaStream_t st);
-bool attn_split_table(const Index& ix, int Hkv, void* buf, size_t bytes, SplitTable* t);
+bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* buf, size_t bytes, SplitTable* t);
 int32_t attn_split_launch(const Index& ix, int G, int Hkv, const SplitTable& t, cudaStream_t st);
 int32_t attn_split_reduce(const Index& ix, int Hkv, const SplitTable& t, void* dk_, void* dv_, cudaStream_t st);
 
@@ -344,8 +344,8 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
         return HARTS_ECUDA;
     const Index ix = make_index(hi, di);
     SplitTable split;
-    const bool cut = attn_split_table(ix, Hkv, dq, (size_t)n_rows * Hq * D * 2, &split);
-    if (cut) {        // small problems: the units' partial sums use dq's memory before dq is computed
+    const bool cut = attn_split_table(ix, hi, Hq / Hkv, Hkv, dq, (size_t)n_rows * Hq * D * 2, &split);
+    if (cut) {        // small, skewed problems: the units' partial sums use dq's memory before dq is computed
         if ((rc = attn_split_launch(ix, Hq / Hkv, Hkv, split, st)) != HARTS_OK) return rc;
         if ((rc = attn_dkv_launch(ix, n_rows, q, k, v, lse, dO, delta, dk_, dv_, Hq, Hkv, scale, status, &split, st)) != HARTS_OK) return rc;
         if ((rc = attn_split_reduce(ix, Hkv, split, dk_, dv_, st)) != HARTS_OK) return rc;

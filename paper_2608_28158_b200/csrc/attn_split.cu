@@ -1,9 +1,12 @@
-// Split of the dK / dV work of small problems.  A key tile near the root is seen by every query below it -- for every query
-// head of its group -- so on one tree with grouped queries a few work items are most of the work, and the CTA that draws the
-// largest one is what the launch takes (9,001 tokens, 16 query heads on 4 key heads: 1.02 ms, 0.33 ms with this split).  Here
-// one CTA cuts every item into units of about a quarter of an SM's share of the whole, attn_dkv_kernel leaves the sums of
+// Split of the dK / dV work of small, skewed problems (worth_cutting).  A key tile near the root is seen by every query below
+// it -- for every query head of its group -- so on one tree with grouped queries a few work items are most of the work, and the
+// CTA that draws the largest one is what the launch takes (9,001 tokens, 16 query heads on 4 key heads: 1.02 ms, 0.33 ms with
+// this split).  Here one CTA cuts every item into units of about a quarter of an SM's share of the whole, attn_dkv_kernel leaves the sums of
 // a cut item in fp32, unit by unit, and reduce_kernel adds them in unit order (no atomics: same bits every run).
 // The table and the partial sums live in the dq tensor, which is written only afterwards (the dQ kernel runs last then).
+#include <memory>
+#include <new>
+
 #include "kernels.h"
 
 #include "../../include/harts_attn.h"
@@ -152,10 +155,51 @@ __global__ void __launch_bounds__(256) reduce_kernel(Index ix, int Hkv, SplitTab
 
 }  // namespace
 
-// The table and the partial sums in `buf`; false: too small a buffer, or so much work that it balances by itself (16 items
-// and more per SM: the largest item of 16k-token trees is then 1 in 25 of an SM's share).
-bool attn_split_table(const Index& ix, int Hkv, void* buf, size_t bytes, SplitTable* t) {
-    if ((long long)ix.n_kv_items * Hkv >= 16LL * sm_count()) return false;
+// What cutting would save, from the host's copy of the index: the dK / dV items as they are dealt without a cut (snake order, one
+// CTA per SM), in query tiles (about 1.2 us) with six more for the start and end of an item.  The CTA with the most work
+// against an even share: the cut has to make up for its two extra kernels, the units' starts and ends and the partial sums
+// (both kernels and forward, whole -> cut, us).
+//   worth it    9,001 branchy tokens, 16 query / 4 key heads  1,527 -> 1,224  (most 656 tiles, share 271); 30,001 x 16/4
+//               3,954 -> 3,055 (1,818, 844); 18,001 x 16/8 3,106 -> 2,766 (1,312, 758); 25,001 x 8/8 1,443 -> 1,330 (622, 333)
+//   not         agentic trees, whose items are even: 65,521 x 4/4 5,591 -> 6,105 (1,902, 1,740), 20,001 x 16/2 7,861 -> 8,669
+//               (2,796, 2,476); little work: 5,001 branchy x 32/16 1,080 -> 1,216 (442, 252), 5,001 agentic x 8/4 513 -> 536
+static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
+    const int P = hi[1], n_items = hi[5];
+    const int32_t *len = hi + hi[9], *parent = hi + hi[10], *item = hi + hi[17];
+    auto tiles = [](int rows) { return (rows + 63) / 64; };
+    std::unique_ptr<int32_t[]> mem(new (std::nothrow) int32_t[3 * (size_t)P]());
+    std::unique_ptr<int64_t[]> load(new (std::nothrow) int64_t[sms]());
+    if (!mem || !load) return false;
+    int32_t *below = mem.get(), *kids = below + P, *todo = kids + P, n = 0;     // below: query tiles of all descendants
+    for (int p = 0; p < P; p++)
+        if (parent[p] >= 0) kids[parent[p]]++;
+    for (int p = 0; p < P; p++)
+        if (!kids[p]) todo[n++] = p;
+    while (n) {
+        const int p = todo[--n], a = parent[p];
+        if (a < 0) continue;
+        below[a] += below[p] + tiles(len[p]);
+        if (--kids[a] == 0) todo[n++] = a;
+    }
+    int64_t total = 0, most = 0;
+    for (int i = 0, at = 0, tier = 0; i < n_items; i++) {
+        const int piece = item[2 * i];
+        const int64_t t = (int64_t)G * (below[piece] + tiles(len[piece] - item[2 * i + 1] * 128));
+        total += t * Hkv;
+        for (int h = 0; h < Hkv; h++) {
+            int64_t& l = load[tier & 1 ? sms - 1 - at : at];
+            l += t + 6;
+            most = l > most ? l : most;
+            if (++at == sms) at = 0, tier++;
+        }
+    }
+    return most * sms * 10 >= total * 17 && (most - 240) * sms >= total;
+}
+
+// The table and the partial sums in `buf`; false: too small a buffer, nothing to gain, or 16 items and more per SM (where the
+// largest item is a small part of a share, but for fans: 10,000 replay tokens x 8 heads, 22 per SM, 2,053 us against 1,791 cut).
+bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* buf, size_t bytes, SplitTable* t) {
+    if ((long long)ix.n_kv_items * Hkv >= 16LL * sm_count() || !worth_cutting(hi, G, Hkv, sm_count())) return false;
     const size_t max_units = (size_t)ix.n_kv_items + 5 * sm_count() + 64;       // units of a quarter share, plus one per item
     char* p = static_cast<char*>(buf);
     size_t off = 256;
