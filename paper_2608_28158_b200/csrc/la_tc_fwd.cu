@@ -503,81 +503,75 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// The encoder is a driver call and wants a current context.  A thread that has made no runtime call yet has none (the kernels'
+// own launches would set it, but the maps come first): the device the runtime would use is made current then.
+template <typename... Args>
+int32_t encode(Args... args) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return HARTS_ECUDA;
+    if (fn(args...) == CUDA_SUCCESS) return HARTS_OK;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return HARTS_ECUDA;
+    return fn(args...) == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+}
+
 }  // namespace
 
 // [rows][H][128] bf16 tensor, box = 64 rows x 1 head x 64 columns
 int32_t make_row_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)rows};
     cuuint64_t strides[2] = {256, (cuuint64_t)H * 256};
     cuuint32_t box[3] = {64, 1, 64}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // [n][128][128] bf16 states, box = 1 state x 128 rows x 64 columns
 int32_t make_state_map(CUtensorMap* map, const void* base, int64_t n) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, 128, (cuuint64_t)(n < 1 ? 1 : n)};
     cuuint64_t strides[2] = {256, 32768};
     cuuint32_t box[3] = {64, 128, 1}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // [n][128][128] fp32 states (exported slots, hand-off gradients), box = 1 state x 128 rows x 32 columns
 int32_t make_state32_map(CUtensorMap* map, const void* base, int64_t n) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, 128, (cuuint64_t)(n < 1 ? 1 : n)}, strides[2] = {512, 65536};
     cuuint32_t box[3] = {32, 128, 1}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // 32-column slices of [n][128][128] bf16 states, box = 1 state x 128 rows, 64-byte swizzle
 int32_t make_state_slice_map(CUtensorMap* map, const void* base, int64_t n) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, 128, (cuuint64_t)(n < 1 ? 1 : n)}, strides[2] = {256, 32768};
     cuuint32_t box[3] = {32, 128, 1}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // [rows][H][128] fp32 tensor, box = 64 rows x 1 head x 128 columns, plain rows
 int32_t make_gate_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)rows}, strides[2] = {512, (cuuint64_t)H * 512};
     cuuint32_t box[3] = {128, 1, 64}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 // [rows][H][128] bf16 output tensor, box = 64 rows x 1 head x 128 columns, plain (unswizzled) rows
 int32_t make_out_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return HARTS_ECUDA;
     cuuint64_t dims[3] = {128, (cuuint64_t)H, (cuuint64_t)rows};
     cuuint64_t strides[2] = {256, (cuuint64_t)H * 256};
     cuuint32_t box[3] = {128, 1, 64}, es[3] = {1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? HARTS_OK : HARTS_ECUDA;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 int sm_count() {
