@@ -17,6 +17,7 @@ extern "C" int32_t harts_attn_index(int32_t n_trees, const int32_t* tree_node_pt
     if (n_trees < 0 || !tree_node_ptr || !node_parent || !node_fork_off || !node_len || !n_words) return HARTS_EINVAL;
     if (tree_node_ptr[0] != 0) return HARTS_EINVAL;
     const int32_t n_nodes = tree_node_ptr[n_trees];
+    if (n_nodes < 0) return HARTS_EINVAL;
     std::vector<int64_t> base(n_nodes + 1, 0);
     for (int32_t t = 0; t < n_trees; ++t) {
         const int32_t lo = tree_node_ptr[t], hi = tree_node_ptr[t + 1];

@@ -13,6 +13,7 @@ extern "C" int32_t harts_la_expand(int32_t n_trees, const int32_t* tree_node_ptr
         return HARTS_EINVAL;
     if (tree_node_ptr[0] != 0) return HARTS_EINVAL;
     const int32_t n_nodes = tree_node_ptr[n_trees];
+    if (n_nodes < 0) return HARTS_EINVAL;
     std::vector<int64_t> base(static_cast<size_t>(n_nodes) + 1, 0);      // canonical index of a node's first token
     std::vector<int64_t> depth(n_nodes, 0);                              // tokens on the path before the node
     std::vector<char> continued(n_nodes, 0);                             // a child forks at the node's very end

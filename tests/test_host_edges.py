@@ -67,3 +67,9 @@ def test_attention_index_beyond_the_first_guess():
     _check_index(fo, None)
     ix = H.harts_attn_index(fo.tree_node_ptr, fo.node_parent, fo.node_fork_off, fo.node_len)
     assert len(ix.host) > 4096 + 64 * 2 * n + 2 * n // 16
+
+
+@pytest.mark.parametrize("call", [H.harts_attn_index, H.harts_conv_index, H.harts_la_expand, H.harts_la_plan])
+def test_a_negative_node_count_is_an_error(call):
+    with pytest.raises(H.HartsError):
+        call([0, -5], [], [], [])
