@@ -582,12 +582,17 @@ int32_t launch(const Launch& x) {
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 // The narrower the slices, the shorter a step of the walk and the more often k is read: as narrow as leaves the chains of the
-// (first) round at most one CTA per SM.  One tree x 4 heads (4 chains in round 1): 32 columns 73 us, 64: 79, 128: 131; four
-// trees x 16 heads: 265 / 226 / 275; eight trees x 16 heads: 576 / 485 / 463.
+// (first) round at most one CTA per SM, but never 128 columns in the backward, where a state thread multiplies its columns with
+// S_c besides.  Device time in us with 32 / 64 / 128 columns, cold inputs: 17,695 tokens x 4 heads (4 chains in
+// the first round) forward 78 / 93 / 141, backward 82 / 86 / 187; 65,521 x 16 (64 chains) 298 / 244 / 289, 406 / 293 / 451;
+// 100,003 x 16 (96 chains) 426 / 359 / 345, 606 / 468 / 561; 149,270 x 12 (96 chains) forward 64: 401, 128: 400, backward 546, 573.
 template <bool BWD>
 int32_t launch_sliced(const Launch& x) {
     const int chains = (x.order.n ? x.order.ptr[1] - x.order.ptr[0] : x.seq_hi - x.seq_lo) * x.H;
-    return 4 * chains <= sm_count() ? launch<BWD, 32, false>(x) : 2 * chains <= sm_count() ? launch<BWD, 64, false>(x) : launch<BWD, 128, false>(x);
+    if (4 * chains <= sm_count()) return launch<BWD, 32, false>(x);
+    if constexpr (!BWD)
+        if (2 * chains > sm_count()) return launch<false, 128, false>(x);
+    return launch<BWD, 64, false>(x);
 }
 
 }  // namespace
