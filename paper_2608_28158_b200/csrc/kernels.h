@@ -141,14 +141,18 @@ int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      //
 int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
 int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);     // la_chunk_bwd.cu
-// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs.  The walk kernels (la_tc_*.cu) move 240 KB per item in
-// a whole step, this path 400 KB: with enough chains to fill the GPU the walk wins (4,696 chunks x 32 heads: 9.7 against 11.2
-// ms a step; 2,389 x 16: 3.0 against 3.1; 685 chunks in 21 sequences x 32 heads: 1.70 against 1.85), with few the chain of its
-// 3-6 us chunks is what takes the time (walk -> chunk-parallel: 304 chunks x 4 heads, forward + backward, 0.74 -> 0.24 ms;
-// 1,047 chunks in 28 sequences x 16, forward, 0.87 -> 0.52).  With r = longest path of chunks over the average sequence (5 to
-// 10), the walk's chain is longer than this path's time while n_seq * H < about 100 r.  Many sequences of a chunk or two (fewer
-// than four chunks each, more than 128 pairs) stay with the walk: the scan pays about 5 us for each of them.  The line
-// depends on the tables' totals only, so that a round issued alone takes the path of the whole.
+// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs, with fewer than four chunks a sequence up to 128 pairs.
+// The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 430 KB: with enough chains to fill the GPU the walk
+// wins, with few the chain of its 3-6 us chunks is what takes the time.  Walk / chunk-parallel, time of a step (of the forward
+// alone), 46 forests both ways with cold inputs:
+//   inside the line the chunk path won everywhere: 304 chunks x 4 heads 2.8 (2.9); agentic 16,736 items, 384 pairs 1.78 (1.96);
+//     25,576 items, 632 pairs 1.15 (1.34); 28,668 items, 636 pairs 1.20 (1.34); branchy 7,296 items, 624 pairs 1.16 (1.10);
+//     replay fans, 92 to 233 items, 34 to 127 pairs 2.5 to 2.9
+//   just outside it still won on agentic trees (28,144 items, 736 pairs 1.12 (1.26); 33,472 items, 768 pairs 1.05 (1.20)) and on
+//     small fans (368 to 1,008 items, 136 to 508 pairs 1.6 to 2.2): the line is on the safe side there
+//   further out the walk wins: branchy 9,728 items, 832 pairs 0.97 (0.86); 24,768 items, 2,328 pairs 0.89 (0.76); agentic 51,152
+//     items, 1,264 pairs 0.94 (0.90); 6,949 chunks of replay fans x 16 heads 0.65
+// The line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
 constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640;
 inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
     const int64_t chains = (int64_t)tb.n_seq * H;
@@ -170,13 +174,15 @@ inline size_t scan_flags_offset(const harts_la_tables_t& tb, int32_t H, int32_t 
 inline size_t chunk_parallel_bytes(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
     return scan_flags_offset(tb, H, dk, dv) + (4 + (size_t)(tb.n_seq > tb.n_slots ? tb.n_seq : tb.n_slots) * H * 4) * sizeof(int);
 }
-// The same for the per-channel decay, under the same rule (walk -> chunk-parallel, forward + backward: 1,047 chunks x 16 heads
-// 7.7 -> 3.8 ms; 33 k items of agentic trees 7.4 -> 6.8, of branchy ones 7.0 -> 7.2; 64 k items 12.3 -> 12.9).
+// The same for the per-channel decay, under the same rule.  Walk / chunk-parallel, forward + backward: inside the line 1.16 (branchy
+// 7,296 items, 624 pairs) to 4.0, 1.34 at 28,668 items; outside it the chunk path is ahead up to 51,152 items of agentic trees
+// (1.12) and behind on branchy ones (9,728 items, 832 pairs: 0.97).
 int32_t gk_scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);
 int32_t gk_scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);
 int32_t gk_chunk_fwd(const FwdArgs& a);
 int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);
-// The same for fp32 inputs, d_k = d_v = 64 (la_f32.cu): every problem that brings a chunk-state workspace.  extra: e^{b_n}
+// The same for fp32 inputs, d_k = d_v = 64 (la_f32.cu): every problem that brings a chunk-state workspace (3.5 to 35 times as fast
+// as the walk from 13 to 12,880 items, agentic, branchy and replay; least on short sequences).  extra: e^{b_n}
 // [n_chunks, H] and the gradients of the boundary states [n_chunks, H, dk, dv], fp32, behind the flags.
 inline bool f32_chunks(int32_t dk, int32_t dv, int32_t dtype) { return dtype == HARTS_FP32 && dk == 64 && dv == 64; }
 inline size_t f32_extra_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {

@@ -5,7 +5,7 @@
 // state tile arrive by TMA.  Two CTAs per SM (106 KB of shared memory, 256 tensor-memory columns each), 8 compute warps,
 // one warp whose first lane issues every TMA and MMA, one that prepares the next items (record, gates, row ids).  The
 // state's product does not need P, so it runs under the decay masking; only four MMAs are left after it.
-// What bounds it: 96 KB of traffic per item (80 read, 16 written); 2,389 chunks x 16 heads take 0.56 ms = 6.5 TB/s.
+// What bounds it: 96 KB of traffic per item (80 read, 16 written); 1,047 chunks x 16 heads take 0.25 ms = 6.6 TB/s.
 // Every wait is bounded.
 #include "chunk_item.cuh"
 

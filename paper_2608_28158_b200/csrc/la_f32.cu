@@ -8,8 +8,9 @@
 // The kernels of la_fma.cu walk a sequence's chunks with everything in one CTA: 84 us per chunk, forward and backward, one
 // after the other.  Only the walk is serial here, and its step is one multiply-add per element with the operand prefetched;
 // the 64^3 products of different chunks run side by side.  What bounds it: launches and the latency of one product (256
-// threads x 4x4 outputs, 2,048 cycles at 128 multiply-adds a clock) on small forests, the CUDA cores on large ones.  718
-// tokens x 1 head (two rounds), forward + backward: 1.18 -> 0.080 ms (outer 7 + 7, walk 3 per round, out 13, grad 25 us).
+// threads x 4x4 outputs, 2,048 cycles at 128 multiply-adds a clock) on small forests, the CUDA cores on large ones.  Forward +
+// backward, cold inputs, against the walk: 718 tokens x 1 head (two rounds) 1.33 -> 0.095 ms (outer 9 + 7, walk 3 per round, out 17,
+// grad 30 us), 12,000 branchy x 4 12.0 -> 0.34, 40,000 replay x 8 13.6 -> 3.9, 150,000 agentic x 4 46.4 -> 3.3 (grad 2.0, out 0.7).
 #include "chunk_item.cuh"
 
 namespace harts {

@@ -1,9 +1,12 @@
 // Per-channel-decay recurrence (the Diag(gamma) term of Eq. 1, Section 2.2) for bf16 tensors with d_k = d_v = 128:
 // the same packed chunkwise call (Eq. 16), plan tables, slots, chunk states and scratch layout as la_gk.cu, with
 // every dense product of a chunk on the tensor cores (warp-level mma.sync.m16n8k16, bf16 operands, fp32
-// accumulation) and the running state S (forward) / its gradient dS (backward) held in the accumulator registers of
-// the CTA's eight warps for the whole walk over a sequence.  What cannot be a dense product stays on the CUDA cores
-// in fp32: the decay-dependent pair sums
+// accumulation).  Two ways to drive them.  The walks hold the running state S (forward) / its gradient dS (backward) in the
+// accumulator registers of the CTA's sixteen warps over a whole sequence, which is what register accumulators are for.  The chunk
+// kernels take every (chunk, head) on its own, with S and dS from memory (la_scan.cu); they share the walks' code for the inside
+// of a chunk and hold no state, so nothing but that ties them to mma.sync: 17 us per item of the backward on one CTA per SM,
+// where its 240 KB of traffic would take 5.6.  What cannot be a dense product stays on the CUDA cores in fp32: the
+// decay-dependent pair sums
 //     A_tj      = sum_i q_t[i] k_j[i] e^{b_t[i]-b_j[i]}                          (j <= t)
 //     dq_t[i]  += sum_{j<=t} dA_tj k_j[i] e^{b_t[i]-b_j[i]},   dk_j[i] += sum_{t>=j} dA_tj q_t[i] e^{b_t[i]-b_j[i]}
 // for t and j in the same 16-row block of the chunk; pairs in different blocks become dense products too, through
@@ -530,7 +533,7 @@ __device__ __forceinline__ int owner_of(const harts_la_tables_t& tb, int seq_lo,
 
 // How a kernel is driven.
 // ROUND: one launch per round, item = (sequence, head) = block index, no flags.
-// CHUNKS (backward only): the boundary states and their gradients are in memory (la_scan.cu), item = (chunk, head).
+// CHUNKS (backward only): the boundary states, their gradients and <S, dS> are in memory (la_scan.cu), item = (chunk, head).
 // ONE_LAUNCH: the grid covers the sequences of ALL rounds (numbered round by round).  Every CTA draws its work item
 // from `ticket`, so an item is only ever held by a running CTA; a sequence that starts from an exported state waits for
 // the flag its producer (an earlier round, a smaller ticket, hence running or done) sets after writing the slot.
@@ -677,7 +680,7 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
 // thread.  To fit, everything is worked on in place or over something dead: the running sums' scratch lies under the
 // scores, k becomes the keys anchored at their own block, q becomes q~, V comes in over the anchored queries once the
 // scores are done, the state over the running sums.  One pass over q and k makes all four operands of a mild chunk.
-// Measured, 1,047 chunks x 16 heads: 0.78 ms (one CTA per SM with every tile in a place of its own: 1.08).
+// Measured, 1,047 chunks x 16 heads: 0.80 ms cold, 0.78 warm (one CTA per SM with every tile in a place of its own: 1.08).
 struct SharedC {
     static constexpr int q = 0, k = 16384;                              // bf16 [64][128]; then q~, keys anchored at their block
     static constexpr int b = 32768;                                     // fp32 [64][128] running log-decay; then the state

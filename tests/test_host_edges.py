@@ -73,3 +73,17 @@ def test_attention_index_beyond_the_first_guess():
 def test_a_negative_node_count_is_an_error(call):
     with pytest.raises(H.HartsError):
         call([0, -5], [], [], [])
+
+
+@pytest.mark.parametrize("n_seq,n_chunks,heads,chunks", [
+    (5, 448, 64, True), (5, 449, 64, False), (5, 28672, 1, True), (5, 28673, 1, False),        # 28,672 items
+    (10, 44, 64, True), (10, 44, 65, False),                                                   # 640 (sequence, head) pairs
+    (32, 128, 5, True), (32, 127, 5, False), (32, 127, 4, True)])                              # four chunks a sequence, or 128 pairs
+@pytest.mark.parametrize("sizes", [H.harts_la_workspace_bytes, H.harts_la_gk_workspace_bytes])
+def test_which_problems_bring_the_room_of_the_chunk_parallel_path(sizes, n_seq, n_chunks, heads, chunks):
+    """The rule that picks the path also sizes the workspace: states alone (and flags), or their gradients and <S, dS> besides."""
+    tables = H.binding.Tables(chunk=64, n_rows=64 * n_chunks, n_seq=n_seq, n_chunks=n_chunks)
+    states = n_chunks * heads * 128 * 128 * 2
+    got = sizes(tables, heads, 128, 128, H.HARTS_BF16)[0] - states
+    assert (got >= states + n_chunks * heads * 4 * 128 * 4) == chunks
+    assert chunks or got < states // 2 + 4096
