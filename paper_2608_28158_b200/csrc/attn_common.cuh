@@ -60,6 +60,13 @@ struct TileWalkT {      // enumerates the key tiles (W rows) of one item in orde
         return n;
     }
     __device__ bool next(KvTile& t) {
+        if (!in_own && off + W < cur_len) {       // inside a run
+            t.row = cur_row0 + off;
+            t.n_valid = W;
+            t.shift = NO_DIAG;
+            off += W;
+            return true;
+        }
         if (!in_own) {
             t.row = cur_row0 + off;
             t.n_valid = min(W, cur_len - off);
@@ -102,7 +109,7 @@ struct SplitTable {
     int cap_slots;
 };
 
-// The query tiles (64 rows) that see the key tile `kt` (128 rows) of a piece: for every query head of the group,
+// The query tiles (128 rows) that see the key tile `kt` (128 rows) of a piece: for every query head of the group,
 // the rest of the piece from the key tile's first row on (causal inside), then all rows of every descendant piece.
 // Key row i is seen by query column j iff jmin(i) <= j < n_valid, with jmin(i) = max(0, i - lead) for own tiles
 // (lead = first query row of the tile minus first key row of the key tile) and 0 for descendants.
@@ -115,7 +122,7 @@ struct QWalk {
     int left = 0x7fffffff;              // tiles still to deliver (a unit of a cut item)
     bool in_own;
     __device__ QWalk(const Index& ix_, int piece_, int kt, int hk, int G_) : ix(ix_), piece(piece_), G(G_) {
-        k0 = kt * 128;
+        k0 = kt * BQ;
         own_len = ix.piece_len[piece];
         own_row0 = ix.piece_row0[piece];
         head0 = hk * G;
@@ -140,8 +147,8 @@ struct QWalk {
         d = ix.desc_ptr[piece];
     }
     __device__ int count() const {
-        int n = (own_len - k0 + 63) / 64;
-        for (int e = ix.desc_ptr[piece]; e < d_end; e++) n += (ix.piece_len[ix.desc_piece[e]] + 63) / 64;
+        int n = (own_len - k0 + BQ - 1) / BQ;
+        for (int e = ix.desc_ptr[piece]; e < d_end; e++) n += (ix.piece_len[ix.desc_piece[e]] + BQ - 1) / BQ;
         return n * G;
     }
     __device__ bool next(QTile& t) {
@@ -151,10 +158,10 @@ struct QWalk {
             if (in_own) {
                 if (off < own_len) {
                     t.row = own_row0 + off;
-                    t.n_valid = min(64, own_len - off);
+                    t.n_valid = min(BQ, own_len - off);
                     t.lead = off - k0;
                     t.head = head0 + g;
-                    off += 64;
+                    off += BQ;
                     return true;
                 }
                 in_own = false;
@@ -166,10 +173,10 @@ struct QWalk {
             }
             if (d < d_end) {
                 t.row = cur_row0 + off;
-                t.n_valid = min(64, cur_len - off);
+                t.n_valid = min(BQ, cur_len - off);
                 t.lead = -1;
                 t.head = head0 + g;
-                off += 64;
+                off += BQ;
                 if (off >= cur_len) {
                     off = 0;
                     if (++d < d_end) {
@@ -183,6 +190,45 @@ struct QWalk {
         }
     }
 };
+
+// Position in a ring of N stages that runs on over a CTA's work items: the stage, and the parity of its barriers in this lap.
+template <int N>
+struct Ring {
+    int st = 0;
+    uint32_t ph = 0;
+    __device__ void next() {
+        if (++st == N) {
+            st = 0;
+            ph ^= 1;
+        }
+    }
+};
+
+// Two fp32 values at a time (one instruction on sm_100a): the element-wise passes of the backward.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_split(F2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
 
 }  // namespace attn
 }  // namespace harts

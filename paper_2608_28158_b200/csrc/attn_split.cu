@@ -26,7 +26,7 @@ __device__ __forceinline__ int warp_sum(int x) {
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(~0u, x, o);
     return x;
 }
-__device__ __forceinline__ int tiles_of(int rows) { return (rows + 63) / 64; }
+__device__ __forceinline__ int tiles_of(int rows) { return (rows + BQ - 1) / BQ; }
 
 // One CTA of 1024 threads, a warp per item.
 __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, int sms, SplitTable t) {
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) len = max(16, (int)(((long long)total * Hkv + 4 * sms - 1) / (4 * sms)));
+    if (threadIdx.x == 0) len = max(8, (int)(((long long)total * Hkv + 4 * sms - 1) / (4 * sms)));
     for (int tries = 0; tries < 20; tries++) {                // the longest unit such that the partial sums fit
         if (threadIdx.x == 0) slots = 0;
         __syncthreads();
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
             x.g = at / per_head;
             int r = at % per_head;
             x.in_own = r < own;
-            x.off = kt * 128 + r * 64;
+            x.off = kt * 128 + r * BQ;
             x.d = ix.desc_ptr[piece];
             if (!x.in_own) {
                 r -= own;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
                     if (here) {
                         const int l = __ffs(here) - 1;
                         x.d = d0 + l;
-                        x.off = (r - (__shfl_sync(~0u, sum, l) - __shfl_sync(~0u, n, l))) * 64;
+                        x.off = (r - (__shfl_sync(~0u, sum, l) - __shfl_sync(~0u, n, l))) * BQ;
                         break;
                     }
                     r -= __shfl_sync(~0u, sum, 31);
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(Index ix, int Hkv, SplitTab
 static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
     const int P = hi[1], n_items = hi[5];
     const int32_t *len = hi + hi[9], *parent = hi + hi[10], *item = hi + hi[17];
-    auto tiles = [](int rows) { return (rows + 63) / 64; };
+    auto tiles = [](int rows) { return (rows + BQ - 1) / BQ; };
     std::unique_ptr<int32_t[]> mem(new (std::nothrow) int32_t[3 * (size_t)P]());
     std::unique_ptr<int64_t[]> load(new (std::nothrow) int64_t[sms]());
     if (!mem || !load) return false;
@@ -189,12 +189,12 @@ static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
         total += t * Hkv;
         for (int h = 0; h < Hkv; h++) {
             int64_t& l = load[tier & 1 ? sms - 1 - at : at];
-            l += t + 6;
+            l += t + 4;
             most = l > most ? l : most;
             if (++at == sms) at = 0, tier++;
         }
     }
-    return most * sms * 10 >= total * 17 && (most - 240) * sms >= total;
+    return most * sms * 10 >= total * 17 && (most - 120) * sms >= total;
 }
 
 // The table and the partial sums in `buf`; false: too small a buffer, nothing to gain, or 16 items and more per SM (where the
