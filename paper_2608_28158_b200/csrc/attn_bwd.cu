@@ -11,7 +11,11 @@
 //                  S^T = K Q^T,  dP^T = V dO^T,  dV += P^T dO,  dK += dS^T Q.
 //                  The gradient of a shared ancestor's K/V is thus accumulated on chip over all its descendants and
 //                  written once: this replaces the scatter-add of the gather's backward.
-// S/dP live in two tensor-memory buffers, so the MMAs of tile n+1 run under the element-wise pass of tile n.
+// dq_kernel: S lives in two tensor-memory buffers and dP is taken into registers first, so the MMAs of tile n+1 run under the
+// element-wise pass of tile n, and the roles meet at mbarriers only, so that the loads and first products of an item run under the
+// output of the one before.  24 MMAs of 64 cycles a 128 x 128 tile (1,536); it takes 2,800 cycles, bound by the power limit on long
+// sequences (1.36 GHz).  3,970 with eleven instructions an element instead of six: scalar fp32, the scale on every dS, a test for
+// hidden columns on every element.  65,521 agentic tokens x 16 heads: 8.1 -> 6.3 ms.
 #include "kernels.h"
 #include "tc_common.cuh"
 
@@ -64,7 +68,7 @@ struct SmemQ {
     static constexpr int bytes = misc + 256;
 };
 struct MiscQ {
-    uint64_t bar_q, bar_k[KST], bar_v[2], bar_kfree[KST], bar_vfree[2], bar_s, bar_dpfree, bar_p[2], bar_o, bar_exit;
+    uint64_t bar_q, bar_qfree, bar_k[KST], bar_v[2], bar_kfree[KST], bar_s[2], bar_dpfree, bar_p[2], bar_o, bar_ofree, bar_exit;
     int dead;        // latch: a wait of this CTA ran out, the CTA is abandoning its work
     uint32_t tmem;
 };
@@ -74,7 +78,7 @@ using WalkW = TileWalkT<BKW>;
 __global__ void __launch_bounds__(NT, 1)
 attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUtensorMap map_q,
                const __grid_constant__ CUtensorMap map_do, const __grid_constant__ CUtensorMap map_k,
-               const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_dq,
+               const __grid_constant__ CUtensorMap map_v,
                const float* __restrict__ lse, const float* __restrict__ delta, __nv_bfloat16* __restrict__ dq,
                int* status) {
     extern __shared__ unsigned char smem_raw[];
@@ -83,7 +87,7 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
     unsigned char* sDO = smem + SmemQ::dO;
     MiscQ& m = *reinterpret_cast<MiscQ*>(smem + SmemQ::misc);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool is_softmax = warp < NS / 32, is_issuer = tid == NS, is_producer = tid == NS + 32;
+    const bool is_softmax = warp < NS / 32, is_issuer = warp == NS / 32, is_producer = tid == NS + 32;
     if (tid == 0) {
         mbar_init(&m.bar_q, 1);
         for (int st = 0; st < KST; st++) {
@@ -92,13 +96,14 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
         }
         for (int st = 0; st < 2; st++) {
             mbar_init(&m.bar_v[st], 1);
-            mbar_init(&m.bar_vfree[st], 1);
+            mbar_init(&m.bar_s[st], 1);
         }
-        mbar_init(&m.bar_s, 1);
         mbar_init(&m.bar_dpfree, NS / 32);
         mbar_init(&m.bar_p[0], NS / 32);
         mbar_init(&m.bar_p[1], NS / 32);
+        mbar_init(&m.bar_qfree, 1);
         mbar_init(&m.bar_o, 1);
+        mbar_init(&m.bar_ofree, NS / 32);
         mbar_init(&m.bar_exit, 1);
         m.dead = 0;
         fence_barrier_init();
@@ -109,19 +114,22 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
     tc_fence_after();
     const uint32_t tmem = m.tmem;
     const uint32_t tm_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    constexpr uint32_t I_S = instr_desc(BQ, BKW, 0, 0);    // [128 x 128] = (Q | dO) (K-major) . (K | V) (K-major)
     constexpr uint32_t I_DQ = instr_desc(BQ, D, 0, 1);     // dQ[128 x 128] += dS (tensor memory) . K (rows = keys)
     const uint64_t dQd = desc_kmajor_base(smem_u32(sQ)), dDOd = desc_kmajor_base(smem_u32(sDO));
     const float scale_log2 = scale * LOG2E;
 
-    uint32_t ph_q = 0, ph_k[KST] = {}, ph_v[2] = {0, 0}, ph_kfree[KST] = {}, ph_vfree[2] = {0, 0}, ph_s = 0, ph_p[2] = {0, 0},
-             ph_dpfree = 0, ph_o = 0;
+    // where this thread's role stands in the rings, which run on over the work items (a fresh barrier counts as free: parity 1
+    // has passed)
+    Ring<KST> rk;
+    Ring<2> r2;              // V, S and the barriers that come in twos
+    uint32_t ph_q = 0, ph_dpfree = 0, ph_o = 0;
     const int n_work = ix.n_q_items * Hq;
     // work items come most work first; dealt in a snake pattern (tier by tier, every second tier in reverse), so that no
     // CTA gets the largest item of every tier
     for (int tier = 0; tier * (int)gridDim.x < n_work; tier++) {
         const int w = tier * (int)gridDim.x + ((tier & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
         if (w >= n_work) continue;
+        if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the work
         const int item = w / Hq, h = w % Hq, hk = h / G;
         const int piece = ix.q_item[2 * item], qt = ix.q_item[2 * item + 1];
         const int q_row0 = ix.piece_row0[piece] + qt * BQ;
@@ -131,185 +139,207 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
             // ---- TMA producer: Q and dO tiles, then K and V tiles two deep (released separately) --------------------
             WalkW lw(ix, piece, qt);
             KvTile lt;
+            mbar_wait(&m.bar_qfree, ph_q ^ 1, status, &m.dead);      // the last item's S and dP products have read the tiles
+            ph_q ^= 1;
             mbar_expect_tx(&m.bar_q, 2 * Q_BYTES);
             for (int p = 0; p < 2; p++)
                 for (int r = 0; r < 2; r++) {
                     tma_load_3d(sQ + p * (Q_BYTES / 2) + r * (Q_BYTES / 4), &map_q, p * 64, h, q_row0 + r * 64, &m.bar_q);
                     tma_load_3d(sDO + p * (Q_BYTES / 2) + r * (Q_BYTES / 4), &map_do, p * 64, h, q_row0 + r * 64, &m.bar_q);
                 }
-            for (int n = 0; lw.next(lt); n++) {
+            for (; lw.next(lt); rk.next(), r2.next()) {
                 if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const int stage = n & 1, kst = n % KST;
-                unsigned char* sK = smem + SmemQ::k0 + kst * KW_BYTES;
-                unsigned char* sV = smem + SmemQ::v0 + stage * KW_BYTES;
-                if (n >= KST) {
-                    mbar_wait(&m.bar_kfree[kst], ph_kfree[kst], status, &m.dead);         // released after dQ of tile n - KST
-                    ph_kfree[kst] ^= 1;
-                }
-                mbar_expect_tx(&m.bar_k[kst], KW_BYTES);
-                for (int p = 0; p < 2; p++)
-                    for (int r = 0; r < 2; r++)
-                        tma_load_3d(sK + p * (KW_BYTES / 2) + r * (KW_BYTES / 4), &map_k, p * 64, hk, lt.row + r * 64, &m.bar_k[kst]);
-                if (n >= 2) {
-                    mbar_wait(&m.bar_vfree[stage], ph_vfree[stage], status, &m.dead);     // released after dP of tile n - 2
-                    ph_vfree[stage] ^= 1;
-                }
-                mbar_expect_tx(&m.bar_v[stage], KW_BYTES);
-                for (int p = 0; p < 2; p++)
-                    for (int r = 0; r < 2; r++)
-                        tma_load_3d(sV + p * (KW_BYTES / 2) + r * (KW_BYTES / 4), &map_v, p * 64, hk, lt.row + r * 64, &m.bar_v[stage]);
+                const int halves = lt.n_valid > 64 ? 2 : 1;      // rows past the 64th are read by nothing then
+                unsigned char* sK = smem + SmemQ::k0 + rk.st * KW_BYTES;
+                unsigned char* sV = smem + SmemQ::v0 + r2.st * KW_BYTES;
+                mbar_wait(&m.bar_kfree[rk.st], rk.ph ^ 1, status, &m.dead);      // dQ of the stage's last tile is done
+                mbar_expect_tx(&m.bar_k[rk.st], halves * (KW_BYTES / 2));
+                for (int r = 0; r < halves; r++)
+                    for (int p = 0; p < 2; p++)
+                        tma_load_3d(sK + p * (KW_BYTES / 2) + r * (KW_BYTES / 4), &map_k, p * 64, hk, lt.row + r * 64, &m.bar_k[rk.st]);
+                // S and dP of the stage's last tile are done; the next phase of this barrier needs the tile loaded here
+                mbar_wait(&m.bar_s[r2.st], r2.ph ^ 1, status, &m.dead);
+                mbar_expect_tx(&m.bar_v[r2.st], halves * (KW_BYTES / 2));
+                for (int r = 0; r < halves; r++)
+                    for (int p = 0; p < 2; p++)
+                        tma_load_3d(sV + p * (KW_BYTES / 2) + r * (KW_BYTES / 4), &map_v, p * 64, hk, lt.row + r * 64, &m.bar_v[r2.st]);
             }
         }
         if (is_issuer) {
-            // ---- MMA issue: this thread does nothing else, a tcgen05.mma holds it until the pipe has room ---------
-            const int n_tiles = WalkW(ix, piece, qt).count();
-            auto issue_s = [&](int n) {      // S(n) into buffer n & 1
-                const int stage = n & 1, kst = n % KST;
-                mbar_wait(&m.bar_k[kst], ph_k[kst], status, &m.dead);
-                ph_k[kst] ^= 1;
+            // ---- MMA issue: a tcgen05.mma holds its thread until the pipe has room, so this warp does nothing else ---------
+            // Pipe order S(n+1), dP(n+1), dQ(n): the first two run under the pass of tile n (S has a second buffer, and the pass
+            // takes dP(n) into registers first and says so).  S / dP are as wide as the tile has keys (steps of 16), dQ as deep.
+            WalkW iw(ix, piece, qt);
+            KvTile tn;
+            Ring<KST> rk0 = rk;        // stages of tile n; rk and r2: of tile n + 1
+            Ring<2> r0 = r2;
+            KvTile tl;                 // looked up one further: whether tile n + 1 is the last
+            bool more = iw.next(tn), more2 = iw.next(tl);
+            auto issue_s = [&]() {
+                mbar_wait_warp(&m.bar_k[rk.st], rk.ph, status, &m.dead);
                 tc_fence_after();
-                const uint64_t dK = desc_kmajor_base(smem_u32(smem + SmemQ::k0 + kst * KW_BYTES));
+                const uint32_t idesc = instr_desc(BQ, (tn.n_valid + 15) & ~15, 0, 0);     // (Q | dO) (K-major) . (K | V) (K-major)
+                const uint64_t dK = desc_kmajor_base(smem_u32(smem + SmemQ::k0 + rk.st * KW_BYTES));
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)
-                    mma_ss(tmem + stage * 128, dQd + kstep_kmajor<BQ>(ks), dK + kstep_kmajor<BKW>(ks), I_S, ks > 0);
+                    for (int ks = 0; ks < 8; ks++)
+                        mma_ss(tmem + r2.st * 128, dQd + kstep_kmajor<BQ>(ks), dK + kstep_kmajor<BKW>(ks), idesc, ks > 0);
+                }
+                __syncwarp();
+                rk.next();
             };
-            auto issue_dp = [&](int n) {     // dP(n); its commit also covers S(n), issued before it
-                const int stage = n & 1;
-                mbar_wait(&m.bar_v[stage], ph_v[stage], status, &m.dead);
-                ph_v[stage] ^= 1;
+            auto issue_dp = [&](bool ahead) {     // ahead: more key tiles follow; its commit also covers S, issued before it
+                mbar_wait_warp(&m.bar_v[r2.st], r2.ph, status, &m.dead);
                 tc_fence_after();
-                const uint64_t dV = desc_kmajor_base(smem_u32(smem + SmemQ::v0 + stage * KW_BYTES));
+                const uint32_t idesc = instr_desc(BQ, (tn.n_valid + 15) & ~15, 0, 0);
+                const uint64_t dV = desc_kmajor_base(smem_u32(smem + SmemQ::v0 + r2.st * KW_BYTES));
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)
-                    mma_ss(tmem + COL_DP, dDOd + kstep_kmajor<BQ>(ks), dV + kstep_kmajor<BKW>(ks), I_S, ks > 0);
-                mma_commit(&m.bar_s);
-                if (n + 2 < n_tiles) mma_commit(&m.bar_vfree[stage]);
+                    for (int ks = 0; ks < 8; ks++)
+                        mma_ss(tmem + COL_DP, dDOd + kstep_kmajor<BQ>(ks), dV + kstep_kmajor<BKW>(ks), idesc, ks > 0);
+                    mma_commit(&m.bar_s[r2.st]);
+                    if (!ahead) mma_commit(&m.bar_qfree);
+                }
+                __syncwarp();
+                r2.next();
             };
-            mbar_wait(&m.bar_q, ph_q, status, &m.dead);
+            mbar_wait_warp(&m.bar_q, ph_q, status, &m.dead);
             ph_q ^= 1;
-            issue_s(0);
-            issue_dp(0);
-            for (int n = 0; n < n_tiles; n++) {
+            issue_s();
+            issue_dp(more2);
+            mbar_wait_warp(&m.bar_ofree, ph_q, status, &m.dead);     // the last item's dQ has been read (ph_q: this item's parity, turned)
+            for (int n = 0; more; n++) {
                 if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const int stage = n & 1;
-                // S(n+1) and dP(n+1) run under the element-wise pass of tile n: S has a second buffer, and the pass
-                // takes dP(n) into registers first and says so
-                if (n + 1 < n_tiles) {
-                    issue_s(n + 1);
-                    mbar_wait(&m.bar_dpfree, ph_dpfree, status, &m.dead);
-                    ph_dpfree ^= 1;
+                const int steps = (tn.n_valid + 15) >> 4;
+                more = more2;
+                if (more) {
+                    tn = tl;
+                    more2 = iw.next(tl);
+                    issue_s();
+                }
+                mbar_wait_warp(&m.bar_dpfree, ph_dpfree, status, &m.dead);
+                ph_dpfree ^= 1;
+                if (more) {
                     tc_fence_after();
-                    issue_dp(n + 1);
+                    issue_dp(more2);
                 }
                 // dS(n) written, S(n) read.  One barrier per S buffer: a warp that is done with tile n may already work
                 // on tile n+1 (its S and dP are complete) and arrive for it, and that arrival must not count for tile n.
-                mbar_wait(&m.bar_p[stage], ph_p[stage], status, &m.dead);
-                ph_p[stage] ^= 1;
+                mbar_wait_warp(&m.bar_p[r0.st], r0.ph, status, &m.dead);
                 tc_fence_after();
-                const uint64_t dKm = desc_mnmajor_base<BKW>(smem_u32(smem + SmemQ::k0 + (n % KST) * KW_BYTES));
+                const uint64_t dKm = desc_mnmajor_base<BKW>(smem_u32(smem + SmemQ::k0 + rk0.st * KW_BYTES));
+                const uint32_t a = tmem + r0.st * 128;
+                if (elect_one()) {
+                    if (steps == 8) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)
-                    mma_ts(tmem + COL_DQ, tmem + stage * 128 + (ks >> 2) * 64 + (ks & 3) * 8, dKm + kstep_mnmajor(ks), I_DQ,
-                           n > 0 || ks > 0);
-                if (n + KST < n_tiles) mma_commit(&m.bar_kfree[n % KST]);
-                if (n + 1 == n_tiles) mma_commit(&m.bar_o);
+                        for (int ks = 0; ks < 8; ks++)
+                            mma_ts(tmem + COL_DQ, a + (ks >> 2) * 64 + (ks & 3) * 8, dKm + kstep_mnmajor(ks), I_DQ, n > 0 || ks > 0);
+                    } else {
+#pragma unroll 1
+                        for (int ks = 0; ks < steps; ks++)
+                            mma_ts(tmem + COL_DQ, a + (ks >> 2) * 64 + (ks & 3) * 8, dKm + kstep_mnmajor(ks), I_DQ, n > 0 || ks > 0);
+                    }
+                    mma_commit(&m.bar_kfree[rk0.st]);
+                    if (!more) mma_commit(&m.bar_o);
+                }
+                __syncwarp();
+                rk0.next();
+                r0.next();
             }
         }
         if (is_softmax) {
             WalkW walk(ix, piece, qt);
             KvTile t;
             const int i = tid & 127, c = tid >> 7;           // query row, and which 64 of a tile's 128 key columns
-            const bool row_ok = i < q_valid;
-            // rows past the end of the piece: lse = +inf makes every probability 0
-            const float lse2 = row_ok ? lse[(size_t)(q_row0 + i) * Hq + h] * LOG2E : INFINITY;
+            const bool row_ok = i < q_valid;                 // other rows are other pieces' queries: computed, never stored
+            const float lse2 = row_ok ? lse[(size_t)(q_row0 + i) * Hq + h] * LOG2E : 0.f;
             const float dl = row_ok ? delta[(size_t)(q_row0 + i) * Hq + h] : 0.f;
-            for (int n = 0; walk.next(t); n++) {
+            const F2 scale2 = f2(scale_log2, scale_log2), nl = f2(-lse2, -lse2), nd = f2(-dl, -dl);
+            for (; walk.next(t); r2.next()) {
                 if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const int b = n & 1;
-                mbar_wait_warp(&m.bar_s, ph_s, status, &m.dead);
-                ph_s ^= 1;
+                const uint32_t at = tm_lane + r2.st * 128 + c * 64;
+                const bool any = c * 64 < t.n_valid;      // columns past the tile's keys are read by nothing
+                mbar_wait_warp(&m.bar_s[r2.st], r2.ph, status, &m.dead);
                 tc_fence_after();
-                const int limit = min(t.n_valid, t.shift == NO_DIAG ? BKW : i - t.shift + 1);
-                // dP of this thread's 64 columns into registers, so that the buffer can take dP of the next tile
-                uint32_t xp[64];
-                tmem_ld32(tm_lane + COL_DP + c * 64, xp);
-                tmem_ld32(tm_lane + COL_DP + c * 64 + 32, xp + 32);
-                tmem_ld_wait();
-                tc_fence_before();
-                __syncwarp();
-                const bool last_tile = walk.in_own && walk.off >= walk.own_end;     // no dP follows the last tile
-                if (lane == 0 && !last_tile) mbar_arrive(&m.bar_dpfree);
-#pragma unroll
-                for (int cc = 0; cc < 2; cc++) {
-                    const int j0 = c * 64 + cc * 32;
-                    uint32_t xs[32], pk[16];
-                    tmem_ld32(tm_lane + b * 128 + j0, xs);
+                uint32_t xs[32], xp[64];
+                if (any) {      // dP of this thread's 64 columns into registers: its buffer can take the next tile
+                    tmem_ld32(tm_lane + COL_DP + c * 64, xp);
+                    tmem_ld32(tm_lane + COL_DP + c * 64 + 32, xp + 32);
+                    tmem_ld32(at, xs);
                     tmem_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        float ds[2];
-#pragma unroll
-                        for (int u = 0; u < 2; u++) {
-                            const float p = j0 + e + u < limit ? ex2(fmaf(__uint_as_float(xs[e + u]), scale_log2, -lse2)) : 0.f;
-                            ds[u] = p * (__uint_as_float(xp[cc * 32 + e + u]) - dl) * scale;
-                        }
-                        pk[e >> 1] = pack_bf16(ds[0], ds[1]);
-                    }
-                    // over this thread's own half of S (columns it has already read)
-                    tmem_st16(tm_lane + b * 128 + c * 64 + cc * 16, pk);
                 }
-                tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&m.bar_p[b]);
+                if (lane == 0) mbar_arrive(&m.bar_dpfree);
+                if (any) {
+                    const int limit = min(t.n_valid, t.shift == NO_DIAG ? BKW : i - t.shift + 1) - c * 64;     // visible: j < limit
+                    const bool masked = !__all_sync(0xffffffffu, limit >= 64);
+#pragma unroll
+                    for (int cc = 0; cc < 2; cc++) {
+                        uint32_t pk[16];
+                        if (cc) {
+                            tmem_ld32(at + 32, xs);
+                            tmem_ld_wait();
+                        }
+#pragma unroll
+                        for (int e = cc * 32; e < cc * 32 + 32; e += 2) {
+                            float p0, p1, d0, d1;
+                            f2_split(f2_fma(f2(__uint_as_float(xs[e & 31]), __uint_as_float(xs[(e & 31) + 1])), scale2, nl), p0, p1);
+                            p0 = ex2(p0);
+                            p1 = ex2(p1);
+                            if (masked) {
+                                p0 = e < limit ? p0 : 0.f;
+                                p1 = e + 1 < limit ? p1 : 0.f;
+                            }
+                            f2_split(f2_mul(f2(p0, p1), f2_add(f2(__uint_as_float(xp[e]), __uint_as_float(xp[e + 1])), nd)), d0, d1);
+                            pk[(e & 31) >> 1] = pack_bf16(d0, d1);
+                        }
+                        tmem_st16(at + cc * 16, pk);      // dS / scale, over this thread's own half of S
+                    }
+                    tmem_st_wait();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&m.bar_p[r2.st]);
             }
             // ---- epilogue: dQ -> bf16 ------------------------------------------------------------------------------
             mbar_wait_warp(&m.bar_o, ph_o, status, &m.dead);
             tc_fence_after();
-            const bool full = q_valid == BQ;
 #pragma unroll
             for (int cc = 0; cc < 2; cc++) {
                 const int c4 = c * 2 + cc;
                 uint32_t x[32];
                 tmem_ld32(tm_lane + COL_DQ + c4 * 32, x);
                 tmem_ld_wait();
+                if (cc == 1) {                 // dQ has been read: the next item's may start
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&m.bar_ofree);
+                }
 #pragma unroll
-                for (int v4 = 0; v4 < 4; v4++) {
-                    uint4 pk;
-                    pk.x = pack_bf16(__uint_as_float(x[v4 * 8 + 0]), __uint_as_float(x[v4 * 8 + 1]));
-                    pk.y = pack_bf16(__uint_as_float(x[v4 * 8 + 2]), __uint_as_float(x[v4 * 8 + 3]));
-                    pk.z = pack_bf16(__uint_as_float(x[v4 * 8 + 4]), __uint_as_float(x[v4 * 8 + 5]));
-                    pk.w = pack_bf16(__uint_as_float(x[v4 * 8 + 6]), __uint_as_float(x[v4 * 8 + 7]));
-                    const int col = c4 * 32 + v4 * 8;
-                    if (full)
-                        *reinterpret_cast<uint4*>(sQ + (col >> 6) * (Q_BYTES / 2) + sw128_chunk(i, (col & 63) >> 3)) = pk;
-                    else if (row_ok)
-                        *reinterpret_cast<uint4*>(dq + ((size_t)(q_row0 + i) * Hq + h) * D + col) = pk;
+                for (int e = 0; e < 32; e++) x[e] = __float_as_uint(__uint_as_float(x[e]) * scale);
+                if (row_ok) {
+#pragma unroll
+                    for (int v4 = 0; v4 < 4; v4++) {
+                        uint4 pk;
+                        pk.x = pack_bf16(__uint_as_float(x[v4 * 8 + 0]), __uint_as_float(x[v4 * 8 + 1]));
+                        pk.y = pack_bf16(__uint_as_float(x[v4 * 8 + 2]), __uint_as_float(x[v4 * 8 + 3]));
+                        pk.z = pack_bf16(__uint_as_float(x[v4 * 8 + 4]), __uint_as_float(x[v4 * 8 + 5]));
+                        pk.w = pack_bf16(__uint_as_float(x[v4 * 8 + 6]), __uint_as_float(x[v4 * 8 + 7]));
+                        *reinterpret_cast<uint4*>(dq + ((size_t)(q_row0 + i) * Hq + h) * D + c4 * 32 + v4 * 8) = pk;
+                    }
                 }
             }
-            if (full) fence_async_smem();
+            ph_o ^= 1;
         }
-        ph_o ^= 1;
-        tc_fence_before();
-        if (__syncthreads_or(m.dead)) break;
-        tc_fence_after();
-        if (is_issuer && q_valid == BQ) {
-            for (int p = 0; p < 2; p++)
-                for (int r = 0; r < 2; r++)
-                    tma_store_3d(&map_dq, sQ + p * (Q_BYTES / 2) + r * (Q_BYTES / 4), p * 64, h, q_row0 + r * 64);
-            tma_store_commit();
-            tma_store_wait_read();
-        }
-        __syncthreads();
     }
     if (__syncthreads_or(m.dead)) {               // abandoned: let the loads and MMAs in flight finish (bounded)
-        if (is_issuer) {
+        if (tid == NS) {
             mma_commit(&m.bar_exit);
             mbar_wait_drain(&m.bar_exit, 0);
         }
         drain_delay();
     }
-    if (is_issuer) tma_store_wait_all();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc<TMEM_Q>(tmem);
@@ -332,13 +362,12 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
     const long long n = (long long)n_rows * Hq;
     delta_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)dO,
                                                                   delta, n);
-    CUtensorMap mq, mdo, mk, mv, mdq;
+    CUtensorMap mq, mdo, mk, mv;
     int32_t rc;
     if ((rc = make_row_map(&mq, q, n_rows, Hq)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mdo, dO, n_rows, Hq)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mk, k, n_rows, Hkv)) != HARTS_OK) return rc;
     if ((rc = make_row_map(&mv, v, n_rows, Hkv)) != HARTS_OK) return rc;
-    if ((rc = make_row_map(&mdq, dq, n_rows, Hq)) != HARTS_OK) return rc;
     if (cudaFuncSetAttribute(attn_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SmemQ::bytes + 1024) !=
         cudaSuccess)
         return HARTS_ECUDA;
@@ -352,7 +381,7 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
     }
     const long long n_work = (long long)ix.n_q_items * Hq;
     const int grid = (int)(n_work < sm_count() ? n_work : sm_count());
-    attn_dq_kernel<<<grid, NT, SmemQ::bytes + 1024, st>>>(ix, Hq, Hq / Hkv, scale, mq, mdo, mk, mv, mdq, lse, delta,
+    attn_dq_kernel<<<grid, NT, SmemQ::bytes + 1024, st>>>(ix, Hq, Hq / Hkv, scale, mq, mdo, mk, mv, lse, delta,
                                                          (__nv_bfloat16*)dq, status);
     if (cudaGetLastError() != cudaSuccess) return HARTS_ECUDA;
     return cut ? HARTS_OK : attn_dkv_launch(ix, n_rows, q, k, v, lse, dO, delta, dk_, dv_, Hq, Hkv, scale, status, nullptr, st);
