@@ -35,7 +35,8 @@ namespace {
 using namespace tc;
 
 constexpr int BT = 64, D = 128;
-constexpr int GATES = 4, RAW = 8, ITEMS = 4;      // rings: weights, raw log-decays, items
+constexpr int GATES = 4, RAW = 8, ITEMS = 4, EXPORTS = 4;      // rings: weights, raw log-decays, items, slots written (the state
+                                                               // is at most OUTS = 3 tiles ahead of their stores)
 constexpr int PANEL = BT * 128, S_PANEL = D * 128;
 constexpr float LOG2E = 1.4426950408889634f;
 
@@ -62,7 +63,7 @@ struct Misc {
     float gammas[GATES][D];      // per-channel decay: e^{b_n} of every state row
     float part[2][4][D];         // and the sums of four groups of 16 rows, of every second step
     uint64_t full[5], weighted[5], stage_empty[5], u_full[2], u_empty[2], gates_full[GATES], gates_empty[GATES], out_full[3],
-        out_empty[3], item_full[ITEMS], item_empty[ITEMS], part_full[2];
+        out_empty[3], item_full[ITEMS], item_empty[ITEMS], part_full[2], exported[EXPORTS];
     Item items[ITEMS];
     int2 tile[3];            // backward: the tile (index, slice) a buffer is for
     uint32_t tmem;
@@ -109,6 +110,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             mbar_init(&m.item_full[i], 1);
             mbar_init(&m.item_empty[i], (NS + NWT) / 32 + (GK ? 2 : 3));
         }
+        for (int i = 0; i < EXPORTS; i++) mbar_init(&m.exported[i], NS / 32);
         m.dead = 0;
         fence_barrier_init();
     }
@@ -130,7 +132,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
         // ---- state: row L, columns col0 .. col0 + CW - 1 of the slice ------------------------------------------------------
         const int L = (warp & 3) * 32 + lane, col0 = (warp >> 2) * CW;
         const uint32_t tm = tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0;
-        int gs = 0, gt = 0;                   // steps and tiles since the kernel began
+        int gs = 0, gt = 0, n_exported = 0;   // steps, tiles and exports since the kernel began
         bool alive = true;
         for (int k = 0; alive && wait_warp(&m.item_full[k % ITEMS], k / ITEMS); k++) {
             const Item it = m.items[k % ITEMS];
@@ -144,7 +146,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             if (!BWD && it.init_slot >= 0) {
                 const size_t from = (size_t)it.init_slot * H + it.h;
                 const float4* src = reinterpret_cast<const float4*>(slots + from * (D * D) + in_state);
-                if (order.n) alive = flag_wait_warp(flags + from * SLICES + it.slice, NS / 32, status, &m.dead);
+                if (order.n) alive = flag_wait_warp(flags + from * SLICES + it.slice, 1, status, &m.dead);
 #pragma unroll
                 for (int e = 0; e < CW / 4; e++) *reinterpret_cast<float4*>(x + 4 * e) = __ldcg(src + e);
             }
@@ -202,7 +204,9 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     float4* dst = reinterpret_cast<float4*>(slots + to * (D * D) + in_state);
 #pragma unroll
                     for (int e = 0; e < CW / 4; e++) dst[e] = *reinterpret_cast<const float4*>(x + 4 * e);
-                    if (order.n) flag_add_warp(flags + to * SLICES + it.slice);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&m.exported[n_exported % EXPORTS]);      // the store warp publishes it: no fence in the chain
+                    n_exported++;
                     req++;
                     boundary = req < it.req_hi ? tb.slot_chunk[req] : -1;
                 }
@@ -518,10 +522,12 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             }
             tma_store_wait_all();
         } else if (lane == 0) {
+            int n_exported = 0;
             for (int k = 0; alive && wait(&m.item_full[k % ITEMS], k / ITEMS); k++) {
                 const Item it = m.items[k % ITEMS];
                 mbar_arrive(&m.item_empty[k % ITEMS]);
                 if (it.seq < 0) break;
+                int req = it.req_lo, boundary = req < it.req_hi ? tb.slot_chunk[req] : -1;
                 for (int i = 0; i < it.n_chunks; i++, gt++) {
                     if (!(alive = wait(&m.out_full[gt % OUTS], gt / OUTS))) break;
                     const int idx = (it.chunk_base + chunk_of(it, i)) * H + it.h;
@@ -530,6 +536,13 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     tma_store_commit();
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");      // the tile before this one has left its buffer
                     if (gt > 0) mbar_arrive(&m.out_empty[(gt - 1) % OUTS]);
+                    if (boundary == i) {          // the state warps have written this boundary's slot: tell the sequences that wait
+                        if (!(alive = wait(&m.exported[n_exported % EXPORTS], n_exported / EXPORTS))) break;
+                        n_exported++;
+                        if (order.n) flag_set(flags + ((size_t)req * H + it.h) * SLICES + it.slice);
+                        req++;
+                        boundary = req < it.req_hi ? tb.slot_chunk[req] : -1;
+                    }
                 }
             }
             tma_store_wait_all();

@@ -139,10 +139,10 @@ __device__ __forceinline__ bool flag_wait(const int* flag, int* status, volatile
     return false;
 }
 
-// Counting form for producers that finish warp by warp: a (converged) warp adds one once its lanes' data is written; the
-// consumer warp waits until `target` warps have (its first lane acquires, the warp barrier hands that on to the others).
+// Counting form for producers that finish warp by warp: a (converged) warp adds one once its lanes' data is written -- the warp
+// barrier orders the lanes' writes before the first lane's release, which is cumulative: no fence per lane -- and the consumer
+// warp waits until `target` warps have (its first lane acquires, the warp barrier hands that on to the others).
 __device__ __forceinline__ void flag_add_warp(int* flag) {
-    __threadfence();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(flag) : "memory");
 }
