@@ -1,0 +1,36 @@
+"""Fans of short branches through the chunk-parallel path: both sides of its line, and slots exported by one chunk after another."""
+import pytest
+import torch
+
+import paper_2608_28158_b200 as H
+from parity_util import compare, oracle_subset, run_gpu
+from test_gpu_parity import check
+from workloads import make_forest, make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads", [16, 17])
+def test_both_sides_of_the_line_of_fans(heads):
+    """32 sequences of fewer than four chunks: 512 (sequence, head) pairs take the chunk-parallel path, 544 the walk."""
+    fo = make_forest([([-1] + [0] * 31, [0] + [1 + 4 * i for i in range(31)], [130] + [2 * i + 1 for i in range(31)])])
+    inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 13, device="cuda")
+    plan, out = run_gpu(fo, inp)
+    assert plan.n_seq == 32 and plan.n_chunks < 4 * plan.n_seq
+    tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1])
+    check(compare(out, tok, [0, heads - 1], ref, rows=True), "bf16")
+    _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
+    for n in out:
+        assert torch.equal(out[n], rounds[n]), n
+
+
+@pytest.mark.parametrize("heads", [1, 40, 80])
+def test_a_slot_from_every_chunk(heads):
+    """Forks in each of 24 consecutive chunks (32, 64 and 128 columns of state at a time): slots are published in turn."""
+    n = 24
+    fo = make_forest([([-1] + [0] * n, [0] + [64 * i + 65 for i in range(n)], [64 * n + 70] + [5] * n)])
+    inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 17, device="cuda")
+    plan, out = run_gpu(fo, inp)
+    assert plan.n_slots >= n - 1
+    tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1] if heads > 1 else [0])
+    check(compare(out, tok, [0, heads - 1] if heads > 1 else [0], ref, rows=True), "bf16")
