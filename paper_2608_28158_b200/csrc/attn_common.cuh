@@ -96,7 +96,7 @@ using TileWalk = TileWalkT<BK>;
 // dK / dV work of small problems, cut into units (attn_split.cu): a unit is a run of the query tiles of one key tile, in the
 // order of QWalk; slot: where its partial sums go, -1: the item is not cut.
 struct DkvUnit {
-    int piece, kt, n_tiles, slot, g, in_own, off, d;
+    int piece, kt, n_tiles, slot, g, row, end, lead, d;
 };
 struct SplitItem {
     int n_tiles, n_units, first_unit, first_slot;
@@ -109,86 +109,44 @@ struct SplitTable {
     int cap_slots;
 };
 
-// The query tiles (128 rows) that see the key tile `kt` (128 rows) of a piece: for every query head of the group,
-// the rest of the piece from the key tile's first row on (causal inside), then all rows of every descendant piece.
-// Key row i is seen by query column j iff jmin(i) <= j < n_valid, with jmin(i) = max(0, i - lead) for own tiles
-// (lead = first query row of the tile minus first key row of the key tile) and 0 for descendants.
-struct QTile {
-    int row, n_valid, lead, head;       // lead < 0: descendant piece (no diagonal)
-};
-struct QWalk {
+// The query rows that see the key tile `kt` (128 rows) of a piece, as runs [row, end) of physical rows: the rest of the piece from
+// the key tile's first row on (causal inside), then all rows of every descendant piece.  Descendants that follow each other in
+// memory make one run -- they all see the whole key tile -- and so does the first of them with the piece's own rest: fans of short
+// branches fill their query tiles (17,111 replay tokens x 16 heads, two to a key head: dK / dV 3.0 ms piece by piece, 0.82 so; 1,773
+// agentic x 32 heads 145 -> 79 us).  Used by a whole warp.
+// Key row i is seen by row lead + j of the first run iff i <= lead + j; lead < 0: a run without a diagonal.
+struct QRuns {
     const Index& ix;
-    int piece, k0, own_len, own_row0, G, head0, g, off, d, d_end, cur_len, cur_row0;
-    int left = 0x7fffffff;              // tiles still to deliver (a unit of a cut item)
-    bool in_own;
-    __device__ QWalk(const Index& ix_, int piece_, int kt, int hk, int G_) : ix(ix_), piece(piece_), G(G_) {
-        k0 = kt * BQ;
-        own_len = ix.piece_len[piece];
-        own_row0 = ix.piece_row0[piece];
-        head0 = hk * G;
+    int piece, k0, d, d_end, row, end, lead, lane;
+    __device__ QRuns(const Index& ix_, int piece_, int kt) : ix(ix_), piece(piece_), k0(kt * BQ), lane(threadIdx.x & 31) {
         d_end = ix.desc_ptr[piece + 1];
-        start_head(0);
     }
-    __device__ void start_at(const DkvUnit& u) {
-        g = u.g;
-        in_own = u.in_own;
-        off = u.off;
-        d = u.d;
-        left = u.n_tiles;
-        if (!in_own && d < d_end) {
-            cur_len = ix.piece_len[ix.desc_piece[d]];
-            cur_row0 = ix.piece_row0[ix.desc_piece[d]];
-        }
-    }
-    __device__ void start_head(int g_) {
-        g = g_;
-        in_own = true;
-        off = k0;
-        d = ix.desc_ptr[piece];
-    }
-    __device__ int count() const {
-        int n = (own_len - k0 + BQ - 1) / BQ;
-        for (int e = ix.desc_ptr[piece]; e < d_end; e++) n += (ix.piece_len[ix.desc_piece[e]] + BQ - 1) / BQ;
-        return n * G;
-    }
-    __device__ bool next(QTile& t) {
-        if (left-- <= 0) return false;
+    __device__ void extend(int last) {          // the run's end: behind piece `last` and those that follow it, d: the next one
         while (true) {
-            if (g >= G) return false;
-            if (in_own) {
-                if (off < own_len) {
-                    t.row = own_row0 + off;
-                    t.n_valid = min(BQ, own_len - off);
-                    t.lead = off - k0;
-                    t.head = head0 + g;
-                    off += BQ;
-                    return true;
-                }
-                in_own = false;
-                off = 0;
-                if (d < d_end) {
-                    cur_len = ix.piece_len[ix.desc_piece[d]];
-                    cur_row0 = ix.piece_row0[ix.desc_piece[d]];
-                }
-            }
-            if (d < d_end) {
-                t.row = cur_row0 + off;
-                t.n_valid = min(BQ, cur_len - off);
-                t.lead = -1;
-                t.head = head0 + g;
-                off += BQ;
-                if (off >= cur_len) {
-                    off = 0;
-                    if (++d < d_end) {
-                        cur_len = ix.piece_len[ix.desc_piece[d]];
-                        cur_row0 = ix.piece_row0[ix.desc_piece[d]];
-                    }
-                }
-                return true;
-            }
-            start_head(g + 1);
+            const bool follows = d + lane < d_end && ix.desc_piece[d + lane] == last + 1 + lane;
+            const unsigned m = __ballot_sync(0xffffffffu, follows);
+            const int k = m == 0xffffffffu ? 32 : __ffs(~m) - 1;
+            last += k;
+            d += k;
+            if (k < 32) break;
         }
+        end = ix.piece_row0[last] + ix.piece_len[last];
     }
+    __device__ void first() {
+        d = ix.desc_ptr[piece];
+        row = ix.piece_row0[piece] + k0;
+        lead = 0;
+        extend(piece);
+    }
+    __device__ bool next() {
+        if (d >= d_end) return false;
+        const int p = ix.desc_piece[d++];
+        row = ix.piece_row0[p];
+        lead = -1;
+        extend(p);
+        return true;
+    }
+    __device__ int tiles() const { return (end - row + BQ - 1) / BQ; }
 };
 
 // Position in a ring of N stages that runs on over a CTA's work items: the stage, and the parity of its barriers in this lap.

@@ -3,8 +3,8 @@
 //
 // One work item = (piece, tile of 128 key rows, kv head).  Key rows sit on the tensor-memory lanes; the CTA keeps the
 // K and V tiles in shared memory and streams every query tile (128 rows) that sees them: the rest of the key tile's
-// own piece (causal inside the tile, Eq. 22), then all rows of all descendant pieces, for each query head of the GQA
-// group.  Per query tile:
+// own piece (causal inside the tile, Eq. 22) and all rows of all descendant pieces, whatever follows each other in memory as one
+// run (QRuns; one warp walks them and tells the others, tile by tile), for each query head of the GQA group.  Per query tile:
 //     S^T = K Q^T,  dP^T = V dO^T            operands in shared memory, results in tensor memory
 //     P^T = exp2(S^T - lse_q),  dS^T = P^T (dP^T - delta_q)     one key row per thread; bf16 back over S^T / dP^T
 //     dV += P^T dO,  dK += dS^T Q            A operand from tensor memory, Q / dO tiles read row-major as B
@@ -31,24 +31,26 @@ namespace {
 using namespace tc;
 using namespace attn;
 
-constexpr int NS = 256, NT = NS + 96;     // 8 element-wise warps: warp w and w + 4 share a lane quarter and split the columns
+constexpr int NS = 256, NT = NS + 128;    // 8 element-wise warps: warp w and w + 4 share a lane quarter and split the columns
 constexpr int BKV = 128;
 constexpr int TILE = BQ * D * 2;          // 32 KB: two panels [128 rows][64 columns]
-constexpr int QST = 3, DST = 2, VST = 2;  // stages: Q (held from S^T to dK), dO (from dP^T to dV), vectors
+constexpr int QST = 3, DST = 2, VST = 2, TST = 4;  // stages: Q (held from S^T to dK), dO (from dP^T to dV), vectors, tile records
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr int COL_S = 0, COL_DP = 128, COL_DV = 256, COL_DK = 384, TMEM_COLS = 512;
 
 struct Smem {
     static constexpr int k = 0, v = TILE, q0 = 2 * TILE, do0 = q0 + QST * TILE, vec = do0 + DST * TILE, misc = vec + VST * 2 * BQ * 4;
-    static constexpr int bytes = misc + 256;
+    static constexpr int bytes = misc + 384;
 };
 struct Misc {
-    uint64_t bar_kv, bar_kvfree, bar_q[QST], bar_do[DST], bar_vec[VST], bar_vfree[VST], bar_s, bar_dp, bar_p, bar_ds, bar_o,
+    uint64_t bar_kv, bar_kvfree, bar_q[QST], bar_do[DST], bar_vec[VST], bar_vfree[VST], bar_tile[TST], bar_tfree[TST], bar_s, bar_dp, bar_p, bar_ds, bar_o,
         bar_ofree, bar_exit;
+    int4 tile[TST];  // {first row, rows, lead, 2 head + 1 if it is the item's last}: what the walker tells the other roles
+    int4 vinfo[VST]; // the same, beside a tile's vectors
     int dead;        // latch: a wait of this CTA ran out, the CTA is abandoning its work
     uint32_t tmem;
 };
-static_assert(sizeof(Misc) <= 256, "barriers");
+static_assert(sizeof(Misc) <= 384, "barriers");
 
 // SPLIT: the work is the unit list of attn_split.cu, and a unit of a cut item leaves fp32 sums.
 template <bool SPLIT>
@@ -64,7 +66,8 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
     float* sVec = reinterpret_cast<float*>(smem + Smem::vec);       // [stage][-lse (log2 units) | -delta][128]
     Misc& m = *reinterpret_cast<Misc*>(smem + Smem::misc);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool is_softmax = warp < NS / 32, is_issuer = warp == NS / 32, is_producer = tid == NS + 32, is_loader = warp == NS / 32 + 2;
+    const bool is_softmax = warp < NS / 32, is_issuer = warp == NS / 32, is_producer = tid == NS + 32, is_loader = warp == NS / 32 + 2,
+               is_walker = warp == NS / 32 + 3;
     if (smem_u32(smem) & 1023) {              // never on sm_100a; the swizzled tiles would be misread
         if (tid == 0 && status) atomicExch(status, STATUS_TIMEOUT);
         return;
@@ -74,6 +77,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         for (int s = 0; s < QST; s++) mbar_init(&m.bar_q[s], 1);
         for (int s = 0; s < DST; s++) mbar_init(&m.bar_do[s], 1);
         for (int s = 0; s < VST; s++) { mbar_init(&m.bar_vec[s], 32); mbar_init(&m.bar_vfree[s], NS / 32); }
+        for (int s = 0; s < TST; s++) { mbar_init(&m.bar_tile[s], 1); mbar_init(&m.bar_tfree[s], 3); }
         mbar_init(&m.bar_s, 1);
         mbar_init(&m.bar_dp, 1);
         mbar_init(&m.bar_p, NS / 32);
@@ -99,6 +103,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
     Ring<QST> rq;
     Ring<DST> rd;
     Ring<VST> rv;
+    Ring<TST> rt;
     uint32_t ph_kv = 0, ph_s = 0, ph_dp = 0, ph_p = 0, ph_ds = 0, ph_o = 0;
     const int n_work = (SPLIT ? split.n_units[0] : ix.n_kv_items) * Hkv;
     // work items come most work first; dealt in a snake pattern (tier by tier, every second tier in reverse), so that no
@@ -117,9 +122,6 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
 
         if (is_producer) {
             // ---- TMA producer: the K and V tiles, then the query / dO tiles STAGES deep -----------------------------
-            QWalk lw(ix, piece, kt, hk, G);
-            if (SPLIT) lw.start_at(unit);
-            QTile lt;
             mbar_wait(&m.bar_kvfree, ph_kv ^ 1, status, &m.dead);    // the last item's S^T and dP^T products have read the tiles
             ph_kv ^= 1;
             mbar_expect_tx(&m.bar_kv, 2 * TILE);
@@ -128,9 +130,12 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
                     tma_load_3d(sK + p * (TILE / 2) + r * (TILE / 4), &map_k, p * 64, hk, kv_row0 + r * 64, &m.bar_kv);
                     tma_load_3d(sV + p * (TILE / 2) + r * (TILE / 4), &map_v, p * 64, hk, kv_row0 + r * 64, &m.bar_kv);
                 }
-            for (; lw.next(lt); rq.next(), rd.next()) {
-                if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const int halves = lt.n_valid > 64 ? 2 : 1;      // rows past the 64th are read by nothing then
+            for (int4 t{}; !(t.w & 1); rq.next(), rd.next()) {
+                if (!mbar_wait(&m.bar_tile[rt.st], rt.ph, status, &m.dead)) break;       // a wait ran out: abandon the item
+                t = m.tile[rt.st];
+                mbar_arrive(&m.bar_tfree[rt.st]);
+                rt.next();
+                const int halves = t.y > 64 ? 2 : 1;      // rows past the 64th are read by nothing then
                 // S^T of the tile before (over all items) done: so are dK of three tiles ago and dV of two tiles ago, issued before
                 // it, which read these stages last.  The tile is not needed before that tile's dV, 1,500 cycles later.  (Every phase
                 // is waited for, and the next cannot complete before: parity is enough.)
@@ -141,29 +146,63 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
                 mbar_expect_tx(&m.bar_q[rq.st], halves * (TILE / 2));
                 for (int r = 0; r < halves; r++)
                     for (int p = 0; p < 2; p++)
-                        tma_load_3d(sQ + p * (TILE / 2) + r * (TILE / 4), &map_q, p * 64, lt.head, lt.row + r * 64, &m.bar_q[rq.st]);
+                        tma_load_3d(sQ + p * (TILE / 2) + r * (TILE / 4), &map_q, p * 64, t.w >> 1, t.x + r * 64, &m.bar_q[rq.st]);
                 mbar_expect_tx(&m.bar_do[rd.st], halves * (TILE / 2));
                 for (int r = 0; r < halves; r++)
                     for (int p = 0; p < 2; p++)
-                        tma_load_3d(sDO + p * (TILE / 2) + r * (TILE / 4), &map_do, p * 64, lt.head, lt.row + r * 64, &m.bar_do[rd.st]);
+                        tma_load_3d(sDO + p * (TILE / 2) + r * (TILE / 4), &map_do, p * 64, t.w >> 1, t.x + r * 64, &m.bar_do[rd.st]);
+            }
+        }
+        if (is_walker) {
+            // ---- the query tiles of this item, in order, TST ahead of the slowest role that uses them ---------------------
+            QRuns r(ix, piece, kt);
+            int g = 0, left = 0x7fffffff;
+            if (SPLIT) {
+                g = unit.g;
+                left = unit.n_tiles;
+                r.row = unit.row;
+                r.end = unit.end;
+                r.lead = unit.lead;
+                r.d = unit.d;
+            } else {
+                r.first();
+            }
+            for (bool more = true; more; rt.next()) {
+                int4 t = make_int4(r.row, min(BQ, r.end - r.row), r.lead, 2 * (hk * G + g));
+                r.row += BQ;
+                if (r.lead >= 0) r.lead += BQ;
+                if (--left == 0) more = false;
+                if (more && r.row >= r.end && !r.next()) {
+                    more = ++g < G;
+                    if (more) r.first();
+                }
+                t.w |= !more;
+                if (!mbar_wait_warp(&m.bar_tfree[rt.st], rt.ph ^ 1, status, &m.dead)) break;       // a wait ran out: abandon the item
+                if (lane == 0) {
+                    m.tile[rt.st] = t;
+                    mbar_arrive(&m.bar_tile[rt.st]);
+                }
+                __syncwarp();
             }
         }
         if (is_loader) {
             // ---- per-column -lse (log2 units) and -delta of the query tiles, in flight while the ring is full -----------
-            QWalk lw(ix, piece, kt, hk, G);
-            if (SPLIT) lw.start_at(unit);
-            QTile lt;
-            for (; lw.next(lt); rv.next()) {
-                if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
+            for (int4 t{}; !(t.w & 1); rv.next()) {
+                if (!mbar_wait_warp(&m.bar_tile[rt.st], rt.ph, status, &m.dead)) break;  // a wait ran out: abandon the item
+                t = m.tile[rt.st];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&m.bar_tfree[rt.st]);
+                rt.next();
                 float l4[4], d4[4];
 #pragma unroll
                 for (int e = 0; e < 4; e++) {
                     const int j = lane + e * 32;
-                    const size_t at = (size_t)(lt.row + j) * Hq + lt.head;
-                    l4[e] = j < lt.n_valid ? -lse[at] * LOG2E : -INFINITY;     // columns past the end: probability 0
-                    d4[e] = j < lt.n_valid ? -delta[at] : 0.f;
+                    const size_t at = (size_t)(t.x + j) * Hq + (t.w >> 1);
+                    l4[e] = j < t.y ? -lse[at] * LOG2E : -INFINITY;     // columns past the end: probability 0
+                    d4[e] = j < t.y ? -delta[at] : 0.f;
                 }
                 mbar_wait_warp(&m.bar_vfree[rv.st], rv.ph ^ 1, status, &m.dead);
+                if (lane == 0) m.vinfo[rv.st] = t;
                 float* to = sVec + rv.st * 2 * BQ + lane;
 #pragma unroll
                 for (int e = 0; e < 4; e++) {
@@ -177,17 +216,21 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
             // ---- MMA issue: a tcgen05.mma holds its thread until the pipe has room, so this warp does nothing else ---------
             // Pipe order dV(n), S^T(n+1), dK(n), dP^T(n+1): P of tile n+1 is made under the last two, dS of tile n under the
             // first two.  S^T / dP^T are as wide as the tile has queries (steps of 16), dV / dK as deep.
-            QWalk iw(ix, piece, kt, hk, G);
-            if (SPLIT) iw.start_at(unit);
-            QTile tn;
+            int4 tn{};                 // tile n + 1
+            auto read_tile = [&]() {
+                const bool ok = mbar_wait_warp(&m.bar_tile[rt.st], rt.ph, status, &m.dead);
+                tn = m.tile[rt.st];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&m.bar_tfree[rt.st]);
+                rt.next();
+                return ok;
+            };
             Ring<QST> rq0 = rq;        // stages of tile n; rq and rd: of tile n + 1
             Ring<DST> rd0 = rd;
-            QTile tl;                  // looked up one further: whether tile n + 1 is the last
-            bool more = iw.next(tn), more2 = iw.next(tl);
             auto issue_s = [&]() {
                 mbar_wait_warp(&m.bar_q[rq.st], rq.ph, status, &m.dead);
                 tc_fence_after();
-                const uint32_t idesc = instr_desc(BKV, (tn.n_valid + 15) & ~15, 0, 0);
+                const uint32_t idesc = instr_desc(BKV, (tn.y + 15) & ~15, 0, 0);
                 const uint64_t dQ = desc_kmajor_base(smem_u32(smem + Smem::q0 + rq.st * TILE));
                 if (elect_one()) {
 #pragma unroll
@@ -200,13 +243,13 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
             auto issue_dp = [&]() {
                 mbar_wait_warp(&m.bar_do[rd.st], rd.ph, status, &m.dead);
                 tc_fence_after();
-                const uint32_t idesc = instr_desc(BKV, (tn.n_valid + 15) & ~15, 0, 0);
+                const uint32_t idesc = instr_desc(BKV, (tn.y + 15) & ~15, 0, 0);
                 const uint64_t dDO = desc_kmajor_base(smem_u32(smem + Smem::do0 + rd.st * TILE));
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < 8; ks++) mma_ss(tmem + COL_DP, dVd + kstep_kmajor<BKV>(ks), dDO + kstep_kmajor<BQ>(ks), idesc, ks > 0);
                     mma_commit(&m.bar_dp);
-                    if (!more2) mma_commit(&m.bar_kvfree);
+                    if (tn.w & 1) mma_commit(&m.bar_kvfree);
                 }
                 __syncwarp();
                 rd.next();
@@ -226,15 +269,15 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
             };
             mbar_wait_warp(&m.bar_kv, ph_kv, status, &m.dead);
             ph_kv ^= 1;
+            bool more = read_tile();
             issue_s();
             issue_dp();
             mbar_wait_warp(&m.bar_ofree, ph_kv, status, &m.dead);    // the last item's sums have been read (ph_kv: this item's parity, turned)
             for (int n = 0; more; n++) {
                 if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const int steps = (tn.n_valid + 15) >> 4;
-                more = more2;
-                tn = tl;
-                if (more) more2 = iw.next(tl);
+                const int steps = (tn.y + 15) >> 4;
+                more = !(tn.w & 1);
+                if (more) read_tile();
                 mbar_wait_warp(&m.bar_p, ph_p, status, &m.dead);
                 ph_p ^= 1;
                 tc_fence_after();
@@ -252,22 +295,20 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
             __syncwarp();
         }
         if (is_softmax) {
-            QWalk walk(ix, piece, kt, hk, G);
-            if (SPLIT) walk.start_at(unit);
-            QTile t;
             const int i = tid & 127, c = tid >> 7;             // key row inside the tile, and which 64 of the 128 query columns
             const F2 scale2 = f2(scale_log2, scale_log2);
-            for (; walk.next(t); rv.next()) {
-                if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the item
-                const bool any = c * 64 < t.n_valid;      // columns past the tile's queries are read by nothing
+            for (bool more = true; more; rv.next()) {
+                if (!mbar_wait_warp(&m.bar_vec[rv.st], rv.ph, status, &m.dead)) break;   // a wait ran out: abandon the item
+                const int4 t = m.vinfo[rv.st];
+                more = !(t.w & 1);
+                const bool any = c * 64 < t.y;      // columns past the tile's queries are read by nothing
                 // query column j of an own tile sees key row i iff j >= i - lead; only warps on the diagonal have hidden ones.
                 // Key rows past the end of the piece are other pieces' rows: computed, never stored.
-                const bool masked = t.lead >= 0 && (warp & 3) * 32 + 31 - t.lead > c * 64;
-                const int jmin = i - t.lead - c * 64;
+                const bool masked = t.z >= 0 && (warp & 3) * 32 + 31 - t.z > c * 64;
+                const int jmin = i - t.z - c * 64;
                 const float* vl = sVec + rv.st * 2 * BQ + c * 64;
                 F2 p[32];
                 // ---- P^T = exp2(S^T - lse), bf16 over this warp's half of S^T (the other warp may still read its half) ------
-                mbar_wait_warp(&m.bar_vec[rv.st], rv.ph, status, &m.dead);
                 mbar_wait_warp(&m.bar_s, ph_s, status, &m.dead);
                 ph_s ^= 1;
                 tc_fence_after();

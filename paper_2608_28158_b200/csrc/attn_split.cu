@@ -21,13 +21,6 @@ namespace {
 
 using namespace attn;
 
-__device__ __forceinline__ int warp_sum(int x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(~0u, x, o);
-    return x;
-}
-__device__ __forceinline__ int tiles_of(int rows) { return (rows + BQ - 1) / BQ; }
-
 // One CTA of 1024 threads, a warp per item.
 __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, int sms, SplitTable t) {
     __shared__ int total, slots, len;
@@ -35,10 +28,11 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
     if (threadIdx.x == 0) total = 0;
     __syncthreads();
     for (int i = warp; i < ix.n_kv_items; i += 32) {          // tiles of every item
-        const int piece = ix.kv_item[2 * i], kt = ix.kv_item[2 * i + 1];
-        int n = 0;
-        for (int d = ix.desc_ptr[piece] + lane; d < ix.desc_ptr[piece + 1]; d += 32) n += tiles_of(ix.piece_len[ix.desc_piece[d]]);
-        n = (warp_sum(n) + tiles_of(ix.piece_len[piece] - kt * 128)) * G;
+        QRuns r(ix, ix.kv_item[2 * i], ix.kv_item[2 * i + 1]);
+        r.first();
+        int n = r.tiles();
+        while (r.next()) n += r.tiles();
+        n *= G;
         if (lane == 0) {
             t.item[i].n_tiles = n;
             atomicAdd(&total, n);
@@ -88,40 +82,22 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
     __syncthreads();
     for (int i = warp; i < ix.n_kv_items; i += 32) {          // where every unit begins
         const SplitItem it = t.item[i];
-        const int piece = ix.kv_item[2 * i], kt = ix.kv_item[2 * i + 1], own = tiles_of(ix.piece_len[piece] - kt * 128);
         const int per_head = it.n_tiles / G, step = (it.n_tiles + it.n_units - 1) / it.n_units;
         for (int u = 0; u < it.n_units; u++) {
             DkvUnit x;
-            x.piece = piece;
-            x.kt = kt;
+            x.piece = ix.kv_item[2 * i];
+            x.kt = ix.kv_item[2 * i + 1];
             x.n_tiles = max(0, min(step, it.n_tiles - u * step));
             x.slot = it.n_units > 1 ? it.first_slot + u : -1;
             const int at = min(u * step, it.n_tiles - 1);
             x.g = at / per_head;
-            int r = at % per_head;
-            x.in_own = r < own;
-            x.off = kt * 128 + r * BQ;
-            x.d = ix.desc_ptr[piece];
-            if (!x.in_own) {
-                r -= own;
-                for (int d0 = x.d; d0 < ix.desc_ptr[piece + 1]; d0 += 32) {
-                    const int d = d0 + lane, n = d < ix.desc_ptr[piece + 1] ? tiles_of(ix.piece_len[ix.desc_piece[d]]) : 0;
-                    int sum = n;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(~0u, sum, o);
-                        if (lane >= o) sum += y;
-                    }
-                    const unsigned here = __ballot_sync(~0u, r < sum);
-                    if (here) {
-                        const int l = __ffs(here) - 1;
-                        x.d = d0 + l;
-                        x.off = (r - (__shfl_sync(~0u, sum, l) - __shfl_sync(~0u, n, l))) * BQ;
-                        break;
-                    }
-                    r -= __shfl_sync(~0u, sum, 31);
-                }
-            }
+            int skip = at % per_head;
+            QRuns r(ix, x.piece, x.kt);
+            for (r.first(); skip >= r.tiles(); r.next()) skip -= r.tiles();
+            x.row = r.row + skip * BQ;
+            x.end = r.end;
+            x.lead = r.lead < 0 ? -1 : skip * BQ;
+            x.d = r.d;
             if (lane == 0) t.unit[it.first_unit + u] = x;
         }
     }
@@ -171,7 +147,7 @@ static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
     std::unique_ptr<int32_t[]> mem(new (std::nothrow) int32_t[3 * (size_t)P]());
     std::unique_ptr<int64_t[]> load(new (std::nothrow) int64_t[sms]());
     if (!mem || !load) return false;
-    int32_t *below = mem.get(), *kids = below + P, *todo = kids + P, n = 0;     // below: query tiles of all descendants
+    int32_t *below = mem.get(), *kids = below + P, *todo = kids + P, n = 0;     // below: rows of all descendants
     for (int p = 0; p < P; p++)
         if (parent[p] >= 0) kids[parent[p]]++;
     for (int p = 0; p < P; p++)
@@ -179,13 +155,13 @@ static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
     while (n) {
         const int p = todo[--n], a = parent[p];
         if (a < 0) continue;
-        below[a] += below[p] + tiles(len[p]);
+        below[a] += below[p] + len[p];
         if (--kids[a] == 0) todo[n++] = a;
     }
     int64_t total = 0, most = 0;
     for (int i = 0, at = 0, tier = 0; i < n_items; i++) {
         const int piece = item[2 * i];
-        const int64_t t = (int64_t)G * (below[piece] + tiles(len[piece] - item[2 * i + 1] * 128));
+        const int64_t t = (int64_t)G * tiles(below[piece] + len[piece] - item[2 * i + 1] * 128);
         total += t * Hkv;
         for (int h = 0; h < Hkv; h++) {
             int64_t& l = load[tier & 1 ? sms - 1 - at : at];
