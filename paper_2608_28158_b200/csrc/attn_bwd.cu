@@ -38,7 +38,8 @@ constexpr float LOG2E = 1.4426950408889634f;
 
 __global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16* __restrict__ o,
                                                     const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
-                                                    long long n) {       // n = rows * Hq; one warp per (row, head)
+                                                    long long n, int* ticket) {       // n = rows * Hq; one warp per (row, head)
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;       // of attn_dkv_kernel
     const long long w = (blockIdx.x * 256LL + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= n) return;
@@ -349,7 +350,7 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
 
 int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* k, const void* v, const float* lse,
                         const void* dO, const float* delta, void* dk_, void* dv_, int Hq, int Hkv, float scale,
-                        int32_t* status, const SplitTable* split, cudaStream_t st);
+                        int* ticket, int32_t* status, const SplitTable* split, cudaStream_t st);
 bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* buf, size_t bytes, SplitTable* t);
 int32_t attn_split_launch(const Index& ix, int G, int Hkv, const SplitTable& t, cudaStream_t st);
 int32_t attn_split_reduce(const Index& ix, int Hkv, const SplitTable& t, void* dk_, void* dv_, cudaStream_t st);
@@ -360,8 +361,9 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
     const int n_rows = hi[0];
     if (n_rows == 0 || hi[4] == 0) return HARTS_OK;
     const long long n = (long long)n_rows * Hq;
-    delta_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)dO,
-                                                                  delta, n);
+    // the dK / dV kernel runs first: its work counter and, on skewed problems, its units and their sums lie in dq's memory
+    int* ticket = static_cast<int*>(dq) + 1;
+    delta_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)dO, delta, n, ticket);
     CUtensorMap mq, mdo, mk, mv;
     int32_t rc;
     if ((rc = make_row_map(&mq, q, n_rows, Hq)) != HARTS_OK) return rc;
@@ -374,17 +376,15 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
     const Index ix = make_index(hi, di);
     SplitTable split;
     const bool cut = attn_split_table(ix, hi, Hq / Hkv, Hkv, dq, (size_t)n_rows * Hq * D * 2, &split);
-    if (cut) {        // small, skewed problems: the units' partial sums use dq's memory before dq is computed
-        if ((rc = attn_split_launch(ix, Hq / Hkv, Hkv, split, st)) != HARTS_OK) return rc;
-        if ((rc = attn_dkv_launch(ix, n_rows, q, k, v, lse, dO, delta, dk_, dv_, Hq, Hkv, scale, status, &split, st)) != HARTS_OK) return rc;
-        if ((rc = attn_split_reduce(ix, Hkv, split, dk_, dv_, st)) != HARTS_OK) return rc;
-    }
+    if (cut && (rc = attn_split_launch(ix, Hq / Hkv, Hkv, split, st)) != HARTS_OK) return rc;
+    if ((rc = attn_dkv_launch(ix, n_rows, q, k, v, lse, dO, delta, dk_, dv_, Hq, Hkv, scale, ticket, status, cut ? &split : nullptr, st)) != HARTS_OK)
+        return rc;
+    if (cut && (rc = attn_split_reduce(ix, Hkv, split, dk_, dv_, st)) != HARTS_OK) return rc;
     const long long n_work = (long long)ix.n_q_items * Hq;
     const int grid = (int)(n_work < sm_count() ? n_work : sm_count());
     attn_dq_kernel<<<grid, NT, SmemQ::bytes + 1024, st>>>(ix, Hq, Hq / Hkv, scale, mq, mdo, mk, mv, lse, delta,
                                                          (__nv_bfloat16*)dq, status);
-    if (cudaGetLastError() != cudaSuccess) return HARTS_ECUDA;
-    return cut ? HARTS_OK : attn_dkv_launch(ix, n_rows, q, k, v, lse, dO, delta, dk_, dv_, Hq, Hkv, scale, status, nullptr, st);
+    return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
 }  // namespace harts

@@ -34,7 +34,7 @@ using namespace attn;
 constexpr int NS = 256, NT = NS + 128;    // 8 element-wise warps: warp w and w + 4 share a lane quarter and split the columns
 constexpr int BKV = 128;
 constexpr int TILE = BQ * D * 2;          // 32 KB: two panels [128 rows][64 columns]
-constexpr int QST = 3, DST = 2, VST = 2, TST = 4;  // stages: Q (held from S^T to dK), dO (from dP^T to dV), vectors, tile records
+constexpr int QST = 3, DST = 2, VST = 2, TST = 4, IST = 2;  // stages: Q (held from S^T to dK), dO (from dP^T to dV), vectors, tile records, items
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr int COL_S = 0, COL_DP = 128, COL_DV = 256, COL_DK = 384, TMEM_COLS = 512;
 
@@ -43,9 +43,10 @@ struct Smem {
     static constexpr int bytes = misc + 384;
 };
 struct Misc {
-    uint64_t bar_kv, bar_kvfree, bar_q[QST], bar_do[DST], bar_vec[VST], bar_vfree[VST], bar_tile[TST], bar_tfree[TST], bar_s, bar_dp, bar_p, bar_ds, bar_o,
+    uint64_t bar_kv, bar_kvfree, bar_q[QST], bar_do[DST], bar_vec[VST], bar_vfree[VST], bar_tile[TST], bar_tfree[TST], bar_item[IST], bar_ifree[IST], bar_s, bar_dp, bar_p, bar_ds, bar_o,
         bar_ofree, bar_exit;
     int4 tile[TST];  // {first row, rows, lead, 2 head + 1 if it is the item's last}: what the walker tells the other roles
+    int item[IST];   // the work numbers this CTA drew
     int4 vinfo[VST]; // the same, beside a tile's vectors
     int dead;        // latch: a wait of this CTA ran out, the CTA is abandoning its work
     uint32_t tmem;
@@ -59,7 +60,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
                 const __grid_constant__ CUtensorMap map_do, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const float* __restrict__ lse,
                 const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk_, __nv_bfloat16* __restrict__ dv_,
-                int* status, SplitTable split) {
+                int* ticket, int* status, SplitTable split) {
     extern __shared__ __align__(1024) unsigned char smem[];       // no static shared memory: the dynamic window starts 1024-byte aligned
     unsigned char* sK = smem + Smem::k;
     unsigned char* sV = smem + Smem::v;
@@ -78,6 +79,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         for (int s = 0; s < DST; s++) mbar_init(&m.bar_do[s], 1);
         for (int s = 0; s < VST; s++) { mbar_init(&m.bar_vec[s], 32); mbar_init(&m.bar_vfree[s], NS / 32); }
         for (int s = 0; s < TST; s++) { mbar_init(&m.bar_tile[s], 1); mbar_init(&m.bar_tfree[s], 3); }
+        for (int s = 0; s < IST; s++) { mbar_init(&m.bar_item[s], 1); mbar_init(&m.bar_ifree[s], 3 + NS / 32); }
         mbar_init(&m.bar_s, 1);
         mbar_init(&m.bar_dp, 1);
         mbar_init(&m.bar_p, NS / 32);
@@ -104,14 +106,36 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
     Ring<DST> rd;
     Ring<VST> rv;
     Ring<TST> rt;
+    Ring<IST> ri;
     uint32_t ph_kv = 0, ph_s = 0, ph_dp = 0, ph_p = 0, ph_ds = 0, ph_o = 0;
     const int n_work = (SPLIT ? split.n_units[0] : ix.n_kv_items) * Hkv;
-    // work items come most work first; dealt in a snake pattern (tier by tier, every second tier in reverse), so that no
-    // CTA gets the largest item of every tier
-    for (int tier = 0; tier * (int)gridDim.x < n_work; tier++) {
-        const int w = tier * (int)gridDim.x + ((tier & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
-        if (w >= n_work) continue;
-        if (*(volatile int*)&m.dead) break;       // a wait ran out: abandon the work
+    // Work items come most work first and are drawn from a counter (by the walker, when it has handed out the tiles of the one
+    // before): what a key tile takes differs by the length of its tree and its depth in it, and dealt in a fixed pattern the fullest
+    // CTA had 1.05 (65,521 agentic tokens) to 1.9 times (67,731 branchy) an even share.  Which CTA an item falls to does not enter
+    // its sums.
+    while (is_softmax || is_issuer || is_producer || is_loader || is_walker) {
+        int w;
+        if (is_walker) {
+            if (lane == 0) w = atomicAdd(ticket, 1);
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (!mbar_wait_warp(&m.bar_ifree[ri.st], ri.ph ^ 1, status, &m.dead)) break;       // a wait ran out: abandon the work
+            if (lane == 0) {
+                m.item[ri.st] = w;
+                mbar_arrive(&m.bar_item[ri.st]);
+            }
+            __syncwarp();
+        } else if (is_producer) {
+            if (!mbar_wait(&m.bar_item[ri.st], ri.ph, status, &m.dead)) break;
+            w = m.item[ri.st];
+            mbar_arrive(&m.bar_ifree[ri.st]);
+        } else {
+            if (!mbar_wait_warp(&m.bar_item[ri.st], ri.ph, status, &m.dead)) break;
+            w = m.item[ri.st];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&m.bar_ifree[ri.st]);
+        }
+        ri.next();
+        if (w >= n_work) break;
         const int item = w / Hkv, hk = w % Hkv;
         DkvUnit unit{};
         if (SPLIT) unit = split.unit[item];
@@ -434,7 +458,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
 
 int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* k, const void* v, const float* lse,
                         const void* dO, const float* delta, void* dk_, void* dv_, int Hq, int Hkv, float scale,
-                        int32_t* status, const SplitTable* split, cudaStream_t st) {
+                        int* ticket, int32_t* status, const SplitTable* split, cudaStream_t st) {
     CUtensorMap mq, mdo, mk, mv;
     int32_t rc;
     if ((rc = make_row_map(&mq, q, n_rows, Hq)) != HARTS_OK) return rc;
@@ -446,7 +470,7 @@ int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* 
     const long long n_work = (long long)ix.n_kv_items * Hkv;
     const int grid = split || n_work > sm_count() ? sm_count() : (int)n_work;
     kernel<<<grid, NT, Smem::bytes, st>>>(ix, Hq, Hkv, Hq / Hkv, scale, mq, mdo, mk, mv, lse,
-                                                          delta, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_, status,
+                                                          delta, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_, ticket, status,
                                                  split ? *split : SplitTable{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }

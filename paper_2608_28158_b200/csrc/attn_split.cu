@@ -1,7 +1,7 @@
 // Split of the dK / dV work of small, skewed problems (worth_cutting).  A key tile near the root is seen by every query below
 // it -- for every query head of its group -- so on one tree with grouped queries a few work items are most of the work, and the
-// CTA that draws the largest one is what the launch takes (9,001 tokens, 16 query heads on 4 key heads: 0.89 ms; 0.34 ms
-// with this split, 0.02 of them in split_kernel and reduce_kernel).  Here one CTA cuts every item into units of about a quarter of
+// CTA that draws the largest one is what the launch takes (9,001 tokens, 16 query heads on 4 key heads: both backward kernels 0.62
+// ms; 0.39 ms with this split, 0.03 of them in split_kernel and reduce_kernel).  Here one CTA cuts every item into units of about a quarter of
 // an SM's share of the whole, attn_dkv_kernel leaves the sums of a cut item in fp32, unit by unit, and reduce_kernel adds them
 // in unit order (no atomics: same bits every run).
 // The table and the partial sums live in the dq tensor, which is written only afterwards (the dQ kernel runs last then).
@@ -21,6 +21,8 @@ namespace {
 
 using namespace attn;
 
+constexpr int LEAST_UNIT = 8;          // query tiles
+
 // One CTA of 1024 threads, a warp per item.
 __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, int sms, SplitTable t) {
     __shared__ int total, slots, len;
@@ -39,7 +41,7 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) len = max(8, (int)(((long long)total * Hkv + 4 * sms - 1) / (4 * sms)));
+    if (threadIdx.x == 0) len = max(LEAST_UNIT, (int)(((long long)total * Hkv + 4 * sms - 1) / (4 * sms)));
     for (int tries = 0; tries < 20; tries++) {                // the longest unit such that the partial sums fit
         if (threadIdx.x == 0) slots = 0;
         __syncthreads();
@@ -132,21 +134,22 @@ __global__ void __launch_bounds__(256) reduce_kernel(Index ix, int Hkv, SplitTab
 
 }  // namespace
 
-// What cutting would save, from the host's copy of the index: the dK / dV items as they are dealt without a cut (snake order, one
-// CTA per SM), in query tiles (about 1.2 us) with six more for the start and end of an item.  The CTA with the most work
-// against an even share: the cut has to make up for its two extra kernels, the units' starts and ends and the partial sums
-// (both kernels and forward, whole -> cut, us).
-//   worth it    9,001 branchy tokens, 16 query / 4 key heads  1,527 -> 1,224  (most 656 tiles, share 271); 30,001 x 16/4
-//               3,954 -> 3,055 (1,818, 844); 18,001 x 16/8 3,106 -> 2,766 (1,312, 758); 25,001 x 8/8 1,443 -> 1,330 (622, 333)
-//   not         agentic trees, whose items are even: 65,521 x 4/4 5,591 -> 6,105 (1,902, 1,740), 20,001 x 16/2 7,861 -> 8,669
-//               (2,796, 2,476); little work: 5,001 branchy x 32/16 1,080 -> 1,216 (442, 252), 5,001 agentic x 8/4 513 -> 536
-static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
+// What cutting would save, from the host's copy of the index, in query tiles (1.3 to 1.5 us): uncut, a launch takes as long as its
+// largest item or an even share of all, cut as long as its longest unit (split_kernel's length, from the room for partial sums) or
+// the share.  That has to make up for two extra kernels, the units' starts and ends and the partial sums: 60 tiles.  Both
+// backward kernels, whole -> cut, us (largest item, share):
+//   worth it    9,001 branchy tokens, 16 query / 4 key heads  615 -> 385 (284, 74); 12,001 x 8/2 758 -> 418 (376, 80); 3,001 x 16/2
+//               349 -> 132 (192, 20); 30,001 x 16/4 2,149 -> 1,973 (492, 429); 5,001 agentic x 8/2 367 -> 278 (160, 41);
+//               6,007 replay x 8/1 806 -> 462 (376, 68)
+//   not         25,001 branchy x 8/8 836 -> 855 (98, 167), 1,773 agentic x 32/32 173 -> 184 (14, 26); too little room for sums:
+//               10,001 agentic x 4/1 658 -> 680 (316, 77; longest unit 304), 1,964 x 4/1 135 -> 145 (64, 4)
+constexpr int CUT_LEAST = 60;
+static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms, int cap_slots) {
     const int P = hi[1], n_items = hi[5];
     const int32_t *len = hi + hi[9], *parent = hi + hi[10], *item = hi + hi[17];
     auto tiles = [](int rows) { return (rows + BQ - 1) / BQ; };
     std::unique_ptr<int32_t[]> mem(new (std::nothrow) int32_t[3 * (size_t)P]());
-    std::unique_ptr<int64_t[]> load(new (std::nothrow) int64_t[sms]());
-    if (!mem || !load) return false;
+    if (!mem) return false;
     int32_t *below = mem.get(), *kids = below + P, *todo = kids + P, n = 0;     // below: rows of all descendants
     for (int p = 0; p < P; p++)
         if (parent[p] >= 0) kids[parent[p]]++;
@@ -158,25 +161,31 @@ static bool worth_cutting(const int32_t* hi, int G, int Hkv, int sms) {
         below[a] += below[p] + len[p];
         if (--kids[a] == 0) todo[n++] = a;
     }
+    std::unique_ptr<int32_t[]> n_tiles(new (std::nothrow) int32_t[n_items]);
+    if (!n_tiles) return false;
     int64_t total = 0, most = 0;
-    for (int i = 0, at = 0, tier = 0; i < n_items; i++) {
+    for (int i = 0; i < n_items; i++) {
         const int piece = item[2 * i];
-        const int64_t t = (int64_t)G * tiles(below[piece] + len[piece] - item[2 * i + 1] * 128);
-        total += t * Hkv;
-        for (int h = 0; h < Hkv; h++) {
-            int64_t& l = load[tier & 1 ? sms - 1 - at : at];
-            l += t + 4;
-            most = l > most ? l : most;
-            if (++at == sms) at = 0, tier++;
-        }
+        const int32_t t = G * tiles(below[piece] + len[piece] - item[2 * i + 1] * 128);
+        n_tiles[i] = t;
+        total += (int64_t)t * Hkv;
+        most = t > most ? t : most;
     }
-    return most * sms * 10 >= total * 17 && (most - 120) * sms >= total;
+    const int64_t share = (total + sms - 1) / sms;
+    if (most - share < CUT_LEAST) return false;
+    int64_t unit = (total + 4 * sms - 1) / (4 * sms);
+    if (unit < LEAST_UNIT) unit = LEAST_UNIT;
+    for (; unit < most; unit *= 2) {          // as split_kernel does
+        int64_t slots = 0;
+        for (int i = 0; i < n_items; i++)
+            if (n_tiles[i] > unit) slots += (n_tiles[i] + unit - 1) / unit;
+        if (slots <= cap_slots) break;
+    }
+    return most - (unit > share ? unit : share) >= CUT_LEAST;
 }
 
-// The table and the partial sums in `buf`; false: too small a buffer, nothing to gain, or 16 items and more per SM (where the
-// largest item is a small part of a share, but for fans: 10,000 replay tokens x 8 heads, 22 per SM, 2,053 us against 1,791 cut).
+// The table and the partial sums in `buf`; false: too small a buffer, or nothing to gain.
 bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* buf, size_t bytes, SplitTable* t) {
-    if ((long long)ix.n_kv_items * Hkv >= 16LL * sm_count() || !worth_cutting(hi, G, Hkv, sm_count())) return false;
     const size_t max_units = (size_t)ix.n_kv_items + 5 * sm_count() + 64;       // units of a quarter share, plus one per item
     char* p = static_cast<char*>(buf);
     size_t off = 256;
@@ -188,7 +197,7 @@ bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* 
     t->sums = reinterpret_cast<float*>(p + off);
     if (bytes <= off) return false;
     t->cap_slots = (int)((bytes - off) / ((size_t)Hkv * 2 * 128 * D * sizeof(float)));
-    return t->cap_slots > 1;
+    return t->cap_slots > 1 && worth_cutting(hi, G, Hkv, sm_count(), t->cap_slots);
 }
 int32_t attn_split_launch(const Index& ix, int G, int Hkv, const SplitTable& t, cudaStream_t st) {
     split_kernel<<<1, 1024, 0, st>>>(ix, G, Hkv, sm_count(), t);
