@@ -335,7 +335,7 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
         }
     }
     if (__syncthreads_or(m.dead)) {               // abandoned: let the loads and MMAs in flight finish (bounded)
-        if (tid == NS) {
+        if (is_issuer && elect_one()) {
             mma_commit(&m.bar_exit);
             mbar_wait_drain(&m.bar_exit, 0);
         }

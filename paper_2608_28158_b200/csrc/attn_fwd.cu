@@ -311,7 +311,7 @@ attn_fwd_kernel(Index ix, int Hq, int G, float scale_log2, const __grid_constant
         }
     }
     if (__syncthreads_or(m.dead)) {               // abandoned: let the loads and MMAs in flight finish (bounded)
-        if (tid == NS) {
+        if (is_issuer && elect_one()) {
             mma_commit(&m.bar_exit);
             mbar_wait_drain(&m.bar_exit, 0);
         }

@@ -141,25 +141,26 @@ int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      //
 int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
 int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);     // la_chunk_bwd.cu
-// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs, with fewer than four chunks a sequence up to 512 pairs.
+// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs, with fewer than four chunks a sequence up to 1,152 pairs.
 // The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 430 KB: with enough chains to fill the GPU the walk
 // wins, with few the chain of its 3-6 us chunks is what takes the time.  Walk / chunk-parallel, time of a step (of the forward
 // alone), 46 forests both ways with cold inputs:
 //   inside the line the chunk path won everywhere: 304 chunks x 4 heads 2.8 (2.9); agentic 16,736 items, 384 pairs 1.78 (1.96);
 //     25,576 items, 632 pairs 1.15 (1.34); 28,668 items, 636 pairs 1.20 (1.34); branchy 7,296 items, 624 pairs 1.16 (1.10);
-//     replay fans, 92 to 233 items, 34 to 127 pairs 2.5 to 2.9; 422 items, 254 pairs 2.0 (2.9; gate per channel 2.6); 645 items, 393
-//     pairs 1.9; 782 items, 478 pairs 1.8
+//     replay fans, 422 items, 254 pairs 3.5 (2.9; gate per channel 3.4); 645 items, 393 pairs 3.4; 782 items, 478 pairs 3.3; 1,564
+//     items, 956 pairs 2.5; beyond the line 3,128 items, 1,912 pairs 0.95, 6,256 items, 3,824 pairs 0.83 (up to 1,184 pairs the walk
+//     runs all rounds in one launch, and one CTA sums all gradients of a boundary; the scan reads them 512 bytes at a time)
 //   just outside it still won on agentic trees (28,144 items, 736 pairs 1.12 (1.26); 33,472 items, 768 pairs 1.05 (1.20)): the
 //     line is on the safe side there
 //   further out the walk wins: branchy 9,728 items, 832 pairs 0.97 (0.86); 24,768 items, 2,328 pairs 0.89 (0.76); agentic 51,152
 //     items, 1,264 pairs 0.94 (0.90); 6,949 chunks of replay fans x 16 heads 0.65
 // The line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
-constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640, CHUNK_PARALLEL_FANS = 512;
+constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640, CHUNK_PARALLEL_FANS = 1152;
 inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
     const int64_t chains = (int64_t)tb.n_seq * H;
     return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 &&
-           (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX && chains <= CHUNK_PARALLEL_CHAINS &&
-           (tb.n_chunks >= 4 * (int64_t)tb.n_seq || chains <= CHUNK_PARALLEL_FANS);
+           (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
+           chains <= (tb.n_chunks >= 4 * (int64_t)tb.n_seq ? CHUNK_PARALLEL_CHAINS : CHUNK_PARALLEL_FANS);
 }
 // the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then
 // <S_c, dS_c> in parts, fp32 [n_chunks, H, 4 blocks of 32 columns, dk], then the scan's ticket and counters

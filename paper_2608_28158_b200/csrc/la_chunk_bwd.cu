@@ -75,7 +75,7 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                   *sDP = smem + Smem::dp, *sS = smem + Smem::s, *sDS = smem + Smem::ds;
     Misc& m = *reinterpret_cast<Misc*>(smem + Smem::misc);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool is_compute = warp < NC / 32, is_issuer = tid == NC, is_aux = warp == NC / 32 + 1;
+    const bool is_compute = warp < NC / 32, is_issuer = tid == NC, is_mma = warp == NC / 32, is_aux = warp == NC / 32 + 1;
     const int grp = warp >> 2, L = (warp & 3) * 32 + lane;
 
     const int chunk_lo = tb.seq_chunk_ptr[seq_lo], n_items = (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H;
@@ -176,31 +176,37 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             fence_async_smem();
             __syncthreads();
         }
-        if (is_issuer) {
-            bool ok = mbar_wait(&m.bar_tiles, ph, status, &m.dead);
+        if (is_mma) {                      // an elected lane issues: operands in uniform registers
+            bool ok = mbar_wait_warp(&m.bar_tiles, ph, status, &m.dead);
             tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ks++) mma_ss(tmem + COL_A, dQk + kstep_kmajor<BT>(ks), dKk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
+                for (int ks = 0; ks < 8; ks++) mma_ss(tmem + COL_A, dQk + kstep_kmajor<BT>(ks), dKk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
 #pragma unroll
-            for (int ks = 0; ks < 8; ks++)
-                mma_ss(tmem + COL_DA, dDOk_hi + kstep_kmajor<BT>(ks), dVk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
-            mma_commit(&m.bar_a);
-            ok = mbar_wait(&m.bar_states, ph, status, &m.dead) && ok;
+                for (int ks = 0; ks < 8; ks++)
+                    mma_ss(tmem + COL_DA, dDOk_hi + kstep_kmajor<BT>(ks), dVk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
+                mma_commit(&m.bar_a);
+            }
+            __syncwarp();
+            ok = mbar_wait_warp(&m.bar_states, ph, status, &m.dead) && ok;
             if (ok) tiles_pending = false;
             tc_fence_after();
-            if (has_ds) {
+            if (elect_one()) {
+                if (has_ds) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)           // dS V^T
-                    mma_ss(tmem + COL_DKE, dDSk + kstep_kmajor<D>(ks), dVk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
+                    for (int ks = 0; ks < 8; ks++)       // dS V^T
+                        mma_ss(tmem + COL_DKE, dDSk + kstep_kmajor<D>(ks), dVk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)           // dS^T K^T
-                    mma_ss(tmem + COL_DVE, dDSm + kstep_mnmajor(ks), dKk + kstep_kmajor<BT>(ks), I_MK64, ks > 0);
+                    for (int ks = 0; ks < 8; ks++)       // dS^T K^T
+                        mma_ss(tmem + COL_DVE, dDSm + kstep_mnmajor(ks), dKk + kstep_kmajor<BT>(ks), I_MK64, ks > 0);
+                }
+                if (has_s)
+#pragma unroll
+                    for (int ks = 0; ks < 8; ks++)       // S dO^T
+                        mma_ss(tmem + COL_DQE, dSk + kstep_kmajor<D>(ks), dDOk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
             }
-            if (has_s)
-#pragma unroll
-                for (int ks = 0; ks < 8; ks++)           // S dO^T
-                    mma_ss(tmem + COL_DQE, dSk + kstep_kmajor<D>(ks), dDOk + kstep_kmajor<BT>(ks), I_KK64, ks > 0);
-            tma_store_wait_read();         // the previous item's outputs have left the staging tiles
+            __syncwarp();
+            if (is_issuer) tma_store_wait_read();     // the previous item's outputs have left the staging tiles
         }
         if (is_aux && i + 1 < n_mine) store_rows(m.rows[(i + 1) % 3], nx_code, nx_g, lane);
         float g_part = 0.f;                // this thread's share of <S_{c+1}, dS_{c+1}>
@@ -242,16 +248,21 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
         tc_fence_before();
         __syncthreads();                   // (A) P and dP are in place, the staging tiles are free, the next record is visible
         tc_fence_after();
+        if (is_mma) {
+            if (elect_one()) {
+#pragma unroll
+                for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DK, dQm + kstep_mnmajor(ks), dDPm + kstep_mnmajor(ks), I_MM64, ks > 0);
+                mma_commit(&m.bar_o);
+#pragma unroll
+                for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DV, dDOm + kstep_mnmajor(ks), dPm + kstep_mnmajor(ks), I_MM64, ks > 0);
+                mma_commit(&m.bar_o2);
+#pragma unroll
+                for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DQ, dKm + kstep_mnmajor(ks), dDPk + kstep_kmajor<BT>(ks), I_MK64, ks > 0);
+                mma_commit(&m.bar_o3);
+            }
+            __syncwarp();
+        }
         if (is_issuer) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DK, dQm + kstep_mnmajor(ks), dDPm + kstep_mnmajor(ks), I_MM64, ks > 0);
-            mma_commit(&m.bar_o);
-#pragma unroll
-            for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DV, dDOm + kstep_mnmajor(ks), dPm + kstep_mnmajor(ks), I_MM64, ks > 0);
-            mma_commit(&m.bar_o2);
-#pragma unroll
-            for (int ks = 0; ks < 4; ks++) mma_ss(tmem + COL_DQ, dKm + kstep_mnmajor(ks), dDPk + kstep_kmajor<BT>(ks), I_MK64, ks > 0);
-            mma_commit(&m.bar_o3);
             mbar_wait(&m.bar_o3, ph, status, &m.dead);
             mbar_wait(&m.bar_qk_read, ph, status, &m.dead);      // the compute warps have taken their q and k values
             if (i + 1 < n_mine) {
@@ -417,10 +428,13 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             }
         }
     }
-    if (__syncthreads_or(m.dead) && is_issuer) {      // abandoned: let copies and MMAs in flight finish (bounded)
-        if (tiles_pending) drain_delay();
-        mma_commit(&m.bar_exit);
-        mbar_wait_drain(&m.bar_exit, 0);
+    if (__syncthreads_or(m.dead) && is_mma) {         // abandoned: let copies and MMAs in flight finish (bounded)
+        if (is_issuer && tiles_pending) drain_delay();
+        __syncwarp();
+        if (elect_one()) {
+            mma_commit(&m.bar_exit);
+            mbar_wait_drain(&m.bar_exit, 0);
+        }
     }
     if (is_issuer) tma_store_wait_all();
     tc_fence_before();

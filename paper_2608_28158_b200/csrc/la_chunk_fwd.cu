@@ -51,7 +51,7 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                   *sO = smem + Smem::stage;
     Misc& m = *reinterpret_cast<Misc*>(smem + Smem::misc);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool is_compute = warp < NC / 32, is_issuer = tid == NC, is_aux = warp == NC / 32 + 1;
+    const bool is_compute = warp < NC / 32, is_issuer = tid == NC, is_mma = warp == NC / 32, is_aux = warp == NC / 32 + 1;
     const int grp = warp >> 2, L = (warp & 3) * 32 + lane;
 
     const int chunk_lo = tb.seq_chunk_ptr[seq_lo], n_items = (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H;
@@ -89,6 +89,8 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
     const uint32_t tmem = m.tmem, tm_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
 
     const uint32_t aQ = smem_u32(sQ), aK = smem_u32(sK), aV = smem_u32(sV), aP = smem_u32(sP), aS = smem_u32(sS), aO = smem_u32(sO);
+    const uint64_t dQk = desc_kmajor_base(aQ), dKk = desc_kmajor_base(aK), dPk = desc_kmajor_base(aP);
+    const uint64_t dVm = desc_mnmajor_base<BT>(aV), dSm = desc_mnmajor_base<D>(aS);
     constexpr uint32_t IDESC_A = instr_desc(128, 64, 0, 0);    // Q x K, both K-major (rows 64..127 of A unused)
     constexpr uint32_t IDESC_O = instr_desc(128, 64, 1, 0);    // V^T x P, S^T x Q
 
@@ -135,17 +137,20 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             fence_async_smem();
             __syncthreads();
         }
-        if (is_issuer) {
-            if (mbar_wait(&m.bar_tiles, ph, status, &m.dead)) tiles_pending = false;
+        if (is_mma) {                      // an elected lane issues: operands in uniform registers
+            if (mbar_wait_warp(&m.bar_tiles, ph, status, &m.dead)) tiles_pending = false;
             tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ks++) mma_ss(tmem + COL_A, desc_kmajor<BT>(aQ, ks), desc_kmajor<BT>(aK, ks), IDESC_A, ks > 0);
-            mma_commit(&m.bar_a);
-            if (!zero_state)
+                for (int ks = 0; ks < 8; ks++) mma_ss(tmem + COL_A, dQk + kstep_kmajor<BT>(ks), dKk + kstep_kmajor<BT>(ks), IDESC_A, ks > 0);
+                mma_commit(&m.bar_a);
+                if (!zero_state)
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)
-                    mma_ss(tmem + COL_O2, desc_mnmajor<D>(aS, ks), desc_kmajor<BT>(aQ, ks), IDESC_O, ks > 0);
-            tma_store_wait_read();         // the previous item's outputs have left the staging tile
+                    for (int ks = 0; ks < 8; ks++)
+                        mma_ss(tmem + COL_O2, dSm + kstep_mnmajor(ks), dQk + kstep_kmajor<BT>(ks), IDESC_O, ks > 0);
+            }
+            __syncwarp();
+            if (is_issuer) tma_store_wait_read();     // the previous item's outputs have left the staging tile
         }
         if (is_aux && i + 1 < n_mine) store_rows(m.rows[(i + 1) % 3], nx_code, nx_g, lane);
         if (is_compute && (warp & 3) < 2) {           // P = A .* decay: lanes 0..63 hold the rows
@@ -174,11 +179,16 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
         tc_fence_before();
         __syncthreads();                   // (A) P is in place, the staging tile is free, the next record is visible
         tc_fence_after();
-        if (is_issuer) {
+        if (is_mma) {
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ks++)
-                mma_ss(tmem + COL_O1, desc_mnmajor<BT>(aV, ks), desc_kmajor<BT>(aP, ks), IDESC_O, ks > 0);
-            mma_commit(&m.bar_o);
+                for (int ks = 0; ks < 4; ks++)
+                    mma_ss(tmem + COL_O1, dVm + kstep_mnmajor(ks), dPk + kstep_kmajor<BT>(ks), IDESC_O, ks > 0);
+                mma_commit(&m.bar_o);
+            }
+            __syncwarp();
+        }
+        if (is_issuer) {
             mbar_wait(&m.bar_o, ph, status, &m.dead);
             if (i + 1 < n_mine) {          // every MMA that read the tiles is done
                 issue_tiles(m.items[(i + 1) % 3]);
@@ -237,10 +247,13 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             }
         }
     }
-    if (__syncthreads_or(m.dead) && is_issuer) {      // abandoned: let copies and MMAs in flight finish (bounded)
-        if (tiles_pending) drain_delay();
-        mma_commit(&m.bar_exit);
-        mbar_wait_drain(&m.bar_exit, 0);
+    if (__syncthreads_or(m.dead) && is_mma) {         // abandoned: let copies and MMAs in flight finish (bounded)
+        if (is_issuer && tiles_pending) drain_delay();
+        __syncwarp();
+        if (elect_one()) {
+            mma_commit(&m.bar_exit);
+            mbar_wait_drain(&m.bar_exit, 0);
+        }
     }
     if (is_issuer) tma_store_wait_all();
     tc_fence_before();

@@ -140,6 +140,12 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             if (lane == 0) mbar_arrive(&m.item_empty[k % ITEMS]);
             if (it.seq < 0) break;
             const size_t in_state = (size_t)L * D + it.slice * NV + col0;
+            // gradients of initial states, which only these threads write and read: [32 columns][32 rows][four of the columns][row],
+            // whatever the slices' width, so that a warp's access is 512 bytes in a row
+            auto ds0_of = [&](size_t seq_head) {
+                return reinterpret_cast<float4*>(ds0 + seq_head * (D * D)) + ((it.slice * NV + col0) / 32 * 4 + (warp & 3)) * 256 + lane;
+            };
+            auto ds0_step = [](int e) { return (e >> 3) * 1024 + (e & 7) * 32; };
             float x[CW];
 #pragma unroll
             for (int e = 0; e < CW; e++) x[e] = 0.f;
@@ -155,13 +161,20 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             for (int i = 0; i < it.n_chunks && alive; i++) {
                 const int c = chunk_of(it, i);
                 if (BWD && boundary == c + 1) {   // gradients of every sequence that started from this boundary, in table order
-                    for (int u = tb.slot_cons_ptr[req]; u < tb.slot_cons_ptr[req + 1]; u++) {
+                    unsigned there = 0;       // whose flag is up already: a lane each looks, 32 at a time
+                    for (int u = tb.slot_cons_ptr[req], k = 0; u < tb.slot_cons_ptr[req + 1]; u++, k++) {
+                        if (order.n && (k & 31) == 0) {
+                            const bool mine = u + lane < tb.slot_cons_ptr[req + 1] &&
+                                              ld_acquire(flags + ((size_t)tb.slot_cons_seq[u + lane] * H + it.h) * SLICES + it.slice) >= NS / 32;
+                            there = __ballot_sync(0xffffffffu, mine);
+                            __syncwarp();     // hands on what the lanes acquired
+                        }
                         const size_t from = (size_t)tb.slot_cons_seq[u] * H + it.h;
-                        const float4* src = reinterpret_cast<const float4*>(ds0 + from * (D * D) + in_state);
-                        if (order.n) alive = flag_wait_warp(flags + from * SLICES + it.slice, NS / 32, status, &m.dead) && alive;
+                        if (order.n && !(there >> (k & 31) & 1)) alive = flag_wait_warp(flags + from * SLICES + it.slice, NS / 32, status, &m.dead) && alive;
+                        const float4* src = ds0_of(from);
 #pragma unroll
                         for (int e = 0; e < CW / 4; e++) {
-                            const float4 y = __ldcg(src + e);
+                            const float4 y = __ldcg(src + ds0_step(e));
                             x[4 * e] += y.x, x[4 * e + 1] += y.y, x[4 * e + 2] += y.z, x[4 * e + 3] += y.w;
                         }
                     }
@@ -232,9 +245,9 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
             }
             if (BWD && it.init_slot >= 0 && alive) {     // the hand-off into the sequence that exported this state
                 const size_t to = (size_t)it.seq * H + it.h;
-                float4* dst = reinterpret_cast<float4*>(ds0 + to * (D * D) + in_state);
+                float4* dst = ds0_of(to);
 #pragma unroll
-                for (int e = 0; e < CW / 4; e++) dst[e] = *reinterpret_cast<const float4*>(x + 4 * e);
+                for (int e = 0; e < CW / 4; e++) dst[ds0_step(e)] = *reinterpret_cast<const float4*>(x + 4 * e);
                 if (order.n) flag_add_warp(flags + to * SLICES + it.slice);
             }
         }

@@ -1,18 +1,20 @@
 """Fans of short branches through the chunk-parallel path: both sides of its line, and slots exported by one chunk after another."""
+import numpy as np
 import pytest
 import torch
 
 import paper_2608_28158_b200 as H
 from parity_util import compare, oracle_subset, run_gpu
+from test_gpu_gk import check as check_gk, run_gk
 from test_gpu_parity import check
 from workloads import make_forest, make_inputs
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("heads", [16, 17])
+@pytest.mark.parametrize("heads", [36, 37])
 def test_both_sides_of_the_line_of_fans(heads):
-    """32 sequences of fewer than four chunks: 512 (sequence, head) pairs take the chunk-parallel path, 544 the walk."""
+    """32 sequences of fewer than four chunks: 1,152 (sequence, head) pairs take the chunk-parallel path, 1,184 the walk."""
     fo = make_forest([([-1] + [0] * 31, [0] + [1 + 4 * i for i in range(31)], [130] + [2 * i + 1 for i in range(31)])])
     inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 13, device="cuda")
     plan, out = run_gpu(fo, inp)
@@ -34,3 +36,24 @@ def test_a_slot_from_every_chunk(heads):
     assert plan.n_slots >= n - 1
     tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1] if heads > 1 else [0])
     check(compare(out, tok, [0, heads - 1] if heads > 1 else [0], ref, rows=True), "bf16")
+
+
+@pytest.mark.parametrize("kids", [33, 70])
+@pytest.mark.parametrize("gk", [False, True])
+def test_a_boundary_with_many_consumers(kids, gk):
+    """One boundary that more than 32 (64) sequences start from: their flags are looked at 32 at a time, their gradients summed in
+    table order, with the same bits in one launch and round by round."""
+    fo = make_forest([([-1] + [0] * kids, [0] + [64 + 1 + i % 60 for i in range(kids)], [130] + [1 + i % 7 for i in range(kids)])])
+    if gk:
+        plan, errs = run_gk(fo, 2, 128, "bf16", 19)
+        check_gk(errs, "bf16")
+        (_, out), (_, rounds) = (run_gk(fo, 2, 128, "bf16", 19, raw=True, flags=f) for f in (0, H.HARTS_FLAG_ROUND_LAUNCHES))
+    else:
+        inp = make_inputs(fo.n_tokens, 2, 128, 128, "bf16", 19)
+        plan, out = run_gpu(fo, inp)
+        tok, ref = oracle_subset(fo, inp, [0], [0, 1])
+        check(compare(out, tok, [0, 1], ref, rows=True), "bf16")
+        _, rounds = run_gpu(fo, inp, flags=H.HARTS_FLAG_ROUND_LAUNCHES)
+    assert max(np.diff(plan.slot_cons_ptr)) >= kids - 1
+    for n in out:
+        assert np.array_equal(np.asarray(torch.as_tensor(out[n]).float().cpu()), np.asarray(torch.as_tensor(rounds[n]).float().cpu())), n
