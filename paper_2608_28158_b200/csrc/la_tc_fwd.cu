@@ -315,6 +315,9 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
         __syncthreads();                          // (3) b2 / eb / w / gamma visible
         // ---- state pass: S_c^T -> bf16 operand tile (+ slot), S^T <- gamma S^T ----------------------------
+        // nobody reads the state at the end of a sequence: its last chunk neither scales nor updates it (6,949 short-sequence chunks
+        // x 16 heads 3.16 -> 2.86 ms, 4,696 long-sequence chunks x 32 heads 3.01 -> 2.93)
+        const bool last = c == s.n_chunks - 1;
         {
             const bool export_slot = next_boundary == c;
             float* slot_dst = export_slot ? slots + ((size_t)next_req * H + h) * state_elems + (size_t)L * D : nullptr;
@@ -340,6 +343,7 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                     int col = blk * 32 + v4 * 8;           // first of 8 consecutive j'
                     *reinterpret_cast<uint4*>(sS + (col >> 6) * S_PANEL + sw128_chunk(L, (col & 63) >> 3)) = pk;
                 }
+                if (last) continue;
 #pragma unroll
                 for (int i = 0; i < 32; i++) x[i] = __float_as_uint(__uint_as_float(x[i]) * gamma);
                 tmem_st32(tm_lane + COL_S + blk * 32, x);
@@ -382,7 +386,7 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                     *reinterpret_cast<uint4*>(sP + sw128_chunk(t, half * 4 + v4)) = pk;
                 }
             }
-        } else {
+        } else if (!last) {
             for (int e = ((warp & 3) - 2) * 32 + lane + 64 * grp; e < BT * 16; e += 128) {
                 uint32_t off = e * 16;
                 float wj = m.w[(off % PANEL) >> 7];
@@ -415,8 +419,9 @@ tc_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                 mma_ss(tmem + COL_O1, desc_mnmajor<BT>(aV, ks), desc_kmajor<BT>(aP, ks), IDESC_O1, ks > 0);
             for (int ks = 0; ks < 8; ks++)
                 mma_ss(tmem + COL_A, desc_mnmajor<D>(aS, ks), desc_kmajor<BT>(aQ, ks), IDESC_O2, ks > 0);
-            for (int ks = 0; ks < 4; ks++)
-                mma_ss(tmem + COL_S, desc_mnmajor<BT>(aK, ks), desc_mnmajor<BT>(aV, ks), IDESC_S, true);
+            if (!last)
+                for (int ks = 0; ks < 4; ks++)
+                    mma_ss(tmem + COL_S, desc_mnmajor<BT>(aK, ks), desc_mnmajor<BT>(aV, ks), IDESC_S, true);
             mma_commit(&m.bar_o);
         }
         if constexpr (!ONE_LAUNCH) {
