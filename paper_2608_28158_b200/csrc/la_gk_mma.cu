@@ -518,6 +518,28 @@ __device__ __forceinline__ void global_to_tile128(const __nv_bfloat16* src, unsi
     }
 }
 
+// A warp's 16 x 32 block (rows 16 * mb, columns 32 * nq) of a [64][128] product: bf16 rows to global memory, 16 bytes a lane, by way of
+// the block's own place in a tile nobody reads any more.  Straight from the fragments a store is 4 bytes of eight rows: with dq,
+// dk, dv so, the rows' outputs were 0.2 of the backward's time.  Rows without an output (code < 0) are left out.
+__device__ __forceinline__ void block_to_rows(const float (&acc)[4][4], unsigned char* tile, int mb, int nq, const int* srow,
+                                              __nv_bfloat16* __restrict__ out, int H, int h, int lane) {
+#pragma unroll
+    for (int n2 = 0; n2 < 2; n2++) {
+        const int row = 16 * mb + ((lane >> 3) & 1) * 8 + (lane & 7), c16 = 4 * nq + 2 * n2 + (lane >> 4);
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(s_u32(tile + sw256(row, c16))),
+                     "r"(pack2(acc[2 * n2][0], acc[2 * n2][1])), "r"(pack2(acc[2 * n2][2], acc[2 * n2][3])),
+                     "r"(pack2(acc[2 * n2 + 1][0], acc[2 * n2 + 1][1])), "r"(pack2(acc[2 * n2 + 1][2], acc[2 * n2 + 1][3])) : "memory");
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int row = 16 * mb + 8 * u + (lane >> 2), c16 = 4 * nq + (lane & 3), code = srow[row];
+        const uint4 y = *reinterpret_cast<const uint4*>(tile + sw256(row, c16));
+        if (code >= 0) *reinterpret_cast<uint4*>(out + ((size_t)code * H + h) * D + c16 * 8) = y;
+    }
+    __syncwarp();
+}
+
 // the sequence of [seq_lo, seq_hi) that owns chunk gc (every warp searches, 32 ways at a time)
 __device__ __forceinline__ int owner_of(const harts_la_tables_t& tb, int seq_lo, int seq_hi, int gc) {
     const int lane = threadIdx.x & 31;
@@ -700,12 +722,18 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
     float *sB = reinterpret_cast<float*>(sm + SharedC::b), *sTmp = reinterpret_cast<float*>(sP), *sR = reinterpret_cast<float*>(sQa);
     int* srow = reinterpret_cast<int*>(sm + SharedC::row);
     const uint32_t aQ = s_u32(sQ), aK = s_u32(sK), aP = s_u32(sP), aV = s_u32(sV), aS = s_u32(sB);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
     const int chunk_lo = tb.seq_chunk_ptr[seq_lo], n_items = (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H;
+    SeqInfo s;
+    s.chunk_base = s.n_chunks = 0;
+    int seq = seq_lo;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int h = item % H, gc = chunk_lo + item / H;
-        const SeqInfo s = seq_info(tb, owner_of(tb, seq_lo, seq_hi, gc));
+        if (gc >= s.chunk_base + s.n_chunks) {             // chunks come in order: often still the last one's sequence
+            seq = owner_of(tb, seq, seq_hi, gc);
+            s = seq_info(tb, seq);
+        }
         const int c = gc - s.chunk_base;
         const bool has_s = c > 0 || s.init_slot >= 0;     // the state of a sequence that starts from zero is not read
         __syncthreads();                                   // the previous item's readers of every tile are through
@@ -784,13 +812,7 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
             }
-        const int row_lo = srow[m0 + g], row_hi = srow[m0 + g + 8];
-#pragma unroll
-        for (int n = 0; n < 4; n++) {
-            const int col = n_base + n * 8 + tq * 2;
-            if (row_lo >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
-            if (row_hi >= 0) *reinterpret_cast<uint32_t*>(o + ((size_t)row_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
-        }
+        block_to_rows(acc, sK, mb, nq, srow, o, H, h, lane);       // k has been read: its anchored forms carry it
     }
 }
 
@@ -864,6 +886,9 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
     const int chunk_lo = CHUNKS ? tb.seq_chunk_ptr[seq_lo] : 0, n_items = CHUNKS ? (tb.seq_chunk_ptr[seq_hi] - chunk_lo) * H : 0;
     int item = blockIdx.x;
+    SeqInfo s;
+    s.chunk_base = s.n_chunks = 0;
+    int seq = seq_lo;
     do {
     if (CHUNKS && item >= n_items) break;
     int seq_pos = seq_lo + item / H, h = item % H;
@@ -883,9 +908,11 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             else j -= cnt;
         }
     }
-    const int seq = CHUNKS ? owner_of(tb, seq_lo, seq_hi, gc) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+    if (!CHUNKS || gc >= s.chunk_base + s.n_chunks) {     // chunks come in order: often still the last one's sequence
+        seq = CHUNKS ? owner_of(tb, seq, seq_hi, gc) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+        s = seq_info(tb, seq);
+    }
     const int mb = warp & 3, nq = warp >> 2;          // this warp's 16-row block and 32-column quarter of [64][128] products
-    const SeqInfo s = seq_info(tb, seq);
     const size_t state_elems = (size_t)D * D;
 
     float ds[8][4];                                   // dS, laid out over the warps like the forward's state
@@ -1150,23 +1177,22 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                     tail.x += x.x + (b2 > mb ? y.x : 0.f);
                     tail.y += x.y + (b2 > mb ? y.y : 0.f);
                 }
-                auto put = [&](int code, int r, float2 dqv, float2 dkv, float2 dgv) {      // replayed rows: fp32 to the scratch
+                auto put = [&](int code, int r, float2 dkv, float2 dgv) {      // replayed rows: fp32 to the scratch
                     if (code >= 0) {
-                        const size_t off = ((size_t)code * H + h) * D + col;
-                        *reinterpret_cast<uint32_t*>(dq + off) = pack2(dqv.x, dqv.y);
-                        *reinterpret_cast<uint32_t*>(dk_ + off) = pack2(dkv.x, dkv.y);
-                        *reinterpret_cast<float2*>(dgk + off) = dgv;
+                        *reinterpret_cast<float2*>(dgk + ((size_t)code * H + h) * D + col) = dgv;
                     } else if (code < -1) {
                         const size_t off = ((size_t)(s.replay_base + r) * H + h) * D + col;
                         *reinterpret_cast<float2*>(rk + off) = dkv;
                         *reinterpret_cast<float2*>(rg + off) = dgv;
                     }
                 };
-                put(code_lo, r_lo, make_float2(iq[n][0], iq[n][1]), make_float2(ik[n][0], ik[n][1]),
+                put(code_lo, r_lo, make_float2(ik[n][0], ik[n][1]),
                     make_float2(z[n][0] + tail.x, z[n][1] + tail.y));
-                put(code_hi, r_hi, make_float2(iq[n][2], iq[n][3]), make_float2(ik[n][2], ik[n][3]),
+                put(code_hi, r_hi, make_float2(ik[n][2], ik[n][3]),
                     make_float2(z[n][2] + tail.x, z[n][3] + tail.y));
             }
+            block_to_rows(iq, sQa, mb, nq, srow, dq, H, h, lane);      // over the anchored operands, which have been multiplied
+            block_to_rows(ik, sKa, mb, nq, srow, dk_, H, h, lane);
         } else {
             __syncthreads();                              // the anchored operands are dead, the step factors visible
             scores_diagonal(sQ, sK, sR, sP, warp, lane);
@@ -1296,11 +1322,10 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = 32 * nq + 8 * n + 2 * tq;
-                if (row_lo >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)row_lo * H + h) * D + col) = pack2(acc[n][0], acc[n][1]);
-                else if (row_lo < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_lo) * H + h) * D + col) = make_float2(acc[n][0], acc[n][1]);
-                if (row_hi >= 0) *reinterpret_cast<uint32_t*>(dv_ + ((size_t)row_hi * H + h) * D + col) = pack2(acc[n][2], acc[n][3]);
-                else if (row_hi < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_hi) * H + h) * D + col) = make_float2(acc[n][2], acc[n][3]);
+                if (row_lo < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_lo) * H + h) * D + col) = make_float2(acc[n][0], acc[n][1]);
+                if (row_hi < -1) *reinterpret_cast<float2*>(rv + ((size_t)(s.replay_base + r_hi) * H + h) * D + col) = make_float2(acc[n][2], acc[n][3]);
             }
+            block_to_rows(acc, sQa, mb, nq, srow, dv_, H, h, lane);
         }
         // ---- dS <- Diag(e^{b_n}) dS + q~^T dO ---------------------------------------------------------------------------
         if (!CHUNKS) state_update(ds, sB, aQt, aDO, warp, lane);
