@@ -9,8 +9,10 @@
 // after the other.  Only the walk is serial here, and its step is one multiply-add per element with the operand prefetched;
 // the 64^3 products of different chunks run side by side.  What bounds it: launches and the latency of one product (256
 // threads x 4x4 outputs, 2,048 cycles at 128 multiply-adds a clock) on small forests, the CUDA cores on large ones.  Forward +
-// backward, cold inputs, against the walk: 718 tokens x 1 head (two rounds) 1.33 -> 0.095 ms (outer 9 + 7, walk 3 per round, out 17,
-// grad 30 us), 12,000 branchy x 4 12.0 -> 0.34, 40,000 replay x 8 13.6 -> 3.9, 150,000 agentic x 4 46.4 -> 3.3 (grad 2.0, out 0.7).
+// backward, cold inputs, against the walk: 718 tokens x 1 head (two rounds) 1.33 -> 0.086 ms (outer 9 + 7, walk 3 per round, out 13,
+// grad 25 us), 12,000 branchy x 4 12.0 -> 0.32, 40,000 replay x 8 13.6 -> 3.9, 150,000 agentic x 4 46.4 -> 3.3 (grad 2.0, out 0.7).
+// grad_kernel has one CTA an SM (141 KB): sixteen warps of 2x4 outputs instead of eight of 4x4 -- more shared-memory reads, twice the
+// warps to hide them -- and diagonals that are not unrolled took it from 31.3 to 24.8 us on 13 items, 174 to 159 on 796.
 #include "chunk_item.cuh"
 
 namespace harts {
@@ -28,33 +30,41 @@ using tc::ex2;
 constexpr int D = 64, NT = 256, LD = D + 4;      // rows of shared-memory tiles are padded: 16-byte aligned, conflict-free by column
 constexpr int TILE = BT * LD;                    // floats
 
-// Thread (ty, tx) = (tid / 16, tid % 16) owns outputs (4 ty + r, tx + 16 c), r, c = 0..3; a warp owns eight rows.
-using Acc = float[4][4];
-__device__ __forceinline__ void clear(Acc& a) {
+// Thread (ty, tx) = (tid / 16, tid % 16) owns outputs (R ty + r, tx + 16 c), r = 0..R-1, c = 0..3; a warp owns 2 R rows.  R = 4 with 256
+// threads, R = 2 with 512.
+template <int R>
+struct AccT {
+    float a[R][4];
+    __device__ float* operator[](int r) { return a[r]; }
+    __device__ const float* operator[](int r) const { return a[r]; }
+};
+template <int R>
+__device__ __forceinline__ void clear(AccT<R>& a) {
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int r = 0; r < R; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) a[r][c] = 0.f;
 }
 // a += X Y^T over column blocks 0..n_col-1 of 16
-template <int N_COL>
-__device__ __forceinline__ void mul_nt(Acc& a, const float* x, const float* y, int ty, int tx) {
+template <int N_COL, int R>
+__device__ __forceinline__ void mul_nt(AccT<R>& a, const float* x, const float* y, int ty, int tx) {
 #pragma unroll 4
     for (int i = 0; i < D; i += 4) {
-        float4 xv[4];
+        float4 xv[R];
 #pragma unroll
-        for (int r = 0; r < 4; r++) xv[r] = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + i);
+        for (int r = 0; r < R; r++) xv[r] = *reinterpret_cast<const float4*>(x + (R * ty + r) * LD + i);
 #pragma unroll
         for (int c = 0; c < N_COL; c++) {
             const float4 yv = *reinterpret_cast<const float4*>(y + (tx + 16 * c) * LD + i);
 #pragma unroll
-            for (int r = 0; r < 4; r++) a[r][c] += xv[r].x * yv.x + xv[r].y * yv.y + xv[r].z * yv.z + xv[r].w * yv.w;
+            for (int r = 0; r < R; r++) a[r][c] += xv[r].x * yv.x + xv[r].y * yv.y + xv[r].z * yv.z + xv[r].w * yv.w;
         }
     }
 }
 // the same where only columns <= the warp's last row are wanted (the rest of a stays as it is)
-__device__ __forceinline__ void mul_nt_causal(Acc& a, const float* x, const float* y, int ty, int tx) {
-    switch (ty >> 2) {                           // 16-row groups: two warps each
+template <int R>
+__device__ __forceinline__ void mul_nt_causal(AccT<R>& a, const float* x, const float* y, int ty, int tx) {
+    switch (R * ty >> 4) {                       // 16-row groups
         case 0: mul_nt<1>(a, x, y, ty, tx); break;
         case 1: mul_nt<2>(a, x, y, ty, tx); break;
         case 2: mul_nt<3>(a, x, y, ty, tx); break;
@@ -62,68 +72,76 @@ __device__ __forceinline__ void mul_nt_causal(Acc& a, const float* x, const floa
     }
 }
 // a += X[:, k0..k1) Y[k0..k1, :)
-__device__ __forceinline__ void mul_nn(Acc& a, const float* x, const float* y, int k0, int k1, int ty, int tx) {
+template <int R>
+__device__ __forceinline__ void mul_nn(AccT<R>& a, const float* x, const float* y, int k0, int k1, int ty, int tx) {
 #pragma unroll 2
     for (int k = k0; k < k1; k += 4) {
-        float4 xv[4];
+        float4 xv[R];
 #pragma unroll
-        for (int r = 0; r < 4; r++) xv[r] = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + k);
+        for (int r = 0; r < R; r++) xv[r] = *reinterpret_cast<const float4*>(x + (R * ty + r) * LD + k);
 #pragma unroll
         for (int kk = 0; kk < 4; kk++)
 #pragma unroll
             for (int c = 0; c < 4; c++) {
                 const float yv = y[(k + kk) * LD + tx + 16 * c];
 #pragma unroll
-                for (int r = 0; r < 4; r++) a[r][c] += (kk == 0 ? xv[r].x : kk == 1 ? xv[r].y : kk == 2 ? xv[r].z : xv[r].w) * yv;
+                for (int r = 0; r < R; r++) a[r][c] += (kk == 0 ? xv[r].x : kk == 1 ? xv[r].y : kk == 2 ? xv[r].z : xv[r].w) * yv;
             }
     }
 }
 // a += X[t0..64, :)^T Y[t0..64, :)
-__device__ __forceinline__ void mul_tn(Acc& a, const float* x, const float* y, int t0, int ty, int tx) {
+template <int R>
+__device__ __forceinline__ void load_r(float (&x)[R], const float* from) {       // R floats in a row, aligned so
+    if constexpr (R == 4) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(from);
+    else *reinterpret_cast<float2*>(x) = *reinterpret_cast<const float2*>(from);
+}
+template <int R>
+__device__ __forceinline__ void mul_tn(AccT<R>& a, const float* x, const float* y, int t0, int ty, int tx) {
 #pragma unroll 4
     for (int t = t0; t < BT; t++) {
-        const float4 xv = *reinterpret_cast<const float4*>(x + t * LD + 4 * ty);
+        float xv[R];
+        load_r<R>(xv, x + t * LD + R * ty);
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const float yv = y[t * LD + tx + 16 * c];
-            a[0][c] += xv.x * yv;
-            a[1][c] += xv.y * yv;
-            a[2][c] += xv.z * yv;
-            a[3][c] += xv.w * yv;
+#pragma unroll
+            for (int r = 0; r < R; r++) a[r][c] += xv[r] * yv;
         }
     }
 }
 
-// The eight columns (rows) at the diagonal of a warp's rows: what lies past the diagonal is left out, not multiplied by zero, so
+// The 2 R columns (rows) at the diagonal of a warp's rows: what lies past the diagonal is left out, not multiplied by zero, so
 // that an infinity or a NaN in a later row stays out of the rows before it.
-// a += P[:, k0..k0+8) Y[k0..k0+8, :), columns up to the row
-__device__ __forceinline__ void mul_nn_diagonal(Acc& a, const float* x, const float* y, int k0, int ty, int tx) {
+// a += P[:, k0..k0+2R) Y[k0..k0+2R, :), columns up to the row
+template <int R>
+__device__ __forceinline__ void mul_nn_diagonal(AccT<R>& a, const float* x, const float* y, int k0, int ty, int tx) {
+#pragma unroll 1
+    for (int k = k0; k < k0 + 2 * R; k += 4) {
+        float xv[R][4];
 #pragma unroll
-    for (int k = k0; k < k0 + 8; k += 4) {
-        float xv[4][4];
-#pragma unroll
-        for (int r = 0; r < 4; r++) *reinterpret_cast<float4*>(xv[r]) = *reinterpret_cast<const float4*>(x + (4 * ty + r) * LD + k);
+        for (int r = 0; r < R; r++) *reinterpret_cast<float4*>(xv[r]) = *reinterpret_cast<const float4*>(x + (R * ty + r) * LD + k);
 #pragma unroll
         for (int kk = 0; kk < 4; kk++)
 #pragma unroll
             for (int c = 0; c < 4; c++) {
                 const float yv = y[(k + kk) * LD + tx + 16 * c];
 #pragma unroll
-                for (int r = 0; r < 4; r++) a[r][c] = k + kk <= 4 * ty + r ? a[r][c] + xv[r][kk] * yv : a[r][c];
+                for (int r = 0; r < R; r++) a[r][c] = k + kk <= R * ty + r ? a[r][c] + xv[r][kk] * yv : a[r][c];
             }
     }
 }
-// a += P[t0..t0+8, :)^T Y[t0..t0+8, :), rows from the column on
-__device__ __forceinline__ void mul_tn_diagonal(Acc& a, const float* x, const float* y, int t0, int ty, int tx) {
-#pragma unroll
-    for (int t = t0; t < t0 + 8; t++) {
-        float xv[4];
-        *reinterpret_cast<float4*>(xv) = *reinterpret_cast<const float4*>(x + t * LD + 4 * ty);
+// a += P[t0..t0+2R, :)^T Y[t0..t0+2R, :), rows from the column on
+template <int R>
+__device__ __forceinline__ void mul_tn_diagonal(AccT<R>& a, const float* x, const float* y, int t0, int ty, int tx) {
+#pragma unroll 2
+    for (int t = t0; t < t0 + 2 * R; t++) {
+        float xv[R];
+        load_r<R>(xv, x + t * LD + R * ty);
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const float yv = y[t * LD + tx + 16 * c];
 #pragma unroll
-            for (int r = 0; r < 4; r++) a[r][c] = t >= 4 * ty + r ? a[r][c] + xv[r] * yv : a[r][c];
+            for (int r = 0; r < R; r++) a[r][c] = t >= R * ty + r ? a[r][c] + xv[r] * yv : a[r][c];
         }
     }
 }
@@ -160,7 +178,7 @@ __device__ __forceinline__ void store_gates(Rows& rd, const float (&gv)[2], int 
 
 // Rows of a chunk into a tile; `own`: replayed rows (and rows past the end) are zero, else only rows past the end.
 __device__ __forceinline__ void load_tile(float* dst, const float* src, const Rows& rd, bool own, int h, int H) {
-    for (int e = threadIdx.x; e < BT * 16; e += NT) {
+    for (int e = threadIdx.x; e < BT * 16; e += blockDim.x) {
         const int t = e >> 4, ch = e & 15, code = rd.code[t], r = code >= 0 ? code : -2 - code;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (own ? code >= 0 : code != -1) x = *reinterpret_cast<const float4*>(src + ((size_t)r * H + h) * D + ch * 4);
@@ -168,7 +186,7 @@ __device__ __forceinline__ void load_tile(float* dst, const float* src, const Ro
     }
 }
 __device__ __forceinline__ void load_state(float* dst, const float* src) {
-    for (int e = threadIdx.x; e < D * 16; e += NT)
+    for (int e = threadIdx.x; e < D * 16; e += blockDim.x)
         *reinterpret_cast<float4*>(dst + (e >> 4) * LD + (e & 15) * 4) = *reinterpret_cast<const float4*>(src + e * 4);
 }
 // The CTA's item `idx` of the range: warp 0 finds it and prepares its row data.  False: the range has no such item.  On return
@@ -224,7 +242,7 @@ __global__ void __launch_bounds__(NT, 5) outer_kernel(const harts_la_tables_t tb
     }
     __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    Acc acc;
+    AccT<4> acc;
     clear(acc);
     mul_tn(acc, s.x, s.y, 0, ty, tx);
     float* dst = sums + ((size_t)it.gc * H + it.h) * (D * D);
@@ -301,7 +319,8 @@ struct __align__(16) OutSmem {
     Rows rd;
     Item it;
 };
-__global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
+template <int R>
+__global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
                                                  const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
                                                  const float* __restrict__ states, float* __restrict__ o, const int32_t* gate) {
     if (gate_closed(gate)) return;
@@ -315,30 +334,30 @@ __global__ void __launch_bounds__(NT) out_kernel(const harts_la_tables_t tb, int
     if (!it.zero_state) load_state(s.s, states + ((size_t)it.gc * H + it.h) * (D * D));
     __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16, warp = threadIdx.x / 32;
-    Acc acc;
+    AccT<R> acc;
     clear(acc);
     mul_nt_causal(acc, s.q, s.k, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int r = 0; r < R; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const int t = 4 * ty + r, j = tx + 16 * c;
+            const int t = R * ty + r, j = tx + 16 * c;
             s.p[t * LD + j] = j <= t ? acc[r][c] * s.rd.decay(t, j) : 0.f;
         }
     __syncwarp();                                // a warp reads the rows it wrote
     clear(acc);
     if (!it.zero_state) mul_nn(acc, s.q, s.s, 0, D, ty, tx);
-    Acc in;                                      // the chunk's own share, summed by itself: it is small beside the state's
+    AccT<R> in;                                      // the chunk's own share, summed by itself: it is small beside the state's
     clear(in);
-    mul_nn(in, s.p, s.v, 0, 8 * warp, ty, tx);
-    mul_nn_diagonal(in, s.p, s.v, 8 * warp, ty, tx);
+    mul_nn(in, s.p, s.v, 0, 2 * R * warp, ty, tx);
+    mul_nn_diagonal(in, s.p, s.v, 2 * R * warp, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int code = s.rd.code[4 * ty + r];
+    for (int r = 0; r < R; r++) {
+        const int code = s.rd.code[R * ty + r];
         if (code >= 0)
 #pragma unroll
             for (int c = 0; c < 4; c++)
-                o[((size_t)code * H + it.h) * D + tx + 16 * c] = it.zero_state ? in[r][c] : __fmaf_rn(s.rd.eb[4 * ty + r], acc[r][c], in[r][c]);
+                o[((size_t)code * H + it.h) * D + tx + 16 * c] = it.zero_state ? in[r][c] : __fmaf_rn(s.rd.eb[R * ty + r], acc[r][c], in[r][c]);
     }
     }
 }
@@ -347,9 +366,10 @@ struct __align__(16) GradSmem {
     float q[TILE], k[TILE], v[TILE], dO[TILE], s[TILE], ds[TILE], p[TILE], dp[TILE];
     Rows rd;
     Item it;
-    float z[BT], part[NT / 32];
+    float z[BT], part[16];
 };
-__global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
+template <int R>
+__global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
                                                   const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
                                                   const float* __restrict__ dO, const float* __restrict__ states,
                                                   const float* __restrict__ ds_tiles, float* __restrict__ dq, float* __restrict__ dk_,
@@ -371,16 +391,16 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     if (has_ds) load_state(s.ds, ds_tiles + tile);
     __syncthreads();
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, warp = tid / 32, lane = tid & 31;
-    Acc acc, dacc;
+    AccT<R> acc, dacc;
     clear(acc);
     clear(dacc);
     mul_nt_causal(acc, s.q, s.k, ty, tx);
     mul_nt_causal(dacc, s.dO, s.v, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int r = 0; r < R; r++)
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const int t = 4 * ty + r, j = tx + 16 * c;
+            const int t = R * ty + r, j = tx + 16 * c;
             const float w = j <= t ? s.rd.decay(t, j) : 0.f;
             s.p[t * LD + j] = j <= t ? acc[r][c] * w : 0.f;
             s.dp[t * LD + j] = j <= t ? dacc[r][c] * w : 0.f;
@@ -388,16 +408,16 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     __syncthreads();
     const float gamma = s.rd.gamma;
     float g_part = 0.f;                          // this thread's share of <S_{c+1}, dS_{c+1}>
-    float z[4] = {0.f, 0.f, 0.f, 0.f};           // its share of q.dq - k.dk, per row
+    float z[R] = {};           // its share of q.dq - k.dk, per row
     // ---- dq = e^{b_t} dO S^T + dP K
     clear(acc);
     clear(dacc);
     if (has_s) mul_nt<4>(acc, s.dO, s.s, ty, tx);
-    mul_nn(dacc, s.dp, s.k, 0, 8 * warp, ty, tx);         // the chunk's own share by itself, as in out_kernel
-    mul_nn_diagonal(dacc, s.dp, s.k, 8 * warp, ty, tx);
+    mul_nn(dacc, s.dp, s.k, 0, 2 * R * warp, ty, tx);         // the chunk's own share by itself, as in out_kernel
+    mul_nn_diagonal(dacc, s.dp, s.k, 2 * R * warp, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int t = 4 * ty + r, code = s.rd.code[t];
+    for (int r = 0; r < R; r++) {
+        const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const float x = has_s ? __fmaf_rn(s.rd.eb[t], acc[r][c], dacc[r][c]) : dacc[r][c];
@@ -409,11 +429,11 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     clear(acc);
     clear(dacc);
     if (has_ds) mul_nt<4>(acc, s.v, s.ds, ty, tx);
-    mul_tn_diagonal(dacc, s.dp, s.q, 8 * warp, ty, tx);
-    mul_tn(dacc, s.dp, s.q, 8 * warp + 8, ty, tx);
+    mul_tn_diagonal(dacc, s.dp, s.q, 2 * R * warp, ty, tx);
+    mul_tn(dacc, s.dp, s.q, 2 * R * warp + 2 * R, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int t = 4 * ty + r, code = s.rd.code[t];
+    for (int r = 0; r < R; r++) {
+        const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const float kv = s.k[t * LD + tx + 16 * c], inter = has_ds ? acc[r][c] * s.rd.w[t] : 0.f, x = dacc[r][c] + inter;
@@ -427,11 +447,11 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     clear(acc);
     clear(dacc);
     if (has_ds) mul_nn(acc, s.k, s.ds, 0, D, ty, tx);
-    mul_tn_diagonal(dacc, s.p, s.dO, 8 * warp, ty, tx);
-    mul_tn(dacc, s.p, s.dO, 8 * warp + 8, ty, tx);
+    mul_tn_diagonal(dacc, s.p, s.dO, 2 * R * warp, ty, tx);
+    mul_tn(dacc, s.p, s.dO, 2 * R * warp + 2 * R, ty, tx);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int t = 4 * ty + r, code = s.rd.code[t];
+    for (int r = 0; r < R; r++) {
+        const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const float x = has_ds ? __fmaf_rn(s.rd.w[t], acc[r][c], dacc[r][c]) : dacc[r][c];
@@ -442,17 +462,17 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
     // ---- dg_t = sum_{tau>=t} z_tau + e^{b_n} <S_c, dS> + sum_j k_j . (w_j dS v_j), every sum in a fixed order
     if (has_s && has_ds) {
         float dot = 0.f;
-        for (int e = tid; e < D * D; e += NT) dot += s.s[(e >> 6) * LD + (e & 63)] * s.ds[(e >> 6) * LD + (e & 63)];
+        for (int e = tid; e < D * D; e += 1024 / R) dot += s.s[(e >> 6) * LD + (e & 63)] * s.ds[(e >> 6) * LD + (e & 63)];
         g_part += gamma * dot;
     }
 #pragma unroll
     for (int o_ = 16; o_ > 0; o_ >>= 1) g_part += __shfl_xor_sync(~0u, g_part, o_);
     if (lane == 0) s.part[warp] = g_part;
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
+    for (int r = 0; r < R; r++) {
 #pragma unroll
         for (int o_ = 8; o_ > 0; o_ >>= 1) z[r] += __shfl_xor_sync(~0u, z[r], o_);
-        if (tx == 0) s.z[4 * ty + r] = z[r];
+        if (tx == 0) s.z[R * ty + r] = z[r];
     }
     __syncthreads();
     if (warp == 0) {
@@ -467,7 +487,7 @@ __global__ void __launch_bounds__(NT, 1) grad_kernel(const harts_la_tables_t tb,
         }
         const float half = __shfl_sync(~0u, hi, 0);
 #pragma unroll
-        for (int w = 0; w < NT / 32; w++) G += s.part[w];
+        for (int w = 0; w < 32 / R; w++) G += s.part[w];
         const float out[2] = {lo + half + G, hi + G};
 #pragma unroll
         for (int r = 0; r < 2; r++) {
@@ -501,10 +521,15 @@ int32_t f32_fwd(const FwdArgs& a, float* extra, const int32_t* range, int32_t n)
     for (int32_t r = 0; r < n; r++)
         if (range[r] < range[r + 1])
             walk_kernel<false><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, states, gammas, a.slots, nullptr, gate);
-    if (cudaFuncSetAttribute(out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(OutSmem)) != cudaSuccess) return HARTS_ECUDA;
-    out_kernel<<<grid_of(a.tb, a.H, OUT_PER_SM), NT, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g,
-                                                        states, (float*)a.o, gate);
-    return done();
+    // an item a CTA: sixteen warps hide its latency (13 items 16.4 -> 13.4 us); more: two CTAs of eight warps an SM, whose 4 x 4 outputs a
+    // thread read shared memory less (796 items 55 us, 71 with sixteen)
+    auto outputs = [&](auto kernel, int threads) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(OutSmem)) != cudaSuccess) return HARTS_ECUDA;
+        kernel<<<grid_of(a.tb, a.H, OUT_PER_SM), threads, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k,
+                                                                                       (const float*)a.v, a.g, states, (float*)a.o, gate);
+        return done();
+    };
+    return (int64_t)a.tb.n_chunks * a.H <= sm_count() ? outputs(out_kernel<2>, 512) : outputs(out_kernel<4>, 256);
 }
 
 int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n) {
@@ -518,8 +543,8 @@ int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n)
     for (int32_t r = n - 1; r >= 0; r--)
         if (range[r] < range[r + 1])
             walk_kernel<true><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, tiles, gammas, nullptr, ds0, gate);
-    if (cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem)) != cudaSuccess) return HARTS_ECUDA;
-    grad_kernel<<<grid_of(a.tb, a.H, GRAD_PER_SM), NT, sizeof(GradSmem), a.stream>>>(
+    if (cudaFuncSetAttribute(grad_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem)) != cudaSuccess) return HARTS_ECUDA;
+    grad_kernel<2><<<grid_of(a.tb, a.H, GRAD_PER_SM), 512, sizeof(GradSmem), a.stream>>>(
         a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g, (const float*)a.dO, (const float*)a.chunk_states,
         tiles, (float*)a.dq, (float*)a.dk_, (float*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv), (float*)(base + sl.rg), gate);
     return done();
