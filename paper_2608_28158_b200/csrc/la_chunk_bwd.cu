@@ -68,6 +68,7 @@ chunk_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                  __nv_bfloat16* __restrict__ dk_, __nv_bfloat16* __restrict__ dv_, float* __restrict__ dg,
                  float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg, const float* __restrict__ dots,
                  int* status, const int32_t* gate) {
+    after_previous();
     if (gate_closed(gate)) return;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -464,7 +465,7 @@ int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) {
     char* base = static_cast<char*>(a.scratch);
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
     const int grid = (int)(n < sm_count() ? n : sm_count());
-    chunk_bwd_kernel<<<grid, NT, Smem::bytes + 1024, a.stream>>>(
+    launch_after(chunk_bwd_kernel, grid, NT, Smem::bytes + 1024, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, mq, mk, mv, mdo, ms, mds, mdq, mdk, mdv, (const __nv_bfloat16*)a.q,
         (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq,
         (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv),

@@ -44,6 +44,7 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
                  const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                  const __nv_bfloat16* __restrict__ v, const float* __restrict__ g, __nv_bfloat16* __restrict__ o,
                  int* status, const int32_t* gate) {
+    after_previous();
     if (gate_closed(gate)) return;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -277,7 +278,7 @@ int32_t chunk_fwd(const FwdArgs& a) {
         return HARTS_ECUDA;
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
     const int grid = (int)(n < 2 * sm_count() ? n : 2 * sm_count());
-    chunk_fwd_kernel<<<grid, NT, Smem::bytes + 1024, a.stream>>>(
+    launch_after(chunk_fwd_kernel, grid, NT, Smem::bytes + 1024, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, mq, mk, mv, mcs, mo, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (__nv_bfloat16*)a.o, a.dev_status, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;

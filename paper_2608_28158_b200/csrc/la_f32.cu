@@ -220,6 +220,8 @@ template <bool BWD>
 __global__ void __launch_bounds__(NT, 5) outer_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ a,
                                                    const float* __restrict__ b, const float* __restrict__ g, float* __restrict__ sums,
                                                    float* __restrict__ gammas, const int32_t* gate) {
+    let_next_launch();
+    after_previous();
     if (gate_closed(gate)) return;
     __shared__ OuterSmem s;
     for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
@@ -259,6 +261,8 @@ constexpr int AHEAD = 8;                         // sums in flight per thread
 template <bool BWD>
 __global__ void __launch_bounds__(NT) walk_kernel(const harts_la_tables_t tb, int seq_lo, int H, float* tiles, const float* gammas,
                                                   float* slots, float* ds0, const int32_t* gate) {
+    let_next_launch();
+    after_previous();
     if (gate_closed(gate)) return;
     const int part = blockIdx.x & 3, item = blockIdx.x >> 2, h = item % H;
     const int pos = seq_lo + item / H, seq = tb.seq_order ? tb.seq_order[pos] : pos;
@@ -323,6 +327,8 @@ template <int R>
 __global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const float* __restrict__ q,
                                                  const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
                                                  const float* __restrict__ states, float* __restrict__ o, const int32_t* gate) {
+    let_next_launch();
+    after_previous();
     if (gate_closed(gate)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OutSmem& s = *reinterpret_cast<OutSmem*>(smem_raw);
@@ -375,6 +381,8 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
                                                   const float* __restrict__ ds_tiles, float* __restrict__ dq, float* __restrict__ dk_,
                                                   float* __restrict__ dv_, float* __restrict__ dg, float* __restrict__ rk,
                                                   float* __restrict__ rv, float* __restrict__ rg, const int32_t* gate) {
+    let_next_launch();
+    after_previous();
     if (gate_closed(gate)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
@@ -520,13 +528,13 @@ int32_t f32_fwd(const FwdArgs& a, float* extra, const int32_t* range, int32_t n)
     outer_kernel<false><<<grid_of(a.tb, a.H, OUTER_PER_SM), NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.k, (const float*)a.v, a.g, states, gammas, gate);
     for (int32_t r = 0; r < n; r++)
         if (range[r] < range[r + 1])
-            walk_kernel<false><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, states, gammas, a.slots, nullptr, gate);
+            launch_after(walk_kernel<false>, (range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream, a.tb, range[r], a.H, states, gammas, a.slots, nullptr, gate);
     // an item a CTA: sixteen warps hide its latency (13 items 16.4 -> 13.4 us); more: two CTAs of eight warps an SM, whose 4 x 4 outputs a
     // thread read shared memory less (796 items 55 us, 71 with sixteen)
     auto outputs = [&](auto kernel, int threads) {
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(OutSmem)) != cudaSuccess) return HARTS_ECUDA;
-        kernel<<<grid_of(a.tb, a.H, OUT_PER_SM), threads, sizeof(OutSmem), a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k,
-                                                                                       (const float*)a.v, a.g, states, (float*)a.o, gate);
+        launch_after(kernel, grid_of(a.tb, a.H, OUT_PER_SM), threads, sizeof(OutSmem), a.stream, a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k,
+                     (const float*)a.v, a.g, states, (float*)a.o, gate);
         return done();
     };
     return (int64_t)a.tb.n_chunks * a.H <= sm_count() ? outputs(out_kernel<2>, 512) : outputs(out_kernel<4>, 256);
@@ -542,9 +550,9 @@ int32_t f32_bwd(const BwdArgs& a, float* extra, const int32_t* range, int32_t n)
     outer_kernel<true><<<grid_of(a.tb, a.H, OUTER_PER_SM), NT, 0, a.stream>>>(a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.dO, a.g, tiles, gammas, gate);
     for (int32_t r = n - 1; r >= 0; r--)
         if (range[r] < range[r + 1])
-            walk_kernel<true><<<(range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream>>>(a.tb, range[r], a.H, tiles, gammas, nullptr, ds0, gate);
+            launch_after(walk_kernel<true>, (range[r + 1] - range[r]) * a.H * 4, NT, 0, a.stream, a.tb, range[r], a.H, tiles, gammas, nullptr, ds0, gate);
     if (cudaFuncSetAttribute(grad_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem)) != cudaSuccess) return HARTS_ECUDA;
-    grad_kernel<2><<<grid_of(a.tb, a.H, GRAD_PER_SM), 512, sizeof(GradSmem), a.stream>>>(
+    launch_after(grad_kernel<2>, grid_of(a.tb, a.H, GRAD_PER_SM), 512, sizeof(GradSmem), a.stream,
         a.tb, lo, hi, a.H, (const float*)a.q, (const float*)a.k, (const float*)a.v, a.g, (const float*)a.dO, (const float*)a.chunk_states,
         tiles, (float*)a.dq, (float*)a.dk_, (float*)a.dv_, a.dg, (float*)(base + sl.rk), (float*)(base + sl.rv), (float*)(base + sl.rg), gate);
     return done();

@@ -437,6 +437,7 @@ __device__ __forceinline__ void add4<__nv_bfloat16>(__nv_bfloat16* p, const floa
 template <typename T>
 __global__ void replay_reduce_kernel(harts_la_tables_t tb, int H, int DK, int DV, T* dk_, T* dv_, float* dg,
                                      const float* rk, const float* rv, const float* rg, int n_items) {
+    after_previous();
     const int per = (DK + DV) / 4;
     const int item = blockIdx.x * (blockDim.x / per) + threadIdx.x / per, part = threadIdx.x % per;
     if (item >= n_items) return;
@@ -586,10 +587,10 @@ int32_t replay_reduce(const harts_la_tables_t& tb, void* dk_, void* dv_, float* 
     if ((dk + dv) % 4 != 0 || dk % 4 != 0 || threads % per != 0) return HARTS_EUNSUPPORTED;
     const int blocks = (n + threads / per - 1) / (threads / per);
     if (dtype == HARTS_FP32)
-        replay_reduce_kernel<float><<<blocks, threads, 0, stream>>>(tb, H, dk, dv, (float*)dk_, (float*)dv_, dg, rk, rv, rg, n);
+        launch_after(replay_reduce_kernel<float>, blocks, threads, 0, stream, tb, H, dk, dv, (float*)dk_, (float*)dv_, dg, rk, rv, rg, n);
     else
-        replay_reduce_kernel<__nv_bfloat16><<<blocks, threads, 0, stream>>>(tb, H, dk, dv, (__nv_bfloat16*)dk_,
-                                                                            (__nv_bfloat16*)dv_, dg, rk, rv, rg, n);
+        launch_after(replay_reduce_kernel<__nv_bfloat16>, blocks, threads, 0, stream, tb, H, dk, dv, (__nv_bfloat16*)dk_,
+                     (__nv_bfloat16*)dv_, dg, rk, rv, rg, n);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
