@@ -82,6 +82,7 @@ attn_dq_kernel(Index ix, int Hq, int G, float scale, const __grid_constant__ CUt
                const __grid_constant__ CUtensorMap map_v,
                const float* __restrict__ lse, const float* __restrict__ delta, __nv_bfloat16* __restrict__ dq,
                int* status) {
+    after_previous();
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     unsigned char* sQ = smem + SmemQ::q;
@@ -382,8 +383,7 @@ int32_t attn_bwd_launch(const int32_t* hi, const int32_t* di, const void* q, con
     if (cut && (rc = attn_split_reduce(ix, Hkv, split, dk_, dv_, st)) != HARTS_OK) return rc;
     const long long n_work = (long long)ix.n_q_items * Hq;
     const int grid = (int)(n_work < sm_count() ? n_work : sm_count());
-    attn_dq_kernel<<<grid, NT, SmemQ::bytes + 1024, st>>>(ix, Hq, Hq / Hkv, scale, mq, mdo, mk, mv, lse, delta,
-                                                         (__nv_bfloat16*)dq, status);
+    launch_after(attn_dq_kernel, grid, NT, SmemQ::bytes + 1024, st, ix, Hq, Hq / Hkv, scale, mq, mdo, mk, mv, lse, delta, (__nv_bfloat16*)dq, status);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

@@ -61,6 +61,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
                 const __grid_constant__ CUtensorMap map_v, const float* __restrict__ lse,
                 const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk_, __nv_bfloat16* __restrict__ dv_,
                 int* ticket, int* status, SplitTable split) {
+    after_previous();
     extern __shared__ __align__(1024) unsigned char smem[];       // no static shared memory: the dynamic window starts 1024-byte aligned
     unsigned char* sK = smem + Smem::k;
     unsigned char* sV = smem + Smem::v;
@@ -469,9 +470,8 @@ int32_t attn_dkv_launch(const Index& ix, int n_rows, const void* q, const void* 
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::bytes) != cudaSuccess) return HARTS_ECUDA;
     const long long n_work = (long long)ix.n_kv_items * Hkv;
     const int grid = split || n_work > sm_count() ? sm_count() : (int)n_work;
-    kernel<<<grid, NT, Smem::bytes, st>>>(ix, Hq, Hkv, Hq / Hkv, scale, mq, mdo, mk, mv, lse,
-                                                          delta, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_, ticket, status,
-                                                 split ? *split : SplitTable{});
+    launch_after(kernel, grid, NT, Smem::bytes, st, ix, Hq, Hkv, Hq / Hkv, scale, mq, mdo, mk, mv, lse, delta, (__nv_bfloat16*)dk_,
+                 (__nv_bfloat16*)dv_, ticket, status, split ? *split : SplitTable{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

@@ -25,6 +25,7 @@ constexpr int LEAST_UNIT = 8;          // query tiles
 
 // One CTA of 1024 threads, a warp per item.
 __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, int sms, SplitTable t) {
+    after_previous();
     __shared__ int total, slots, len;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) total = 0;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(1024) split_kernel(Index ix, int G, int Hkv, i
 // dV and dK of the items that were cut: their units' sums in unit order, eight CTAs per (item, key head).
 __global__ void __launch_bounds__(256) reduce_kernel(Index ix, int Hkv, SplitTable t, __nv_bfloat16* __restrict__ dk_,
                                                      __nv_bfloat16* __restrict__ dv_) {
+    after_previous();
     const int part = blockIdx.x & 7, i = (blockIdx.x >> 3) / Hkv, hk = (blockIdx.x >> 3) % Hkv;
     const SplitItem it = t.item[i];
     if (it.n_units < 2) return;
@@ -200,11 +202,11 @@ bool attn_split_table(const Index& ix, const int32_t* hi, int G, int Hkv, void* 
     return t->cap_slots > 1 && worth_cutting(hi, G, Hkv, sm_count(), t->cap_slots);
 }
 int32_t attn_split_launch(const Index& ix, int G, int Hkv, const SplitTable& t, cudaStream_t st) {
-    split_kernel<<<1, 1024, 0, st>>>(ix, G, Hkv, sm_count(), t);
+    launch_after(split_kernel, 1, 1024, 0, st, ix, G, Hkv, sm_count(), t);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 int32_t attn_split_reduce(const Index& ix, int Hkv, const SplitTable& t, void* dk_, void* dv_, cudaStream_t st) {
-    reduce_kernel<<<ix.n_kv_items * Hkv * 8, 256, 0, st>>>(ix, Hkv, t, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_);
+    launch_after(reduce_kernel, ix.n_kv_items * Hkv * 8, 256, 0, st, ix, Hkv, t, (__nv_bfloat16*)dk_, (__nv_bfloat16*)dv_);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

@@ -715,6 +715,7 @@ __global__ void __launch_bounds__(NT, 2)
 gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
                     const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                     __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ chunk_states, const int32_t* gate) {
+    after_previous();
     if (gate_closed(gate)) return;
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sQ = sm + SharedC::q, *sK = sm + SharedC::k, *sQa = sm + SharedC::qa, *sKa = sm + SharedC::ka,
@@ -862,6 +863,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                   const __nv_bfloat16* __restrict__ ds_tiles, const float* __restrict__ dots,
                   float* __restrict__ ds0, float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg,
                   const int32_t* gate, int* status, int* ds0_flags, int* ticket, const RoundOrder rounds) {
+    after_previous();
     if (gate_closed(gate)) return;
     constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE, CHUNKS = MODE == CHUNKS_MODE;
     __shared__ int s_item, s_dead;
@@ -1422,7 +1424,7 @@ int32_t gk_chunk_fwd(const FwdArgs& a) {
     if (cudaFuncSetAttribute(gk_chunk_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedC::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
-    gk_chunk_fwd_kernel<<<(int)(n < 2 * sm_count() ? n : 2 * sm_count()), NT, SharedC::bytes, a.stream>>>(
+    launch_after(gk_chunk_fwd_kernel, (int)(n < 2 * sm_count() ? n : 2 * sm_count()), NT, SharedC::bytes, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (__nv_bfloat16*)a.o, (const __nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
@@ -1434,7 +1436,7 @@ int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) 
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
     const GkScratchLayout sl = gk_scratch_layout(a.tb, a.H, a.dk, a.dv);
     char* base = static_cast<char*>(a.scratch);
-    gk_mma_bwd_kernel<CHUNKS_MODE><<<(int)(n < sm_count() ? n : sm_count()), NT, SharedB::bytes, a.stream>>>(
+    launch_after(gk_mma_bwd_kernel<CHUNKS_MODE>, (int)(n < sm_count() ? n : sm_count()), NT, SharedB::bytes, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
         (const __nv_bfloat16*)a.chunk_states, (const __nv_bfloat16*)ds_tiles, dots, (float*)(base + sl.ds0), (float*)(base + sl.rk),
