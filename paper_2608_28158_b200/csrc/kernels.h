@@ -162,7 +162,8 @@ int32_t scan_fwd(const FwdArgs& a, int* flags, const RoundOrder& order);      //
 int32_t scan_bwd(const BwdArgs& a, void* ds_tiles, float* dots, int* flags, const RoundOrder& order);   // their gradients, ds0 hand-off
 int32_t chunk_fwd(const FwdArgs& a);                           // la_chunk_fwd.cu
 int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);     // la_chunk_bwd.cu
-// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs, with fewer than four chunks a sequence up to 1,152 pairs.
+// Taken up to 28,672 (chunk, head) items and 640 (sequence, head) pairs, with fewer than four chunks a sequence up to 128 pairs,
+// or 1,152 where two sequences and more start from each exported state (fans).
 // The walk kernels (la_tc_*.cu) move 240 KB per item in a whole step, this path 430 KB: with enough chains to fill the GPU the walk
 // wins, with few the chain of its 3-6 us chunks is what takes the time.  Walk / chunk-parallel, time of a step (of the forward
 // alone), 46 forests both ways with cold inputs:
@@ -176,12 +177,13 @@ int32_t chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots);   
 //   further out the walk wins: branchy 9,728 items, 832 pairs 0.97 (0.86); 24,768 items, 2,328 pairs 0.89 (0.76); agentic 51,152
 //     items, 1,264 pairs 0.94 (0.90); 6,949 chunks of replay fans x 16 heads 0.65
 // The line depends on the tables' totals only, so that a round issued alone takes the path of the whole.
-constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640, CHUNK_PARALLEL_FANS = 1152;
+constexpr int64_t CHUNK_PARALLEL_MAX = 28672, CHUNK_PARALLEL_CHAINS = 640, CHUNK_PARALLEL_FANS = 1152, CHUNK_PARALLEL_FEW = 128;
 inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
     const int64_t chains = (int64_t)tb.n_seq * H;
+    const bool fans = tb.n_slots > 0 && tb.n_seq >= 2 * (int64_t)tb.n_slots;
     return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 &&
            (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
-           chains <= (tb.n_chunks >= 4 * (int64_t)tb.n_seq ? CHUNK_PARALLEL_CHAINS : CHUNK_PARALLEL_FANS);
+           chains <= (tb.n_chunks >= 4 * (int64_t)tb.n_seq ? CHUNK_PARALLEL_CHAINS : fans ? CHUNK_PARALLEL_FANS : CHUNK_PARALLEL_FEW);
 }
 // the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then
 // <S_c, dS_c> in parts, fp32 [n_chunks, H, 4 blocks of 32 columns, dk], then the scan's ticket and counters
