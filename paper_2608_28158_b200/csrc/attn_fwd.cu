@@ -31,7 +31,7 @@ using namespace tc;
 
 using namespace attn;
 constexpr int NS = 128;                 // softmax threads (4 warps), thread = query row = tensor-memory lane
-constexpr int NT = NS + 64;             // plus one warp whose first lane issues the MMAs and one whose first lane issues the TMA loads
+constexpr int NT = NS + 64;             // plus one warp that issues the MMAs and one whose first lane issues the TMA loads
 constexpr int Q_BYTES = BQ * D * 2;     // 32 KB: two panels [128 rows][64 columns]
 constexpr int KV_BYTES = BK * D * 2;    // 16 KB: two panels [64 rows][64 columns]
 constexpr int COL_S = 0, COL_O = 128, TMEM_COLS = 256;     // S / P of tile n at COL_S + 64 (n & 1)

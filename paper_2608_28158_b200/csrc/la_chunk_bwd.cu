@@ -8,10 +8,10 @@
 // tcgen05 MMAs, every product transposed (tensor-memory lane = feature, column = row of the chunk); the 24 MMAs of the
 // three state products do not need P or dP and run under the decay masking, so twelve are left after it.  One CTA per SM:
 // eight 64-column accumulators take all 512 tensor-memory columns, tiles and staging 198 KB of shared memory.  Sixteen
-// compute warps, one warp whose first lane issues every TMA and MMA, one that prepares the next items and finishes dg.
+// compute warps, one warp that issues every TMA (first lane) and MMA (an elected lane), one that prepares the next items and finishes dg.
 // The dS of a sequence's last chunk and the state of a sequence that starts from zero are zero: not read, not multiplied.
-// What bounds it: the dependent phases of one item (4.7 us; 178 KB of traffic would take 4.0): 0.54 ms for 1,047 chunks x 16
-// heads.  Every wait is bounded.
+// What bounds it: the dependent phases of one item (4.5 us; 178 KB of traffic would take 4.0): 0.77 ms for 1,595 chunks x 16
+// heads (0.80 with the MMAs issued by the first lane).  Every wait is bounded.
 #include "chunk_item.cuh"
 
 namespace harts {

@@ -3,7 +3,7 @@
 //     A = Q K^T    P = A .* e^{b_t-b_j} [j<=t]    o_t = P V + e^{b_t} Q S_c
 // tcgen05 MMAs with accumulators in tensor memory (O^T: lane = feature, column = row of the chunk); q, k, v and the
 // state tile arrive by TMA.  Two CTAs per SM (106 KB of shared memory, 256 tensor-memory columns each), 8 compute warps,
-// one warp whose first lane issues every TMA and MMA, one that prepares the next items (record, gates, row ids).  The
+// one warp that issues every TMA (first lane) and MMA (an elected lane), one that prepares the next items (record, gates, row ids).  The
 // state's product does not need P, so it runs under the decay masking; only four MMAs are left after it.
 // What bounds it: 96 KB of traffic per item (80 read, 16 written); 1,047 chunks x 16 heads take 0.25 ms = 6.6 TB/s.
 // Every wait is bounded.

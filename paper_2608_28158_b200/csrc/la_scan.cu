@@ -16,8 +16,8 @@
 // MMA warp, the state warps, and a store warp (TMA).  A (sequence, head) is one item of NV = 128 state columns, or 2 of 64,
 // or 4 of 32 (launch_sliced): the columns do not interact, so the split does not change any result.  All rounds run in one
 // launch (scan_fwd below).
-// Measured, cold inputs: 1.1 us per step of the longest path while the chains leave SMs idle, 1.2 to 1.3 backward (17,695 tokens x
-// 4 heads, 68 steps: 77 and 82 us; 65,521 x 16, 228 steps: 244 and 294); with 96 chains of 100,003 tokens x 16 heads 4.9 TB/s
+// Measured, cold inputs: 1.05 us per step of the longest path while the chains leave SMs idle, 1.05 to 1.3 backward (17,695 tokens x
+// 4 heads, 68 steps: 72 and 71 us; 65,521 x 16, 228 steps: 244 and 294); with 96 chains of 100,003 tokens x 16 heads 4.9 TB/s
 // forward (345 us), 6.1 backward (470 us).
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -610,7 +610,8 @@ int32_t launch(const Launch& x) {
 }
 // The narrower the slices, the shorter a step of the walk and the more often k is read: as narrow as leaves the chains of the
 // (first) round at most one CTA per SM, but never 128 columns in the backward, where a state thread multiplies its columns with
-// S_c besides.  Device time in us with 32 / 64 / 128 columns, cold inputs: 17,695 tokens x 4 heads (4 chains in
+// S_c besides.  Device time in us with 32 / 64 / 128 columns, cold inputs (before slots were published by the store warp and
+// gradients read coalesced: 72 and 71 now where 78 and 82 stand): 17,695 tokens x 4 heads (4 chains in
 // the first round) forward 78 / 93 / 141, backward 82 / 86 / 187; 65,521 x 16 (64 chains) 298 / 244 / 289, 406 / 293 / 451;
 // 100,003 x 16 (96 chains) 426 / 359 / 345, 606 / 468 / 561; 149,270 x 12 (96 chains) forward 64: 401, 128: 400, backward 546, 573.
 template <bool BWD>
