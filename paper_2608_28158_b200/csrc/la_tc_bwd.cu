@@ -79,8 +79,15 @@ struct Misc {
     int item;                // all rounds in one launch: the work item thread 0 drew
     int head;
     SeqInfo seq;
+    // one launch per round: the next work item, looked up by the auxiliary warp under the last chunk of this one
+    int next_head, next_id, id;
+    SeqInfo next_seq;
 };
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
+}
 __device__ __forceinline__ SeqInfo seq_info(const harts_la_tables_t& tb, int seq) {
     SeqInfo s;
     s.own_begin = tb.seq_own_begin[seq];
@@ -191,8 +198,17 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     uint32_t ph_tiles = 0, ph_a = 0, ph_o = 0;
     bool tiles_pending = false, gave_up = false;   // tiles_pending is kept by the issuing thread only
     const int G = gridDim.x;
+    // one launch per round: item of a tier; n_items or more: none
+    auto dealt = [&](int tier) { return (tier & 1) ? tier * G + (G - 1 - (int)blockIdx.x) : tier * G + (int)blockIdx.x; };
+    int cur = 0;                                   // which of the two records of row data the current chunk reads
     for (int tier = 0;; tier++) {
-    int item, seq_pos;
+    // The order of one launch per round is known beforehand: the auxiliary warp looks up the next sequence and prepares its
+    // first chunk's row data under the last chunk of the current one, and asks the L2 for its rows and state.  Looked up at
+    // the switch, those are four dependent trips to memory (3,000 of the 23,500 cycles of a replayed tail of one or two chunks)
+    // with nothing else in flight: 6,949 chunks of such tails x 16 heads 6.7 -> 6.32 ms, 6.22 with the L2 asked.  A ticket
+    // (all rounds in one launch) is still drawn at the switch: held early, it would keep an item from a CTA that is free.
+    const bool ahead = !ONE_LAUNCH && tier > 0;
+    int item, seq_pos = 0;
     if constexpr (ONE_LAUNCH) {
         // all rounds in one launch: whichever CTA is free draws the next item; the order is last round first, and
         // inside a round the plan's order (longest sequence first)
@@ -210,18 +226,24 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
     } else {
         if (tier * G >= n_items) break;
-        item = (tier & 1) ? tier * G + (G - 1 - (int)blockIdx.x) : tier * G + (int)blockIdx.x;
+        item = dealt(tier);
         if (item >= n_items) continue;
         seq_pos = seq_lo + item / H;
     }
-    const int seq = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
     // the item's record lives in shared memory and is read where it is needed: held in registers over the whole walk it
     // would push the kernel over its register budget
-    if (is_issuer) tma_store_wait_read();          // the previous item's dS0 has left the state tiles
     __syncthreads();                               // the previous item's last readers of the record are through
     if (tid == 0) {
-        m.seq = seq_info(tb, seq);
-        m.head = item % H;
+        if (ahead) {
+            m.seq = m.next_seq;
+            m.head = m.next_head;
+            m.id = m.next_id;
+        } else {
+            const int id = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+            m.seq = seq_info(tb, id);
+            m.head = item % H;
+            m.id = id;
+        }
     }
     __syncthreads();
     const SeqInfo& s = m.seq;
@@ -272,7 +294,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             }
     };
     // Row codes and g of chunk c for rows `lane` and `lane + 32` (the auxiliary warp prepares a chunk's row data on its own).
-    auto load_rows = [&](int c, int (&code)[2], float (&gv)[2]) {
+    auto load_rows = [&](const SeqInfo& s, int h, int c, int (&code)[2], float (&gv)[2]) {
 #pragma unroll
         for (int r = 0; r < 2; r++) {
             code[r] = -1;
@@ -309,23 +331,43 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         if (lane == 0) rd.gamma = ex2(bn * LOG2E);
     };
 
+    // The rows of a chunk that will be fetched at its own start (replayed tails) or at the switch to the next item: into the L2,
+    // while the current chunk runs.
+    auto warm_rows = [&](int h, const int (&code)[2]) {
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            if (code[r] == -1) continue;
+            const size_t off = ((size_t)(code[r] >= 0 ? code[r] : -2 - code[r]) * H + h) * D;
+            for (int half = 0; half < 2; half++) {
+                prefetch_l2(k + off + half * 64);
+                prefetch_l2(v + off + half * 64);
+                if (code[r] < 0) continue;
+                prefetch_l2(q + off + half * 64);
+                prefetch_l2(dO + off + half * 64);
+            }
+        }
+    };
+
     const bool gather_first = s.n_replay > 0;
     int next_req = s.req_hi - 1;
     // chunk index of the next exported boundary on the way down (kept in a register: no global load per chunk)
     int next_boundary = next_req >= s.req_lo ? tb.slot_chunk[next_req] : -1;
     int aux_req = next_req, aux_boundary = next_boundary;    // the auxiliary warp's own walk over the boundaries
-    if (is_issuer) issue_tiles(s.n_chunks - 1, !(gather_first && s.n_chunks == 1));
+    if (is_issuer) {
+        tma_store_wait_read();                     // the previous item's dS0 has left the state tiles
+        issue_tiles(s.n_chunks - 1, !(gather_first && s.n_chunks == 1));
+    }
     int nx_code[2];
     float nx_g[2];
-    if (is_aux) {
-        load_rows(s.n_chunks - 1, nx_code, nx_g);
-        store_rows(m.rows[0], nx_code, nx_g);
+    if (!ahead) {
+        if (is_aux) {
+            load_rows(s, h, s.n_chunks - 1, nx_code, nx_g);
+            store_rows(m.rows[cur], nx_code, nx_g);
+        }
+        tc_fence_before();
+        __syncthreads();                          // row data of the first chunk visible
+        tc_fence_after();
     }
-    int cur = 0;
-
-    tc_fence_before();
-    __syncthreads();                              // row data of the first chunk visible
-    tc_fence_after();
 
     // Two block-wide barriers per chunk: (A) before the MMA batch, (B) at the end of the epilogue.  After (B) the
     // compute warps go straight on to the next chunk, while the issuing thread sends the staged outputs off and the
@@ -369,7 +411,21 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
         if (got_tiles) ph_tiles ^= 1;
         if (is_aux) {
-            load_rows(c - 1, nx_code, nx_g);              // next chunk's rows and g, in flight during this chunk
+            if (ONE_LAUNCH || c > 0) {
+                load_rows(s, h, c - 1, nx_code, nx_g);    // next chunk's rows and g, in flight during this chunk
+                if (c == 1 && gather_first) warm_rows(h, nx_code);
+            } else if (const int next = dealt(tier + 1); next < n_items) {
+                if (lane == 0) {
+                    const int id = tb.seq_order ? tb.seq_order[seq_lo + next / H] : seq_lo + next / H;
+                    m.next_seq = seq_info(tb, id);
+                    m.next_head = next % H;
+                    m.next_id = id;
+                }
+                __syncwarp();
+                load_rows(m.next_seq, m.next_head, m.next_seq.n_chunks - 1, nx_code, nx_g);
+                warm_rows(m.next_head, nx_code);
+                if (lane < 2) tma_prefetch_3d(&map_cs, lane * 64, 0, (m.next_seq.chunk_base + m.next_seq.n_chunks - 1) * H + m.next_head);
+            }
             if (aux_boundary == c + 1) {                  // the boundary this chunk's dS pass is crossing
                 aux_req--;
                 aux_boundary = aux_req >= s.req_lo ? tb.slot_chunk[aux_req] : -1;
@@ -554,7 +610,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             }
             __syncwarp();
         }
-        if (is_aux && c > 0) store_rows(m.rows[cur ^ 1], nx_code, nx_g);   // visible to the others at barrier (B)
+        if (is_aux && (c > 0 || (!ONE_LAUNCH && dealt(tier + 1) < n_items))) store_rows(m.rows[cur ^ 1], nx_code, nx_g);   // visible to the others at barrier (B)
         if (is_compute) {
             const int c4 = lane & 3, Lq = (warp & 3) * 32, t0 = grp * 16;
             Frag fr;
@@ -735,12 +791,12 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
         __syncthreads();
         if (is_issuer) {
-            for (int p = 0; p < 4; p++) tma_store_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, seq * H + h);
+            for (int p = 0; p < 4; p++) tma_store_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, m.id * H + h);
             tma_store_commit();
         }
     }
     if (ONE_LAUNCH && is_compute && s.init_slot >= 0) {
-        float* dst = ds0 + ((size_t)seq * H + h) * state_elems + (size_t)L * D;
+        float* dst = ds0 + ((size_t)m.id * H + h) * state_elems + (size_t)L * D;
         uint32_t x[32];
         tmem_ld32(tm_lane + COL_DS + grp * 32, x);
         tmem_ld_wait();
@@ -752,7 +808,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         __threadfence();                           // this thread's part, before the flag that follows the barrier below
     }
     if (ONE_LAUNCH && s.init_slot >= 0) {           // publish: the gradient of this sequence's initial state is in place
-        if (!__syncthreads_or(m.dead) && tid == 0) flag_set(ds0_flags + (size_t)seq * H + h);
+        if (!__syncthreads_or(m.dead) && tid == 0) flag_set(ds0_flags + (size_t)m.id * H + h);
     }
     }   // work items
     const bool abandoned = __syncthreads_or(m.dead) != 0;
