@@ -128,6 +128,7 @@ int32_t harts_la_fwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
     const int32_t range[2] = {seq_lo, seq_hi};
     if (chunk_states && harts::f32_chunks(dk, dv, dtype)) return harts::f32_fwd(a, f32_extra(a.tb, chunk_states, H, dk, dv), range, 1);
+    if (harts::pipe_forward(*tb, H, dk, dv, dtype, flags)) return harts::pipe_fwd(a, nullptr, 0);
     if (chunk_states && harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) return chunk_parallel_fwd(a, range, 1);
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_fwd(a);
     return harts::fma_fwd(a);
@@ -190,6 +191,9 @@ int32_t harts_la_fwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
         }
         if (harts::f32_chunks(dk, dv, dtype))
             return harts::f32_fwd(a, f32_extra(tb, chunk_states, H, dk, dv), p->round_seq_ptr.data(), p->n_rounds);
+        if (harts::pipe_forward(tb, H, dk, dv, dtype, flags))
+            return harts::pipe_fwd(a, reinterpret_cast<int*>(static_cast<char*>(chunk_states) + harts::chunk_state_payload(tb, H, dk, dv, 2)),
+                                   p->round_seq_ptr[1] - p->round_seq_ptr[0]);
         if (harts::chunk_parallel(tb, H, dk, dv, dtype, flags))
             return chunk_parallel_fwd(a, p->round_seq_ptr.data(), p->n_rounds);
         int* fl = reinterpret_cast<int*>(static_cast<char*>(chunk_states) + harts::chunk_state_payload(tb, H, dk, dv, 2));

@@ -185,6 +185,19 @@ inline bool chunk_parallel(const harts_la_tables_t& tb, int32_t H, int32_t dk, i
            (int64_t)tb.n_chunks * H <= CHUNK_PARALLEL_MAX &&
            chains <= (tb.n_chunks >= 4 * (int64_t)tb.n_seq ? CHUNK_PARALLEL_CHAINS : fans ? CHUNK_PARALLEL_FANS : CHUNK_PARALLEL_FEW);
 }
+// The pipelined forward walk (la_pipe_fwd.cu) wherever sequences have four chunks and more on average and their (sequence, head) pairs
+// give every SM one, and in place of the synchronous walk also with fewer.  Time of a forward, other path / this one, cold inputs, 47
+// forests: agentic 192 pairs 1.07, 384 pairs 1.23, 688 1.84, 768 1.65, 3,360 1.19; branchy 314 pairs 1.26, 436 1.24, 480 1.39, 5,024
+// 1.35, 10,048 1.15.  With fewer pairs the chain of chunks decides, and the scan's 32-column slices take 0.55 us a step against 1.1:
+// agentic 172 pairs 0.90, 96 pairs 0.74, 24 pairs 0.56 (120 branchy pairs 0.84).  Sequences of one or two chunks are bound by their
+// start states, which the synchronous walk's two CTAs per SM overlap: replay fans, 17,088 pairs 0.97, 68,128 pairs 0.89.
+// The backward has a line of its own (chunk_parallel): the chunk states are the same whoever wrote them.
+constexpr int64_t PIPE_PAIRS = 192;
+inline bool pipe_forward(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv, int32_t dtype, uint32_t flags) {
+    return !(flags & HARTS_FLAG_FMA_KERNELS) && dtype == HARTS_BF16 && dk == 128 && dv == 128 && tb.n_chunks >= 4 * (int64_t)tb.n_seq &&
+           ((int64_t)tb.n_seq * H >= PIPE_PAIRS || !chunk_parallel(tb, H, dk, dv, dtype, flags));
+}
+int32_t pipe_fwd(const FwdArgs& a, int* flags, int first_round);
 // the boundary-state gradients of the chunk-parallel backward: bf16 [n_chunks, H, dk, dv] behind the flags, then
 // <S_c, dS_c> in parts, fp32 [n_chunks, H, 4 blocks of 32 columns, dk], then the scan's ticket and counters
 inline size_t ds_tiles_offset(const harts_la_tables_t& tb, int32_t H, int32_t dk, int32_t dv) {
