@@ -73,7 +73,9 @@ inline const int32_t* status_gate(uint32_t flags, const int32_t* dev_status) {
 }
 #ifdef __CUDACC__
 // A kernel that follows another one of the library in the same call is launched ahead of it (launch_after): its CTAs are on the
-// SMs, and it waits here, before it reads or writes anything, until that kernel is complete and its memory visible.  A launch
+// SMs, and it waits here until that kernel is complete and its memory visible: before it writes anything, and before it reads anything
+// but what the call was given (a call's first kernel is launched the ordinary way, so tables and inputs are complete).  Every CTA waits,
+// also one without work, so that a kernel is complete only when all before it are.  A launch
 // costs about a microsecond less so (nine kernels, 718 tokens x 1 head fp32: 77.6 -> 69.8 us a step; two to five kernels: 2 to 6 us).  In a kernel launched the ordinary way
 // the wait does nothing.
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

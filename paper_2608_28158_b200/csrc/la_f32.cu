@@ -11,6 +11,9 @@
 // threads x 4x4 outputs, 2,048 cycles at 128 multiply-adds a clock) on small forests, the CUDA cores on large ones.  Forward +
 // backward, cold inputs, against the walk: 718 tokens x 1 head (two rounds) 1.33 -> 0.086 ms (outer 9 + 7, walk 3 per round, out 13,
 // grad 25 us), 12,000 branchy x 4 12.0 -> 0.32, 40,000 replay x 8 13.6 -> 3.9, 150,000 agentic x 4 46.4 -> 3.3 (grad 2.0, out 0.7).
+// All but the first kernel of a call are on the SMs before the one ahead of them is done (launch_after).  What needs the call's inputs
+// alone they do before they wait: a walk its tables, outputs and gradients the lookup, the rows, the scores and a chunk's own share --
+// 718 tokens 69.7 -> 51.2 us a step, 796 items 313 -> 293, 3,824 items 1,255 -> 1,235.
 // grad_kernel has one CTA an SM (141 KB): sixteen warps of 2x4 outputs instead of eight of 4x4 -- more shared-memory reads, twice the
 // warps to hide them -- and diagonals that are not unrolled took it from 31.3 to 24.8 us on 13 items, 174 to 159 on 796.
 #include "chunk_item.cuh"
@@ -262,8 +265,7 @@ template <bool BWD>
 __global__ void __launch_bounds__(NT) walk_kernel(const harts_la_tables_t tb, int seq_lo, int H, float* tiles, const float* gammas,
                                                   float* slots, float* ds0, const int32_t* gate) {
     let_next_launch();
-    after_previous();
-    if (gate_closed(gate)) return;
+    if (gate_closed(gate)) return after_previous();
     const int part = blockIdx.x & 3, item = blockIdx.x >> 2, h = item % H;
     const int pos = seq_lo + item / H, seq = tb.seq_order ? tb.seq_order[pos] : pos;
     const int chunk_base = tb.seq_chunk_ptr[seq], n_chunks = tb.seq_chunk_ptr[seq + 1] - chunk_base;
@@ -282,10 +284,11 @@ __global__ void __launch_bounds__(NT) walk_kernel(const harts_la_tables_t tb, in
     };
     float4 u[AHEAD], un[AHEAD], x = make_float4(0.f, 0.f, 0.f, 0.f);
     float gm[AHEAD], gn[AHEAD];
-    load(0, u, gm);
-    if (!BWD && init_slot >= 0) x = *reinterpret_cast<const float4*>(slots + (size_t)init_slot * stride + el);
     int req = BWD ? req_hi - 1 : req_lo;
     int boundary = (BWD ? req >= req_lo : req < req_hi) ? tb.slot_chunk[req] : -1;
+    after_previous();                            // the tables are the call's inputs, the sums are not
+    load(0, u, gm);
+    if (!BWD && init_slot >= 0) x = *reinterpret_cast<const float4*>(slots + (size_t)init_slot * stride + el);
     for (int i0 = 0; i0 < n_chunks; i0 += AHEAD) {
         load(i0 + AHEAD, un, gn);
 #pragma unroll
@@ -328,8 +331,8 @@ __global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t t
                                                  const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ g,
                                                  const float* __restrict__ states, float* __restrict__ o, const int32_t* gate) {
     let_next_launch();
-    after_previous();
-    if (gate_closed(gate)) return;
+    if (gate_closed(gate)) return after_previous();
+    bool waited = false;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OutSmem& s = *reinterpret_cast<OutSmem*>(smem_raw);
     for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
@@ -337,7 +340,8 @@ __global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t t
     load_tile(s.q, q, s.rd, true, it.h, H);
     load_tile(s.k, k, s.rd, false, it.h, H);
     load_tile(s.v, v, s.rd, false, it.h, H);
-    if (!it.zero_state) load_state(s.s, states + ((size_t)it.gc * H + it.h) * (D * D));
+    const float* state = states + ((size_t)it.gc * H + it.h) * (D * D);
+    if (waited && !it.zero_state) load_state(s.s, state);
     __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16, warp = threadIdx.x / 32;
     AccT<R> acc;
@@ -351,12 +355,18 @@ __global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t t
             s.p[t * LD + j] = j <= t ? acc[r][c] * s.rd.decay(t, j) : 0.f;
         }
     __syncwarp();                                // a warp reads the rows it wrote
-    clear(acc);
-    if (!it.zero_state) mul_nn(acc, s.q, s.s, 0, D, ty, tx);
     AccT<R> in;                                      // the chunk's own share, summed by itself: it is small beside the state's
     clear(in);
     mul_nn(in, s.p, s.v, 0, 2 * R * warp, ty, tx);
     mul_nn_diagonal(in, s.p, s.v, 2 * R * warp, ty, tx);
+    if (!waited) {                               // so far the call's inputs alone: the first item's share is made while the states are
+        after_previous();
+        waited = true;
+        if (!it.zero_state) load_state(s.s, state);
+        __syncthreads();
+    }
+    clear(acc);
+    if (!it.zero_state) mul_nn(acc, s.q, s.s, 0, D, ty, tx);
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const int code = s.rd.code[R * ty + r];
@@ -366,6 +376,7 @@ __global__ void __launch_bounds__(1024 / R) out_kernel(const harts_la_tables_t t
                 o[((size_t)code * H + it.h) * D + tx + 16 * c] = it.zero_state ? in[r][c] : __fmaf_rn(s.rd.eb[R * ty + r], acc[r][c], in[r][c]);
     }
     }
+    if (!waited) after_previous();               // no item: the kernel behind this one must not get ahead of the one before it
 }
 
 struct __align__(16) GradSmem {
@@ -382,8 +393,8 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
                                                   float* __restrict__ dv_, float* __restrict__ dg, float* __restrict__ rk,
                                                   float* __restrict__ rv, float* __restrict__ rg, const int32_t* gate) {
     let_next_launch();
-    after_previous();
-    if (gate_closed(gate)) return;
+    if (gate_closed(gate)) return after_previous();
+    bool waited = false;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
     for (int idx = blockIdx.x; begin_item(tb, seq_lo, seq_hi, H, g, idx, s.rd, s.it); idx += gridDim.x) {
@@ -395,8 +406,10 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
     load_tile(s.v, v, s.rd, false, h, H);
     load_tile(s.dO, dO, s.rd, true, h, H);
     const size_t tile = ((size_t)it.gc * H + h) * (D * D);
-    if (has_s) load_state(s.s, states + tile);
-    if (has_ds) load_state(s.ds, ds_tiles + tile);
+    if (waited) {
+        if (has_s) load_state(s.s, states + tile);
+        if (has_ds) load_state(s.ds, ds_tiles + tile);
+    }
     __syncthreads();
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, warp = tid / 32, lane = tid & 31;
     AccT<R> acc, dacc;
@@ -414,37 +427,49 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
             s.dp[t * LD + j] = j <= t ? dacc[r][c] * w : 0.f;
         }
     __syncthreads();
+    // the chunk's own shares, by themselves as in out_kernel: of the call's inputs alone, the first item's made while the states are
+    AccT<R> own_q, own_k, own_v;
+    clear(own_q);
+    clear(own_k);
+    clear(own_v);
+    mul_nn(own_q, s.dp, s.k, 0, 2 * R * warp, ty, tx);
+    mul_nn_diagonal(own_q, s.dp, s.k, 2 * R * warp, ty, tx);
+    mul_tn_diagonal(own_k, s.dp, s.q, 2 * R * warp, ty, tx);
+    mul_tn(own_k, s.dp, s.q, 2 * R * warp + 2 * R, ty, tx);
+    mul_tn_diagonal(own_v, s.p, s.dO, 2 * R * warp, ty, tx);
+    mul_tn(own_v, s.p, s.dO, 2 * R * warp + 2 * R, ty, tx);
+    if (!waited) {
+        after_previous();
+        waited = true;
+        if (has_s) load_state(s.s, states + tile);
+        if (has_ds) load_state(s.ds, ds_tiles + tile);
+        __syncthreads();
+    }
     const float gamma = s.rd.gamma;
     float g_part = 0.f;                          // this thread's share of <S_{c+1}, dS_{c+1}>
     float z[R] = {};           // its share of q.dq - k.dk, per row
     // ---- dq = e^{b_t} dO S^T + dP K
     clear(acc);
-    clear(dacc);
     if (has_s) mul_nt<4>(acc, s.dO, s.s, ty, tx);
-    mul_nn(dacc, s.dp, s.k, 0, 2 * R * warp, ty, tx);         // the chunk's own share by itself, as in out_kernel
-    mul_nn_diagonal(dacc, s.dp, s.k, 2 * R * warp, ty, tx);
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const float x = has_s ? __fmaf_rn(s.rd.eb[t], acc[r][c], dacc[r][c]) : dacc[r][c];
+            const float x = has_s ? __fmaf_rn(s.rd.eb[t], acc[r][c], own_q[r][c]) : own_q[r][c];
             z[r] += s.q[t * LD + tx + 16 * c] * x;
             if (code >= 0) dq[((size_t)code * H + h) * D + tx + 16 * c] = x;
         }
     }
     // ---- dk = w_j V dS^T + dP^T Q
     clear(acc);
-    clear(dacc);
     if (has_ds) mul_nt<4>(acc, s.v, s.ds, ty, tx);
-    mul_tn_diagonal(dacc, s.dp, s.q, 2 * R * warp, ty, tx);
-    mul_tn(dacc, s.dp, s.q, 2 * R * warp + 2 * R, ty, tx);
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const float kv = s.k[t * LD + tx + 16 * c], inter = has_ds ? acc[r][c] * s.rd.w[t] : 0.f, x = dacc[r][c] + inter;
+            const float kv = s.k[t * LD + tx + 16 * c], inter = has_ds ? acc[r][c] * s.rd.w[t] : 0.f, x = own_k[r][c] + inter;
             g_part += kv * inter;
             z[r] -= kv * x;
             if (code >= 0) dk_[((size_t)code * H + h) * D + tx + 16 * c] = x;
@@ -453,16 +478,13 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
     }
     // ---- dv = w_j K dS + P^T dO
     clear(acc);
-    clear(dacc);
     if (has_ds) mul_nn(acc, s.k, s.ds, 0, D, ty, tx);
-    mul_tn_diagonal(dacc, s.p, s.dO, 2 * R * warp, ty, tx);
-    mul_tn(dacc, s.p, s.dO, 2 * R * warp + 2 * R, ty, tx);
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const int t = R * ty + r, code = s.rd.code[t];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const float x = has_ds ? __fmaf_rn(s.rd.w[t], acc[r][c], dacc[r][c]) : dacc[r][c];
+            const float x = has_ds ? __fmaf_rn(s.rd.w[t], acc[r][c], own_v[r][c]) : own_v[r][c];
             if (code >= 0) dv_[((size_t)code * H + h) * D + tx + 16 * c] = x;
             else if (code < -1) rv[((size_t)(it.replay_base + t) * H + h) * D + tx + 16 * c] = x;
         }
@@ -505,6 +527,7 @@ __global__ void __launch_bounds__(1024 / R, 1) grad_kernel(const harts_la_tables
         }
     }
     }
+    if (!waited) after_previous();
 }
 
 // A grid no larger than what is resident at once: the number of items of a range is in the tables on the device, and one launch

@@ -437,14 +437,14 @@ __device__ __forceinline__ void add4<__nv_bfloat16>(__nv_bfloat16* p, const floa
 template <typename T>
 __global__ void replay_reduce_kernel(harts_la_tables_t tb, int H, int DK, int DV, T* dk_, T* dv_, float* dg,
                                      const float* rk, const float* rv, const float* rg, int n_items) {
-    after_previous();
     const int per = (DK + DV) / 4;
     const int item = blockIdx.x * (blockDim.x / per) + threadIdx.x / per, part = threadIdx.x % per;
-    if (item >= n_items) return;
+    if (item >= n_items) return after_previous();
     const int m = item / H, h = item % H;
     const int row = tb.rg_row[m];
     const int lo = tb.rg_ptr[m], hi = tb.rg_ptr[m + 1];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    after_previous();                            // the tables are the call's inputs, the gradients are not
     if (part * 4 < DK) {
         const int i = part * 4;
         for (int e = lo; e < hi; e++) {
