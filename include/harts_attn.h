@@ -65,7 +65,8 @@ int32_t harts_attn_fwd(const int32_t* host_index, const int32_t* dev_index, cons
 
 /*
  * Backward of L = sum_t <dO_t, o_t>.  o and lse are the forward's.  delta: fp32 [n_rows, Hq] scratch (rowsum(dO*o)),
- * overwritten.  Writes dq, dk, dv for every row.
+ * overwritten.  Writes dq, dk, dv for every row.  dq is work memory until its values are written: it may be o's memory (o is read
+ * first), and must not overlap any other argument.
  */
 int32_t harts_attn_bwd(const int32_t* host_index, const int32_t* dev_index, const void* q, const void* k,
                        const void* v, const void* o, const float* lse, const void* dO, void* dq, void* dk_, void* dv_,

@@ -36,10 +36,9 @@ constexpr int NS = 256, NT = NS + 64;     // 8 element-wise warps: warp w and w 
 constexpr int Q_BYTES = BQ * D * 2;       // 32 KB
 constexpr float LOG2E = 1.4426950408889634f;
 
-__global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16* __restrict__ o,
+__global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16* o,
                                                     const __nv_bfloat16* __restrict__ dO, float* __restrict__ delta,
                                                     long long n, int* ticket) {       // n = rows * Hq; one warp per (row, head)
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;       // of attn_dkv_kernel
     const long long w = (blockIdx.x * 256LL + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= n) return;
@@ -55,6 +54,8 @@ __global__ void __launch_bounds__(256) delta_kernel(const __nv_bfloat16* __restr
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
     if (lane == 0) delta[w] = s;
+    // of attn_dkv_kernel.  It lies in dq's first eight bytes, and dq may be o's memory: written by the lane that read these bytes of o
+    if (w == 0 && lane == 0) *ticket = 0;
 }
 
 // ------------------------------------------------------------------------------------------------------------------

@@ -3,8 +3,10 @@
 import pytest
 import torch
 
+import paper_2608_28158_b200 as H
 from oracle import attn_oracle as ao
 from test_gpu_attn import SCALE, _backward, _forward, _rel, _setup
+from test_gpu_attn_split import _is_cut
 from workloads import make_forest
 
 pytestmark = pytest.mark.gpu
@@ -37,3 +39,21 @@ def test_runs_around_a_tile_edge(edge, Hq, Hkv):
         n = 128 + edge + d
         lens = [n, edge + d, edge, edge + 1, 2 * edge + d]
         _check(make_forest([([-1, 0, 0, 1, 1], [0, n, edge + d, edge + d, max(1, edge // 2)], lens)]), Hq, Hkv)
+
+
+@pytest.mark.parametrize("root,Hq,Hkv,cut", [(300, 2, 2, False), (1500, 16, 1, True)])
+def test_dq_over_o(root, Hq, Hkv, cut):
+    """dq is work memory until its values are written, and may be o's memory: the gradients are those of a call with memory of its own,
+    row by row, whole and cut."""
+    fo = make_forest([([-1, 0, 0], [0, root, root // 2], [root, 130, 70])])
+    inp, phys, index, rows = _setup(fo, Hq, Hkv, 12)
+    assert _is_cut(fo, Hq, Hkv) == cut
+    o, lse = _forward(phys, index)
+    want = _backward(phys, index, o, lse)
+    dk, dv = torch.empty_like(phys["k"]), torch.empty_like(phys["v"])
+    delta = torch.empty_like(lse)
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    H.harts_attn_bwd(index, phys["q"], phys["k"], phys["v"], o, lse, phys["dO"], o, dk, dv, delta, SCALE, dev_status=status)
+    H.harts_la_check(status)
+    for a, b in zip((o, dk, dv), want):
+        assert torch.equal(a, b)
