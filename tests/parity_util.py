@@ -46,6 +46,15 @@ def to_physical(plan, canon: dict, device="cuda"):
     return out
 
 
+def kernels_of(call):
+    """Names of the kernels that a call launches, as the profiler prints them, in one text."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        call()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in p.key_averages())
+
+
 GUARD = 4096      # elements of guard band on either side of every output tensor
 
 

@@ -4,8 +4,9 @@ import pytest
 import torch
 
 import paper_2608_28158_b200 as H
-from parity_util import compare, oracle_subset, run_gpu
-from test_gpu_gk import check as check_gk, run_gk
+from oracle import gk_oracle as go
+from parity_util import compare, kernels_of, oracle_subset, rel_err, row_err, run_gpu
+from test_gpu_gk import check as check_gk, make_gk, run_gk
 from test_gpu_parity import check
 from workloads import make_forest, make_inputs
 
@@ -26,16 +27,50 @@ def test_both_sides_of_the_line_of_fans(heads):
         assert torch.equal(out[n], rounds[n]), n
 
 
-@pytest.mark.parametrize("heads", [1, 40, 80])
-def test_a_slot_from_every_chunk(heads):
-    """Forks in each of 24 consecutive chunks (32, 64 and 128 columns of state at a time): slots are published in turn."""
-    n = 24
-    fo = make_forest([([-1] + [0] * n, [0] + [64 * i + 65 for i in range(n)], [64 * n + 70] + [5] * n)])
+def _slots_in_a_row():
+    """Two short branches from each of seven consecutive chunks."""
+    forks = [64 * (i // 2 + 1) + 1 + 4 * i for i in range(14)]
+    return make_forest([([-1] + [0] * 14, [0] + forks, [64 * 9 + 6] + [5 + i for i in range(14)])])
+
+
+@pytest.mark.parametrize("heads,columns", [(1, 32), (40, 64), (75, 128)])
+def test_a_slot_from_every_chunk(heads, columns):
+    """Forks in each of seven consecutive chunks, the scan over 32, 64 and 128 columns of state at a time: slots are published in turn."""
+    fo = _slots_in_a_row()
     inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 17, device="cuda")
-    plan, out = run_gpu(fo, inp)
-    assert plan.n_slots >= n - 1
-    tok, ref = oracle_subset(fo, inp, [0], [0, heads - 1] if heads > 1 else [0])
-    check(compare(out, tok, [0, heads - 1] if heads > 1 else [0], ref, rows=True), "bf16")
+    got = {}
+
+    def run():
+        got["plan"], got["out"] = run_gpu(fo, inp)
+
+    names = kernels_of(run)
+    assert "chunk_fwd_kernel" in names and f"scan_kernel<false, {columns}, false>" in names, names
+    assert got["plan"].n_slots == 7
+    pick = sorted({0, heads - 1})
+    tok, ref = oracle_subset(fo, inp, [0], pick)
+    check(compare(got["out"], tok, pick, ref, rows=True), "bf16")
+
+
+@pytest.mark.parametrize("heads,columns", [(1, 64), (75, 128)])
+def test_a_slot_from_every_chunk_per_channel(heads, columns):
+    fo = _slots_in_a_row()
+    got = {}
+
+    def run():
+        got["plan"], got["out"] = run_gk(fo, heads, 128, "bf16", 18, raw=True)
+
+    names = kernels_of(run)
+    assert "gk_chunk_fwd_kernel" in names and f"scan_kernel<false, {columns}, true>" in names, names
+    assert got["plan"].n_slots == 7
+    inp = make_inputs(fo.n_tokens, heads, 128, 128, "bf16", 18)
+    inp["g"] = make_gk(fo.n_tokens, heads, 128, 18)
+    pick = sorted({0, heads - 1})
+    one = {n: x[:, pick].contiguous() for n, x in inp.items()}
+    ref = go.forest_eval(fo, one["q"], one["k"], one["v"], one["g"], one["dO"])
+    errs = {}
+    for n, x in got["out"].items():
+        errs[n], errs[n + ".row"] = rel_err(x[:, pick], ref[n]), row_err(x[:, pick], ref[n])
+    check_gk(errs, "bf16")
 
 
 @pytest.mark.parametrize("kids", [33, 70])
