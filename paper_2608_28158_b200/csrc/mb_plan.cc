@@ -9,10 +9,13 @@
 //    into a microbatch of its own costs least, until K mod D = 0;
 //  * the slot schedule sorts microbatches by work, heaviest first.
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
+#include <exception>
 #include <limits>
 #include <new>
 #include <set>
+#include <thread>
 #include <vector>
 
 #include "../../include/harts_mb.h"
@@ -666,6 +669,36 @@ int path_lcp(const Traj& a, const Traj& b) {
     return n;
 }
 
+// job(0) .. job(n - 1), taken in order by this thread and, from THREADED trajectories on, by up to three more that end with the call.
+// The jobs do not depend on one another and each writes results of its own, so the plan is the same whatever the threads do.  What a
+// thread costs (15 to 40 us) is less than the greedy passes take from there on (1.5 us a trajectory): 1,084 trajectories 2.21 -> 1.30 ms,
+// 307 0.94 -> 0.67, 217 0.53 -> 0.37; 103 0.17 alone and 0.19 with four threads.
+constexpr int THREADED = 192, MAX_THREADS = 4;
+template <class Job>
+void run_jobs(int n, int n_traj, const Job& job) {
+    std::atomic<int> next{0};
+    std::exception_ptr failed[MAX_THREADS];
+    auto work = [&](int who) {
+        try {
+            for (int i; (i = next.fetch_add(1)) < n;) job(i);
+        } catch (...) {
+            failed[who] = std::current_exception();
+        }
+    };
+    std::thread more[MAX_THREADS - 1];
+    const int threads = n_traj < THREADED ? 1 : std::min<int>(MAX_THREADS, std::max(1u, std::thread::hardware_concurrency()));
+    for (int t = 1; t < threads; ++t) try {
+            more[t - 1] = std::thread(work, t);
+        } catch (const std::exception&) {         // no thread to be had: those there are do the work
+            break;
+        }
+    work(0);
+    for (auto& t : more)
+        if (t.joinable()) t.join();
+    for (auto& e : failed)
+        if (e) std::rethrow_exception(e);
+}
+
 int32_t build(harts_mb_plan_t& p, int32_t n_trees, int32_t D, i64 T) {
     enumerate(p, n_trees, p.traj);
     const int N = static_cast<int>(p.traj.size());
@@ -691,12 +724,22 @@ int32_t build(harts_mb_plan_t& p, int32_t n_trees, int32_t D, i64 T) {
     const int Kmax = std::max(Kmin, std::min(D * ((K0 + D - 1) / D), D * (N / D)));
     std::vector<int> ks;
     for (int K = Kmin; K <= Kmax; K += D) ks.push_back(K);
-    const size_t n_base_begin = cands.size();
-    if (N <= N_EXACT) {
-        ExactDP dp(c, T, std::min(Kmax, N));
-        for (int K : ks)
-            if (K <= N && dp.feasible(K)) cands.push_back(dp.plan(K));
-    } else {
+    // greedy: four processing orders x two placement policies, one candidate (fewest microbatches, then least work)
+    const std::vector<std::vector<int>> orders = greedy_orders(c);
+    struct Placed {
+        Grouping g;
+        i64 work = 0;
+        bool ok = false;
+    };
+    std::vector<Placed> placed(2 * orders.size());
+    std::vector<Grouping> base;
+    auto base_candidates = [&] {
+        if (N <= N_EXACT) {
+            ExactDP dp(c, T, std::min(Kmax, N));
+            for (int K : ks)
+                if (K <= N && dp.feasible(K)) base.push_back(dp.plan(K));
+            return;
+        }
         std::vector<int> pick;
         if (static_cast<int>(ks.size()) <= Q_MAX) {
             pick = ks;
@@ -706,25 +749,26 @@ int32_t build(harts_mb_plan_t& p, int32_t n_trees, int32_t D, i64 T) {
             for (int i = 0; i < 14; ++i) chosen.insert(ks[16 + (ks.size() - 17) * (i + 1) / 15]);
             pick.assign(chosen.begin(), chosen.end());
         }
-        evolve(c, T, nat, pick, cands);
-    }
+        evolve(c, T, nat, pick, base);
+    };
+    run_jobs(1 + static_cast<int>(placed.size()), N, [&](int job) {
+        if (job == 0) return base_candidates();
+        const size_t i = placed.size() - job;                    // the orders by length jump about and take longest: first
+        Placed& to = placed[i];
+        to.ok = greedy_plan(c, T, D, orders[i / 2], i % 2 == 0, &to.g);
+        if (to.ok) to.work = total_work(c, to.g);
+    });
+    const size_t n_base_begin = cands.size();
+    for (Grouping& g : base) cands.push_back(std::move(g));
     const size_t n_base_end = cands.size();
-
-    // greedy: four processing orders x two placement policies, one candidate (fewest microbatches, then least work)
-    const std::vector<std::vector<int>> orders = greedy_orders(c);
     bool have_greedy = false;
     Grouping greedy;
     i64 greedy_work = 0;
-    for (const auto& order : orders)
-        for (int policy = 0; policy < 2; ++policy) {
-            Grouping g;
-            if (!greedy_plan(c, T, D, order, policy == 0, &g)) continue;
-            const i64 w = total_work(c, g);
-            if (!have_greedy || g.mb.size() < greedy.mb.size() || (g.mb.size() == greedy.mb.size() && w < greedy_work)) {
-                greedy = std::move(g);
-                greedy_work = w;
-                have_greedy = true;
-            }
+    for (Placed& x : placed)
+        if (x.ok && (!have_greedy || x.g.mb.size() < greedy.mb.size() || (x.g.mb.size() == greedy.mb.size() && x.work < greedy_work))) {
+            greedy = std::move(x.g);
+            greedy_work = x.work;
+            have_greedy = true;
         }
     if (have_greedy) cands.push_back(greedy);
 

@@ -1,5 +1,7 @@
 """harts_mb_plan (C ABI, host) against the oracle pieces: costs, guarantees, brute force over contiguous cuts."""
+import os
 import random
+from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import pytest
@@ -183,3 +185,26 @@ def test_greedy_increments_and_destinations_follow_eq10():
                 assert got == want, (trial, order, policy)
                 shared_steps += sum(1 for (i, _, c, d) in want if not c and d < len(trajs[i]))
     assert shared_steps > 200                                    # sharing did decide many placements
+
+
+@pytest.mark.parametrize("n_traj", [191, 192, 520])
+def test_the_plan_does_not_depend_on_threads(n_traj):
+    """On one processor, on all of them, and from four threads at once: both sides of the size from which the planner starts threads,
+    and beyond the exact search."""
+    rnd = random.Random(n_traj)
+    trees = []
+    for i in range(0, n_traj, 8):
+        kids = min(8, n_traj - i) - 1                            # off the root's inside: a trajectory each, and the root's own
+        trees.append(([-1] + [0] * kids, [0] + [rnd.randint(1, 39) for _ in range(kids)], [40] + [rnd.randint(1, 60) for _ in range(kids)]))
+    fo = make_forest(trees)
+    tables = lambda p: [np.array(x) for x in (p.traj_leaf, p.traj_mb, p.mb_work, p.mb_replica, p.mb_slot, p.J)]  # noqa: E731
+    cpus = os.sched_getaffinity(0)
+    os.sched_setaffinity(0, {min(cpus)})
+    try:
+        want = tables(_plan(fo, 2, 400))
+    finally:
+        os.sched_setaffinity(0, cpus)
+    assert len(want[0]) == n_traj
+    with ThreadPoolExecutor(4) as pool:
+        for got in pool.map(lambda _: tables(_plan(fo, 2, 400)), range(12)):
+            assert all(np.array_equal(a, b) for a, b in zip(got, want))
