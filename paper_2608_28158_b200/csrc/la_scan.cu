@@ -19,6 +19,12 @@
 // Measured, cold inputs: 1.05 us per step of the longest path while the chains leave SMs idle, 1.05 to 1.3 backward (17,695 tokens x
 // 4 heads, 68 steps: 72 and 71 us; 65,521 x 16, 228 steps: 244 and 294); with 96 chains of 100,003 tokens x 16 heads 4.9 TB/s
 // forward (345 us), 6.1 backward (470 us).
+// Log-decays per channel: 1.4 us a step forward, 1.5 backward (1,047 agentic chunks x 16 heads 408 and 470 us).  The weighting warps are
+// what a step waits for: with a's values read one by one between the stores, which a load may not pass, 1.6 and 1.75 us; and an item
+// whose first chunk has replayed rows began 12 us after its start state was there while a warp copied them with half its lanes, and the
+// gates 16 bytes at a time (454 and 539 us).
+#include <type_traits>
+
 #include "kernels.h"
 #include "tc_common.cuh"
 
@@ -294,11 +300,14 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     }
                     if (grp == 0) *reinterpret_cast<float2*>(&m.gammas[gs % GATES][i0]) = make_float2(ex2(bn.x), ex2(bn.y));
                     unsigned char* sa = smem + S::a + st * S::A + (i0 >> 6) * PANEL + (i0 & 7) * 2;
+                    __nv_bfloat162 x[16];         // all of them first: a load does not pass a store whose address may be the same
+#pragma unroll
+                    for (int u = 0; u < 16; u++) x[u] = *reinterpret_cast<const __nv_bfloat162*>(sa + sw128_chunk(16 * grp + u, (i0 & 63) >> 3));
 #pragma unroll
                     for (int u = 0; u < 16; u++) {
                         const int t = 16 * grp + u;
                         uint32_t* at = reinterpret_cast<uint32_t*>(sa + sw128_chunk(t, (i0 & 63) >> 3));
-                        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(at));
+                        const float2 f = __bfloat1622float2(x[u]);
                         const float b0 = before.x + run[u].x, b1 = before.y + run[u].y;
                         const uint32_t y = pack_bf16(f.x * ex2(BWD ? b0 : bn.x - b0), f.y * ex2(BWD ? b1 : bn.y - b1));
                         *at = BWD && (t < first || t >= n_rows) ? 0u : y;
@@ -392,21 +401,29 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                         const int t = lane + 32 * u;
                         row[u] = t < it.n_replay ? tb.replay_row[it.replay_base + t] : min(it.own_begin + t - it.n_replay, tb.n_rows - 1);
                     }
-#pragma unroll 4
-                    for (int t = 0; t < BT; t++) {
-                        const size_t r = ((size_t)__shfl_sync(~0u, t < 32 ? row[0] : row[1], t & 31) * H + it.h) * D;
-                        const int ch = lane & 15;
-                        if (!BWD || t >= it.n_replay) {
-                            if (lane < 16)
-                                cp_async16(sa + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7), a + r + ch * 8, true);
-                            else if (ch < S::B / PANEL * 8)
-                                cp_async16(sb + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7), b + r + b0 + ch * 8, true);
-                        } else {
-                            *reinterpret_cast<uint4*>((lane < 16 ? sa : sb) + (lane < 16 || S::B > PANEL ? (ch >> 3) * PANEL : 0) + sw128_chunk(t, ch & 7)) =
-                                make_uint4(0, 0, 0, 0);
-                        }
-                        if (GK) cp_async16(smem + S::g + st * S::G + t * (D * 4) + lane * 16, g + r + lane * 4, true);
+                    if (GK) {                     // a row's 128 log-decays are one piece
+                        if (lane == 0) mbar_expect_tx_only(&m.full[st], S::G);
+                        __syncwarp();
+#pragma unroll
+                        for (int u = 0; u < 2; u++)
+                            bulk_load(smem + S::g + st * S::G + (lane + 32 * u) * (D * 4), g + ((size_t)row[u] * H + it.h) * D, D * 4, &m.full[st]);
                     }
+                    // every lane carries 16 bytes of every instruction: CH pieces a row, 32 / CH rows at once
+                    auto gather = [&](auto ch_count, const __nv_bfloat16* from, unsigned char* to, int col) {
+                        constexpr int CH = decltype(ch_count)::value, ROWS = 32 / CH;
+                        const int ch = lane % CH;
+#pragma unroll 8
+                        for (int t0 = 0; t0 < BT; t0 += ROWS) {
+                            const int t = t0 + lane / CH, r0 = __shfl_sync(~0u, row[0], t & 31), r1 = __shfl_sync(~0u, row[1], t & 31);
+                            unsigned char* dst = to + (ch >> 3) * PANEL + sw128_chunk(t, ch & 7);
+                            if (!BWD || t >= it.n_replay)
+                                cp_async16(dst, from + ((size_t)(t0 < 32 ? r0 : r1) * H + it.h) * D + col + ch * 8, true);
+                            else
+                                *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
+                        }
+                    };
+                    gather(std::integral_constant<int, 16>(), a, sa, 0);
+                    gather(std::integral_constant<int, S::B / PANEL * 8>(), b, sb, b0);
                     cp_async_wait_all();
                     fence_async_smem();
                     __syncwarp();
