@@ -22,6 +22,9 @@
 
 namespace harts {
 
+int32_t make_row_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
+int32_t make_state_map(CUtensorMap* map, const void* base, int64_t n);
+int32_t make_gate_map(CUtensorMap* map, const void* base, int64_t rows, int32_t H);
 int sm_count();
 
 namespace {
@@ -33,8 +36,10 @@ constexpr int NW = NT / 32;
 constexpr float LOG2E = 1.4426950408889634f;
 
 // ---- shared-memory addressing ---------------------------------------------------------------------------------------
-// [rows][128] bf16 (256-byte rows) and [rows][64] bf16 (128-byte rows); c16 = index of the 16-byte piece in the row
-__device__ __forceinline__ uint32_t sw256(int r, int c16) { return (uint32_t)(r * 256 + ((c16 ^ (r & 7)) << 4)); }
+// [rows][128] bf16 and [rows][64] bf16 (128-byte rows); c16 = index of the 16-byte piece in the row
+// (a tile of 128 columns is two panels of 64, as TMA leaves them)
+template <int ROWS = BT>
+__device__ __forceinline__ uint32_t sw256(int r, int c16) { return (uint32_t)((c16 >> 3) * (ROWS * 128) + r * 128 + (((c16 & 7) ^ (r & 7)) << 4)); }
 __device__ __forceinline__ uint32_t sw128(int r, int c16) { return (uint32_t)(r * 128 + ((c16 ^ (r & 7)) << 4)); }
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -63,31 +68,31 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// Fragment loaders.  `tile` is the shared-memory address of a swizzled tile, PITCH its row pitch in bytes.
+// Fragment loaders.  `tile` is the shared-memory address of a swizzled tile, ROWS its rows if it has 128 columns, 0 if it has 64.
 // A operand (16 x 16) of a matrix stored [m][k]: rows m0.., columns k0..
-template <int PITCH>
+template <int ROWS>
 __device__ __forceinline__ void frag_a(uint32_t (&a)[4], uint32_t tile, int m0, int k0, int lane) {
     const int r = m0 + (lane & 7) + ((lane >> 3) & 1) * 8, c = (k0 >> 3) + (lane >> 4);
-    ldsm4(a, tile + (PITCH == 256 ? sw256(r, c) : sw128(r, c)));
+    ldsm4(a, tile + (ROWS ? sw256<ROWS>(r, c) : sw128(r, c)));
 }
 // A operand (16 x 16) of the TRANSPOSE of a matrix stored [k][m]: A[m][k] = stored[k][m]
-template <int PITCH>
+template <int ROWS>
 __device__ __forceinline__ void frag_a_t(uint32_t (&a)[4], uint32_t tile, int m0, int k0, int lane) {
     const int r = k0 + (lane & 7) + (lane >> 4) * 8, c = (m0 >> 3) + ((lane >> 3) & 1);
-    ldsm4t(a, tile + (PITCH == 256 ? sw256(r, c) : sw128(r, c)));
+    ldsm4t(a, tile + (ROWS ? sw256<ROWS>(r, c) : sw128(r, c)));
 }
 // B operands of TWO adjacent n-tiles (n0.., n0+8..) for one k-step, matrix stored [k][n]: b[0],b[1] -> tile n0;
 // b[2],b[3] -> tile n0+8
-template <int PITCH>
+template <int ROWS>
 __device__ __forceinline__ void frag_b_kn(uint32_t (&b)[4], uint32_t tile, int k0, int n0, int lane) {
     const int r = k0 + (lane & 7) + ((lane >> 3) & 1) * 8, c = (n0 >> 3) + (lane >> 4);
-    ldsm4t(b, tile + (PITCH == 256 ? sw256(r, c) : sw128(r, c)));
+    ldsm4t(b, tile + (ROWS ? sw256<ROWS>(r, c) : sw128(r, c)));
 }
 // the same for a matrix stored [n][k] (B = stored^T)
-template <int PITCH>
+template <int ROWS>
 __device__ __forceinline__ void frag_b_nk(uint32_t (&b)[4], uint32_t tile, int k0, int n0, int lane) {
     const int r = n0 + (lane & 7) + (lane >> 4) * 8, c = (k0 >> 3) + ((lane >> 3) & 1);
-    ldsm4(b, tile + (PITCH == 256 ? sw256(r, c) : sw128(r, c)));
+    ldsm4(b, tile + (ROWS ? sw256<ROWS>(r, c) : sw128(r, c)));
 }
 
 struct SeqInfo {
@@ -108,16 +113,14 @@ __device__ __forceinline__ SeqInfo seq_info(const harts_la_tables_t& tb, int seq
     return s;
 }
 
-// row codes of chunk c: physical row >= 0 (own), -2 - row (replayed), -1 (past the end)
+// code of row t of chunk c: physical row >= 0 (own), -2 - row (replayed), -1 (past the end)
+__device__ __forceinline__ int row_code(const harts_la_tables_t& tb, const SeqInfo& s, int c, int t) {
+    const int vr = c * BT + t;
+    if (vr >= s.n_virtual) return -1;
+    return vr < s.n_replay ? -2 - tb.replay_row[s.replay_base + vr] : s.own_begin + (vr - s.n_replay);
+}
 __device__ __forceinline__ void load_codes(const harts_la_tables_t& tb, const SeqInfo& s, int c, int* srow) {
-    const int tid = threadIdx.x;
-    if (tid < BT) {
-        const int vr = c * BT + tid;
-        int code = -1;
-        if (vr < s.n_virtual)
-            code = vr < s.n_replay ? -2 - tb.replay_row[s.replay_base + vr] : s.own_begin + (vr - s.n_replay);
-        srow[tid] = code;
-    }
+    if (threadIdx.x < BT) srow[threadIdx.x] = row_code(tb, s, c, threadIdx.x);
 }
 
 // The loads of a chunk go to shared memory by cp.async, all of them in flight at once (through registers they were a round
@@ -126,21 +129,23 @@ using tc::cp_async16;
 
 // One [BT][128] bf16 tile of a [rows, H, 128] tensor into a swizzled tile, 16 bytes at a time.  need_own: only rows
 // with an output are taken (q, dO); otherwise every valid row (k, v).  Rows that are not taken become zero.
-__device__ __forceinline__ void load_tile_bf16(const __nv_bfloat16* src, int H, int h, const int* srow, bool need_own,
+template <class Code>
+__device__ __forceinline__ void load_tile_bf16(const __nv_bfloat16* src, int H, int h, const Code& code_of, bool need_own,
                                                unsigned char* dst) {
 #pragma unroll
     for (int u = 0; u < BT * 16 / NT; u++) {
-        const int p = threadIdx.x + u * NT, t = p >> 4, c16 = p & 15, code = srow[t];
+        const int p = threadIdx.x + u * NT, t = p >> 4, c16 = p & 15, code = code_of(t);
         const int r = code >= 0 ? code : code == -1 ? 0 : -2 - code;
         cp_async16(dst + sw256(t, c16), src + ((size_t)r * H + h) * D + c16 * 8, need_own ? code >= 0 : code != -1);
     }
 }
 
 // g of the chunk's valid rows (fp32 [rows, H, 128]) into sB [BT][128], zero elsewhere
-__device__ __forceinline__ void load_g(const float* gk, int H, int h, const int* srow, float* sB) {
+template <class Code>
+__device__ __forceinline__ void load_g(const float* gk, int H, int h, const Code& code_of, float* sB) {
 #pragma unroll
     for (int u = 0; u < BT * 32 / NT; u++) {
-        const int p = threadIdx.x + u * NT, t = p >> 5, c4 = p & 31, code = srow[t];
+        const int p = threadIdx.x + u * NT, t = p >> 5, c4 = p & 31, code = code_of(t);
         const int r = code >= 0 ? code : code == -1 ? 0 : -2 - code;
         cp_async16(reinterpret_cast<unsigned char*>(sB) + p * 16, gk + ((size_t)r * H + h) * D + c4 * 4, code != -1);
     }
@@ -172,9 +177,32 @@ __device__ __forceinline__ NextItem next_item(const SeqInfo& s, int c, int gc, i
     if (nx >= n_items || n.c >= s.n_chunks) n.c = -1;
     return n;
 }
-__device__ __forceinline__ void prefetch_state(const __nv_bfloat16* tiles, int gc, int h, int H) {
-    const char* st = reinterpret_cast<const char*>(tiles + ((size_t)gc * H + h) * (D * D));
-    for (int p = threadIdx.x; p < D * D * 2 / 128; p += NT) asm volatile("prefetch.global.L2 [%0];" ::"l"(st + p * 128));
+
+// The chunk kernels' loads.  All 64 rows of most chunks are the sequence's own, one after the other: their tiles come by TMA, asked for by
+// one thread.  By cp.async they took the threads' time (160 KB at 16 bytes a lane: 5 k of the backward's 31 k cycles an item).  Chunks with
+// replayed rows or an end still come that way.
+struct ChunkMaps {
+    CUtensorMap q, k, v, dO, g, s, ds;
+};
+__device__ __forceinline__ bool whole_chunk(const SeqInfo& s, int c) { return c * BT >= s.n_replay && (c + 1) * BT <= s.n_virtual; }
+__device__ __forceinline__ void tma_rows(unsigned char* tile, const CUtensorMap* map, const SeqInfo& s, int c, int h, uint64_t* bar) {
+    for (int p = 0; p < 2; p++) tc::tma_load_3d(tile + p * (BT * 128), map, p * 64, h, s.own_begin - s.n_replay + c * BT, bar);
+}
+__device__ __forceinline__ void tma_state(unsigned char* tile, const CUtensorMap* map, int gc, int h, int H, uint64_t* bar) {
+    for (int p = 0; p < 2; p++) tc::tma_load_3d(tile + p * (D * 128), map, p * 64, 0, gc * H + h, bar);
+}
+// asks the L2 for what the CTA's next item loads, one thread
+__device__ __forceinline__ void prefetch_chunk(const ChunkMaps& m, bool backward, const SeqInfo& s, const NextItem& nx, int H) {
+    const int row0 = s.own_begin - s.n_replay + nx.c * BT;
+    for (int p = 0; p < 2; p++) {
+        tc::tma_prefetch_3d(&m.q, p * 64, nx.h, row0);
+        tc::tma_prefetch_3d(&m.k, p * 64, nx.h, row0);
+        tc::tma_prefetch_3d(&m.v, p * 64, nx.h, row0);
+        if (backward) tc::tma_prefetch_3d(&m.dO, p * 64, nx.h, row0);
+        tc::tma_prefetch_3d(&m.s, p * 64, 0, nx.gc * H + nx.h);
+        if (backward) tc::tma_prefetch_3d(&m.ds, p * 64, 0, nx.gc * H + nx.h);
+    }
+    tc::tma_prefetch_3d(&m.g, 0, nx.h, row0);
 }
 
 // log-decays -> their running sum over the rows in log2 units, per channel: four threads per channel (16 rows each, scanned in registers), joined through
@@ -249,7 +277,7 @@ __device__ __forceinline__ void anchored_operands(const unsigned char* sQ, const
         }
         // the local row index of a k^(I) sub-tile is dst_row - its row offset; the offsets are multiples of 8, so the
         // swizzle of the stacked tile equals that of the sub-tile
-        *reinterpret_cast<uint4*>((is_q ? sQa : sKa) + sw256(dst_row, c16)) = x;
+        *reinterpret_cast<uint4*>(is_q ? sQa + sw256(dst_row, c16) : sKa + sw256<96>(dst_row, c16)) = x;
     }
 }
 
@@ -300,7 +328,7 @@ __device__ __forceinline__ void mild_operands(const unsigned char* sQ, const uns
         for (int I = blk + 1; I < 4; I++) {
             row8(ba, 16 * I);
             // the row offsets of the k^(I) sub-tiles are multiples of 8, so the swizzle of the stacked tile equals theirs
-            *reinterpret_cast<uint4*>(sKa + sw256(ka_row0(I) + t, c16)) = scaled(kv, [&](int e) { return ba[e] - bs[e]; });
+            *reinterpret_cast<uint4*>(sKa + sw256<96>(ka_row0(I) + t, c16)) = scaled(kv, [&](int e) { return ba[e] - bs[e]; });
         }
         if (sKt) {
             row8(ba, BT - 1);
@@ -321,8 +349,8 @@ __device__ __forceinline__ void scores_off_diagonal(uint32_t aQa, uint32_t aKa, 
 #pragma unroll
         for (int ks = 0; ks < 8; ks++) {
             uint32_t a[4], b[4];
-            frag_a<256>(a, aQa, 16 * I, ks * 16, lane);
-            frag_b_nk<256>(b, aKd, ks * 16, 16 * I, lane);
+            frag_a<BT>(a, aQa, 16 * I, ks * 16, lane);
+            frag_b_nk<BT>(b, aKd, ks * 16, 16 * I, lane);
             mma16816(acc[0], a, b[0], b[1]);
             mma16816(acc[1], a, b[2], b[3]);
         }
@@ -343,8 +371,8 @@ __device__ __forceinline__ void scores_off_diagonal(uint32_t aQa, uint32_t aKa, 
 #pragma unroll
         for (int ks = 0; ks < 8; ks++) {
             uint32_t a[4], b[4];
-            frag_a<256>(a, aQa, 16 * I, ks * 16, lane);
-            frag_b_nk<256>(b, aKa, ks * 16, ka_row0(I) + 16 * J, lane);
+            frag_a<BT>(a, aQa, 16 * I, ks * 16, lane);
+            frag_b_nk<96>(b, aKa, ks * 16, ka_row0(I) + 16 * J, lane);
             mma16816(acc[0], a, b[0], b[1]);
             mma16816(acc[1], a, b[2], b[3]);
         }
@@ -453,8 +481,8 @@ __device__ __forceinline__ void state_to_operand(const float (&st)[8][4], unsign
     const int g = lane >> 2, tq = lane & 3, r0 = (warp & 7) * 16 + g, c0 = (warp >> 3) * 8;
 #pragma unroll
     for (int n = 0; n < 8; n++) {
-        *reinterpret_cast<uint32_t*>(sSb + sw256(r0, c0 + n) + tq * 4) = pack2(st[n][0], st[n][1]);
-        *reinterpret_cast<uint32_t*>(sSb + sw256(r0 + 8, c0 + n) + tq * 4) = pack2(st[n][2], st[n][3]);
+        *reinterpret_cast<uint32_t*>(sSb + sw256<D>(r0, c0 + n) + tq * 4) = pack2(st[n][0], st[n][1]);
+        *reinterpret_cast<uint32_t*>(sSb + sw256<D>(r0 + 8, c0 + n) + tq * 4) = pack2(st[n][2], st[n][3]);
     }
 }
 // state fragments <-> fp32 [128][128] in global memory (slots, initial-state gradients)
@@ -492,11 +520,11 @@ __device__ __forceinline__ void state_update(float (&st)[8][4], const float* sB,
 #pragma unroll
     for (int ks = 0; ks < 4; ks++) {
         uint32_t a[4];
-        frag_a_t<256>(a, aX, r0, ks * 16, lane);
+        frag_a_t<BT>(a, aX, r0, ks * 16, lane);
 #pragma unroll
         for (int n2 = 0; n2 < 4; n2++) {
             uint32_t b[4];
-            frag_b_kn<256>(b, aY, ks * 16, c0 + n2 * 16, lane);
+            frag_b_kn<BT>(b, aY, ks * 16, c0 + n2 * 16, lane);
             mma16816(st[2 * n2], a, b[0], b[1]);
             mma16816(st[2 * n2 + 1], a, b[2], b[3]);
         }
@@ -506,7 +534,7 @@ __device__ __forceinline__ void state_update(float (&st)[8][4], const float* sB,
 template <int ROWS>
 __device__ __forceinline__ void tile_to_global(const unsigned char* tile, __nv_bfloat16* dst) {
     for (int p = threadIdx.x; p < ROWS * 16; p += NT)
-        reinterpret_cast<uint4*>(dst)[p] = *reinterpret_cast<const uint4*>(tile + sw256(p >> 4, p & 15));
+        reinterpret_cast<uint4*>(dst)[p] = *reinterpret_cast<const uint4*>(tile + sw256<ROWS>(p >> 4, p & 15));
 }
 
 // plain row-major [128][128] bf16 in global memory -> swizzled tile
@@ -514,7 +542,7 @@ __device__ __forceinline__ void global_to_tile128(const __nv_bfloat16* src, unsi
 #pragma unroll
     for (int u = 0; u < D * 16 / NT; u++) {
         const int p = threadIdx.x + u * NT;
-        cp_async16(tile + sw256(p >> 4, p & 15), src + p * 8, true);
+        cp_async16(tile + sw256<D>(p >> 4, p & 15), src + p * 8, true);
     }
 }
 
@@ -613,10 +641,11 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
         __syncthreads();                                   // the previous chunk's readers of every tile are through
         load_codes(tb, s, c, srow);
         __syncthreads();
-        load_tile_bf16(k, H, h, srow, false, sK);
-        load_tile_bf16(q, H, h, srow, true, sQ);
-        load_tile_bf16(v, H, h, srow, false, sV);
-        load_g(gk, H, h, srow, sB);
+        auto code_of = [&](int t) { return srow[t]; };
+        load_tile_bf16(k, H, h, code_of, false, sK);
+        load_tile_bf16(q, H, h, code_of, true, sQ);
+        load_tile_bf16(v, H, h, code_of, false, sV);
+        load_g(gk, H, h, code_of, sB);
         if (c + 1 < s.n_chunks) {
             prefetch_rows(k, H, h, s, c + 1);
             prefetch_rows(q, H, h, s, c + 1);
@@ -661,11 +690,11 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
             for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
             for (int ks = 0; ks <= mb; ks++) {              // P is zero right of the diagonal block
                 uint32_t a[4];
-                frag_a<128>(a, aP, m0, ks * 16, lane);
+                frag_a<0>(a, aP, m0, ks * 16, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
                     uint32_t b[4];
-                    frag_b_kn<256>(b, aV, ks * 16, n_base + n2 * 16, lane);
+                    frag_b_kn<BT>(b, aV, ks * 16, n_base + n2 * 16, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -673,11 +702,11 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4];
-                frag_a<256>(a, aQ, m0, ks * 16, lane);
+                frag_a<BT>(a, aQ, m0, ks * 16, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
                     uint32_t b[4];
-                    frag_b_kn<256>(b, aSb, ks * 16, n_base + n2 * 16, lane);
+                    frag_b_kn<D>(b, aSb, ks * 16, n_base + n2 * 16, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -707,17 +736,37 @@ struct SharedC {
     static constexpr int q = 0, k = 16384;                              // bf16 [64][128]; then q~, keys anchored at their block
     static constexpr int b = 32768;                                     // fp32 [64][128] running log-decay; then the state
     static constexpr int qa = 65536, ka = qa + 16384;                   // anchored operands; then V; step factors (not mild)
-    static constexpr int p = ka + 96 * 256, row = p + 8192, bytes = row + 256;
+    static constexpr int p = ka + 96 * 256, row = p + 8192, misc = row + 256, bytes = misc + 64;
 };
 static_assert(2 * (SharedC::bytes + 1024 + 64) <= 228 * 1024, "two CTAs per SM");
 
 __global__ void __launch_bounds__(NT, 2)
 gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __nv_bfloat16* __restrict__ q,
                     const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
-                    __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ chunk_states, const int32_t* gate) {
+                    __nv_bfloat16* __restrict__ o, const __grid_constant__ ChunkMaps maps, int* status, const int32_t* gate) {
     after_previous();
-    if (gate_closed(gate)) return;
-    extern __shared__ __align__(1024) unsigned char sm[];
+    extern __shared__ __align__(1024) unsigned char sm[];       // no static shared memory: the dynamic window starts 1024-byte aligned
+    struct Misc {
+        uint64_t bar_g, bar_qk, bar_s;
+        int dead, closed;
+    };
+    Misc& m = *reinterpret_cast<Misc*>(sm + SharedC::misc);
+    if (threadIdx.x == 0) {
+        tc::mbar_init(&m.bar_g, 1);
+        tc::mbar_init(&m.bar_qk, 1);
+        tc::mbar_init(&m.bar_s, 1);
+        m.dead = 0;
+        m.closed = gate && *gate != 0;
+        if (s_u32(sm) & 1023) {                   // never on sm_100a; the swizzled tiles would be misread
+            m.closed = 1;
+            if (status) atomicExch(status, tc::STATUS_TIMEOUT);
+        }
+        tc::fence_barrier_init();
+    }
+    __syncthreads();
+    if (m.closed) return;
+    uint32_t ph_rows = 0, ph_s = 0;
+    bool ok = true;
     unsigned char *sQ = sm + SharedC::q, *sK = sm + SharedC::k, *sQa = sm + SharedC::qa, *sKa = sm + SharedC::ka,
                   *sP = sm + SharedC::p, *sV = sQa, *sS = sm + SharedC::b;
     float *sB = reinterpret_cast<float*>(sm + SharedC::b), *sTmp = reinterpret_cast<float*>(sP), *sR = reinterpret_cast<float*>(sQa);
@@ -737,29 +786,50 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
         }
         const int c = gc - s.chunk_base;
         const bool has_s = c > 0 || s.init_slot >= 0;     // the state of a sequence that starts from zero is not read
+        const bool whole = whole_chunk(s, c);
+        tc::fence_async_smem();                            // what was written into the tiles, before TMA writes there
         __syncthreads();                                   // the previous item's readers of every tile are through
         load_codes(tb, s, c, srow);
-        __syncthreads();
-        load_tile_bf16(q, H, h, srow, true, sQ);
-        load_tile_bf16(k, H, h, srow, false, sK);
-        load_g(gk, H, h, srow, sB);
-        const NextItem nx = next_item(s, c, gc, item, H, n_items);
-        if (nx.c >= 0) {
-            prefetch_rows(k, H, nx.h, s, nx.c);
-            prefetch_rows(q, H, nx.h, s, nx.c);
-            prefetch_rows(v, H, nx.h, s, nx.c);
-            prefetch_rows(gk, H, nx.h, s, nx.c);
-            prefetch_state(chunk_states, nx.gc, nx.h, H);
+        if (whole) {
+            if (tid == 0) {
+                tc::mbar_expect_tx(&m.bar_g, BT * D * 4);
+                tc::tma_load_3d(sB, &maps.g, 0, h, s.own_begin - s.n_replay + c * BT, &m.bar_g);
+                tc::mbar_expect_tx(&m.bar_qk, 2 * BT * D * 2);
+                tma_rows(sQ, &maps.q, s, c, h, &m.bar_qk);
+                tma_rows(sK, &maps.k, s, c, h, &m.bar_qk);
+            }
+        } else {
+            auto code_of = [&](int t) { return row_code(tb, s, c, t); };
+            load_g(gk, H, h, code_of, sB);
+            tc::cp_async_commit();
+            load_tile_bf16(q, H, h, code_of, true, sQ);
+            load_tile_bf16(k, H, h, code_of, false, sK);
+            tc::cp_async_commit();
         }
-        tc::cp_async_wait_all();
+        const NextItem nx = next_item(s, c, gc, item, H, n_items);
+        if (nx.c >= 0 && tid == 32) prefetch_chunk(maps, false, s, nx, H);
+        if (whole) ok = tc::mbar_wait_warp(&m.bar_g, ph_rows, status, &m.dead) && ok;
+        else tc::cp_async_wait_group<1>();
         __syncthreads();
-        cumsum_rows(sB, sTmp);
-        const bool mild = chunk_is_mild(sB);
+        cumsum_rows(sB, sTmp);                             // while the rows come
+        if (whole) {
+            ok = tc::mbar_wait_warp(&m.bar_qk, ph_rows, status, &m.dead) && ok;
+            ph_rows ^= 1;
+        } else {
+            tc::cp_async_wait_all();
+        }
+        const bool mild = chunk_is_mild(sB);               // (a barrier: every thread's rows are there)
         if (mild) mild_operands(sQ, sK, sB, sQa, sKa, sK, sQ, nullptr);
         else anchored_operands(sQ, sK, sB, sQa, sKa);
+        tc::fence_async_smem();
         __syncthreads();
-        const __nv_bfloat16* state = chunk_states + ((size_t)gc * H + h) * (D * D);      // goes over the running sums
-        if (mild && has_s) global_to_tile128(state, sS);
+        auto load_state = [&] {                            // over the running sums
+            if (has_s && tid == 0) {
+                tc::mbar_expect_tx(&m.bar_s, D * D * 2);
+                tma_state(sS, &maps.s, gc, h, H, &m.bar_s);
+            }
+        };
+        if (mild) load_state();
         uint4 vv[BT * 16 / NT];                            // V, on its way while the scores are computed
 #pragma unroll
         for (int u = 0; u < BT * 16 / NT; u++) {
@@ -774,16 +844,23 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
             scores_diagonal(sQ, sK, sR, sP, warp, lane);
             __syncthreads();
             scale_qk<true, false>(sQ, sK, sB, sQ, sK);
+            tc::fence_async_smem();
             __syncthreads();
-            if (has_s) global_to_tile128(state, sS);
+            load_state();
         }
 #pragma unroll
         for (int u = 0; u < BT * 16 / NT; u++) {
             const int p = tid + u * NT;
             *reinterpret_cast<uint4*>(sV + sw256(p >> 4, p & 15)) = vv[u];
         }
-        tc::cp_async_wait_all();
-        __syncthreads();
+        if (has_s) {
+            ok = tc::mbar_wait_warp(&m.bar_s, ph_s, status, &m.dead) && ok;
+            ph_s ^= 1;
+        }
+        if (__syncthreads_or(!ok)) {                       // a wait ran out (status word set): let what is in flight land
+            tc::drain_delay();
+            return;
+        }
         // ---- o = P V + q~ S_c : warp -> rows 16 * mb, columns 32 * nq ----------------------------------------------
         const int m0 = mb * 16, n_base = nq * 32;
         float acc[4][4];
@@ -791,11 +868,11 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
         for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
         for (int ks = 0; ks <= mb; ks++) {              // P is zero right of the diagonal block
             uint32_t a[4];
-            frag_a<128>(a, aP, m0, ks * 16, lane);
+            frag_a<0>(a, aP, m0, ks * 16, lane);
 #pragma unroll
             for (int n2 = 0; n2 < 2; n2++) {
                 uint32_t b[4];
-                frag_b_kn<256>(b, aV, ks * 16, n_base + n2 * 16, lane);
+                frag_b_kn<BT>(b, aV, ks * 16, n_base + n2 * 16, lane);
                 mma16816(acc[2 * n2], a, b[0], b[1]);
                 mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
             }
@@ -804,11 +881,11 @@ gk_chunk_fwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const _
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4];
-                frag_a<256>(a, aQ, m0, ks * 16, lane);
+                frag_a<BT>(a, aQ, m0, ks * 16, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
                     uint32_t b[4];
-                    frag_b_kn<256>(b, aS, ks * 16, n_base + n2 * 16, lane);
+                    frag_b_kn<D>(b, aS, ks * 16, n_base + n2 * 16, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -841,12 +918,14 @@ struct SharedB {
     static constexpr int rowdot = tmp + 2048;                           // fp32 [2][128]
     static constexpr int gi = rowdot + 1024;                            // fp32 [4][128]
     static constexpr int row = gi + 2048;                               // int [64]
-    static constexpr int bytes = row + 256;
+    static constexpr int misc = row + 256;
+    static constexpr int bytes = misc + 64;
 };
-static_assert(SharedB::bytes <= 232448, "backward tiles do not fit in shared memory");
+static_assert(SharedB::bytes + 1024 <= 232448, "backward tiles do not fit in shared memory");
 
+template <int ROWS = BT>
 __device__ __forceinline__ float2 ld_bf2(const unsigned char* tile, int r, int col) {      // [r][col], [r][col+1]; col even
-    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + sw256(r, col >> 3) + (col & 7) * 2));
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(tile + sw256<ROWS>(r, col >> 3) + (col & 7) * 2));
 }
 
 
@@ -860,14 +939,29 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ gk,
                   const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk_,
                   __nv_bfloat16* __restrict__ dv_, float* __restrict__ dgk, const __nv_bfloat16* __restrict__ chunk_states,
-                  const __nv_bfloat16* __restrict__ ds_tiles, const float* __restrict__ dots,
-                  float* __restrict__ ds0, float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg,
-                  const int32_t* gate, int* status, int* ds0_flags, int* ticket, const RoundOrder rounds) {
+                  const float* __restrict__ dots, float* __restrict__ ds0, float* __restrict__ rk, float* __restrict__ rv, float* __restrict__ rg,
+                  const int32_t* gate, int* status, int* ds0_flags, int* ticket, const RoundOrder rounds, const __grid_constant__ ChunkMaps maps) {
     after_previous();
     if (gate_closed(gate)) return;
     constexpr bool ONE_LAUNCH = MODE == ONE_LAUNCH_MODE, CHUNKS = MODE == CHUNKS_MODE;
     __shared__ int s_item, s_dead;
-    extern __shared__ __align__(1024) unsigned char sm[];
+    extern __shared__ __align__(1024) unsigned char sm[];       // (the static variables ahead of it are padded to 1,024 bytes)
+    uint64_t *bar_first = reinterpret_cast<uint64_t*>(sm + SharedB::misc), *bar_rest = bar_first + 1;
+    uint32_t ph_first = 0, ph_rest = 0;
+    bool ok = true;
+    if (CHUNKS) {
+        if (s_u32(sm) & 1023) {                       // never on sm_100a; the swizzled tiles would be misread
+            if (threadIdx.x == 0 && status) atomicExch(status, tc::STATUS_TIMEOUT);
+            return;
+        }
+        if (threadIdx.x == 0) {
+            tc::mbar_init(bar_first, 1);
+            tc::mbar_init(bar_rest, 1);
+            s_dead = 0;
+            tc::fence_barrier_init();
+        }
+        __syncthreads();
+    }
     unsigned char *sQ = sm + SharedB::q, *sK = sm + SharedB::k, *sV = sm + SharedB::v, *sDO = sm + SharedB::dO,
                   *sSc = sm + SharedB::sc, *sdSb = sm + SharedB::dsb, *sQa = sm + SharedB::qa, *sKa = sm + SharedB::ka,
                   *sP = sm + SharedB::p, *sdAb = sm + SharedB::dab;
@@ -891,6 +985,24 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
     SeqInfo s;
     s.chunk_base = s.n_chunks = 0;
     int seq = seq_lo;
+    // CHUNKS: q, k and the log-decays of a chunk; asked for under the outputs of a mild one before it
+    bool first_there = false;
+    auto load_first = [&](const SeqInfo& s_, int c_, int h_) {
+        if (whole_chunk(s_, c_)) {
+            if (tid == 0) {
+                tc::mbar_expect_tx(bar_first, BT * D * 8);
+                tc::tma_load_3d(sB, &maps.g, 0, h_, s_.own_begin - s_.n_replay + c_ * BT, bar_first);
+                tma_rows(sQ, &maps.q, s_, c_, h_, bar_first);
+                tma_rows(sK, &maps.k, s_, c_, h_, bar_first);
+            }
+            return;
+        }
+        auto code_of = [&](int t) { return row_code(tb, s_, c_, t); };
+        load_g(gk, H, h_, code_of, sB);
+        load_tile_bf16(q, H, h_, code_of, true, sQ);
+        load_tile_bf16(k, H, h_, code_of, false, sK);
+        tc::cp_async_commit();
+    };
     do {
     if (CHUNKS && item >= n_items) break;
     int seq_pos = seq_lo + item / H, h = item % H;
@@ -926,6 +1038,8 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
     for (int c = c_hi; c >= c_lo; c--) {
         // zero, and neither read nor multiplied: the state of a sequence that starts from zero, the gradient after a last chunk
         const bool has_s = !CHUNKS || c > 0 || s.init_slot >= 0, has_ds = !CHUNKS || c + 1 < s.n_chunks;
+        const bool whole = CHUNKS && whole_chunk(s, c);
+        if (CHUNKS) tc::fence_async_smem();           // what was written into the tiles, before TMA writes there
         __syncthreads();                              // the previous chunk's readers of every tile are through
         // gradient arriving at boundary c+1 from the sequences that started there: one launch per round -- summed into
         // the first consumer's buffer by handoff_reduce; all rounds in one launch -- awaited and summed here, same order
@@ -953,24 +1067,41 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             next_req--;
         }
         load_codes(tb, s, c, srow);
-        __syncthreads();
-        load_tile_bf16(k, H, h, srow, false, sK);
-        load_tile_bf16(q, H, h, srow, true, sQ);
-        load_tile_bf16(v, H, h, srow, false, sV);
-        load_tile_bf16(dO, H, h, srow, true, sDO);
-        load_g(gk, H, h, srow, sB);
-        if (has_s) global_to_tile128(chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems, sSc);
+        float dot = 0.f;                              // CHUNKS: <S_c[i,:], dS[i,:]> in four parts of 32 columns, from the scan (dS is fp32 there)
+        if constexpr (CHUNKS) {
+            if (!first_there) load_first(s, c, h);
+            if (tid == 0 && (whole || has_s || has_ds)) {
+                tc::mbar_expect_tx(bar_rest, (whole ? 2 * BT * D * 2 : 0) + (has_s ? D * D * 2 : 0) + (has_ds ? D * D * 2 : 0));
+                if (whole) {
+                    tma_rows(sV, &maps.v, s, c, h, bar_rest);
+                    tma_rows(sDO, &maps.dO, s, c, h, bar_rest);
+                }
+                if (has_s) tma_state(sSc, &maps.s, gc, h, H, bar_rest);
+                if (has_ds) tma_state(sdSb, &maps.ds, gc, h, H, bar_rest);
+            }
+            if (!whole) {
+                auto code_of = [&](int t) { return row_code(tb, s, c, t); };
+                load_tile_bf16(v, H, h, code_of, false, sV);
+                load_tile_bf16(dO, H, h, code_of, true, sDO);
+                tc::cp_async_commit();
+            }
+            if (tid < 2 * D && has_s && has_ds) {
+                const float* part = dots + ((size_t)gc * H + h) * (4 * D) + (tid >> 7) * (2 * D) + (tid & (D - 1));
+                dot = part[0] + part[D];
+            }
+        } else {
+            __syncthreads();
+            auto code_of = [&](int t) { return srow[t]; };
+            load_tile_bf16(k, H, h, code_of, false, sK);
+            load_tile_bf16(q, H, h, code_of, true, sQ);
+            load_tile_bf16(v, H, h, code_of, false, sV);
+            load_tile_bf16(dO, H, h, code_of, true, sDO);
+            load_g(gk, H, h, code_of, sB);
+        }
+        if (!CHUNKS) global_to_tile128(chunk_states + ((size_t)(s.chunk_base + c) * H + h) * state_elems, sSc);
         if (CHUNKS) {
             const NextItem nx = next_item(s, c, gc, item, H, n_items);
-            if (nx.c >= 0) {
-                prefetch_rows(k, H, nx.h, s, nx.c);
-                prefetch_rows(q, H, nx.h, s, nx.c);
-                prefetch_rows(v, H, nx.h, s, nx.c);
-                prefetch_rows(dO, H, nx.h, s, nx.c);
-                prefetch_rows(gk, H, nx.h, s, nx.c);
-                prefetch_state(chunk_states, nx.gc, nx.h, H);
-                prefetch_state(ds_tiles, nx.gc, nx.h, H);
-            }
+            if (nx.c >= 0 && tid == 32) prefetch_chunk(maps, true, s, nx, H);
         } else if (c >= 1) {      // the next chunk of the walk (chunk 0 of a sequence with replayed rows is not consecutive)
             if (c - 1 >= 1 || s.n_replay == 0) {
                 prefetch_rows(k, H, h, s, c - 1);
@@ -982,11 +1113,24 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             const char* st = reinterpret_cast<const char*>(chunk_states + ((size_t)(s.chunk_base + c - 1) * H + h) * state_elems);
             for (int p = tid; p < D * D * 2 / 128; p += NT) asm volatile("prefetch.global.L2 [%0];" ::"l"(st + p * 128));
         }
-        if (!CHUNKS) state_to_operand(ds, sdSb, warp, lane);
-        else if (has_ds) global_to_tile128(ds_tiles + ((size_t)gc * H + h) * state_elems, sdSb);
-        tc::cp_async_wait_all();
+        if (!CHUNKS) {
+            state_to_operand(ds, sdSb, warp, lane);
+            tc::cp_async_wait_all();
+        } else if (whole) {
+            ok = tc::mbar_wait_warp(bar_first, ph_first, status, &s_dead) && ok;
+            ph_first ^= 1;
+        } else {
+            tc::cp_async_wait_group<1>();
+        }
         __syncthreads();
-        cumsum_rows(sB, sTmp);
+        cumsum_rows(sB, sTmp);                        // while the rest comes
+        if (CHUNKS) {
+            if (whole || has_s || has_ds) {
+                ok = tc::mbar_wait_warp(bar_rest, ph_rest, status, &s_dead) && ok;
+                ph_rest ^= 1;
+            }
+            tc::cp_async_wait_all();                  // (published by the barrier in chunk_is_mild)
+        }
         const bool mild = chunk_is_mild(sB);          // diagonal blocks as dense products too (see chunk_is_mild)
         const int r_lo = 16 * mb + g, r_hi = r_lo + 8;            // this thread's rows in the [64][128] products
         // ---- dA = dO V^T, iq = dO S_c^T, ik = V dS^T, <S_c, dS> per channel -------------------------------------------
@@ -1003,22 +1147,22 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4], b[4];
-                frag_a<256>(a, aDO, 16 * mb, ks * 16, lane);
-                frag_b_nk<256>(b, aV, ks * 16, 16 * nq, lane);          // dA: columns (keys) 16 * nq ..
+                frag_a<BT>(a, aDO, 16 * mb, ks * 16, lane);
+                frag_b_nk<BT>(b, aV, ks * 16, 16 * nq, lane);          // dA: columns (keys) 16 * nq ..
                 mma16816(da[0], a, b[0], b[1]);
                 mma16816(da[1], a, b[2], b[3]);
                 if (has_s)
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
-                    frag_b_nk<256>(b, aSc, ks * 16, 32 * nq + 16 * n2, lane);
+                    frag_b_nk<D>(b, aSc, ks * 16, 32 * nq + 16 * n2, lane);
                     mma16816(iq[2 * n2], a, b[0], b[1]);
                     mma16816(iq[2 * n2 + 1], a, b[2], b[3]);
                 }
                 if (!has_ds) continue;
-                frag_a<256>(a, aV, 16 * mb, ks * 16, lane);
+                frag_a<BT>(a, aV, 16 * mb, ks * 16, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
-                    frag_b_nk<256>(b, adSb, ks * 16, 32 * nq + 16 * n2, lane);
+                    frag_b_nk<D>(b, adSb, ks * 16, 32 * nq + 16 * n2, lane);
                     mma16816(ik[2 * n2], a, b[0], b[1]);
                     mma16816(ik[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -1040,17 +1184,14 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                 }
             }
         }
-        if constexpr (CHUNKS) {      // <S_c[i,:], dS[i,:]> in four parts of 32 columns, from the scan (dS is fp32 there)
-            if (tid < 2 * D) {
-                const float* part = dots + ((size_t)gc * H + h) * (4 * D) + (tid >> 7) * (2 * D) + (tid & (D - 1));
-                sRowdot[tid] = has_s && has_ds ? part[0] + part[D] : 0.f;
-            }
+        if constexpr (CHUNKS) {
+            if (tid < 2 * D) sRowdot[tid] = dot;
         } else {   // <S_c[i,:], dS[i,:]> over this warp's 64 columns of its 16 state rows i (the two column halves meet later)
             const int i0 = (warp & 7) * 16 + g, c0 = (warp >> 3) * 64 + tq * 2;
             float d_lo = 0.f, d_hi = 0.f;
 #pragma unroll
             for (int n = 0; n < 8; n++) {
-                const float2 s_lo = ld_bf2(sSc, i0, c0 + n * 8), s_hi = ld_bf2(sSc, i0 + 8, c0 + n * 8);
+                const float2 s_lo = ld_bf2<D>(sSc, i0, c0 + n * 8), s_hi = ld_bf2<D>(sSc, i0 + 8, c0 + n * 8);
                 d_lo += s_lo.x * ds[n][0] + s_lo.y * ds[n][1];
                 d_hi += s_hi.x * ds[n][2] + s_hi.y * ds[n][3];
             }
@@ -1078,7 +1219,15 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             if (g == 0) *reinterpret_cast<float2*>(sGi + mb * D + col) = make_float2(g0, g1);
         }
         // ---- scores and the anchored operands ------------------------------------------------------------------------
-        __syncthreads();                              // S_c and V are dead from here on; dA is visible
+        // S_c and V are dead from here on; dA is visible
+        if constexpr (CHUNKS) {
+            if (__syncthreads_or(!ok)) {              // a wait ran out (status word set): let what is in flight land
+                tc::drain_delay();
+                return;
+            }
+        } else {
+            __syncthreads();
+        }
         // a mild chunk's own-block keys and q~ (where the walk goes on) over S_c, its k~ over V; otherwise step factors over S_c
         unsigned char *sKd = sSc, *sQt = sSc + 16384;
         const uint32_t aKd = aSc;
@@ -1098,11 +1247,11 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
             for (int ks = 0; ks < mb + (mild ? 1 : 0); ks++) {
                 uint32_t a[4], b[4];
-                frag_a<128>(a, adAb, 16 * mb, 16 * ks, lane);
+                frag_a<0>(a, adAb, 16 * mb, 16 * ks, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
-                    if (ks < mb) frag_b_kn<256>(b, aKa, ka_row0(mb) + 16 * ks, 32 * nq + 16 * n2, lane);
-                    else frag_b_kn<256>(b, aKd, 16 * mb, 32 * nq + 16 * n2, lane);
+                    if (ks < mb) frag_b_kn<96>(b, aKa, ka_row0(mb) + 16 * ks, 32 * nq + 16 * n2, lane);
+                    else frag_b_kn<BT>(b, aKd, 16 * mb, 32 * nq + 16 * n2, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -1124,10 +1273,10 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
             uint32_t a[4], b[4];
-            frag_a_t<128>(a, adAb, 16 * mb, 16 * I, lane);
+            frag_a_t<0>(a, adAb, 16 * mb, 16 * I, lane);
 #pragma unroll
             for (int n2 = 0; n2 < 2; n2++) {
-                frag_b_kn<256>(b, aQa, 16 * I, 32 * nq + 16 * n2, lane);
+                frag_b_kn<BT>(b, aQa, 16 * I, 32 * nq + 16 * n2, lane);
                 mma16816(acc[2 * n2], a, b[0], b[1]);
                 mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
             }
@@ -1164,15 +1313,34 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                 z[n][1] += __shfl_sync(~0u, z[n][3], tq);
                 if (g == 0) *reinterpret_cast<float2*>(sTmp + mb * D + col) = make_float2(z[n][0], z[n][1]);
             }
+            float2 gamma[4];
+#pragma unroll
+            for (int n = 0; n < 4; n++) {
+                const float2 bn = *reinterpret_cast<const float2*>(sB + (BT - 1) * D + 32 * nq + 8 * n + 2 * tq);
+                gamma[n] = make_float2(ex2(bn.x), ex2(bn.y));
+            }
+            if (CHUNKS) tc::fence_async_smem();
             __syncthreads();
+            if constexpr (CHUNKS) {                   // q, k and the running sums have been read: the next item's come in over them
+                const int next = item + gridDim.x, gc2 = chunk_lo + next / H;
+                first_there = next < n_items;
+                if (first_there) {
+                    if (gc2 < s.chunk_base + s.n_chunks) {
+                        load_first(s, gc2 - s.chunk_base, next % H);
+                    } else {
+                        const SeqInfo s2 = seq_info(tb, owner_of(tb, seq, seq_hi, gc2));
+                        load_first(s2, gc2 - s2.chunk_base, next % H);
+                    }
+                }
+            }
             const int code_lo = srow[r_lo], code_hi = srow[r_hi];
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = 32 * nq + 8 * n + 2 * tq;
                 auto at = [&](const float* x) { return *reinterpret_cast<const float2*>(x + col); };
                 // <S_{c+1}[i,:], dS[i,:]> = e^{b_n} <S_c, dS> + sum_j k_j ew_j ik_j, and the blocks below this one
-                const float2 bn = at(sB + (BT - 1) * D), d0 = at(sRowdot), d1 = at(sRowdot + D);
-                float2 tail = make_float2(ex2(bn.x) * (d0.x + d1.x), ex2(bn.y) * (d0.y + d1.y));
+                const float2 d0 = at(sRowdot), d1 = at(sRowdot + D);
+                float2 tail = make_float2(gamma[n].x * (d0.x + d1.x), gamma[n].y * (d0.y + d1.y));
 #pragma unroll
                 for (int b2 = 0; b2 < 4; b2++) {
                     const float2 x = at(sGi + b2 * D), y = at(sTmp + b2 * D);
@@ -1196,6 +1364,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             block_to_rows(iq, sQa, mb, nq, srow, dq, H, h, lane);      // over the anchored operands, which have been multiplied
             block_to_rows(ik, sKa, mb, nq, srow, dk_, H, h, lane);
         } else {
+            first_there = false;
             __syncthreads();                              // the anchored operands are dead, the step factors visible
             scores_diagonal(sQ, sK, sR, sP, warp, lane);
 #pragma unroll
@@ -1300,10 +1469,10 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             for (int n = 0; n < 4; n++) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
             for (int ks = mb; ks < 4; ks++) {             // A_tj = 0 for t < j
                 uint32_t a[4], b[4];
-                frag_a_t<128>(a, aP, 16 * mb, 16 * ks, lane);
+                frag_a_t<0>(a, aP, 16 * mb, 16 * ks, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
-                    frag_b_kn<256>(b, aDO, 16 * ks, 32 * nq + 16 * n2, lane);
+                    frag_b_kn<BT>(b, aDO, 16 * ks, 32 * nq + 16 * n2, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -1312,10 +1481,10 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int ks = 0; ks < 8; ks++) {
                 uint32_t a[4], b[4];
-                frag_a<256>(a, aKt, 16 * mb, 16 * ks, lane);
+                frag_a<BT>(a, aKt, 16 * mb, 16 * ks, lane);
 #pragma unroll
                 for (int n2 = 0; n2 < 2; n2++) {
-                    frag_b_kn<256>(b, adSb, 16 * ks, 32 * nq + 16 * n2, lane);
+                    frag_b_kn<D>(b, adSb, 16 * ks, 32 * nq + 16 * n2, lane);
                     mma16816(acc[2 * n2], a, b[0], b[1]);
                     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
                 }
@@ -1372,8 +1541,8 @@ int32_t gk_mma_bwd(const BwdArgs& a) {
     gk_mma_bwd_kernel<ROUND><<<n, NT, SharedB::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, nullptr, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
-        (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
+        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{}, ChunkMaps{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
@@ -1413,24 +1582,43 @@ int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrd
     gk_mma_bwd_kernel<ONE_LAUNCH_MODE><<<(int)n, NT, SharedB::bytes, a.stream>>>(
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, nullptr, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
-        (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, flags, ticket, rounds);
+        (const __nv_bfloat16*)a.chunk_states, nullptr, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
+        (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, flags, ticket, rounds, ChunkMaps{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
 // Every (chunk, head) of sequences [seq_lo, seq_hi) on its own; the scan has left the states (and their gradients).
+static int32_t chunk_maps(ChunkMaps* m, const harts_la_tables_t& tb, int32_t H, const void* q, const void* k, const void* v, const void* dO, const float* g,
+                          const void* states, const void* ds_tiles) {
+    const int64_t rows = tb.n_rows, tiles = (int64_t)tb.n_chunks * H;
+    int32_t rc;
+    if ((rc = make_row_map(&m->q, q, rows, H)) != HARTS_OK || (rc = make_row_map(&m->k, k, rows, H)) != HARTS_OK ||
+        (rc = make_row_map(&m->v, v, rows, H)) != HARTS_OK || (rc = make_gate_map(&m->g, g, rows, H)) != HARTS_OK ||
+        (rc = make_state_map(&m->s, states, tiles)) != HARTS_OK)
+        return rc;
+    m->dO = m->v;
+    m->ds = m->s;
+    if (dO && ((rc = make_row_map(&m->dO, dO, rows, H)) != HARTS_OK || (rc = make_state_map(&m->ds, ds_tiles, tiles)) != HARTS_OK)) return rc;
+    return HARTS_OK;
+}
 int32_t gk_chunk_fwd(const FwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    ChunkMaps maps;
+    const int32_t rc = chunk_maps(&maps, a.tb, a.H, a.q, a.k, a.v, nullptr, a.g, a.chunk_states, nullptr);
+    if (rc != HARTS_OK) return rc;
     if (cudaFuncSetAttribute(gk_chunk_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedC::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
     launch_after(gk_chunk_fwd_kernel, (int)(n < 2 * sm_count() ? n : 2 * sm_count()), NT, SharedC::bytes, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
-        (__nv_bfloat16*)a.o, (const __nv_bfloat16*)a.chunk_states, status_gate(a.flags, a.dev_status));
+        (__nv_bfloat16*)a.o, maps, a.dev_status, status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
+    ChunkMaps maps;
+    const int32_t rc = chunk_maps(&maps, a.tb, a.H, a.q, a.k, a.v, a.dO, a.g, a.chunk_states, ds_tiles);
+    if (rc != HARTS_OK) return rc;
     if (cudaFuncSetAttribute(gk_mma_bwd_kernel<CHUNKS_MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SharedB::bytes) != cudaSuccess)
         return HARTS_ECUDA;
     const int64_t n = (int64_t)a.tb.n_chunks * a.H;
@@ -1439,8 +1627,8 @@ int32_t gk_chunk_bwd(const BwdArgs& a, const void* ds_tiles, const float* dots) 
     launch_after(gk_mma_bwd_kernel<CHUNKS_MODE>, (int)(n < sm_count() ? n : sm_count()), NT, SharedB::bytes, a.stream,
         a.tb, a.seq_lo, a.seq_hi, a.H, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.g,
         (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_, (__nv_bfloat16*)a.dv_, a.dg,
-        (const __nv_bfloat16*)a.chunk_states, (const __nv_bfloat16*)ds_tiles, dots, (float*)(base + sl.ds0), (float*)(base + sl.rk),
-        (float*)(base + sl.rv), (float*)(base + sl.rg), status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{});
+        nullptr, dots, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv), (float*)(base + sl.rg),
+        status_gate(a.flags, a.dev_status), a.dev_status, nullptr, nullptr, RoundOrder{}, maps);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 

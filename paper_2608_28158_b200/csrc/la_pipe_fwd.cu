@@ -142,11 +142,6 @@ __device__ __forceinline__ void mma_steps(uint32_t d, uint32_t a, uint32_t b, ui
     for (int ks = 1; ks < STEPS; ks++) mma_lo<true>(d, a + ks * SA + (ks >> 2) * GA, b + ks * SB + (ks >> 2) * GB, idesc);
 }
 
-// asks the L2 for a tile that will be loaded later
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
-}
-
 template <int NV>
 __global__ void __launch_bounds__(NT, 1)
 pipe_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __grid_constant__ CUtensorMap map_q,

@@ -85,9 +85,6 @@ struct Misc {
 };
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
-    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
-}
 __device__ __forceinline__ SeqInfo seq_info(const harts_la_tables_t& tb, int seq) {
     SeqInfo s;
     s.own_begin = tb.seq_own_begin[seq];
