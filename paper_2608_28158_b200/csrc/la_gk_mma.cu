@@ -41,6 +41,11 @@ constexpr float LOG2E = 1.4426950408889634f;
 template <int ROWS = BT>
 __device__ __forceinline__ uint32_t sw256(int r, int c16) { return (uint32_t)((c16 >> 3) * (ROWS * 128) + r * 128 + (((c16 & 7) ^ (r & 7)) << 4)); }
 __device__ __forceinline__ uint32_t sw128(int r, int c16) { return (uint32_t)(r * 128 + ((c16 ^ (r & 7)) << 4)); }
+// The running log-decays [64][128] fp32: where (r, col) lies.  Groups of four floats are XOR-ed so that the 8 rows x 8 columns of a fragment
+// and the 32-byte pieces of two rows are read without bank conflicts (laid out plainly: 3.9 k of 17.8 k wavefronts an item of the backward).
+__device__ __forceinline__ int b_at(int r, int col) {
+    return r * D + ((((col >> 2) ^ ((col >> 5) & 1) ^ ((r & 3) << 1)) << 2) | (col & 3));
+}
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
@@ -205,7 +210,7 @@ __device__ __forceinline__ void prefetch_chunk(const ChunkMaps& m, bool backward
     tc::tma_prefetch_3d(&m.g, 0, nx.h, row0);
 }
 
-// log-decays -> their running sum over the rows in log2 units, per channel: four threads per channel (16 rows each, scanned in registers), joined through
+// log-decays, laid out plainly -> their running sum over the rows in log2 units (b_at), per channel: four threads per channel (16 rows each, scanned in registers), joined through
 // sTmp[4][128]
 __device__ __forceinline__ void cumsum_rows(float* sB, float* sTmp) {
     const int tid = threadIdx.x, i = tid & (D - 1), part = tid >> 7;
@@ -219,7 +224,7 @@ __device__ __forceinline__ void cumsum_rows(float* sB, float* sTmp) {
     float base = 0.f;
     for (int pp = 0; pp < part; pp++) base += sTmp[pp * D + i];
 #pragma unroll
-    for (int u = 0; u < 16; u++) sB[(part * 16 + u) * D + i] = x[u] + base;
+    for (int u = 0; u < 16; u++) sB[b_at(part * 16 + u, i)] = x[u] + base;
     __syncthreads();
 }
 
@@ -267,8 +272,8 @@ __device__ __forceinline__ void anchored_operands(const unsigned char* sQ, const
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const int i = c16 * 8 + e * 2;
-            const float2 bs = *reinterpret_cast<const float2*>(sB + src_row * D + i);
-            const float2 ba = *reinterpret_cast<const float2*>(sB + anchor_row * D + i);
+            const float2 bs = *reinterpret_cast<const float2*>(sB + b_at(src_row, i));
+            const float2 ba = *reinterpret_cast<const float2*>(sB + b_at(anchor_row, i));
             const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[e]));
             // q^: e^{b_t - a_I};  k^(I): e^{a_I - b_j}
             const float e0 = is_q ? ex2(bs.x - ba.x) : ex2(ba.x - bs.x);
@@ -291,7 +296,7 @@ constexpr float MILD_LOG2 = 100.f;
 
 __device__ __forceinline__ bool chunk_is_mild(const float* sB) {
     const int i = threadIdx.x & (D - 1), blk = threadIdx.x >> 7;       // 512 threads: 4 blocks x 128 channels
-    const float fall = sB[16 * blk * D + i] - sB[(16 * blk + 15) * D + i];
+    const float fall = sB[b_at(16 * blk, i)] - sB[b_at(16 * blk + 15, i)];
     return __syncthreads_or(!(fall <= MILD_LOG2)) == 0;                  // also false for a NaN gate
 }
 
@@ -306,8 +311,8 @@ __device__ __forceinline__ void mild_operands(const unsigned char* sQ, const uns
         const uint32_t off = sw256(t, c16);
         float bs[8], ba[8];
         auto row8 = [&](float (&x)[8], int r) {
-            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(sB + r * D + c16 * 8);
-            *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(sB + r * D + c16 * 8 + 4);
+            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(sB + b_at(r, c16 * 8));
+            *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(sB + b_at(r, c16 * 8 + 4));
         };
         auto scaled = [&](const uint4& x, auto exponent) {
             const uint32_t w[4] = {x.x, x.y, x.z, x.w};
@@ -391,8 +396,8 @@ __device__ __forceinline__ void step_factors(const float* sB, float* sR) {
     for (int p = threadIdx.x; p < BT * 32; p += NT) {
         const int t = p >> 5, c4 = p & 31;
         if (t == 0) continue;
-        const float4 hi = *reinterpret_cast<const float4*>(sB + t * D + c4 * 4);
-        const float4 lo = *reinterpret_cast<const float4*>(sB + (t - 1) * D + c4 * 4);
+        const float4 hi = *reinterpret_cast<const float4*>(sB + b_at(t, c4 * 4));
+        const float4 lo = *reinterpret_cast<const float4*>(sB + b_at(t - 1, c4 * 4));
         *reinterpret_cast<float4*>(sR + t * D + c4 * 4) = make_float4(ex2(hi.x - lo.x), ex2(hi.y - lo.y), ex2(hi.z - lo.z), ex2(hi.w - lo.w));
     }
 }
@@ -449,8 +454,8 @@ __device__ __forceinline__ void scale_qk(const unsigned char* sQ, const unsigned
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             const int i = c16 * 8 + e * 2;
-            const float2 bt = *reinterpret_cast<const float2*>(sB + t * D + i);
-            const float2 bn = *reinterpret_cast<const float2*>(sB + (BT - 1) * D + i);
+            const float2 bt = *reinterpret_cast<const float2*>(sB + b_at(t, i));
+            const float2 bn = *reinterpret_cast<const float2*>(sB + b_at(BT - 1, i));
             const float2 qf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qw[e]));
             const float2 kf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kw[e]));
             if (Q) qw[e] = pack2(qf.x * ex2(bt.x), qf.y * ex2(bt.y));
@@ -512,7 +517,7 @@ __device__ __forceinline__ void state_to_global(const float (&st)[8][4], float* 
 // stored [row][128]
 __device__ __forceinline__ void state_update(float (&st)[8][4], const float* sB, uint32_t aX, uint32_t aY, int warp, int lane) {
     const int g = lane >> 2, r0 = (warp & 7) * 16, c0 = (warp >> 3) * 64;
-    const float g_lo = ex2(sB[(BT - 1) * D + r0 + g]), g_hi = ex2(sB[(BT - 1) * D + r0 + g + 8]);
+    const float g_lo = ex2(sB[b_at(BT - 1, r0 + g)]), g_hi = ex2(sB[b_at(BT - 1, r0 + g + 8)]);
 #pragma unroll
     for (int n = 0; n < 8; n++) {
         st[n][0] *= g_lo; st[n][1] *= g_lo; st[n][2] *= g_hi; st[n][3] *= g_hi;
@@ -1203,9 +1208,9 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
         for (int n = 0; n < 4; n++) {
             const int col = 32 * nq + 8 * n + 2 * tq;
-            const float2 b_lo = *reinterpret_cast<const float2*>(sB + r_lo * D + col);
-            const float2 b_hi = *reinterpret_cast<const float2*>(sB + r_hi * D + col);
-            const float2 b_n = *reinterpret_cast<const float2*>(sB + (BT - 1) * D + col);
+            const float2 b_lo = *reinterpret_cast<const float2*>(sB + b_at(r_lo, col));
+            const float2 b_hi = *reinterpret_cast<const float2*>(sB + b_at(r_hi, col));
+            const float2 b_n = *reinterpret_cast<const float2*>(sB + b_at(BT - 1, col));
             const float2 k_lo = ld_bf2(sK, r_lo, col), k_hi = ld_bf2(sK, r_hi, col);
             iq[n][0] *= ex2(b_lo.x); iq[n][1] *= ex2(b_lo.y); iq[n][2] *= ex2(b_hi.x); iq[n][3] *= ex2(b_hi.y);
             ik[n][0] *= ex2(b_n.x - b_lo.x); ik[n][1] *= ex2(b_n.y - b_lo.y);
@@ -1259,9 +1264,9 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = 32 * nq + 8 * n + 2 * tq;
-                const float2 b_lo = *reinterpret_cast<const float2*>(sB + r_lo * D + col);
-                const float2 b_hi = *reinterpret_cast<const float2*>(sB + r_hi * D + col);
-                const float2 an = *reinterpret_cast<const float2*>(sB + 16 * mb * D + col);
+                const float2 b_lo = *reinterpret_cast<const float2*>(sB + b_at(r_lo, col));
+                const float2 b_hi = *reinterpret_cast<const float2*>(sB + b_at(r_hi, col));
+                const float2 an = *reinterpret_cast<const float2*>(sB + b_at(16 * mb, col));
                 iq[n][0] += ex2(b_lo.x - an.x) * acc[n][0]; iq[n][1] += ex2(b_lo.y - an.y) * acc[n][1];
                 iq[n][2] += ex2(b_hi.x - an.x) * acc[n][2]; iq[n][3] += ex2(b_hi.y - an.y) * acc[n][3];
             }
@@ -1283,9 +1288,9 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
 #pragma unroll
             for (int n = 0; n < 4; n++) {
                 const int col = 32 * nq + 8 * n + 2 * tq;
-                const float2 b_lo = *reinterpret_cast<const float2*>(sB + r_lo * D + col);
-                const float2 b_hi = *reinterpret_cast<const float2*>(sB + r_hi * D + col);
-                const float2 an = *reinterpret_cast<const float2*>(sB + 16 * I * D + col);
+                const float2 b_lo = *reinterpret_cast<const float2*>(sB + b_at(r_lo, col));
+                const float2 b_hi = *reinterpret_cast<const float2*>(sB + b_at(r_hi, col));
+                const float2 an = *reinterpret_cast<const float2*>(sB + b_at(16 * I, col));
                 ik[n][0] += ex2(an.x - b_lo.x) * acc[n][0]; ik[n][1] += ex2(an.y - b_lo.y) * acc[n][1];
                 ik[n][2] += ex2(an.x - b_hi.x) * acc[n][2]; ik[n][3] += ex2(an.y - b_hi.y) * acc[n][3];
             }
@@ -1316,7 +1321,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
             float2 gamma[4];
 #pragma unroll
             for (int n = 0; n < 4; n++) {
-                const float2 bn = *reinterpret_cast<const float2*>(sB + (BT - 1) * D + 32 * nq + 8 * n + 2 * tq);
+                const float2 bn = *reinterpret_cast<const float2*>(sB + b_at(BT - 1, 32 * nq + 8 * n + 2 * tq));
                 gamma[n] = make_float2(ex2(bn.x), ex2(bn.y));
             }
             if (CHUNKS) tc::fence_async_smem();
@@ -1399,7 +1404,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                     for (int tt = 0; tt < 16; tt++) {
                         const int t = t0 + tt;
                         const float qt = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(sQ + sw256(t, i >> 3) + (i & 7) * 2));
-                        const float bt = sB[t * D + i];
+                        const float bt = sB[b_at(t, i)];
                         const float r = ex2(bt - b_prev);
                         b_prev = bt;
                         xr[tt] = 1.f;
@@ -1428,7 +1433,7 @@ gk_mma_bwd_kernel(harts_la_tables_t tb, int seq_lo, int seq_hi, int H, const __n
                 sTmp[blk * D + i] = total;
                 __syncthreads();
                 // dg_t = suffix over the rows + <S_{c+1}[i,:], dS[i,:]> = e^{b_n} <S_c, dS> + sum_j k_j ew_j ik_j
-                float suffix = ex2(sB[(BT - 1) * D + i]) * (sRowdot[i] + sRowdot[D + i]) + sGi[i] + sGi[D + i] + sGi[2 * D + i] +
+                float suffix = ex2(sB[b_at(BT - 1, i)]) * (sRowdot[i] + sRowdot[D + i]) + sGi[i] + sGi[D + i] + sGi[2 * D + i] +
                                sGi[3 * D + i];
                 for (int b2 = 3; b2 > blk; b2--) suffix += sTmp[b2 * D + i];
 #pragma unroll
