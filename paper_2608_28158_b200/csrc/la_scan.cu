@@ -162,20 +162,39 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
 #pragma unroll
                 for (int e = 0; e < CW / 4; e++) *reinterpret_cast<float4*>(x + 4 * e) = __ldcg(src + e);
             }
+            // what the next export (backward: the next boundary with gradients) needs is asked for at the one before it: a table entry
+            // that is used as soon as it is loaded holds the chain up by 0.35 us
+            const int req_end = BWD ? it.req_lo - 1 : it.req_hi, way = BWD ? -1 : 1;
             int req = BWD ? it.req_hi - 1 : it.req_lo;
-            int boundary = (BWD ? req >= it.req_lo : req < it.req_hi) ? tb.slot_chunk[req] : -1;
+            int boundary = req != req_end ? tb.slot_chunk[req] : -1, boundary2 = req != req_end && req + way != req_end ? tb.slot_chunk[req + way] : -1;
+            int cons_lo = 0, cons_hi = 0, who = 0;      // backward: the sequences that started from it; a lane's one of 32
+            auto consumers = [&] {
+                if (BWD && req != req_end) {
+                    cons_lo = tb.slot_cons_ptr[req];
+                    cons_hi = tb.slot_cons_ptr[req + 1];
+                }
+            };
+            auto advance = [&] {
+                req += way;
+                boundary = boundary2;
+                boundary2 = req != req_end && req + way != req_end ? tb.slot_chunk[req + way] : -1;
+                consumers();
+            };
+            consumers();
             for (int i = 0; i < it.n_chunks && alive; i++) {
                 const int c = chunk_of(it, i);
                 if (BWD && boundary == c + 1) {   // gradients of every sequence that started from this boundary, in table order
                     unsigned there = 0;       // whose flag is up already: a lane each looks, 32 at a time
-                    for (int u = tb.slot_cons_ptr[req], k = 0; u < tb.slot_cons_ptr[req + 1]; u++, k++) {
-                        if (order.n && (k & 31) == 0) {
-                            const bool mine = u + lane < tb.slot_cons_ptr[req + 1] &&
-                                              ld_acquire(flags + ((size_t)tb.slot_cons_seq[u + lane] * H + it.h) * SLICES + it.slice) >= NS / 32;
-                            there = __ballot_sync(0xffffffffu, mine);
-                            __syncwarp();     // hands on what the lanes acquired
+                    for (int u = cons_lo, k = 0; u < cons_hi; u++, k++) {
+                        if ((k & 31) == 0) {
+                            if ((k > 0 || i == 0) && u + lane < cons_hi) who = tb.slot_cons_seq[u + lane];
+                            if (order.n) {
+                                const bool mine = u + lane < cons_hi && ld_acquire(flags + ((size_t)who * H + it.h) * SLICES + it.slice) >= NS / 32;
+                                there = __ballot_sync(0xffffffffu, mine);
+                                __syncwarp();     // hands on what the lanes acquired
+                            }
                         }
-                        const size_t from = (size_t)tb.slot_cons_seq[u] * H + it.h;
+                        const size_t from = (size_t)__shfl_sync(0xffffffffu, who, k & 31) * H + it.h;
                         if (order.n && !(there >> (k & 31) & 1)) alive = flag_wait_warp(flags + from * SLICES + it.slice, NS / 32, status, &m.dead) && alive;
                         const float4* src = ds0_of(from);
 #pragma unroll
@@ -184,9 +203,9 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                             x[4 * e] += y.x, x[4 * e + 1] += y.y, x[4 * e + 2] += y.z, x[4 * e + 3] += y.w;
                         }
                     }
-                    req--;
-                    boundary = req >= it.req_lo ? tb.slot_chunk[req] : -1;
+                    advance();
                 }
+                if (BWD && boundary == c && cons_lo + lane < cons_hi) who = tb.slot_cons_seq[cons_lo + lane];      // of the next step
                 if (!BWD || i > 0) {              // the state before this step as a bf16 tile (backward: zero after the last chunk)
                     // backward: the buffer holds S_c, which is multiplied with the gradient before that is rounded over it
                     if ((BWD || gt >= OUTS) && !wait_warp(&m.out_empty[gt % OUTS], BWD ? gt / OUTS : gt / OUTS - 1)) alive = false;
@@ -220,14 +239,21 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 }
                 if (!BWD && boundary == c) {
                     const size_t to = (size_t)req * H + it.h;
-                    float4* dst = reinterpret_cast<float4*>(slots + to * (D * D) + in_state);
+                    float* dst = slots + to * (D * D) + in_state;
+                    // a thread's row is 512 bytes from the next one's: whole sectors at a time, where the array allows it
+                    if ((reinterpret_cast<uintptr_t>(slots) & 31) == 0) {
 #pragma unroll
-                    for (int e = 0; e < CW / 4; e++) dst[e] = *reinterpret_cast<const float4*>(x + 4 * e);
+                        for (int e = 0; e < CW; e += 8)
+                            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + e), "f"(x[e]), "f"(x[e + 1]), "f"(x[e + 2]),
+                                         "f"(x[e + 3]), "f"(x[e + 4]), "f"(x[e + 5]), "f"(x[e + 6]), "f"(x[e + 7]) : "memory");
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < CW; e += 4) *reinterpret_cast<float4*>(dst + e) = *reinterpret_cast<const float4*>(x + e);
+                    }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&m.exported[n_exported % EXPORTS]);      // the store warp publishes it: no fence in the chain
                     n_exported++;
-                    req++;
-                    boundary = req < it.req_hi ? tb.slot_chunk[req] : -1;
+                    advance();
                 }
                 if (i >= it.n_steps) break;
                 if (!wait_warp(&m.gates_full[gs % GATES], gs / GATES) || !wait_warp(&m.u_full[gs & 1], gs >> 1)) alive = false;
@@ -319,7 +345,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 const float* w = m.w[gs % GATES];
 #pragma unroll
                 for (int u = 0; u < BT * NV / 8 / NWT; u++) {
-                    const int e = wt + u * NWT, t = NV == 32 ? e >> 2 : (e >> 3) & 63, p = NV == 32 ? 0 : e >> 9;
+                    const int e = wt + u * NWT, t = NV == 32 ? (e >> 5) * 8 + (e >> 2 & 1) * 4 + (e >> 3 & 3) : (e >> 3) & 63, p = NV == 32 ? 0 : e >> 9;
                     const int ch = NV == 32 ? (slice & 1) * 4 + (e & 3) : e & 7;
                     uint4* at = reinterpret_cast<uint4*>(sb + p * PANEL + sw128_chunk(t, ch));
                     uint4 y = *at;
