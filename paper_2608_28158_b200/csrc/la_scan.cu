@@ -256,7 +256,10 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                     advance();
                 }
                 if (i >= it.n_steps) break;
-                if (!wait_warp(&m.gates_full[gs % GATES], gs / GATES) || !wait_warp(&m.u_full[gs & 1], gs >> 1)) alive = false;
+                // both tries in flight together (per channel, where the weights are late, the second one is better made after the first)
+                const bool gates = !GK && mbar_try(&m.gates_full[gs % GATES], gs / GATES & 1), sum = !GK && mbar_try(&m.u_full[gs & 1], gs >> 1 & 1);
+                if ((GK || !__all_sync(~0u, gates && sum)) && (!wait_warp(&m.gates_full[gs % GATES], gs / GATES) || !wait_warp(&m.u_full[gs & 1], gs >> 1)))
+                    alive = false;
                 const float gamma = GK ? m.gammas[gs % GATES][L] : m.gamma[gs % GATES];
                 tc_fence_after();
 #pragma unroll
@@ -269,10 +272,7 @@ scan_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const __
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&m.u_empty[gs & 1]);
-                    mbar_arrive(&m.gates_empty[gs % GATES]);
-                }
+                if (lane < 2) mbar_arrive(lane ? &m.gates_empty[gs % GATES] : &m.u_empty[gs & 1]);
                 gs++;
             }
             if (BWD && it.init_slot >= 0 && alive) {     // the hand-off into the sequence that exported this state
