@@ -50,7 +50,7 @@ template <int NV, bool GK>
 struct Shape {
     static constexpr int NS = NV == 32 ? 128 : 256, NWT = NS, NT = NS + NWT + 128;   // state threads, weighting threads, four warps
     static constexpr int CW = NV * 128 / NS;               // state columns per state thread
-    static constexpr int STAGES = GK ? 2 : NV == 64 ? 5 : 3;        // chunks of rows in shared memory
+    static constexpr int STAGES = GK ? NV == 64 ? 3 : 2 : NV == 64 ? 5 : 3;        // chunks of rows in shared memory
     static constexpr int OUTS = GK ? 2 : 3;                // state tiles on their way out
     // a 32-column slice loads the 64-column panel it lies in
     static constexpr int A = 2 * PANEL, B = (NV + 63) / 64 * PANEL, G = GK ? BT * D * 4 : 0,
