@@ -29,6 +29,25 @@ inline bool use_tc(int32_t dtype, int32_t dk, int32_t dv, uint32_t flags) {
 float* f32_extra(const harts_la_tables_t& tb, const void* chunk_states, int32_t H, int32_t dk, int32_t dv) {
     return reinterpret_cast<float*>(const_cast<char*>(static_cast<const char*>(chunk_states)) + harts::f32_extra_offset(tb, H, dk, dv));
 }
+// Whether round r of the walk backward sums its hand-off gradients in runs, and the positions of slot_cons_seq that its sequences are.  Where
+// sequences are short a 64 KB gradient each is what a round writes and the next reads; in runs of eight it is an eighth of that (171,829
+// replay tokens x 16 heads, 4,258 sequences of one to three chunks: reductions 759 -> 187 us, walk 5,580 -> 5,767, a step 9,644 -> 9,240; in runs
+// of sixteen 134, 5,893 and 9,334).  Not where sequences are long, whose dealing by length matters
+// more, nor where the runs would be fewer than four an SM.  Only inside a call for all rounds: a round issued alone leaves every sequence's own.
+bool handoff_runs(const harts::Plan& p, const harts_la_tables_t& tb, int32_t r, int32_t H, int32_t (&run)[2]) {
+    const int32_t lo = p.round_seq_ptr[r - 1], hi = p.round_seq_ptr[r];
+    if (tb.n_chunks >= 4 * (int64_t)tb.n_seq || (int64_t)(hi - lo) * H < 4 * harts::HANDOFF_RUN * (int64_t)harts::sm_count()) return false;
+    int32_t first = tb.n_slots, last = -1;
+    for (int32_t s = lo; s < hi; s++) {
+        if (p.seq_init_slot[s] < 0) return false;
+        first = p.seq_init_slot[s] < first ? p.seq_init_slot[s] : first;
+        last = p.seq_init_slot[s] > last ? p.seq_init_slot[s] : last;
+    }
+    if (p.slot_cons_ptr[last + 1] - p.slot_cons_ptr[first] != hi - lo) return false;
+    run[0] = p.slot_cons_ptr[first];
+    run[1] = p.slot_cons_ptr[last + 1];
+    return true;
+}
 // Chunk-parallel path over sequences [range[0], range[n]), range[r]..range[r+1] per round: the scan, then all chunks at once.
 harts::RoundOrder round_order(const int32_t* range, int32_t n) {
     harts::RoundOrder ro;
@@ -134,10 +153,10 @@ int32_t harts_la_fwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
     return harts::fma_fwd(a);
 }
 
-int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t seq_hi, const void* q, const void* k,
-                          const void* v, const float* g, const void* dO, void* dq, void* dk_, void* dv_, float* dg,
-                          const void* chunk_states, void* scratch, int32_t H, int32_t dk, int32_t dv, int32_t dtype,
-                          uint32_t flags, int32_t* dev_status, void* stream) {
+static int32_t bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t seq_hi, const void* q, const void* k,
+                        const void* v, const float* g, const void* dO, void* dq, void* dk_, void* dv_, float* dg,
+                        const void* chunk_states, void* scratch, int32_t H, int32_t dk, int32_t dv, int32_t dtype,
+                        uint32_t flags, int32_t* dev_status, void* stream, int32_t run_lo, int32_t run_hi, bool runs_below) {
     int32_t rc = check_common(tb, seq_lo, seq_hi, H, dk, dv, dtype);
     if (rc != HARTS_OK) return rc;
     if (!q || !k || !v || !g || !dO || !dq || !dk_ || !dv_ || !dg || !chunk_states || !scratch) return HARTS_EINVAL;
@@ -145,7 +164,7 @@ int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
         misaligned(dk_) || misaligned(dv_) || misaligned(dg) || misaligned(chunk_states) || misaligned(scratch))
         return HARTS_EINVAL;
     harts::BwdArgs a{*tb, seq_lo, seq_hi, q, k, v, g, dO, dq, dk_, dv_, dg, chunk_states, scratch, H, dk, dv, dtype,
-                     flags, dev_status, static_cast<cudaStream_t>(stream)};
+                     flags, dev_status, static_cast<cudaStream_t>(stream), run_lo, run_hi, runs_below};
     if (flags & HARTS_FLAG_CHECK_TABLES)
         if ((rc = harts::check_tables(*tb, seq_lo, seq_hi, dev_status, a.stream)) != HARTS_OK) return rc;
     const int32_t range[2] = {seq_lo, seq_hi};
@@ -153,6 +172,13 @@ int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t s
     if (harts::chunk_parallel(*tb, H, dk, dv, dtype, flags)) return chunk_parallel_bwd(a, range, 1);
     if (use_tc(dtype, dk, dv, flags)) return harts::tc_bwd(a);
     return harts::fma_bwd(a);
+}
+
+int32_t harts_la_bwd_seqs(const harts_la_tables_t* tb, int32_t seq_lo, int32_t seq_hi, const void* q, const void* k,
+                          const void* v, const float* g, const void* dO, void* dq, void* dk_, void* dv_, float* dg,
+                          const void* chunk_states, void* scratch, int32_t H, int32_t dk, int32_t dv, int32_t dtype,
+                          uint32_t flags, int32_t* dev_status, void* stream) {
+    return bwd_seqs(tb, seq_lo, seq_hi, q, k, v, g, dO, dq, dk_, dv_, dg, chunk_states, scratch, H, dk, dv, dtype, flags, dev_status, stream, 0, 0, false);
 }
 
 int32_t harts_la_bwd_finish(const harts_la_tables_t* tb, void* dk_, void* dv_, float* dg, const void* scratch,
@@ -253,10 +279,14 @@ int32_t harts_la_bwd(const harts_la_plan_t* plan, const void* dev_blob, int32_t 
         if (rc == HARTS_OK) done = true;
         else if (rc != HARTS_EUNSUPPORTED) return rc;
     }
+    bool runs_below = false;
     for (int32_t r = r1; r >= r0 && !done; r--) {
-        rc = harts_la_bwd_seqs(&tb, p->round_seq_ptr[r - 1], p->round_seq_ptr[r], q, k, v, g, dO, dq, dk_, dv_, dg,
-                               chunk_states, scratch, H, dk, dv, dtype, flags, dev_status, stream);
+        int32_t run[2] = {0, 0};
+        const bool runs = round == 0 && use_tc(dtype, dk, dv, flags) && handoff_runs(*p, tb, r, H, run);
+        rc = bwd_seqs(&tb, p->round_seq_ptr[r - 1], p->round_seq_ptr[r], q, k, v, g, dO, dq, dk_, dv_, dg, chunk_states, scratch, H, dk, dv, dtype, flags,
+                      dev_status, stream, run[0], run[1], runs_below);
         if (rc != HARTS_OK) return rc;
+        runs_below = runs;
     }
     if (r0 == 1) return harts_la_bwd_finish(&tb, dk_, dv_, dg, scratch, H, dk, dv, dtype, stream);
     return HARTS_OK;

@@ -38,10 +38,10 @@ struct KvTile {
 template <int W>
 struct TileWalkT {      // enumerates the key tiles (W rows) of one item in order; run data is read once per run, not per tile
     const Index& ix;
-    int run0, run, run_end, off, own_row0, own_end, q0, cur_row0, cur_len;
+    int run, run_end, off, own_row0, own_end, q0, cur_row0, cur_len;
     bool in_own;
     __device__ TileWalkT(const Index& ix_, int piece, int qt) : ix(ix_) {
-        run0 = run = ix.anc_ptr[piece];
+        run = ix.anc_ptr[piece];
         run_end = ix.anc_ptr[piece + 1];
         off = 0;
         own_row0 = ix.piece_row0[piece];
@@ -53,11 +53,6 @@ struct TileWalkT {      // enumerates the key tiles (W rows) of one item in orde
             cur_row0 = ix.anc_row0[run];
             cur_len = ix.anc_len[run];
         }
-    }
-    __device__ int count() const {          // number of tiles next() will deliver from a fresh walk
-        int n = (own_end + W - 1) / W;
-        for (int r = run0; r < run_end; r++) n += (ix.anc_len[r] + W - 1) / W;
-        return n;
     }
     __device__ bool next(KvTile& t) {
         if (!in_own && off + W < cur_len) {       // inside a run
@@ -93,8 +88,9 @@ struct TileWalkT {      // enumerates the key tiles (W rows) of one item in orde
 };
 using TileWalk = TileWalkT<BK>;
 
-// dK / dV work of small problems, cut into units (attn_split.cu): a unit is a run of the query tiles of one key tile, in the
-// order of QWalk; slot: where its partial sums go, -1: the item is not cut.
+// dK / dV work of small problems, cut into units (attn_split.cu): a unit is some of the query tiles of one key tile, in the
+// order of QRuns: n_tiles from head g of the group, from row `row` of the run that ends at `end` on (lead: that row's distance to the key
+// tile's first row, -1 for descendants; d: the descendant behind the run).  slot: where its partial sums go, -1: the item is not cut.
 struct DkvUnit {
     int piece, kt, n_tiles, slot, g, row, end, lead, d;
 };

@@ -146,7 +146,7 @@ attn_dkv_kernel(Index ix, int Hq, int Hkv, int G, float scale, const __grid_cons
         const int kv_valid = min(BKV, ix.piece_len[piece] - kt * BKV);
 
         if (is_producer) {
-            // ---- TMA producer: the K and V tiles, then the query / dO tiles STAGES deep -----------------------------
+            // ---- TMA producer: the K and V tiles, then the query and dO tiles (QST and DST deep) -----------------------------
             mbar_wait(&m.bar_kvfree, ph_kv ^ 1, status, &m.dead);    // the last item's S^T and dP^T products have read the tiles
             ph_kv ^= 1;
             mbar_expect_tx(&m.bar_kv, 2 * TILE);

@@ -38,6 +38,10 @@ struct BwdArgs {
     uint32_t flags;
     int32_t* dev_status;
     cudaStream_t stream;
+    // hand-off gradients summed in runs (HANDOFF_RUN): this range of slot_cons_seq are the launch's sequences, and each run's sum is left in
+    // its first one's buffer (run_hi = 0: every sequence leaves its own); runs_below: the round after this one left its gradients so
+    int32_t run_lo = 0, run_hi = 0;
+    bool runs_below = false;
 };
 
 // Byte offsets inside the backward scratch buffer (each region 256-byte aligned).
@@ -237,7 +241,11 @@ int32_t gk_mma_fwd_all(const FwdArgs& a, int* flags, int* ticket);     // all ro
 int32_t gk_mma_bwd_all(const BwdArgs& a, int* flags, int* ticket, const RoundOrder& rounds);
 int32_t tc_bwd(const BwdArgs& a);
 int32_t tc_bwd_fused(const BwdArgs& a, int* flags, int* ticket, const RoundOrder& rounds);   // all rounds in one launch
-int32_t handoff_reduce(const BwdArgs& a);
+// The tensor-core walk sums the gradients of a boundary's consumers in runs -- the positions of slot_cons_seq from one multiple of HANDOFF_RUN
+// to the next -- and then the runs, both in table order, whoever does it.  Elsewhere (run = 1) one after the other.
+constexpr int HANDOFF_RUN = 8;
+int sm_count();
+int32_t handoff_reduce(const BwdArgs& a, int run = 1);
 int32_t replay_reduce(const harts_la_tables_t& tb, void* dk_, void* dv_, float* dg, const void* scratch, int32_t H,
                       int32_t dk, int32_t dv, int32_t dtype, cudaStream_t stream);
 

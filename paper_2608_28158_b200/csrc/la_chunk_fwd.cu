@@ -138,7 +138,7 @@ chunk_fwd_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H, cons
             fence_async_smem();
             __syncthreads();
         }
-        if (is_mma) {                      // an elected lane issues: operands in uniform registers
+        if (is_mma) {                      // an elected lane issues
             if (mbar_wait_warp(&m.bar_tiles, ph, status, &m.dead)) tiles_pending = false;
             tc_fence_after();
             if (elect_one()) {

@@ -527,42 +527,59 @@ int32_t fma_fwd(const FwdArgs& a) {
 // sequences [seq_lo, seq_hi) exported: a bandwidth-bound pass, in consumer order (deterministic), so that the
 // backward kernels add one tensor per boundary instead of walking the consumer list under their own latency.
 __global__ void __launch_bounds__(256) handoff_reduce_kernel(const harts_la_tables_t tb, int seq_lo, int seq_hi, int H,
-                                                             int elems, float* __restrict__ ds0, const int32_t* gate) {
+                                                             int elems, float* __restrict__ ds0, int run, bool summed, const int32_t* gate) {
     if (gate_closed(gate)) return;
     const int slot = blockIdx.x;
     if (slot < tb.seq_req_ptr[seq_lo] || slot >= tb.seq_req_ptr[seq_hi]) return;
     const int c0 = tb.slot_cons_ptr[slot], c1 = tb.slot_cons_ptr[slot + 1];
-    if (c1 - c0 < 2) return;
+    if (c1 - c0 < 2 || (summed && c0 / run == (c1 - 1) / run)) return;
     const int h = blockIdx.y;
-    float4* dst = reinterpret_cast<float4*>(ds0 + ((size_t)tb.slot_cons_seq[c0] * H + h) * elems);
+    auto of = [&](int u) { return reinterpret_cast<float4*>(ds0 + ((size_t)tb.slot_cons_seq[u] * H + h) * elems); };
+    float4* dst = of(c0);
     for (int e = blockIdx.z * 256 + threadIdx.x; e < elems / 4; e += gridDim.z * 256) {
         float4 acc = dst[e];
-        int u = c0 + 1;
-        for (; u + 3 < c1; u += 4) {              // four independent loads in flight
-            float4 v[4];
+        if (run == 1 || summed) {                     // one after the other, or the runs' sums: four independent loads in flight
+            auto next = [&](int u) { return (u / run + 1) * run; };
+            for (int u = next(c0); u < c1;) {
+                float4 v[4];
+                int n = 0;
 #pragma unroll
-            for (int i = 0; i < 4; i++)
-                v[i] = reinterpret_cast<const float4*>(ds0 + ((size_t)tb.slot_cons_seq[u + i] * H + h) * elems)[e];
+                for (int i = 0; i < 4; i++)
+                    if (u < c1) {
+                        v[i] = of(u)[e];
+                        u = next(u);
+                        n++;
+                    }
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w;
+                for (int i = 0; i < 4; i++)
+                    if (i < n) acc.x += v[i].x, acc.y += v[i].y, acc.z += v[i].z, acc.w += v[i].w;
             }
-        }
-        for (; u < c1; u++) {
-            const float4 v = reinterpret_cast<const float4*>(ds0 + ((size_t)tb.slot_cons_seq[u] * H + h) * elems)[e];
-            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        } else {                                      // run by run
+            float4 part = acc;
+            bool one = true;
+            for (int u = c0 + 1; u < c1; u++) {
+                const float4 v = of(u)[e];
+                if (u % run == 0) {
+                    acc = one ? part : make_float4(acc.x + part.x, acc.y + part.y, acc.z + part.z, acc.w + part.w);
+                    one = false;
+                    part = v;
+                } else {
+                    part.x += v.x, part.y += v.y, part.z += v.z, part.w += v.w;
+                }
+            }
+            acc = one ? part : make_float4(acc.x + part.x, acc.y + part.y, acc.z + part.z, acc.w + part.w);
         }
         dst[e] = acc;
     }
 }
 
-int32_t handoff_reduce(const BwdArgs& a) {
+int32_t handoff_reduce(const BwdArgs& a, int run) {
     if (a.tb.n_slots == 0 || a.seq_hi == a.seq_lo) return HARTS_OK;
     ScratchLayout sl = scratch_layout(a.tb, a.H, a.dk, a.dv);
     float* ds0 = reinterpret_cast<float*>(static_cast<char*>(a.scratch) + sl.ds0);
     const int elems = a.dk * a.dv;
     dim3 grid(a.tb.n_slots, a.H, (elems / 4 + 1023) / 1024);
-    handoff_reduce_kernel<<<grid, 256, 0, a.stream>>>(a.tb, a.seq_lo, a.seq_hi, a.H, elems, ds0,
+    handoff_reduce_kernel<<<grid, 256, 0, a.stream>>>(a.tb, a.seq_lo, a.seq_hi, a.H, elems, ds0, run, a.runs_below,
                                                       status_gate(a.flags, a.dev_status));
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }

@@ -4,8 +4,9 @@
 // accumulation).  Two ways to drive them.  The walks hold the running state S (forward) / its gradient dS (backward) in the
 // accumulator registers of the CTA's sixteen warps over a whole sequence, which is what register accumulators are for.  The chunk
 // kernels take every (chunk, head) on its own, with S and dS from memory (la_scan.cu); they share the walks' code for the inside
-// of a chunk and hold no state, so nothing but that ties them to mma.sync: 17 us per item of the backward on one CTA per SM,
-// where its 240 KB of traffic would take 5.6.  What cannot be a dense product stays on the CUDA cores in fp32: the
+// of a chunk and hold no state, so nothing but that ties them to mma.sync: 15 us per item of the backward on one CTA per SM,
+// where its 240 KB of traffic would take 5.6; the shared memory's port is busy for two thirds of it (operand tiles that ldmatrix reads
+// four times over: 14.4 k wavefronts an item).  What cannot be a dense product stays on the CUDA cores in fp32: the
 // decay-dependent pair sums
 //     A_tj      = sum_i q_t[i] k_j[i] e^{b_t[i]-b_j[i]}                          (j <= t)
 //     dq_t[i]  += sum_{j<=t} dA_tj k_j[i] e^{b_t[i]-b_j[i]},   dk_j[i] += sum_{t>=j} dA_tj q_t[i] e^{b_t[i]-b_j[i]}
@@ -736,7 +737,8 @@ gk_mma_fwd_kernel(harts_la_tables_t tb, int seq_lo, int H, const __nv_bfloat16* 
 // thread.  To fit, everything is worked on in place or over something dead: the running sums' scratch lies under the
 // scores, k becomes the keys anchored at their own block, q becomes q~, V comes in over the anchored queries once the
 // scores are done, the state over the running sums.  One pass over q and k makes all four operands of a mild chunk.
-// Measured, 1,047 chunks x 16 heads: 0.80 ms cold, 0.78 warm (one CTA per SM with every tile in a place of its own: 1.08).
+// Measured, 1,047 chunks x 16 heads, cold: 0.57 ms (0.78 with loads by cp.async and running sums laid out plainly; one CTA per SM with every
+// tile in a place of its own 1.08).
 struct SharedC {
     static constexpr int q = 0, k = 16384;                              // bf16 [64][128]; then q~, keys anchored at their block
     static constexpr int b = 32768;                                     // fp32 [64][128] running log-decay; then the state

@@ -16,13 +16,13 @@
 // MMA warp, the state warps, and a store warp (TMA).  A (sequence, head) is one item of NV = 128 state columns, or 2 of 64,
 // or 4 of 32 (launch_sliced): the columns do not interact, so the split does not change any result.  All rounds run in one
 // launch (scan_fwd below).
-// Measured, cold inputs: 1.05 us per step of the longest path while the chains leave SMs idle, 1.05 to 1.3 backward (17,695 tokens x
-// 4 heads, 68 steps: 72 and 71 us; 65,521 x 16, 228 steps: 244 and 294); with 96 chains of 100,003 tokens x 16 heads 4.9 TB/s
+// Measured, cold inputs: 0.8 us per step of the longest path while the chains leave SMs idle, 0.85 backward, and 1.5 us from a sequence to the
+// one that starts from it (17,695 tokens x 4 heads, 68 steps and three such: 65 us each way; 72 and 71 with table entries loaded when
+// they were needed, slots written 16 bytes at a time and a step's waits one after the other); with 96 chains of 100,003 tokens x 16 heads 4.9 TB/s
 // forward (345 us), 6.1 backward (470 us).
-// Log-decays per channel: 1.4 us a step forward, 1.5 backward (1,047 agentic chunks x 16 heads 408 and 470 us).  The weighting warps are
-// what a step waits for: with a's values read one by one between the stores, which a load may not pass, 1.6 and 1.75 us; and an item
-// whose first chunk has replayed rows began 12 us after its start state was there while a warp copied them with half its lanes, and the
-// gates 16 bytes at a time (454 and 539 us).
+// Log-decays per channel: 1.3 us a step forward, 1.4 backward (1,047 agentic chunks x 16 heads 367 and 413 us), the weighting warps' chain.
+// 454 and 539 us with a's values read one by one between the stores, which a load may not pass, with a warp that copied the rows of a first
+// chunk by half its lanes and the gates 16 bytes at a time (12 us an item), and with two stages of rows where three fit (406 and 471).
 #include <type_traits>
 
 #include "kernels.h"
@@ -653,10 +653,10 @@ int32_t launch(const Launch& x) {
 }
 // The narrower the slices, the shorter a step of the walk and the more often k is read: as narrow as leaves the chains of the
 // (first) round at most one CTA per SM, but never 128 columns in the backward, where a state thread multiplies its columns with
-// S_c besides.  Device time in us with 32 / 64 / 128 columns, cold inputs (before slots were published by the store warp and
-// gradients read coalesced: 72 and 71 now where 78 and 82 stand): 17,695 tokens x 4 heads (4 chains in
-// the first round) forward 78 / 93 / 141, backward 82 / 86 / 187; 65,521 x 16 (64 chains) 298 / 244 / 289, 406 / 293 / 451;
-// 100,003 x 16 (96 chains) 426 / 359 / 345, 606 / 468 / 561; 149,270 x 12 (96 chains) forward 64: 401, 128: 400, backward 546, 573.
+// S_c besides.  Device time in us with 32 / 64 / 128 columns, cold inputs, as they were when the line was drawn (a step is shorter now with
+// any of them): 17,695 tokens x 4 heads (4 chains in the first round) forward 78 / 93 / 141, backward 82 / 86 / 187; 65,521 x 16 (64 chains)
+// 298 / 244 / 289, 406 / 293 / 451; 100,003 x 16 (96 chains) 426 / 359 / 345, 606 / 468 / 561; 149,270 x 12 (96 chains) forward 64: 401,
+// 128: 400, backward 546, 573.
 template <bool BWD>
 int32_t launch_sliced(const Launch& x) {
     const int chains = (x.order.n ? x.order.ptr[1] - x.order.ptr[0] : x.seq_hi - x.seq_lo) * x.H;

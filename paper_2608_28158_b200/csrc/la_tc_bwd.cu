@@ -81,6 +81,7 @@ struct Misc {
     SeqInfo seq;
     // one launch per round: the next work item, looked up by the auxiliary warp under the last chunk of this one
     int next_head, next_id, id;
+    int next_to, to, next_add, add;      // where the gradient of the initial state goes: sequence, and whether it is added to what is there
     SeqInfo next_seq;
 };
 
@@ -146,7 +147,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
               const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ g,
               const __nv_bfloat16* __restrict__ dO, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk_,
               __nv_bfloat16* __restrict__ dv_, float* __restrict__ dg, float* __restrict__ ds0, float* __restrict__ rk,
-              float* __restrict__ rv, float* __restrict__ rg, int* status, const int32_t* gate, int* ds0_flags,
+              float* __restrict__ rv, float* __restrict__ rg, int run_lo, int run_hi, int* status, const int32_t* gate, int* ds0_flags,
               int* ticket, const RoundOrder rounds) {
     if (gate_closed(gate)) return;
     extern __shared__ unsigned char smem_raw[];
@@ -165,7 +166,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool is_compute = warp < NC / 32;
     const bool is_issuer = tid == NC;              // first lane of the issuing warp: TMA
-    const bool is_mma = warp == NC / 32;           // the issuing warp: MMAs, by an elected lane (operands in uniform registers)
+    const bool is_mma = warp == NC / 32;           // the issuing warp: MMAs, by an elected lane
     const bool is_aux = warp == NC / 32 + 1;       // row data of the next chunk, dg of the finished one
     const int grp = warp >> 2;                    // column group (compute warps)
     const int L = (warp & 3) * 32 + lane;         // tensor-memory lane = feature index (or row t) of this thread
@@ -197,6 +198,33 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     const int G = gridDim.x;
     // one launch per round: item of a tier; n_items or more: none
     auto dealt = [&](int tier) { return (tier & 1) ? tier * G + (G - 1 - (int)blockIdx.x) : tier * G + (int)blockIdx.x; };
+    // In runs (BwdArgs::run_lo): a CTA takes the consumers of a run one after the other and adds their gradients up where the first one's
+    // lies.  An item is then position in slot_cons_seq * H + head, else sequence * H + head; -1: none.
+    const bool runs = !ONE_LAUNCH && run_hi > 0;
+    auto first_of = [&](int tier_) {
+        const int u = dealt(tier_);
+        if (!runs) return u < n_items ? u : -1;
+        const int run = run_lo / HANDOFF_RUN + u / H;
+        return run * HANDOFF_RUN < run_hi ? max(run_lo, run * HANDOFF_RUN) * H + u % H : -1;
+    };
+    auto in_run = [&](int item_) {                 // the next item is of the same run
+        const int at = item_ / H + 1;
+        return runs && at < run_hi && at % HANDOFF_RUN != 0;
+    };
+    auto item_after = [&](int item_, int tier_) { return in_run(item_) ? item_ + H : first_of(tier_ + 1); };
+    auto seq_of = [&](int item_) {
+        const int pos = item_ / H;
+        return runs ? tb.slot_cons_seq[pos] : tb.seq_order ? tb.seq_order[seq_lo + pos] : seq_lo + pos;
+    };
+    auto target = [&](int item_, const SeqInfo& sq, int id, int& to, int& add) {
+        to = id;
+        add = 0;
+        if (!runs) return;
+        const int at = item_ / H, lead = max(tb.slot_cons_ptr[sq.init_slot], at / HANDOFF_RUN * HANDOFF_RUN);
+        to = tb.slot_cons_seq[lead];
+        add = at != lead;
+    };
+    int item_next = ONE_LAUNCH ? 0 : first_of(0), tier_next = 0;
     int cur = 0;                                   // which of the two records of row data the current chunk reads
     for (int tier = 0;; tier++) {
     // The order of one launch per round is known beforehand: the auxiliary warp looks up the next sequence and prepares its
@@ -204,8 +232,8 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
     // the switch, those are four dependent trips to memory (3,000 of the 23,500 cycles of a replayed tail of one or two chunks)
     // with nothing else in flight: 6,949 chunks of such tails x 16 heads 6.7 -> 6.32 ms, 6.22 with the L2 asked.  A ticket
     // (all rounds in one launch) is still drawn at the switch: held early, it would keep an item from a CTA that is free.
-    const bool ahead = !ONE_LAUNCH && tier > 0;
-    int item, seq_pos = 0;
+    const bool ahead = !ONE_LAUNCH && tier > 0;      // (tier counts items)
+    int item, seq_pos = 0, item_tier = 0;
     if constexpr (ONE_LAUNCH) {
         // all rounds in one launch: whichever CTA is free draws the next item; the order is last round first, and
         // inside a round the plan's order (longest sequence first)
@@ -222,10 +250,11 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             else j -= cnt;
         }
     } else {
-        if (tier * G >= n_items) break;
-        item = dealt(tier);
-        if (item >= n_items) continue;
-        seq_pos = seq_lo + item / H;
+        item = item_next;
+        if (item < 0) break;
+        item_tier = tier_next;
+        tier_next += !in_run(item);
+        item_next = item_after(item, item_tier);
     }
     // the item's record lives in shared memory and is read where it is needed: held in registers over the whole walk it
     // would push the kernel over its register budget
@@ -235,11 +264,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             m.seq = m.next_seq;
             m.head = m.next_head;
             m.id = m.next_id;
+            m.to = m.next_to;
+            m.add = m.next_add;
         } else {
-            const int id = tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
+            const int id = !ONE_LAUNCH ? seq_of(item) : tb.seq_order ? tb.seq_order[seq_pos] : seq_pos;
             m.seq = seq_info(tb, id);
             m.head = item % H;
             m.id = id;
+            target(item, m.seq, id, m.to, m.add);
         }
     }
     __syncthreads();
@@ -345,6 +377,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
     };
 
+    int stored = 0;                                // this item's full chunks so far (the issuing thread's)
     const bool gather_first = s.n_replay > 0;
     int next_req = s.req_hi - 1;
     // chunk index of the next exported boundary on the way down (kept in a register: no global load per chunk)
@@ -411,12 +444,13 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             if (ONE_LAUNCH || c > 0) {
                 load_rows(s, h, c - 1, nx_code, nx_g);    // next chunk's rows and g, in flight during this chunk
                 if (c == 1 && gather_first) warm_rows(h, nx_code);
-            } else if (const int next = dealt(tier + 1); next < n_items) {
+            } else if (const int next = item_next; next >= 0) {
                 if (lane == 0) {
-                    const int id = tb.seq_order ? tb.seq_order[seq_lo + next / H] : seq_lo + next / H;
+                    const int id = seq_of(next);
                     m.next_seq = seq_info(tb, id);
                     m.next_head = next % H;
                     m.next_id = id;
+                    target(next, m.next_seq, id, m.next_to, m.next_add);
                 }
                 __syncwarp();
                 load_rows(m.next_seq, m.next_head, m.next_seq.n_chunks - 1, nx_code, nx_g);
@@ -474,11 +508,20 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                         float4 a;
                         if constexpr (ONE_LAUNCH) {       // written during this launch by other CTAs: read past L1
                             a = __ldcg(first + i4);
+                            float4 sum;               // of the runs behind the present one
+                            bool one = true;
                             for (int u = cons_lo + 1; u < cons_hi; u++) {
                                 const float4 b4 = __ldcg(reinterpret_cast<const float4*>(
                                     ds0 + ((size_t)tb.slot_cons_seq[u] * H + h) * state_elems + in_state) + i4);
-                                a.x += b4.x; a.y += b4.y; a.z += b4.z; a.w += b4.w;
+                                if (u % HANDOFF_RUN == 0) {
+                                    sum = one ? a : make_float4(sum.x + a.x, sum.y + a.y, sum.z + a.z, sum.w + a.w);
+                                    one = false;
+                                    a = b4;
+                                } else {
+                                    a.x += b4.x; a.y += b4.y; a.z += b4.z; a.w += b4.w;
+                                }
                             }
+                            if (!one) a = make_float4(sum.x + a.x, sum.y + a.y, sum.z + a.z, sum.w + a.w);
                         } else {
                             a = first[i4];
                         }
@@ -607,7 +650,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
             }
             __syncwarp();
         }
-        if (is_aux && (c > 0 || (!ONE_LAUNCH && dealt(tier + 1) < n_items))) store_rows(m.rows[cur ^ 1], nx_code, nx_g);   // visible to the others at barrier (B)
+        if (is_aux && (c > 0 || (!ONE_LAUNCH && item_next >= 0))) store_rows(m.rows[cur ^ 1], nx_code, nx_g);   // visible to the others at barrier (B)
         if (is_compute) {
             const int c4 = lane & 3, Lq = (warp & 3) * 32, t0 = grp * 16;
             Frag fr;
@@ -738,6 +781,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
                 tma_store_3d(&map_dv, smem + Smem::stage_dv + p * PANEL, p * 64, h, row0);
             }
             tma_store_commit();
+            stored++;
         }
         if (is_aux) {
             // dg_t = sum_{tau >= t} r_tau + <S_{c+1}, dS_{c+1}>, rows `lane` and `lane + 32` per thread of this warp
@@ -788,7 +832,14 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
         }
         __syncthreads();
         if (is_issuer) {
-            for (int p = 0; p < 4; p++) tma_store_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, m.id * H + h);
+            if (m.add) {                          // the run's sum so far is in memory: what came behind it is this item's full chunks
+                if (stored == 0) tma_store_wait_all();
+                else if (stored == 1) tma_store_wait_group<1>();
+                else tma_store_wait_group<2>();
+            }
+            for (int p = 0; p < 4; p++)
+                if (m.add) tma_add_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, m.to * H + h);
+                else tma_store_3d(&map_ds0, sS + p * S_PANEL, p * 32, 0, m.to * H + h);
             tma_store_commit();
         }
     }
@@ -830,7 +881,7 @@ tc_bwd_kernel(const harts_la_tables_t tb, int seq_lo, int n_items, int H, const 
 
 int32_t tc_bwd(const BwdArgs& a) {
     if (a.seq_hi == a.seq_lo) return HARTS_OK;
-    if (int32_t rc0 = handoff_reduce(a); rc0 != HARTS_OK) return rc0;
+    if (int32_t rc0 = handoff_reduce(a, HANDOFF_RUN); rc0 != HARTS_OK) return rc0;
     CUtensorMap mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mds0;
     int32_t rc;
     if ((rc = make_row_map(&mq, a.q, a.tb.n_rows, a.H)) != HARTS_OK) return rc;
@@ -853,7 +904,7 @@ int32_t tc_bwd(const BwdArgs& a) {
         a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mds0, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_,
         (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
-        (float*)(base + sl.rg), a.dev_status, status_gate(a.flags, a.dev_status), nullptr, nullptr, RoundOrder{});
+        (float*)(base + sl.rg), a.run_lo, a.run_hi, a.dev_status, status_gate(a.flags, a.dev_status), nullptr, nullptr, RoundOrder{});
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
@@ -897,7 +948,7 @@ int32_t tc_bwd_fused(const BwdArgs& a, int* flags, int* ticket, const RoundOrder
         a.tb, a.seq_lo, n, a.H, mq, mk, mv, mdo, mcs, mdq, mdk, mdv, mdv, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
         (const __nv_bfloat16*)a.v, a.g, (const __nv_bfloat16*)a.dO, (__nv_bfloat16*)a.dq, (__nv_bfloat16*)a.dk_,
         (__nv_bfloat16*)a.dv_, a.dg, (float*)(base + sl.ds0), (float*)(base + sl.rk), (float*)(base + sl.rv),
-        (float*)(base + sl.rg), a.dev_status, status_gate(a.flags, a.dev_status), flags, ticket, rounds);
+        (float*)(base + sl.rg), 0, 0, a.dev_status, status_gate(a.flags, a.dev_status), flags, ticket, rounds);
     return cudaGetLastError() == cudaSuccess ? HARTS_OK : HARTS_ECUDA;
 }
 
